@@ -304,6 +304,16 @@ int lob_reset(lob_engine* e);
  *                  delta row alone (same generation: children(a) x
  *                  children(b)) whose new facts only set bitmap bits runs
  *                  as one fused cross-product step; 0: two steps    (default 1)
+ *   "bit_matrix"   1: under LOB_UNIT, a program whose derived relations are
+ *                  binary and whose rules link their body atoms into a chain
+ *                  from one head variable to the other runs on bit matrices
+ *                  over the values that occur (up to about 92,000 of them; no
+ *                  sample ids), provided that packed_join, warp_join,
+ *                  bitmap_delta, emit_filter, cross_join, join_index,
+ *                  sort_algo and max_candidates (2^30 or more) are at their
+ *                  defaults, which ask for no other strategy; 0: never.  The
+ *                  relations and the statistics of the iterations are the
+ *                  same either way                                  (default 1)
  *   "packed_backward" 1: the diff-add-mult backward pass replays packed join
  *                  pipelines on the packed kernels (binding words plus the
  *                  rows of the facts matched so far); 0: every arm on the

@@ -1,0 +1,1497 @@
+// Bit-matrix fixpoint of chain programs (unit semiring).
+//
+// A chain program is one whose derived relations are binary and whose rules
+// link their body atoms into a path from one head variable to the other --
+//   path(x,z) :- path(x,y), edge(y,z).
+//   sg(x,y)   :- parent(a,x), sg(a,b), parent(b,y).
+//   pt(r,o)   :- store(p,q), pt(p,r), pt(q,o).
+// Each rule is then a product of boolean matrices, an atom read against its
+// column order being the transpose.  A derived relation is kept as a bit matrix
+// over the values that occur in the program's relations (renumbered in order, so
+// that row-major bit order is the relation's key order) and an input relation as
+// compressed rows.  Rows of a bit matrix are combined 128 bits a lane, so one
+// instruction derives up to 4,096 candidates of a warp; the general path spends
+// an atomic (or a sort of 8 bytes) on each.  Algorithm 1 is unchanged: an
+// iteration evaluates every semi-naive arm on the facts the previous one left
+// (recent set D, full set F), and D' = N & ~F, F |= D' ends it.
+//
+// What bounds it: reading the operand rows, out of L2 (the matrices of the
+// benchmark's closure are 50 MB each), then the read-out of the result.
+//
+// Products are evaluated from the right: U = M_m, U = M_i U for i = m-1 .. 1.
+//   gather   M_i x bits: row r = OR of the rows of U listed in row r of M_i
+//   scatter  M_i x compressed rows: row r is built in shared memory, one
+//            shared atomic OR per derivation
+// The derived relations are stored transposed when that turns scatters into
+// gathers (bit_eligible's rule): a left-recursive closure reads as E' P'.
+//
+// Measured (GB300, fixpoint only, general path before -> bit matrices): closure
+// of the 20,000-node / 100,000-edge power-law graph 11.9 -> 1.6 ms; same
+// generation on a 50,000-node tree 22.6 -> 8.8 ms; points-to on 400,000
+// statements (8.7e9 derivations of 1.8e6 facts, 36-bit keys: sorted before)
+// 418 -> 2.9 ms; closure of 1,000 nodes / 3,000 edges 0.99 -> 0.45 ms.
+#include "bitmat.h"
+
+#include <algorithm>
+#include <cstring>
+
+#include "engine.h"
+#include "scan.cuh"
+
+namespace {
+
+constexpr int kMaxChain = 4;       // body atoms of a chain rule
+constexpr int kMaxBitRels = 16;    // relations the state block holds sizes of
+constexpr u32 kHeavyRow = 512;     // compressed rows longer than this are gathered by a whole block
+constexpr u64 kMatrixBytes = 1ull << 30;  // largest bit matrix (92,000 values): beyond it sparse facts cost too much
+constexpr u64 kMaxValue = 1ull << 28;     // largest id the renumbering's presence bitmap covers
+
+// state block: done flag (1 fixpoint, 2 max_iters), iterations run, new facts
+// of all iterations, derivations, words read (profiling), then per relation
+// |F|, |D| and this iteration's new facts
+enum : int { B_DONE = 0, B_ITER, B_NEW, B_CAND, B_WORDS, B_REL = 8 };
+LOB_HD int rel_slot(int r, int f) { return B_REL + 3 * r + f; }
+constexpr int kStateSlots = B_REL + 3 * kMaxBitRels;
+// ... and, not read back, two list lengths for each of an iteration's products
+constexpr int kMaxLists = 32;
+constexpr int kAllSlots = kStateSlots + 2 * kMaxLists;
+
+enum IndexKind { I_IDENT = 0, I_CSR = 1, I_BITS = 2 };
+
+// A bit matrix.  Row r is empty, whatever its words hold, when cnt[r] (bag[r]
+// when bag is set) is 0.  bag[r]: the derivations row r stands for, duplicates
+// included (a stored relation's is its facts, cnt).
+struct BMat {
+  const u32* bits;
+  const u32* cnt;
+  const u64* bag;
+  LOB_DEV u64 weight(u32 r) const { return bag ? bag[r] : (u64)cnt[r]; }
+};
+struct BCsr {
+  const u32* ptr;
+  const u32* col;
+  const u32* heavy;    // rows longer than kHeavyRow
+  const u32* n_heavy;
+};
+
+struct BOp {
+  u32 rows, words;     // rows, words per row (a multiple of 4)
+  BCsr ic;             // index matrix M_i
+  BMat ib;
+  BCsr mc;             // operand U
+  BMat mb;
+  const u32* need;     // rows of the result that a later product reads (null: all)
+  // listed form: only the result rows some index entry gives anything to, as
+  // k_bit_active found them (long compressed rows apart); null: every row
+  u32* list;
+  u32* hlist;
+  u64* n_list;         // [0] rows listed, [1] long rows listed
+  // result: a temporary (out, obag) ...
+  u32* out;
+  u64* obag;
+  // ... or the head's accumulator N (flagged rows hold something) ...
+  u32* acc;
+  u32* aflag;
+  int diag;            // 0: all, 1: x != z, 2: x == z
+  // ... or, as the iteration's last product into it, straight D' and F
+  int commit;
+  u32* full;
+  u32* next;
+  u32* ncnt;
+  u32* fcnt;
+  u64* n_new;
+  u64* state;
+  int n_skip;          // the arm is skipped when one of these relations has no old facts
+  int skip[kMaxChain];
+};
+
+LOB_DEV bool op_idle(const BOp& P) {
+  if (P.state[B_DONE]) return true;
+  for (int i = 0; i < P.n_skip; i++)
+    if (P.state[rel_slot(P.skip[i], 0)] == P.state[rel_slot(P.skip[i], 1)]) return true;
+  return false;
+}
+
+LOB_DEV void or4(uint4& a, const uint4& b) {
+  a.x |= b.x; a.y |= b.y; a.z |= b.z; a.w |= b.w;
+}
+LOB_DEV bool any4(const uint4& a) { return (a.x | a.y | a.z | a.w) != 0u; }
+LOB_DEV u32 popc4(const uint4& a) { return __popc(a.x) + __popc(a.y) + __popc(a.z) + __popc(a.w); }
+
+// the rule's filter on the words [w, w + 4) of row r
+LOB_DEV void diag4(uint4& a, int diag, u32 r, u32 w) {
+  if (!diag) return;
+  u32 m[4] = {0, 0, 0, 0};
+  if ((r >> 5) >= w && (r >> 5) < w + 4) m[(r >> 5) - w] = 1u << (r & 31u);
+  if (diag == 1) {
+    a.x &= ~m[0]; a.y &= ~m[1]; a.z &= ~m[2]; a.w &= ~m[3];
+  } else {
+    a.x &= m[0]; a.y &= m[1]; a.z &= m[2]; a.w &= m[3];
+  }
+}
+
+// The words [w, w + 4) of result row r go where the product's result goes;
+// returns the new facts among them (commit).
+LOB_DEV u32 put4(const BOp& P, u32 r, u32 w, uint4 a) {
+  const u64 at = ((u64)r * P.words + w) / 4;
+  if (P.out) {
+    reinterpret_cast<uint4*>(P.out)[at] = a;
+    return 0;
+  }
+  diag4(a, P.diag, r, w);
+  if (!P.commit) {
+    if (any4(a)) {
+      uint4* N = reinterpret_cast<uint4*>(P.acc) + at;
+      or4(a, *N);
+      *N = a;
+      P.aflag[r] = 1;
+    }
+    return 0;
+  }
+  if (P.aflag && P.aflag[r]) {
+    uint4* N = reinterpret_cast<uint4*>(P.acc) + at;
+    or4(a, *N);
+    *N = make_uint4(0, 0, 0, 0);
+  }
+  uint4* F = reinterpret_cast<uint4*>(P.full) + at;
+  uint4 f = *F;
+  a.x &= ~f.x; a.y &= ~f.y; a.z &= ~f.z; a.w &= ~f.w;
+  reinterpret_cast<uint4*>(P.next)[at] = a;
+  if (any4(a)) {
+    or4(f, a);
+    *F = f;
+  }
+  return popc4(a);
+}
+
+LOB_DEV void count_new(const BOp& P, u32 r, u32 fresh) {
+  if (!fresh) return;
+  atomicAdd(P.ncnt + r, fresh);
+  atomicAdd(P.fcnt + r, fresh);
+}
+
+// derivations, words read and new facts of a block's threads, one atomic each
+LOB_DEV void block_totals(const BOp& P, u64 cand, u64 words, u64 fresh) {
+  __shared__ u64 tot[3];
+  if (threadIdx.x < 3) tot[threadIdx.x] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    cand += __shfl_xor_sync(0xFFFFFFFFu, cand, o);
+    words += __shfl_xor_sync(0xFFFFFFFFu, words, o);
+    fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (cand) atomicAdd(reinterpret_cast<unsigned long long*>(&tot[0]), cand);
+    if (words) atomicAdd(reinterpret_cast<unsigned long long*>(&tot[1]), words);
+    if (fresh) atomicAdd(reinterpret_cast<unsigned long long*>(&tot[2]), fresh);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long* s = reinterpret_cast<unsigned long long*>(P.state);
+    if (tot[0] && !P.out) atomicAdd(s + B_CAND, tot[0]);
+    if (tot[1]) atomicAdd(s + B_WORDS, tot[1]);
+    if (tot[2]) atomicAdd(reinterpret_cast<unsigned long long*>(P.n_new), tot[2]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// gather: row r of the result = OR of the operand rows listed in row r of the
+// index matrix.
+// A task is 128 words of a result row.  Compressed index rows: a warp a task
+// (an average row of the benchmark's graph lists five operand rows), and a
+// block a task for rows of more than kHeavyRow entries, whose hub of 5,000
+// would otherwise keep one warp busy long after the rest have finished.  Bit
+// index rows: a block a task, its warps sharing the words of the index row.
+// Rows narrower than 128 words leave lanes over: lanes are split into groups of
+// the row's width, each taking other operand rows, and ORed together at the end.
+// Entries whose operand row is empty are dropped first (a ballot), so an
+// iteration with few recent rows reads few words.
+// ---------------------------------------------------------------------------
+constexpr int kGatherWarps = 8;
+constexpr int kListCap = 64;
+
+struct Lanes {  // how the 32 lanes split over a task's words
+  int group;    // lanes per operand row (a power of two)
+  int sub, n_sub;
+  u32 w;        // this lane's first word of the row
+  bool in;
+};
+LOB_DEV Lanes split_lanes(u32 words, u32 chunk) {
+  const int lane = threadIdx.x & 31;
+  const u32 left = words - chunk * 128;
+  int g = 32;
+  while (g > 1 && (u32)(g / 2) * 4 >= left) g >>= 1;
+  Lanes L;
+  L.group = g;
+  L.sub = lane / g;
+  L.n_sub = 32 / g;
+  L.w = chunk * 128 + (u32)(lane % g) * 4;
+  L.in = L.w < words;
+  return L;
+}
+
+// acc |= the words of the n operand rows listed in shared memory
+LOB_DEV void gather_list(const BMat& M, u32 words, const Lanes& L, const u32* list, int n, uint4& acc) {
+  if (!L.in) return;
+  const uint4* base = reinterpret_cast<const uint4*>(M.bits + L.w);
+  const u64 stride = words / 4;
+  int k = L.sub;
+  for (; k + 3 * L.n_sub < n; k += 4 * L.n_sub) {  // four rows in flight
+    const uint4 a = base[list[k] * stride], b = base[list[k + L.n_sub] * stride];
+    const uint4 c = base[list[k + 2 * L.n_sub] * stride], d = base[list[k + 3 * L.n_sub] * stride];
+    or4(acc, a); or4(acc, b); or4(acc, c); or4(acc, d);
+  }
+  for (; k < n; k += L.n_sub) or4(acc, base[list[k] * stride]);
+}
+
+LOB_DEV void or_groups(const Lanes& L, uint4& a) {
+  for (int o = L.group; o < 32; o <<= 1) {
+    a.x |= __shfl_xor_sync(0xFFFFFFFFu, a.x, o);
+    a.y |= __shfl_xor_sync(0xFFFFFFFFu, a.y, o);
+    a.z |= __shfl_xor_sync(0xFFFFFFFFu, a.z, o);
+    a.w |= __shfl_xor_sync(0xFFFFFFFFu, a.w, o);
+  }
+}
+
+// add one warp's batch of up to 32 candidate operand rows (idx, valid) to its
+// list, reading them once the list holds 32 or more; n entries are pending
+LOB_DEV void push_batch(const BMat& M, u32 words, const Lanes& L, u32* list, int& n, u32 idx, bool valid, bool count,
+                        u64& bag, u64& read, uint4& acc, bool& any) {
+  const u64 wgt = valid ? M.weight(idx) : 0ull;
+  const bool act = wgt != 0;
+  if (count) bag += wgt;
+  const u32 m = __ballot_sync(0xFFFFFFFFu, act);
+  if (!m) return;
+  any = true;
+  const int lane = threadIdx.x & 31;
+  if (act) list[n + __popc(m & ((1u << lane) - 1u))] = idx;
+  n += __popc(m);
+  __syncwarp();
+  if (n >= kListCap - 32) {
+    gather_list(M, words, L, list, n, acc);
+    if (lane == 0) read += (u64)n * (u64)min(128u, words);
+    n = 0;
+    __syncwarp();
+  }
+}
+LOB_DEV void flush_list(const BMat& M, u32 words, const Lanes& L, u32* list, int& n, u64& read, uint4& acc) {
+  if (n) {
+    gather_list(M, words, L, list, n, acc);
+    if ((threadIdx.x & 31) == 0) read += (u64)n * (u64)min(128u, words);
+  }
+  n = 0;
+  __syncwarp();
+}
+
+// store a task's combined words; row r of a temporary always gets its weight
+LOB_DEV u32 finish_task(const BOp& P, const Lanes& L, u32 r, bool count, const uint4& acc, bool any, u64 bag) {
+  if (P.out && count && (threadIdx.x & 31) == 0) P.obag[r] = any ? bag : 0ull;
+  const bool flagged = P.commit && P.aflag && P.aflag[r];
+  if (!any && !flagged) return 0;
+  u32 fresh = 0;
+  if (L.in && L.sub == 0) fresh = put4(P, r, L.w, acc);
+  if (P.commit) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
+    if ((threadIdx.x & 31) == 0) {
+      count_new(P, r, fresh);
+      return fresh;
+    }
+  }
+  return 0;
+}
+
+LOB_DEV u64 warp_total(u64 v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+
+// The result rows a product has work for, a lane a row: rows with a non-empty
+// operand row (compressed index; their derivations are summed on the way) or a
+// non-empty index row (bits), and rows whose accumulator waits for the commit.
+// Large matrices only: there most rows have nothing to do in most iterations
+// (a level of same generation is a twelfth of the tree), and visiting all rows
+// x chunks of a 50,000-value matrix takes 100 us where the list takes 5.
+template <int IK>
+__global__ void __launch_bounds__(256) k_bit_active(const __grid_constant__ BOp P, int operand_bits) {
+  if (op_idle(P)) return;
+  const int lane = threadIdx.x & 31;
+  const u64 nwarps = (u64)gridDim.x * 8;
+  u64 cand = 0;
+  for (u64 r0 = ((u64)blockIdx.x * 8 + (threadIdx.x >> 5)) * 32; r0 < P.rows; r0 += nwarps * 32) {
+    const u32 r = (u32)r0 + lane;
+    const bool in = r < P.rows;
+    bool live = in && (!P.need || P.need[r]);
+    u64 bag = 0;
+    u32 len = 0;
+    if constexpr (IK == I_BITS) {
+      live = live && P.ib.weight(r) != 0;
+    } else {
+      u32 j0 = 0;
+      if constexpr (IK == I_CSR) {
+        if (live) {
+          j0 = P.ic.ptr[r];
+          len = P.ic.ptr[r + 1] - j0;
+        }
+      } else {
+        len = live ? 1 : 0;
+      }
+      if (operand_bits) {
+        if (len <= 32)
+          for (u32 j = 0; j < len; j++) bag += P.mb.weight(IK == I_CSR ? P.ic.col[j0 + j] : r);
+        for (u32 m = __ballot_sync(0xFFFFFFFFu, len > 32); m; m &= m - 1) {
+          const int src = __ffs(m) - 1;
+          const u32 a = __shfl_sync(0xFFFFFFFFu, j0, src), n = __shfl_sync(0xFFFFFFFFu, len, src);
+          u64 b = 0;
+          for (u32 j = lane; j < n; j += 32) b += P.mb.weight(P.ic.col[a + j]);
+          b = warp_total(b);
+          if (lane == src) bag = b;
+        }
+        live = bag != 0;
+      } else {
+        live = len != 0 && (IK == I_CSR || P.mc.ptr[r + 1] != P.mc.ptr[r]);
+      }
+    }
+    if (in && P.out && !live) P.obag[r] = 0;
+    if (in && P.out && live && operand_bits && IK != I_BITS) P.obag[r] = bag;
+    cand += bag;
+    live = live || (in && P.commit && P.aflag && P.aflag[r]);
+    const bool heavy = live && IK == I_CSR && operand_bits && len > kHeavyRow;
+    const u32 ml = __ballot_sync(0xFFFFFFFFu, live && !heavy), mh = __ballot_sync(0xFFFFFFFFu, heavy);
+    u32 at = 0, hat = 0;
+    if (lane == 0) {
+      if (ml) at = (u32)atomicAdd(reinterpret_cast<unsigned long long*>(P.n_list), (unsigned long long)__popc(ml));
+      if (mh) hat = (u32)atomicAdd(reinterpret_cast<unsigned long long*>(P.n_list) + 1, (unsigned long long)__popc(mh));
+    }
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+    hat = __shfl_sync(0xFFFFFFFFu, hat, 0);
+    const u32 below = (1u << lane) - 1u;
+    if (heavy) P.hlist[hat + __popc(mh & below)] = r;
+    else if (live) P.list[at + __popc(ml & below)] = r;
+  }
+  block_totals(P, cand, 0, 0);
+}
+
+template <int IK>
+__global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp P) {
+  __shared__ u32 lists[kGatherWarps][kListCap];
+  __shared__ uint4 part[kGatherWarps][32];
+  __shared__ u64 pbag[kGatherWarps];
+  __shared__ u32 pany[kGatherWarps];
+  if (op_idle(P)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 chunks = (P.words + 127) / 128;
+  u32* list = lists[warp];
+  u64 cand = 0, read = 0, fresh = 0;
+  // k_bit_active has summed the derivations of listed compressed rows
+  const bool count_all = !P.list || IK == I_BITS;
+  if constexpr (IK != I_BITS) {
+    const u64 tasks = (P.list ? P.n_list[0] : (u64)P.rows) * chunks;
+    const u64 nwarps = (u64)gridDim.x * kGatherWarps;
+    for (u64 t = (u64)blockIdx.x * kGatherWarps + warp; t < tasks; t += nwarps) {
+      const u32 q = (u32)(t / chunks), chunk = (u32)(t % chunks);
+      const u32 r = P.list ? P.list[q] : q;
+      const bool count = count_all && chunk == 0;
+      const Lanes L = split_lanes(P.words, chunk);
+      uint4 acc = make_uint4(0, 0, 0, 0);
+      u64 bag = 0;
+      int n = 0;
+      bool any = false;
+      if (!P.need || P.need[r]) {
+        if constexpr (IK == I_IDENT) {
+          push_batch(P.mb, P.words, L, list, n, r, lane == 0, count, bag, read, acc, any);
+        } else {
+          const u32 j0 = P.ic.ptr[r], j1 = P.ic.ptr[r + 1];
+          if (j1 - j0 > kHeavyRow && !P.list) continue;  // below, by whole blocks
+          for (u32 j = j0; j < j1; j += 32) {
+            const bool v = j + lane < j1;
+            push_batch(P.mb, P.words, L, list, n, v ? P.ic.col[j + lane] : 0u, v, count, bag, read, acc, any);
+          }
+        }
+        flush_list(P.mb, P.words, L, list, n, read, acc);
+        or_groups(L, acc);
+      }
+      bag = warp_total(bag);
+      if (lane == 0) cand += bag;
+      fresh += finish_task(P, L, r, count, acc, any, bag);
+    }
+  }
+  if constexpr (IK != I_IDENT) {
+    const u32* rows = IK == I_CSR ? (P.list ? P.hlist : P.ic.heavy) : P.list;
+    const u64 nr = IK == I_CSR ? (P.list ? P.n_list[1] : (u64)*P.ic.n_heavy) : (P.list ? P.n_list[0] : (u64)P.rows);
+    const u64 tasks = nr * chunks;
+    for (u64 t = blockIdx.x; t < tasks; t += gridDim.x) {
+      const u32 q = (u32)(t / chunks), chunk = (u32)(t % chunks);
+      const u32 r = rows ? rows[q] : q;
+      const bool count = count_all && chunk == 0;
+      const Lanes L = split_lanes(P.words, chunk);
+      uint4 acc = make_uint4(0, 0, 0, 0);
+      u64 bag = 0;
+      int n = 0;
+      bool any = false;
+      bool live = !P.need || P.need[r];
+      if constexpr (IK == I_BITS) live = live && P.ib.weight(r) != 0;
+      if (!live) {  // the same for the whole block
+        if (warp == 0) fresh += finish_task(P, L, r, count, acc, false, 0);
+        continue;
+      }
+      if constexpr (IK == I_CSR) {
+        const u32 j0 = P.ic.ptr[r], j1 = P.ic.ptr[r + 1];
+        for (u32 j = j0 + warp * 32; j < j1; j += 256) {
+          const bool v = j + lane < j1;
+          push_batch(P.mb, P.words, L, list, n, v ? P.ic.col[j + lane] : 0u, v, count, bag, read, acc, any);
+        }
+      } else {
+        const u32* row = P.ib.bits + (u64)r * P.words;
+        for (u32 w0 = warp * 32; w0 < P.words; w0 += 256) {
+          const u32 mine = w0 + lane < P.words ? row[w0 + lane] : 0u;
+          for (u32 m = __ballot_sync(0xFFFFFFFFu, mine != 0u); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const u32 word = __shfl_sync(0xFFFFFFFFu, mine, src);
+            push_batch(P.mb, P.words, L, list, n, (w0 + src) * 32 + lane, (word >> lane) & 1u, count, bag, read, acc, any);
+          }
+        }
+      }
+      flush_list(P.mb, P.words, L, list, n, read, acc);
+      or_groups(L, acc);
+      bag = warp_total(bag);
+      part[warp][lane] = acc;
+      if (lane == 0) {
+        pbag[warp] = bag;
+        pany[warp] = any;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        for (int v = 1; v < kGatherWarps; v++) {
+          or4(acc, part[v][lane]);
+          bag += pbag[v];
+          any = any || pany[v];
+        }
+        if (lane == 0) cand += bag;
+        fresh += finish_task(P, L, r, count, acc, any, bag);
+      }
+      __syncthreads();  // part is rewritten by the next task
+    }
+  }
+  block_totals(P, cand, read, fresh);
+}
+
+// ---------------------------------------------------------------------------
+// scatter: row r of the result = the union of the compressed operand rows
+// listed in row r of the index matrix (identity: operand row r itself), built
+// in shared memory by one block.  Bounded by the shared atomics, one per
+// derivation, where the global ones of the general path go to L2; rows of up
+// to 92,000 values take 11.5 KB, so 8 blocks an SM stay resident.
+// ---------------------------------------------------------------------------
+LOB_DEV void set_row_bits(const BCsr& M, u32* row, u32 y, bool valid, u64& bag) {
+  u32 j0 = 0, j1 = 0;
+  if (valid) {
+    j0 = M.ptr[y];
+    j1 = M.ptr[y + 1];
+    bag += j1 - j0;
+  }
+  const bool big = j1 - j0 > 16;
+  if (!big)
+    for (u32 j = j0; j < j1; j++) {
+      const u32 c = M.col[j];
+      atomicOr(row + (c >> 5), 1u << (c & 31u));
+    }
+  const int lane = threadIdx.x & 31;
+  for (u32 m = __ballot_sync(0xFFFFFFFFu, big); m; m &= m - 1) {  // long rows: the whole warp
+    const int src = __ffs(m) - 1;
+    const u32 a = __shfl_sync(0xFFFFFFFFu, j0, src), b = __shfl_sync(0xFFFFFFFFu, j1, src);
+    for (u32 j = a + lane; j < b; j += 32) {
+      const u32 c = M.col[j];
+      atomicOr(row + (c >> 5), 1u << (c & 31u));
+    }
+  }
+}
+
+template <int IK>
+__global__ void __launch_bounds__(256) k_bit_scatter(const __grid_constant__ BOp P) {
+  extern __shared__ __align__(16) u32 row[];
+  __shared__ u64 sm[256 / 32 + 1];
+  if (op_idle(P)) return;
+  u64 cand = 0, read = 0, fresh_all = 0;
+  const u32 n_rows = P.list ? (u32)P.n_list[0] : P.rows;
+  for (u32 q = blockIdx.x; q < n_rows; q += gridDim.x) {
+    const u32 r = P.list ? P.list[q] : q;
+    bool live = !P.need || P.need[r];
+    u32 j0 = 0, j1 = 0;
+    if constexpr (IK == I_BITS) {
+      live = live && P.ib.weight(r) != 0;
+    } else {
+      const BCsr& C = IK == I_CSR ? P.ic : P.mc;
+      j0 = C.ptr[r];
+      j1 = C.ptr[r + 1];
+      live = live && j1 > j0;
+    }
+    const bool flagged = P.commit && P.aflag && P.aflag[r];
+    if (!live && !flagged) {
+      if (P.out && threadIdx.x == 0) P.obag[r] = 0;
+      continue;
+    }
+    for (u32 w = threadIdx.x; w < P.words; w += 256) row[w] = 0;
+    __syncthreads();
+    u64 bag = 0;
+    if (live) {
+      if constexpr (IK == I_IDENT) {
+        for (u32 j = j0 + threadIdx.x; j < j1; j += 256) {
+          const u32 c = P.mc.col[j];
+          atomicOr(row + (c >> 5), 1u << (c & 31u));
+          bag++;
+        }
+      } else if constexpr (IK == I_CSR) {
+        for (u32 j = j0; j < j1; j += 256) {
+          const bool v = j + threadIdx.x < j1;
+          set_row_bits(P.mc, row, v ? P.ic.col[j + threadIdx.x] : 0u, v, bag);
+        }
+      } else {
+        const u32* src = P.ib.bits + (u64)r * P.words;
+        for (u32 w0 = 0; w0 < P.words; w0 += 256) {
+          const u32 w = w0 + threadIdx.x;
+          u32 m = w < P.words ? src[w] : 0u;
+          while (__any_sync(0xFFFFFFFFu, m != 0u)) {
+            const u32 y = w * 32 + (m ? (u32)__ffs(m) - 1 : 0u);
+            set_row_bits(P.mc, row, y, m != 0u, bag);
+            m &= m - 1;
+          }
+        }
+        read += threadIdx.x == 0 ? P.words : 0;
+      }
+    }
+    u64 tot;
+    block_exclusive_sum<u64>(bag, sm, &tot);  // also the barrier before the row is read
+    if (threadIdx.x == 0) cand += tot;
+    if (P.out && threadIdx.x == 0) P.obag[r] = tot;
+    u32 fresh = 0;
+    if (!P.out || tot)
+      for (u32 w = threadIdx.x * 4; w < P.words; w += 1024) fresh += put4(P, r, w, *reinterpret_cast<const uint4*>(row + w));
+    if (P.commit) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
+      if ((threadIdx.x & 31) == 0) {
+        count_new(P, r, fresh);
+        fresh_all += fresh;
+      }
+    }
+    __syncthreads();  // the row is cleared for the next one
+  }
+  block_totals(P, cand, read, fresh_all);
+}
+
+// D' = N & ~F, F |= D' of the rows some product added to; N is cleared
+__global__ void __launch_bounds__(256) k_bit_commit(const __grid_constant__ BOp P) {
+  if (P.state[B_DONE]) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 chunks = (P.words + 127) / 128;
+  const u64 tasks = (u64)P.rows * chunks, nwarps = (u64)gridDim.x * kGatherWarps;
+  u64 fresh_all = 0, read = 0;
+  for (u64 t = (u64)blockIdx.x * kGatherWarps + warp; t < tasks; t += nwarps) {
+    const u32 r = (u32)(t / chunks);
+    if (!P.aflag[r]) continue;
+    const u32 w = (u32)(t % chunks) * 128 + lane * 4;
+    u32 fresh = w < P.words ? put4(P, r, w, make_uint4(0, 0, 0, 0)) : 0u;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
+    if (lane == 0) {
+      read += 3ull * min(128u, P.words);
+      count_new(P, r, fresh);
+      fresh_all += fresh;
+    }
+  }
+  block_totals(P, 0, read, fresh_all);
+}
+
+struct BEnd {
+  u32 rows;
+  int n_rel;
+  int rel[kMaxBitRels];
+  u32* old_cnt[kMaxBitRels];   // row counts of the recent set this iteration read: the next one writes there
+  u32* aflag[kMaxBitRels];
+  u32* tcnt[kMaxBitRels];      // row counts of its transposed copy (or null)
+  u32 max_iters;
+  u64* state;
+};
+// End of an iteration: sizes, the stop decision, cleared row counts and flags.
+// Only block 0 writes the state; a block that sees the new done flag skips
+// clearing what no later iteration reads.
+__global__ void __launch_bounds__(256) k_bit_end(const __grid_constant__ BEnd E) {
+  u64* s = E.state;
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  if (s[B_DONE]) return;
+  for (int i = 0; i < E.n_rel; i++)
+    for (u64 q = (u64)blockIdx.x * blockDim.x + threadIdx.x; q < E.rows; q += stride) {
+      E.old_cnt[i][q] = 0;
+      if (E.aflag[i]) E.aflag[i][q] = 0;
+      if (E.tcnt[i]) E.tcnt[i][q] = 0;
+    }
+  if (blockIdx.x || threadIdx.x) return;
+  u64 total = 0;
+  for (int i = 0; i < E.n_rel; i++) {
+    const int r = E.rel[i];
+    const u64 n = s[rel_slot(r, 2)];
+    s[rel_slot(r, 0)] += n;
+    s[rel_slot(r, 1)] = n;
+    s[rel_slot(r, 2)] = 0;
+    total += n;
+  }
+  for (int i = 0; i < 2 * kMaxLists; i++) s[kStateSlots + i] = 0;
+  s[B_NEW] += total;
+  s[B_ITER] += 1;
+  if (!total) s[B_DONE] = 1;
+  else if (s[B_ITER] >= E.max_iters) s[B_DONE] = 2;
+}
+
+// ---------------------------------------------------------------------------
+// transpose: 256 x 256 bits a block.  Each warp takes 32 rows, turns eight
+// 32 x 32 squares by ballots, and the block stores 32-byte pieces of 256 result
+// rows.  With `full`, the same bits are ORed into a second matrix (F' follows D').
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_bit_transpose(BMat src, u32 rows, u32 words, u32* __restrict__ dst,
+                                                       u32* __restrict__ dcnt, u32* __restrict__ full,
+                                                       u32* __restrict__ fcnt, const u64* state) {
+  __shared__ u32 tile[256][9];  // result row within the block, its 8 words (+1: no bank conflicts)
+  if (state && state[B_DONE]) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 bw = (words + 7) / 8;
+  const u64 tiles = (u64)((rows + 255) / 256) * bw;
+  for (u64 t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const u32 r0 = (u32)(t / bw) * 256, w0 = (u32)(t % bw) * 8;
+    const u32 r = r0 + warp * 32 + lane;
+    const bool live = r < rows && src.weight(r) != 0;
+    u32 x[8];
+#pragma unroll
+    for (int j = 0; j < 8; j += 4) {
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (live && w0 + j < words) v = *reinterpret_cast<const uint4*>(src.bits + (u64)r * words + w0 + j);
+      x[j] = v.x; x[j + 1] = v.y; x[j + 2] = v.z; x[j + 3] = v.w;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      u32 mine = 0;
+      if (__any_sync(0xFFFFFFFFu, x[j] != 0u)) {
+#pragma unroll
+        for (int b = 0; b < 32; b++) {
+          const u32 v = __ballot_sync(0xFFFFFFFFu, (x[j] >> b) & 1u);
+          if (lane == b) mine = v;
+        }
+      }
+      tile[j * 32 + lane][warp] = mine;
+    }
+    __syncthreads();
+    const u32 orow = w0 * 32 + threadIdx.x, ow = r0 / 32;
+    if (orow < rows) {
+      u32 c = 0;
+      u32 y[8];
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        y[j] = tile[threadIdx.x][j];
+        c += __popc(y[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; j += 4)
+        if (ow + j < words) {
+          const u64 at = ((u64)orow * words + ow + j) / 4;
+          uint4 v = make_uint4(y[j], y[j + 1], y[j + 2], y[j + 3]);
+          reinterpret_cast<uint4*>(dst)[at] = v;
+          if (full && any4(v)) {
+            uint4* f = reinterpret_cast<uint4*>(full) + at;
+            or4(v, *f);
+            *f = v;
+          }
+        }
+      if (c && dcnt) atomicAdd(dcnt + orow, c);
+      if (c && fcnt) atomicAdd(fcnt + orow, c);
+    }
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// renumbering: the values that occur get consecutive codes in value order
+// ---------------------------------------------------------------------------
+struct KeyCols {
+  const void* keys;
+  int key64;
+  u64 n;
+  int shift[2], width[2];
+};
+struct Codes {       // code of value v: pref[v / 32] + bits of pres[v / 32] below v (null pref: v itself)
+  const u32* pres;
+  const u32* pref;
+  LOB_DEV u32 operator()(u32 v) const {
+    return pref ? pref[v >> 5] + __popc(pres[v >> 5] & ((1u << (v & 31u)) - 1u)) : v;
+  }
+};
+
+__global__ void k_mark_values(KeyCols K, u32* __restrict__ pres) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < K.n; i += stride) {
+    const u64 k = load_key(K.keys, K.key64, i);
+    touch_bit(pres, field_of(k, K.shift[0], K.width[0]));
+    touch_bit(pres, field_of(k, K.shift[1], K.width[1]));
+  }
+}
+__global__ void k_word_bits(const u32* __restrict__ pres, u64 nw, u32* __restrict__ out) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += stride) out[i] = __popc(pres[i]);
+}
+__global__ void k_code_values(const u32* __restrict__ pres, const u32* __restrict__ pref, u64 nw, u32* __restrict__ dict) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += stride) {
+    u32 at = pref[i];
+    for (u32 m = pres[i]; m; m &= m - 1) dict[at++] = (u32)i * 32 + (u32)__ffs(m) - 1;
+  }
+}
+
+// compressed rows of an input relation: row lengths (and which values occur as
+// columns), then, after a scan, the columns; a row's columns are in no
+// particular order (a product does not depend on it)
+__global__ void k_csr_count(KeyCols K, Codes code, int inv, u32* __restrict__ len, u32* __restrict__ colflag) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < K.n; i += stride) {
+    const u64 k = load_key(K.keys, K.key64, i);
+    atomicAdd(len + code((u32)field_of(k, K.shift[inv], K.width[inv])), 1u);
+    colflag[code((u32)field_of(k, K.shift[inv ^ 1], K.width[inv ^ 1]))] = 1u;
+  }
+}
+__global__ void k_csr_fill(KeyCols K, Codes code, int inv, const u32* __restrict__ ptr, u32* __restrict__ used,
+                           u32* __restrict__ col, u32* __restrict__ heavy, u32* __restrict__ n_heavy) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < K.n; i += stride) {
+    const u64 k = load_key(K.keys, K.key64, i);
+    const u32 r = code((u32)field_of(k, K.shift[inv], K.width[inv]));
+    const u32 q = atomicAdd(used + r, 1u);
+    col[ptr[r] + q] = code((u32)field_of(k, K.shift[inv ^ 1], K.width[inv ^ 1]));
+    if (q == kHeavyRow) heavy[atomicAdd(n_heavy, 1u)] = r;  // one entry of a longer row gets here
+  }
+}
+// facts loaded into a derived relation: F and D start with them
+__global__ void k_set_facts(KeyCols K, Codes code, int inv, u32 words, u32* full, u32* recent, u32* cnt, u32* fcnt) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < K.n; i += stride) {
+    const u64 k = load_key(K.keys, K.key64, i);
+    const u32 r = code((u32)field_of(k, K.shift[inv], K.width[inv]));
+    const u32 c = code((u32)field_of(k, K.shift[inv ^ 1], K.width[inv ^ 1]));
+    atomicOr(full + (u64)r * words + (c >> 5), 1u << (c & 31u));
+    atomicOr(recent + (u64)r * words + (c >> 5), 1u << (c & 31u));
+    atomicAdd(cnt + r, 1u);  // keys are distinct
+    atomicAdd(fcnt + r, 1u);
+  }
+}
+
+// bits per row of a matrix (every row's words are valid): a warp a row
+__global__ void __launch_bounds__(256) k_row_counts(const u32* __restrict__ bits, u32 rows, u32 words,
+                                                    u32* __restrict__ cnt) {
+  const int lane = threadIdx.x & 31;
+  const u64 nwarps = (u64)gridDim.x * 8;
+  for (u64 r = (u64)blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += nwarps) {
+    const uint4* a = reinterpret_cast<const uint4*>(bits + r * words);
+    u32 c = 0;
+    for (u32 w = lane; w < words / 4; w += 32) c += popc4(a[w]);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
+    if (lane == 0) cnt[r] = c;
+  }
+}
+
+// Read-out: a warp walks a row 32 words at a time; a scan of the words' bit
+// counts places each lane's columns in the warp's shared-memory stage, and the
+// warp stores the batch's rows of every output column to consecutive addresses.
+__global__ void __launch_bounds__(256) k_bit_read(const u32* __restrict__ bits, u32 rows, u32 words,
+                                                  const u64* __restrict__ off, const u32* __restrict__ dict,
+                                                  u32* __restrict__ c0, u32* __restrict__ c1, float* __restrict__ tags,
+                                                  u32* __restrict__ samples) {
+  __shared__ u32 stages[8][1024];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  u32* stage = stages[warp];
+  const u64 nwarps = (u64)gridDim.x * 8;
+  for (u64 r = (u64)blockIdx.x * 8 + warp; r < rows; r += nwarps) {
+    u64 base = off[r];
+    if (off[r + 1] == base) continue;
+    const u32 x = dict ? dict[r] : (u32)r;
+    const u32* row = bits + r * words;
+    u32 nextw = lane < words ? row[lane] : 0u;
+    for (u32 w0 = 0; w0 < words; w0 += 32) {
+      const u32 m0 = nextw;
+      nextw = w0 + 32 + lane < words ? row[w0 + 32 + lane] : 0u;
+      const u32 c = __popc(m0);
+      const u32 inc = warp_inclusive_sum(c);
+      const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+      if (!tot) continue;
+      u32 pos = inc - c;
+      const u32 kw = (w0 + lane) * 32;
+      for (u32 m = m0; m; m &= m - 1) stage[pos++] = kw + (u32)__ffs(m) - 1;
+      __syncwarp();
+      for (u32 q = lane; q < tot; q += 32) {
+        const u32 y = stage[q];
+        c0[base + q] = x;
+        c1[base + q] = dict ? dict[y] : y;
+        if (tags) tags[base + q] = 1.0f;
+        if (samples) samples[base + q] = 0u;
+      }
+      __syncwarp();
+      base += tot;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// planning
+// ---------------------------------------------------------------------------
+struct Link {
+  u32 rel;
+  int inv;   // 1: read from its second column to its first
+  int atom;  // body position
+};
+struct Chain {
+  u32 head;
+  std::vector<Link> links;  // from head column 0 to head column 1
+  int diag = 0;
+  std::vector<int> order;   // links by body position: order[a] = link of body atom a
+};
+
+bool find_chain(const lob_engine& e, const RuleAst& R, Chain& C) {
+  if (R.computes() || R.head.args.size() != 2 || R.body.empty() || R.body.size() > (size_t)kMaxChain) return false;
+  const Term &hx = R.head.args[0], &hz = R.head.args[1];
+  if (!hx.var || !hz.var || hx.v == hz.v) return false;
+  std::vector<int> uses(R.var_names.size(), 0);
+  for (const AtomAst& a : R.body) {
+    if (a.args.size() != 2 || !a.args[0].var || !a.args[1].var || a.args[0].v == a.args[1].v) return false;
+    uses[a.args[0].v]++;
+    uses[a.args[1].v]++;
+  }
+  for (size_t v = 0; v < uses.size(); v++)
+    if (uses[v] != ((u32)v == hx.v || (u32)v == hz.v ? 1 : 2)) return false;
+  for (const FilterAst& F : R.filters) {  // only x != z or x == z, once
+    if (F.prog || !F.a.var || !F.b.var || C.diag) return false;
+    if (!((F.a.v == hx.v && F.b.v == hz.v) || (F.a.v == hz.v && F.b.v == hx.v))) return false;
+    C.diag = F.eq ? 2 : 1;
+  }
+  C.head = R.head.rel;
+  C.order.assign(R.body.size(), -1);
+  u32 at = hx.v;
+  for (size_t n = 0; n < R.body.size(); n++) {
+    bool found = false;
+    for (size_t i = 0; i < R.body.size() && !found; i++) {
+      if (C.order[i] >= 0) continue;
+      const u32 a = R.body[i].args[0].v, b = R.body[i].args[1].v;
+      if (a != at && b != at) continue;
+      C.order[i] = (int)C.links.size();
+      C.links.push_back({R.body[i].rel, b == at, (int)i});
+      at = b == at ? a : b;
+      found = true;
+    }
+    if (!found) return false;
+  }
+  return at == hz.v;
+}
+
+bool chains_of(const lob_engine& e, std::vector<Chain>& out) {
+  for (const RuleAst& R : e.rules) {
+    Chain C;
+    if (!find_chain(e, R, C)) return false;
+    out.push_back(std::move(C));
+  }
+  return !out.empty();
+}
+
+// Store the derived relations transposed?  Costs of an iteration's products:
+// one per scatter, one per derived relation read both ways (its transposed
+// copy is kept too), half for the final transpose.
+bool store_transposed(const lob_engine& e, const std::vector<Chain>& chains) {
+  double cost[2] = {0, 0.5};
+  for (int t = 0; t < 2; t++) {
+    std::vector<char> both(e.rels.size(), 0);
+    for (const Chain& C : chains) {
+      bool recursive = false;
+      for (const Link& l : C.links) recursive = recursive || e.rels[l.rel].idb;
+      if (!recursive) continue;
+      const Link& last = t ? C.links.front() : C.links.back();
+      if (C.links.size() > 1 && !e.rels[last.rel].idb) cost[t] += 1;
+      for (const Link& l : C.links)
+        if (e.rels[l.rel].idb && l.inv != 0) both[l.rel] = 1;
+    }
+    for (char b : both) cost[t] += b;
+  }
+  return cost[1] < cost[0];
+}
+
+unsigned warp_grid(u64 tasks) {
+  const u64 b = (tasks + kGatherWarps - 1) / kGatherWarps;
+  return (unsigned)std::max<u64>(1, std::min<u64>(b, 152ull * 8));
+}
+unsigned block_grid(u64 tasks) { return (unsigned)std::max<u64>(1, std::min<u64>(tasks, 152ull * 8)); }
+unsigned elem_grid(u64 n) { return (unsigned)std::max<u64>(1, std::min<u64>((n + 255) / 256, 152ull * 16)); }
+
+KeyCols key_cols(const RelSt& r) {
+  const ViewSt& V = r.views[0];
+  KeyCols K{};
+  K.keys = V.keys.p;
+  K.key64 = V.lay.key64;
+  K.n = V.n;
+  for (int j = 0; j < 2; j++) {
+    K.shift[j] = V.lay.shift[j];
+    K.width[j] = V.lay.width[j];
+  }
+  return K;
+}
+
+}  // namespace
+
+bool bit_eligible(const lob_engine& e) {
+  // Options that ask for one of the general path's strategies get that path.
+  if (!e.opt_bit_matrix || e.semiring != SR_UNIT || e.swidth) return false;
+  if (!e.opt_packed_join || e.opt_warp_join != 1 || e.opt_bitmap_delta != 1 || e.opt_emit_filter != 1 ||
+      !e.opt_cross_join || e.opt_join_index || e.opt_sort_algo || e.opt_max_cand < (1ull << 30))
+    return false;
+  if (e.rels.size() > (size_t)kMaxBitRels) return false;
+  for (const RelSt& r : e.rels)
+    if (r.idb && r.arity != 2) return false;
+  std::vector<Chain> chains;
+  if (!chains_of(e, chains)) return false;
+  for (const Chain& C : chains)
+    for (const Link& l : C.links)
+      for (int c = 0; c < 2; c++)
+        if (e.rels[l.rel].width[c] > 28) return false;
+  return true;
+}
+
+namespace {
+
+struct Run {
+  lob_engine& e;
+  BitRun& B;
+  std::vector<Chain> chains;
+  bool linear = true;      // every rule reads at most one derived atom
+  u64 heavy_slots = 0;
+  int n_temp = 0;
+  std::vector<char> accumulates;  // per relation: some iteration has more than one product into it
+
+  explicit Run(lob_engine& en) : e(en), B(*en.bit) {}
+
+  void launch_check(const char* what) {
+    e.after_launch(what);
+    e.launches++;
+  }
+
+  // codes of the program's values; false when a matrix would be too large
+  bool domain() {
+    int width = 1;
+    std::vector<char> used(e.rels.size(), 0);
+    for (auto& C : chains) {
+      used[C.head] = 1;
+      for (auto& l : C.links) used[l.rel] = 1;
+    }
+    for (size_t r = 0; r < e.rels.size(); r++)
+      if (used[r])
+        for (int c = 0; c < 2; c++) width = std::max(width, e.rels[r].width[c]);
+    // widths are bitlen(max + 1): all values are below 2^width
+    u64 D = 1ull << width;
+    if (D > kMaxValue) return false;
+    B.mapped = false;
+    if (D > 4096) {
+      const u64 nw = D / 32;
+      e.ensure(B.pres, nw * 4);
+      e.ensure(B.pref, nw * 4);
+      e.check(cudaMemsetAsync(B.pres.p, 0, nw * 4, e.stream), "values");
+      for (size_t r = 0; r < e.rels.size(); r++)
+        if (used[r] && e.rels[r].views[0].n) {
+          const KeyCols K = key_cols(e.rels[r]);
+          k_mark_values<<<elem_grid(K.n), 256, 0, e.stream>>>(K, B.pres.as<u32>());
+          launch_check("values");
+        }
+      k_word_bits<<<elem_grid(nw), 256, 0, e.stream>>>(B.pres.as<u32>(), nw, B.pref.as<u32>());
+      launch_check("values");
+      e.ensure(e.scratch, scan_scratch_elems(nw) * 4 + 64);
+      e.check(cudaMemsetAsync(e.counts.as<u64>() + 1, 0, sizeof(u64), e.stream), "values");
+      exclusive_scan<u32, u32>(B.pref.as<u32>(), B.pref.as<u32>(), nw, reinterpret_cast<u32*>(e.counts.as<u64>() + 1),
+                               e.scratch.as<u32>(), e.stream);
+      e.after_launch("values");
+      e.launches += scan_launches(nw);
+      D = std::max<u64>(1, e.read_u64(e.counts.as<u64>() + 1) & 0xFFFFFFFFull);
+      B.mapped = true;
+    }
+    B.rows = (u32)D;
+    B.words = (u32)((D + 127) / 128 * 4);
+    if ((u64)B.rows * B.words * 4 > kMatrixBytes) return false;
+    if (B.mapped) {
+      const u64 nw = (1ull << width) / 32;
+      e.ensure(B.dict, (u64)B.rows * 4);
+      k_code_values<<<elem_grid(nw), 256, 0, e.stream>>>(B.pres.as<u32>(), B.pref.as<u32>(), nw, B.dict.as<u32>());
+      launch_check("values");
+    }
+    return true;
+  }
+
+  Codes codes() const {
+    Codes c{};
+    if (B.mapped) {
+      c.pres = B.pres.as<u32>();
+      c.pref = B.pref.as<u32>();
+    }
+    return c;
+  }
+
+  // a link as the stored orientation reads it
+  Link oriented(const Link& l) const { return B.transposed ? Link{l.rel, !l.inv, l.atom} : l; }
+  std::vector<Link> links_of(const Chain& C) const {
+    std::vector<Link> v;
+    for (auto& l : C.links) v.push_back(oriented(l));
+    if (B.transposed) std::reverse(v.begin(), v.end());
+    return v;
+  }
+  bool stored_way(const Link& l) const { return l.inv == (B.transposed ? 1 : 0); }
+
+  BCsr csr(const Link& l) const {
+    const BitRel& R = B.rel[l.rel];
+    const BitCsr& C = R.csr[l.inv];
+    BCsr c{};
+    c.ptr = C.ptr.as<u32>();
+    c.col = C.col.as<u32>();
+    c.heavy = C.heavy.as<u32>();
+    c.n_heavy = C.heavy.as<u32>() + C.heavy_cap;
+    return c;
+  }
+  void build_csr(const Link& l) {
+    BitCsr& C = B.rel[l.rel].csr[l.inv];
+    if (C.built) return;
+    C.built = true;
+    const KeyCols K = key_cols(e.rels[l.rel]);
+    const u64 D = B.rows;
+    C.heavy_cap = (u32)(K.n / kHeavyRow + 1);
+    // lengths (their scan: ptr), fill positions, column flags, heavy rows and their number
+    e.ensure(C.ptr, (D + 1) * 4);
+    e.ensure(C.used, D * 4);
+    e.ensure(C.colflag, D * 4);
+    e.ensure(C.col, std::max<u64>(K.n, 1) * 4);
+    e.ensure(C.heavy, ((u64)C.heavy_cap + 1) * 4);
+    e.check(cudaMemsetAsync(C.ptr.p, 0, (D + 1) * 4, e.stream), "rows");
+    e.check(cudaMemsetAsync(C.used.p, 0, D * 4, e.stream), "rows");
+    e.check(cudaMemsetAsync(C.colflag.p, 0, D * 4, e.stream), "rows");
+    e.check(cudaMemsetAsync(C.heavy.p, 0, ((u64)C.heavy_cap + 1) * 4, e.stream), "rows");
+    if (!K.n) return;
+    ProfScope ps("bit_rows", K.n * (K.key64 ? 8.0 : 4.0) * 2.0 + K.n * 4.0 + D * 12.0, e.stream);
+    k_csr_count<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), l.inv, C.ptr.as<u32>(), C.colflag.as<u32>());
+    launch_check("rows");
+    e.ensure(e.scratch, scan_scratch_elems(D + 1) * 4 + 64);
+    exclusive_scan<u32, u32>(C.ptr.as<u32>(), C.ptr.as<u32>(), D + 1, nullptr, e.scratch.as<u32>(), e.stream);
+    e.after_launch("rows");
+    e.launches += scan_launches(D + 1);
+    k_csr_fill<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), l.inv, C.ptr.as<u32>(), C.used.as<u32>(), C.col.as<u32>(),
+                                                     C.heavy.as<u32>(), C.heavy.as<u32>() + C.heavy_cap);
+    launch_check("rows");
+  }
+
+  u64 mat_bytes() const { return (u64)B.rows * B.words * 4; }
+
+  void allocate() {
+    const u64 mb = mat_bytes(), D = B.rows;
+    for (size_t r = 0; r < e.rels.size(); r++) {
+      BitRel& R = B.rel[r];
+      if (!e.rels[r].idb) continue;
+      e.ensure(R.full, mb);
+      e.check(cudaMemsetAsync(R.full.p, 0, mb, e.stream), "bit matrix");
+      e.ensure(R.fcnt, D * 4);
+      for (int b = 0; b < 2; b++) {
+        e.ensure(R.recent[b], mb);
+        e.ensure(R.rcnt[b], D * 4);
+        e.check(cudaMemsetAsync(R.rcnt[b].p, 0, D * 4, e.stream), "bit matrix");
+      }
+      e.check(cudaMemsetAsync(R.fcnt.p, 0, D * 4, e.stream), "bit matrix");
+      if (accumulates[r]) {
+        e.ensure(R.acc, mb);
+        e.ensure(R.aflag, D * 4);
+        e.check(cudaMemsetAsync(R.acc.p, 0, mb, e.stream), "bit matrix");
+        e.check(cudaMemsetAsync(R.aflag.p, 0, D * 4, e.stream), "bit matrix");
+      }
+      if (R.need_t) {
+        e.ensure(R.trecent, mb);
+        e.ensure(R.trcnt, D * 4);
+        e.check(cudaMemsetAsync(R.trcnt.p, 0, D * 4, e.stream), "bit matrix");
+        if (!linear) {
+          e.ensure(R.tfull, mb);
+          e.ensure(R.tfcnt, D * 4);
+          e.check(cudaMemsetAsync(R.tfull.p, 0, mb, e.stream), "bit matrix");
+          e.check(cudaMemsetAsync(R.tfcnt.p, 0, D * 4, e.stream), "bit matrix");
+        }
+      }
+    }
+    for (int i = 0; i < n_temp; i++) {
+      e.ensure(B.temp[i], mb);
+      e.ensure(B.tbag[i], D * 8);
+    }
+    e.ensure(B.state, kAllSlots * 8);
+    e.check(cudaMemsetAsync(B.state.p, 0, kAllSlots * 8, e.stream), "bit state");
+    if (listed()) {
+      e.ensure(B.list, D * 4);
+      e.ensure(B.hlist, D * 4);
+    }
+  }
+
+  // rows x 128-word chunks beyond about two waves of warps: products list the
+  // rows they have work for first
+  bool listed() const { return (u64)B.rows * ((B.words + 127) / 128) > 152ull * 8 * kGatherWarps * 2; }
+
+
+  // the operand of a link: derived relations by which set the arm reads
+  BMat matrix(const Link& l, bool recent, int cur) const {
+    const BitRel& R = B.rel[l.rel];
+    BMat m{};
+    const bool st = stored_way(l);
+    const DevBuf& bits = recent ? (st ? R.recent[cur] : R.trecent) : (st ? R.full : R.tfull);
+    const DevBuf& cnt = recent ? (st ? R.rcnt[cur] : R.trcnt) : (st ? R.fcnt : R.tfcnt);
+    m.bits = bits.as<u32>();
+    m.cnt = cnt.as<u32>();
+    return m;
+  }
+
+  double words_before = 0;
+  void profile_before() {
+    if (g_prof) words_before = (double)e.read_u64(B.state.as<u64>() + B_WORDS);
+  }
+  void profile_after() {
+    if (g_prof) g_prof->add_last_bytes(4.0 * ((double)e.read_u64(B.state.as<u64>() + B_WORDS) - words_before));
+  }
+
+  // One arm: the chain's product with the recent set at link `delta` (body
+  // position), full sets at the other derived atoms (recent ones too in a
+  // linear program, where there are none).  `commit`: it is the last product
+  // into its head and no product of this iteration reads F.
+  void run_arm(const Chain& C, int delta, bool all_full, bool commit, int cur) {
+    const std::vector<Link> L = links_of(C);
+    const int m = (int)L.size();
+    BOp base{};
+    base.rows = B.rows;
+    base.words = B.words;
+    base.state = B.state.as<u64>();
+    if (!all_full)
+      for (const Link& l : L)
+        if (e.rels[l.rel].idb && l.atom < delta) base.skip[base.n_skip++] = (int)l.rel;
+    auto recent = [&](const Link& l) { return linear || (!all_full && l.atom == delta); };
+    BMat cur_m{};
+    BCsr cur_c{};
+    bool bits = e.rels[L[m - 1].rel].idb;
+    if (bits) cur_m = matrix(L[m - 1], recent(L[m - 1]), cur);
+    else cur_c = csr(L[m - 1]);
+    for (int i = m - 2; i >= -1; i--) {  // i == -1: a single atom, copied
+      if (i == -1 && m > 1) break;
+      BOp P = base;
+      P.mb = cur_m;
+      P.mc = cur_c;
+      int ik = I_IDENT;
+      if (i >= 0) {
+        if (e.rels[L[i].rel].idb) {
+          ik = I_BITS;
+          P.ib = matrix(L[i], recent(L[i]), cur);
+        } else {
+          ik = I_CSR;
+          P.ic = csr(L[i]);
+        }
+      }
+      const bool last = i <= 0;
+      if (!last) {
+        const int t = i % 2;
+        P.out = B.temp[t].as<u32>();
+        P.obag = B.tbag[t].as<u64>();
+        // rows that the next index matrix never lists need not be formed
+        if (!e.rels[L[i - 1].rel].idb) P.need = B.rel[L[i - 1].rel].csr[L[i - 1].inv].colflag.as<u32>();
+      } else {
+        set_head(P, C.head, cur, commit);
+        P.diag = C.diag;
+      }
+      product(P, ik, bits);
+      cur_m = BMat{};
+      cur_m.bits = P.out;
+      cur_m.bag = P.obag;
+      bits = true;
+    }
+  }
+
+  void set_head(BOp& P, u32 head, int cur, bool commit) {
+    BitRel& H = B.rel[head];
+    P.acc = H.acc.as<u32>();
+    P.aflag = H.aflag.as<u32>();
+    P.commit = commit;
+    P.full = H.full.as<u32>();
+    P.next = H.recent[cur ^ 1].as<u32>();
+    P.ncnt = H.rcnt[cur ^ 1].as<u32>();
+    P.fcnt = H.fcnt.as<u32>();
+    P.n_new = B.state.as<u64>() + rel_slot((int)head, 2);
+  }
+
+  int n_lists = 0;  // products of the current iteration that listed their rows
+
+  void product(BOp P, int ik, bool bits) {
+    const u32 chunks = (P.words + 127) / 128;
+    profile_before();
+    if (listed() && n_lists < kMaxLists) {
+      P.list = B.list.as<u32>();
+      P.hlist = B.hlist.as<u32>();
+      P.n_list = B.state.as<u64>() + kStateSlots + 2 * n_lists++;
+      {
+        ProfScope ps("bit_active", P.rows * 12.0, e.stream);
+        const unsigned g = warp_grid((P.rows + 31) / 32);
+        if (ik == I_IDENT) k_bit_active<I_IDENT><<<g, 256, 0, e.stream>>>(P, bits);
+        else if (ik == I_CSR) k_bit_active<I_CSR><<<g, 256, 0, e.stream>>>(P, bits);
+        else k_bit_active<I_BITS><<<g, 256, 0, e.stream>>>(P, bits);
+      }
+      launch_check("bit rows");
+    }
+    if (bits) {
+      {
+        ProfScope ps("bit_gather", 0, e.stream);
+        if (ik == I_IDENT) k_bit_gather<I_IDENT><<<warp_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
+        else if (ik == I_CSR) k_bit_gather<I_CSR><<<warp_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
+        else k_bit_gather<I_BITS><<<block_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
+      }
+      launch_check("bit gather");
+    } else {
+      {
+        ProfScope ps("bit_scatter", 0, e.stream);
+        const size_t sm = (size_t)P.words * 4;
+        if (ik == I_IDENT) k_bit_scatter<I_IDENT><<<block_grid(P.rows), 256, sm, e.stream>>>(P);
+        else if (ik == I_CSR) k_bit_scatter<I_CSR><<<block_grid(P.rows), 256, sm, e.stream>>>(P);
+        else k_bit_scatter<I_BITS><<<block_grid(P.rows), 256, sm, e.stream>>>(P);
+      }
+      launch_check("bit scatter");
+    }
+    profile_after();
+  }
+
+  void transpose_recent(int cur, u64* state) {
+    for (size_t r = 0; r < e.rels.size(); r++) {
+      BitRel& R = B.rel[r];
+      if (!e.rels[r].idb || !R.need_t) continue;
+      BMat m{};
+      m.bits = R.recent[cur].as<u32>();
+      m.cnt = R.rcnt[cur].as<u32>();
+      ProfScope ps("bit_transpose", 2.0 * mat_bytes(), e.stream);
+      const u64 tiles = (u64)((B.rows + 255) / 256) * ((B.words + 7) / 8);
+      k_bit_transpose<<<block_grid(tiles), 256, 0, e.stream>>>(m, B.rows, B.words, R.trecent.as<u32>(), R.trcnt.as<u32>(),
+                                                               R.tfull.as<u32>(), R.tfcnt.as<u32>(), state);
+      launch_check("bit transpose");
+    }
+  }
+
+  // one iteration (k >= 1) on recent buffers `cur`; its results go to cur ^ 1
+  void iteration(u32 k, u32 max_iters, int cur) {
+    // the arms of this iteration: in the first, every loaded fact is recent, so
+    // the arm of each rule's first atom covers the rule; later only derived
+    // atoms have recent facts
+    struct ArmRef { const Chain* c; int delta; };
+    std::vector<ArmRef> arms;
+    for (auto& C : chains) {
+      if (k == 1) {
+        bool empty = false;
+        for (auto& l : C.links) empty = empty || !e.rels[l.rel].views[0].n;
+        if (!empty) arms.push_back({&C, 0});
+        continue;
+      }
+      for (size_t a = 0; a < C.order.size(); a++)
+        if (e.rels[C.links[C.order[a]].rel].idb) arms.push_back({&C, (int)a});
+    }
+    std::vector<int> left(e.rels.size(), 0);
+    n_lists = 0;
+    for (auto& a : arms) left[a.c->head]++;
+    for (auto& a : arms) {
+      const bool commit = linear && --left[a.c->head] == 0;
+      run_arm(*a.c, a.delta, k == 1, commit, cur);
+    }
+    if (!linear) {
+      std::vector<char> has(e.rels.size(), 0);
+      for (auto& a : arms) has[a.c->head] = 1;
+      for (size_t r = 0; r < e.rels.size(); r++) {
+        if (!has[r]) continue;
+        BOp P{};
+        P.rows = B.rows;
+        P.words = B.words;
+        P.state = B.state.as<u64>();
+        set_head(P, (u32)r, cur, true);
+        const u32 chunks = (P.words + 127) / 128;
+        profile_before();
+        {
+          ProfScope ps("bit_commit", 0, e.stream);
+          k_bit_commit<<<warp_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
+        }
+        launch_check("bit commit");
+        profile_after();
+      }
+    }
+    BEnd E{};
+    E.rows = B.rows;
+    E.max_iters = max_iters;
+    E.state = B.state.as<u64>();
+    for (size_t r = 0; r < e.rels.size(); r++) {
+      if (!e.rels[r].idb) continue;
+      const int i = E.n_rel++;
+      BitRel& R = B.rel[r];
+      E.rel[i] = (int)r;
+      E.old_cnt[i] = R.rcnt[cur].as<u32>();
+      E.aflag[i] = R.aflag.as<u32>();
+      E.tcnt[i] = R.need_t ? R.trcnt.as<u32>() : nullptr;
+    }
+    k_bit_end<<<std::min(elem_grid(B.rows), 152u), 256, 0, e.stream>>>(E);
+    launch_check("bit end");
+    transpose_recent(cur ^ 1, B.state.as<u64>());
+  }
+
+  bool run(u32 max_iters, u32& k, u64& new_facts, int* rc) {
+    if (!chains_of(e, chains)) return false;
+    B.transposed = store_transposed(e, chains);
+    B.rel.clear();
+    B.rel.resize(e.rels.size());
+    accumulates.assign(e.rels.size(), 0);
+    std::vector<int> first(e.rels.size(), 0), later(e.rels.size(), 0);
+    for (auto& C : chains) {
+      int idb = 0;
+      for (auto& l : C.links)
+        if (e.rels[l.rel].idb) {
+          idb++;
+          if (!stored_way(oriented(l))) B.rel[l.rel].need_t = true;
+        }
+      if (idb > 1) linear = false;
+      first[C.head]++;
+      later[C.head] += idb;
+      if ((int)C.links.size() > 2) n_temp = std::max(n_temp, std::min(2, (int)C.links.size() - 2));
+    }
+    if (n_temp) n_temp = 2;
+    for (size_t r = 0; r < e.rels.size(); r++) {
+      // the first iteration's rules that have facts, and each later iteration's arms
+      int f = 0;
+      for (auto& C : chains) {
+        bool empty = false;
+        for (auto& l : C.links) empty = empty || !e.rels[l.rel].views[0].n;
+        f += C.head == r && !empty;
+      }
+      accumulates[r] = e.rels[r].idb && (!linear || f > 1 || later[r] > 1);
+    }
+    if (!domain()) return false;
+    allocate();
+    for (auto& C : chains)
+      for (auto& l : C.links)
+        if (!e.rels[l.rel].idb) build_csr(oriented(l));
+    std::vector<u64> h(kStateSlots, 0);
+    bool loaded = false;
+    for (size_t r = 0; r < e.rels.size(); r++) {
+      if (!e.rels[r].idb || !e.rels[r].views[0].n) continue;
+      loaded = true;
+      BitRel& R = B.rel[r];
+      const KeyCols K = key_cols(e.rels[r]);
+      e.check(cudaMemsetAsync(R.recent[0].p, 0, mat_bytes(), e.stream), "bit matrix");
+      k_set_facts<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), B.transposed, B.words, R.full.as<u32>(),
+                                                        R.recent[0].as<u32>(), R.rcnt[0].as<u32>(), R.fcnt.as<u32>());
+      launch_check("bit facts");
+      h[rel_slot((int)r, 0)] = h[rel_slot((int)r, 1)] = K.n;
+    }
+    if (loaded) {
+      e.check(cudaMemcpyAsync(B.state.p, h.data(), h.size() * 8, cudaMemcpyHostToDevice, e.stream), "bit state");
+      e.sync();  // h goes out of scope with the run; the copy is from pageable memory
+      transpose_recent(0, nullptr);
+    }
+    // Iterations are queued in groups without waiting: one that follows the
+    // fixpoint sees the done flag and does nothing (about 2 us a launch), which
+    // is cheaper than a host wait per iteration (about 10 us).
+    u64* s = e.pinned;
+    u32 queued = 0;
+    for (u32 group = 4;; group = std::min(16u, group * 2)) {
+      for (u32 i = 0; i < group && queued < max_iters; i++, queued++) iteration(queued + 1, max_iters, (int)(queued & 1));
+      e.check(cudaMemcpyAsync(s, B.state.p, kStateSlots * 8, cudaMemcpyDeviceToHost, e.stream), "bit state");
+      e.sync();
+      if (s[B_DONE] || queued >= max_iters) break;
+    }
+    *rc = s[B_DONE] == 1 ? LOB_OK : LOB_E_MAXITER;
+    k = (u32)s[B_ITER];
+    new_facts = s[B_NEW];
+    e.cand_emitted = s[B_CAND];
+    for (size_t r = 0; r < e.rels.size(); r++)
+      if (e.rels[r].idb) e.rels[r].views[0].n = s[rel_slot((int)r, 0)];
+    finish();
+    return true;
+  }
+
+  // results in row order, with each row's offset
+  void finish() {
+    const u64 D = B.rows;
+    for (size_t r = 0; r < e.rels.size(); r++) {
+      BitRel& R = B.rel[r];
+      if (!e.rels[r].idb) continue;
+      if (B.transposed) {
+        BMat m{};
+        m.bits = R.full.as<u32>();
+        m.cnt = R.fcnt.as<u32>();
+        {
+          ProfScope ps("bit_transpose", 2.0 * mat_bytes(), e.stream);
+          const u64 tiles = (u64)((B.rows + 255) / 256) * ((B.words + 7) / 8);
+          k_bit_transpose<<<block_grid(tiles), 256, 0, e.stream>>>(m, B.rows, B.words, R.recent[0].as<u32>(), nullptr,
+                                                                   nullptr, nullptr, nullptr);
+        }
+        launch_check("bit transpose");
+        std::swap(R.full, R.recent[0]);
+        {
+          ProfScope ps("bit_counts", (double)mat_bytes(), e.stream);
+          k_row_counts<<<warp_grid(D), 256, 0, e.stream>>>(R.full.as<u32>(), B.rows, B.words, R.fcnt.as<u32>());
+        }
+        launch_check("bit counts");
+      }
+      e.ensure(R.off, (D + 1) * 8);
+      e.ensure(e.scratch, scan_scratch_elems(D) * 8 + 64);
+      exclusive_scan<u32, u64>(R.fcnt.as<u32>(), R.off.as<u64>(), D, R.off.as<u64>() + D, e.scratch.as<u64>(), e.stream);
+      e.after_launch("bit offsets");
+      e.launches += scan_launches(D);
+      for (DevBuf* b : {&R.recent[0], &R.recent[1], &R.rcnt[0], &R.rcnt[1], &R.acc, &R.aflag, &R.trecent, &R.trcnt, &R.tfull,
+                        &R.tfcnt})
+        e.release(*b);
+    }
+    for (int i = 0; i < 2; i++) {
+      e.release(B.temp[i]);
+      e.release(B.tbag[i]);
+    }
+  }
+};
+
+}  // namespace
+
+bool bit_run(lob_engine& e, u32 max_iters, u32& k, u64& new_facts, int* rc) {
+  e.bit.reset(new BitRun());
+  try {
+    Run R(e);
+    if (R.run(max_iters, k, new_facts, rc)) {
+      e.bit->on = true;
+      return true;
+    }
+  } catch (const LobError& x) {
+    bit_release(e);
+    if (x.code != LOB_E_OOM) throw;
+    return false;  // the general path may need less
+  }
+  bit_release(e);
+  return false;
+}
+
+void bit_release(lob_engine& e) {
+  if (!e.bit) return;
+  BitRun& B = *e.bit;
+  for (DevBuf* b : {&B.pres, &B.pref, &B.dict, &B.state, &B.list, &B.hlist, &B.temp[0], &B.temp[1], &B.tbag[0], &B.tbag[1]}) e.release(*b);
+  for (BitRel& R : B.rel) {
+    for (DevBuf* b : {&R.full, &R.fcnt, &R.recent[0], &R.recent[1], &R.rcnt[0], &R.rcnt[1], &R.acc, &R.aflag, &R.trecent,
+                      &R.trcnt, &R.tfull, &R.tfcnt, &R.off})
+      e.release(*b);
+    for (BitCsr& C : R.csr)
+      for (DevBuf* b : {&C.ptr, &C.used, &C.colflag, &C.col, &C.heavy}) e.release(*b);
+  }
+  e.bit.reset();
+}
+
+void bit_read(lob_engine& e, u32 rel, u32* cols, u64 stride, float* tags, u32* samples) {
+  BitRun& B = *e.bit;
+  BitRel& R = B.rel[rel];
+  const u64 n = e.rels[rel].views[0].n;
+  ProfScope ps("bit_read", (double)B.rows * B.words * 4 + n * (8.0 + (tags ? 4.0 : 0.0) + (samples ? 4.0 : 0.0)), e.stream);
+  k_bit_read<<<warp_grid(B.rows), 256, 0, e.stream>>>(R.full.as<u32>(), B.rows, B.words, R.off.as<u64>(),
+                                                      B.mapped ? B.dict.as<u32>() : nullptr, cols, cols + stride, tags,
+                                                      samples);
+}

@@ -15,6 +15,7 @@
 #include <cstring>
 #include <functional>
 
+#include "bitmat.h"
 #include "engine.h"
 #include "scan.cuh"
 
@@ -165,6 +166,7 @@ static void release_derived(lob_engine& e) {
     r.last_cand = r.last_new = r.cand_iter = 0;
   }
   for (DevBuf* b : {&e.arena, &e.top1_state, &e.top1_prob}) e.release(*b);
+  bit_release(e);
   e.arena_tail = e.arena_cap = 0;
   e.plans.clear();
 }
@@ -658,6 +660,11 @@ static void prepare(lob_engine& e, int sem) {
     for (int j = 0; j < kMaxArity; j++) id[j] = j;
     find_view(e, r, id);
   }
+}
+
+// arms, join orders and the secondary views they probe (general path)
+static void prepare_arms(lob_engine& e) {
+  const int sem = e.semiring;
   const bool idem = sem_idempotent(sem);
   for (auto& R : e.rules) {
     RulePlan p;
@@ -865,6 +872,17 @@ static void load_facts(lob_engine& e) {
       e.check(cudaMemcpyAsync(r.rtags.p, V.tags.p, V.n * sb, cudaMemcpyDeviceToDevice, e.stream), "recent tags");
     }
     r.n_recent = V.n;
+  }
+  if (sem_top1(sem)) top1_setup(e, id_base);
+}
+
+// the secondary views of the loaded facts
+static void load_views(lob_engine& e) {
+  const int sb = stored_bytes(e.semiring);
+  const bool stamps = sem_stamps(e.semiring);
+  for (auto& r : e.rels) {
+    const ViewSt& V = r.views[0];
+    if (!V.n) continue;
     for (size_t vi = 1; vi < r.views.size(); vi++) {
       ViewSt& W = r.views[vi];
       auto kt = sort_view_rows(e, r, W, V.keys.p, V.tags.p, V.n);
@@ -882,7 +900,6 @@ static void load_facts(lob_engine& e) {
       }
     }
   }
-  if (sem_top1(sem)) top1_setup(e, id_base);
 }
 
 // ---------------------------------------------------------------------------
@@ -1898,20 +1915,30 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   e.check(cudaEventCreate(&ev.b), "event");
   cudaEvent_t ev0 = ev.a, ev1 = ev.b;
   e.check(cudaEventRecord(ev0, e.stream), "event");
+  e.iter_counts.clear();
+  e.cand_emitted = 0;
+  e.stratum_begin.clear();
+  e.n_strata = 1;
+  e.check(cudaMemsetAsync(sort_err(e), 0, sizeof(u32), e.stream), "sort error word");
+  e.check(cudaMemsetAsync(e.counts.as<u64>() + 13, 0, sizeof(u64), e.stream), "emitted counter");
   prepare(e, sem);
+  // a chain program under the unit semiring runs on bit matrices and needs
+  // neither arms nor secondary views
+  const bool bits = max_iters > 0 && bit_eligible(e);
+  if (!bits) prepare_arms(e);
   load_facts(e);
-  enable_dense(e);
   lob_stats s{};
   s.semiring = (u32)sem;
   int rc = LOB_OK;
   u32 k = 0;
-  e.iter_counts.clear();
-  e.cand_emitted = 0;
-  e.check(cudaMemsetAsync(sort_err(e), 0, sizeof(u32), e.stream), "sort error word");
-  e.check(cudaMemsetAsync(e.counts.as<u64>() + 13, 0, sizeof(u64), e.stream), "emitted counter");
-  e.stratum_begin.clear();
+  const bool bit_done = bits && bit_run(e, max_iters, k, (u64&)s.new_facts, &rc);
+  if (!bit_done) {
+    if (bits) prepare_arms(e);
+    load_views(e);
+  }
+  enable_dense(e);
   int stratum = 0;  // the stratum being run (assign_strata)
-  for (;;) {
+  while (!bit_done) {
     if (k >= max_iters) { rc = LOB_E_MAXITER; break; }
     k++;
     e.iter_counts.emplace_back();
@@ -2358,8 +2385,12 @@ int lob_read_relation(lob_engine* e, uint32_t rel, uint32_t* cols, float* tags, 
     if (!n) return LOB_OK;
     if (!cols) throw LobError(LOB_E_ARG, "null cols");
     const int ks = sem_kernel(e->semiring);
+    const auto rows_out = [&](u32* c, u64 stride, float* t, u32* sm) {
+      if (r.idb && e->bit && e->bit->on) bit_read(*e, rel, c, stride, t, sm);
+      else read_rows(ks, V.lay, V.perm, V.keys.p, V.tags.p, n, c, stride, t, sm, e->stream);
+    };
     if (mem == LOB_MEM_DEVICE) {
-      read_rows(ks, V.lay, V.perm, V.keys.p, V.tags.p, n, cols, capacity, tags, sample_ids, e->stream);
+      rows_out(cols, capacity, tags, sample_ids);
       e->after_launch("read");
       e->sync();
       return LOB_OK;
@@ -2371,7 +2402,7 @@ int lob_read_relation(lob_engine* e, uint32_t rel, uint32_t* cols, float* tags, 
     float* dt = tags ? static_cast<float*>(mapped_range(tags, n * 4)) : nullptr;
     u32* ds = sample_ids ? static_cast<u32*>(mapped_range(sample_ids, n * 4)) : nullptr;
     if (dc && (!tags || dt) && (!sample_ids || ds)) {
-      read_rows(ks, V.lay, V.perm, V.keys.p, V.tags.p, n, dc, capacity, dt, ds, e->stream);
+      rows_out(dc, capacity, dt, ds);
       e->after_launch("read (mapped host)");
       e->sync();
       return LOB_OK;
@@ -2380,8 +2411,7 @@ int lob_read_relation(lob_engine* e, uint32_t rel, uint32_t* cols, float* tags, 
     e->ensure(c, n * r.arity * 4);
     if (tags) e->ensure(t, n * 4);
     if (sample_ids) e->ensure(s, n * 4);
-    read_rows(ks, V.lay, V.perm, V.keys.p, V.tags.p, n, c.as<u32>(), n, tags ? t.as<float>() : nullptr,
-              sample_ids ? s.as<u32>() : nullptr, e->stream);
+    rows_out(c.as<u32>(), n, tags ? t.as<float>() : nullptr, sample_ids ? s.as<u32>() : nullptr);
     e->after_launch("read");
     for (u32 q = 0; q < r.arity; q++)
       e->check(cudaMemcpyAsync(cols + (u64)q * capacity, c.as<u32>() + (u64)q * n, n * 4, cudaMemcpyDeviceToHost, e->stream),
@@ -2616,6 +2646,7 @@ int lob_set_option(lob_engine* e, const char* key, int64_t value) {
     else if (k == "loop_cap_floor" && value >= 256 && value <= (1 << 24)) e->opt_loop_cap_floor = (int)value;
     else if (k == "packed_backward" && (value == 0 || value == 1)) e->opt_packed_backward = (int)value;
     else if (k == "cross_join" && (value == 0 || value == 1)) e->opt_cross_join = (int)value;
+    else if (k == "bit_matrix" && (value == 0 || value == 1)) e->opt_bit_matrix = (int)value;
     else if (k == "proof_cap" && value >= 1 && value <= (1 << 20)) e->opt_proof_cap = (int)value;
     else if (k == "proof_arena_words" && value >= 16 && value <= (1ll << 31)) e->opt_arena_words = (u64)value;
     else throw LobError(LOB_E_ARG, "unknown option or value out of range: " + k);

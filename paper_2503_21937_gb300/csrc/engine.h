@@ -181,6 +181,33 @@ struct EngineProfiler : KernelProfiler {
   ~EngineProfiler();
 };
 
+// ---------------------------------------------------------------------------
+// bit-matrix runs (bitmat.cu)
+// ---------------------------------------------------------------------------
+// compressed rows of an input relation: offsets, columns, fill positions, which
+// values occur as columns, the long rows and (last word) their number
+struct BitCsr {
+  bool built = false;
+  DevBuf ptr, col, used, colflag, heavy;
+  u32 heavy_cap = 0;
+};
+// a derived relation: F, the two recent sets' buffers, the accumulator of an
+// iteration with several products, transposed copies (need_t) -- each with its
+// row counts -- and the final row offsets
+struct BitRel {
+  bool need_t = false;
+  DevBuf full, fcnt, recent[2], rcnt[2], acc, aflag, trecent, trcnt, tfull, tfcnt, off;
+  BitCsr csr[2];  // an input relation read forwards / backwards
+};
+struct BitRun {
+  bool on = false;          // the derived relations live in the matrices
+  bool transposed = false;  // stored transposed while the run lasts
+  bool mapped = false;      // values are renumbered (dict: code -> value)
+  u32 rows = 0, words = 0;
+  DevBuf pres, pref, dict, state, list, hlist, temp[2], tbag[2];
+  std::vector<BitRel> rel;
+};
+
 struct lob_engine {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -193,6 +220,7 @@ struct lob_engine {
   std::map<std::string, u32> rel_ids;
   std::vector<RuleAst> rules;
   std::vector<RulePlan> plans;
+  std::unique_ptr<BitRun> bit;    // set while a bit-matrix run's results are held
   // options
   int opt_join_index = 0, opt_dense_bits = 24, opt_radix_bits = 8, opt_sync_check = 0, opt_profile = 0;
   int opt_hash_slots = 2;         // hash index: slots per view row at least (load factor <= 1 / opt_hash_slots)
@@ -209,6 +237,7 @@ struct lob_engine {
   int opt_loop_cap_floor = 1 << 16;  // smallest buffer capacity (rows) the device loop plans with
   int opt_packed_backward = 1;    // diff-add-mult backward replays packed arms on the packed kernels
   int opt_cross_join = 1;         // unit semiring: fused cross-product step for two probes keyed by the delta row
+  int opt_bit_matrix = 1;         // unit semiring: chain programs on bit matrices
   int opt_proof_cap = 300;        // top-1-proofs: longest proof (input facts) a union may produce
   u64 opt_arena_words = 1ull << 22;  // top-1-proofs: free words of a fresh proof arena (it grows on demand)
   std::map<std::string, u64> loop_caps;  // buffer capacities the device loop needed, kept across runs

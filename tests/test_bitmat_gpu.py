@@ -1,0 +1,99 @@
+"""Chain programs on bit matrices (unit semiring) against the oracle and
+against the general path (option bit_matrix = 0): relations, iterations,
+derivations and new facts are equal on every program shape, both storage
+orientations, renumbered ids, long rows and listed (large) matrices."""
+import numpy as np
+import pytest
+
+from paper_2503_21937_gb300 import workloads as W
+from tests.common import compare, engine_run
+
+pytestmark = pytest.mark.gpu
+
+PROGRAMS = {
+    "left": W.TC_PROGRAM,
+    "right": "path(x,y) :- edge(x,y).\npath(x,z) :- edge(x,y), path(y,z).\n",
+    "nonlinear": "path(x,y) :- edge(x,y).\npath(x,z) :- path(x,y), path(y,z).\n",
+    "same_generation": "path(x,y) :- edge(p,x), edge(p,y), x != y.\npath(x,y) :- edge(a,x), path(a,b), edge(b,y).\n",
+    "reversed": "path(y,x) :- edge(x,y).\npath(x,z) :- path(y,x), edge(y,z), x != z.\n",
+    "four_atoms": "path(x,y) :- edge(x,y).\npath(x,w) :- edge(x,y), path(z,y), edge(z,v), path(v,w).\n",
+    "loops": "path(x,y) :- edge(x,y).\npath(x,z) :- path(x,y), edge(y,z).\nback(x,y) :- path(x,z), path(z,y), x == y.\n",
+    "mutual": "odd(x,y) :- edge(x,y).\nodd(x,z) :- even(x,y), edge(y,z).\neven(x,z) :- odd(x,y), edge(y,z).\n",
+    "two_rules": "path(x,y) :- edge(x,y).\npath(x,y) :- edge(y,x).\npath(x,z) :- path(x,y), edge(y,z).\n"
+                 "path(x,z) :- path(x,y), edge(z,y).\n",
+}
+
+
+def same_as_general(program, inputs, **kw):
+    outs = []
+    for on in (1, 0):
+        e, st, got = engine_run(program, inputs, options={"bit_matrix": on}, **kw)
+        outs.append((st, got))
+        e.close()
+    (a, ga), (b, gb) = outs
+    for k in ("iterations", "derived", "candidates", "new_facts"):
+        assert a[k] == b[k], (k, a[k], b[k])
+    for name in gb:
+        assert np.array_equal(ga[name].cols, gb[name].cols), name
+        assert np.array_equal(ga[name].tags, gb[name].tags), name
+        assert np.array_equal(ga[name].samples, gb[name].samples), name
+    return a
+
+
+@pytest.mark.parametrize("name", list(PROGRAMS))
+@pytest.mark.parametrize("n,m,scale", [(2, 1, 1), (31, 40, 1), (33, 60, 1), (127, 200, 40000), (129, 180, 1)])
+def test_program_shapes(name, n, m, scale):
+    """Rows of one word group and just past one, ids dense and spread out
+    (renumbered), every rule shape; duplicates among the input rows."""
+    s = W.stream(7100 + n)
+    a, b = s.below(m, n) * np.uint32(scale), s.below(m, n) * np.uint32(scale)
+    inputs = {"edge": ((np.concatenate([a, a[:5]]), np.concatenate([b, b[:5]])),)}
+    compare(PROGRAMS[name], inputs)
+    same_as_general(PROGRAMS[name], inputs)
+
+
+@pytest.mark.parametrize("name", ["left", "right", "nonlinear", "mutual", "same_generation"])
+def test_facts_loaded_into_derived_relations(name):
+    s = W.stream(7200)
+    a, b, c, d = (s.below(60, 50) for _ in range(4))
+    head = "odd" if name == "mutual" else "path"
+    inputs = {"edge": ((a, b),), head: ((c[:9], d[:9]),)}
+    compare(PROGRAMS[name], inputs)
+    same_as_general(PROGRAMS[name], inputs)
+
+
+@pytest.mark.parametrize("name", ["left", "right", "same_generation", "two_rules"])
+def test_listed_rows_and_long_rows(name):
+    """Matrices beyond the listing threshold (12,000 values), rows of more than
+    512 entries in both directions (a hub), most rows idle in most iterations."""
+    s = W.stream(7300)
+    n = 12000
+    parent, child, _ = W.random_tree(n, seed_index=7301)
+    hub = np.full(700, 5, np.uint32)
+    leaf = s.below(700, n)
+    a = np.concatenate([parent, hub, leaf[:600]])
+    b = np.concatenate([child, leaf, hub[:600]])
+    if name == "same_generation":
+        a, b = parent, child
+    if name == "two_rules":
+        a, b = a[:3000], b[:3000]
+    same_as_general(PROGRAMS[name], {"edge": ((a, b),)})
+
+
+def test_points_to_and_iteration_limit():
+    A = W.andersen_program(60000, 3000, seed_index=7400)
+    inputs = {k: ((v[0], v[1]),) for k, v in A.items()}
+    compare(W.ANDERSEN_PROGRAM, inputs, rels=["pt"])
+    same_as_general(W.ANDERSEN_PROGRAM, inputs)
+    from paper_2503_21937_gb300 import Engine, LobsterError
+    got = []
+    for on in (1, 0):
+        e = Engine()
+        e.program(W.TC_PROGRAM)
+        e.set_option("bit_matrix", on)
+        e.load("edge", W.ktree_chain(60))
+        with pytest.raises(LobsterError, match="MAXITER"):
+            e.run("unit", max_iters=7)
+        got.append(e.read("path").cols)
+        e.close()
+    assert np.array_equal(got[0], got[1])
