@@ -148,7 +148,11 @@ int lob_add_rule(lob_engine* e, const char* text);
  * buffers chosen through a device pointer table, every size and the stop
  * decision held in device memory, and no host wait between iterations;
  * buffers that turn out too small end the graph early, grow, and the graph is
- * launched again from the last committed iteration. */
+ * launched again from the last committed iteration.  A component of such a
+ * run whose rules read at most one derived atom, joined with one input atom,
+ * runs its iterations after the first in one launch of its own (counted in
+ * graph_launches and device_iterations) on dense arrays over its key space
+ * of up to 2^24 keys; the rest of the program runs beside it as above. */
 int lob_run_to_fixpoint(lob_engine* e, int semiring, uint32_t max_iters, lob_stats* stats);
 
 /* Options chosen by lob_autotune and the timings behind them. */

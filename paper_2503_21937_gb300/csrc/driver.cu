@@ -271,13 +271,14 @@ bool loop_eligible(const lob_engine& e) {
   int narm = 0;
   for (const auto& r : e.rels) {
     if (r.idb && !r.dense) return false;
+    if (r.finished) continue;
     int nv = 0;
     for (size_t vi = 1; vi < r.views.size(); vi++) nv += r.views[vi].maintained;
     if (nv > kGMaxViews) return false;
   }
   for (const auto& p : e.plans)
     for (const auto& A : p.arms) {
-      if (!e.rels[p.ast.body[A.delta].rel].idb) continue;
+      if (!e.rels[p.ast.body[A.delta].rel].idb || e.rels[p.ast.head.rel].finished) continue;
       if (!A.packed.ok || A.steps.size() < 2 || A.steps.size() > (size_t)kGMaxSteps) return false;
       if (A.before_rels.size() > (size_t)kGMaxBefore) return false;
       narm++;
@@ -292,15 +293,15 @@ void plan_loop(lob_engine& e, GLoop& G, u32 max_iters) {
   G.views.assign(nrel, {});
   for (int r = 0; r < nrel; r++) {
     RelSt& R = e.rels[r];
-    G.d.rel_dense[r] = R.idb && R.dense;
+    G.d.rel_dense[r] = R.idb && R.dense && !R.finished;
     int slot = 0;
     for (size_t vi = 1; vi < R.views.size(); vi++)
-      if (R.views[vi].maintained) G.views[r].push_back({r, (int)vi, ++slot});
+      if (R.views[vi].maintained && !R.finished) G.views[r].push_back({r, (int)vi, ++slot});
     G.d.rel_nviews[r] = slot;
   }
   for (const auto& p : e.plans)
     for (const auto& A : p.arms) {
-      if (!e.rels[p.ast.body[A.delta].rel].idb) continue;
+      if (!e.rels[p.ast.body[A.delta].rel].idb || e.rels[p.ast.head.rel].finished) continue;
       const int a = (int)G.arms.size();
       G.arms.push_back({&p, &A});
       G.d.arm_delta[a] = (int)p.ast.body[A.delta].rel;

@@ -17,6 +17,7 @@
 
 #include "bitmat.h"
 #include "engine.h"
+#include "linear.h"
 #include "scan.cuh"
 
 RuleAst parse_rule(const lob_engine& e, const char* text);
@@ -159,7 +160,7 @@ static void release_derived(lob_engine& e) {
                       &r.row_keys, &r.akeys, &r.atags, &r.akeys2, &r.atags2, &r.bitmap, &r.prev_bitmap, &r.dacc,
                       &r.dtouched})
       e.release(*b);
-    r.extract = r.touched = r.keys_stale = r.dense = false;
+    r.extract = r.touched = r.keys_stale = r.dense = r.finished = false;
     r.n_recent = r.n_next = r.n_cand = r.n_acc = 0;
     r.flushed = false;
     r.filter_on = false;
@@ -627,6 +628,7 @@ static void prepare(lob_engine& e, int sem) {
         m = (u32)(e.read_u64(reinterpret_cast<u64*>(dmax)) & 0xFFFFFFFFull);
       }
       r.width[c] = r.n_in ? std::max(1, bitlen((u64)m + 1)) : 1;
+      r.maxv[c] = m;
     }
     if (r.in_has_samples && r.n_in) {
       reduce_max_u32(r.in_samples.as<u32>(), r.n_in, dmax, e.stream);
@@ -635,6 +637,7 @@ static void prepare(lob_engine& e, int sem) {
       any_samples = true;
     }
   }
+  e.max_sample = max_sample;
   e.swidth = any_samples ? bitlen((u64)max_sample + 1) : 0;
   for (auto& r : e.rels) r.idb = false;
   for (auto& R : e.rules) e.rels[R.head.rel].idb = true;
@@ -645,13 +648,18 @@ static void prepare(lob_engine& e, int sem) {
       for (size_t c = 0; c < R.head.args.size(); c++) {
         const Term& t = R.head.args[c];
         int need = 1;
-        if (c < R.head_prog.size() && R.head_prog[c]) need = 32;  // computed: any u32 but 2^32 - 1
-        else if (!t.var) need = bitlen((u64)t.v + 1);
+        u32 top = 0;
+        if (c < R.head_prog.size() && R.head_prog[c]) { need = 32; top = 0xFFFFFFFEu; }  // computed: any u32 but 2^32 - 1
+        else if (!t.var) { need = bitlen((u64)t.v + 1); top = t.v; }
         else
           for (auto& a : R.body)
             for (size_t q = 0; q < a.args.size(); q++)
-              if (a.args[q].var && a.args[q].v == t.v) need = std::max(need, e.rels[a.rel].width[q]);
+              if (a.args[q].var && a.args[q].v == t.v) {
+                need = std::max(need, e.rels[a.rel].width[q]);
+                top = std::max(top, e.rels[a.rel].maxv[q]);
+              }
         if (need > h.width[c]) { h.width[c] = need; changed = true; }
+        if (top > h.maxv[c]) { h.maxv[c] = top; changed = true; }
       }
     }
   }
@@ -1937,6 +1945,7 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
     load_views(e);
   }
   enable_dense(e);
+  LinearOut lin;
   int stratum = 0;  // the stratum being run (assign_strata)
   while (!bit_done) {
     if (k >= max_iters) { rc = LOB_E_MAXITER; break; }
@@ -1981,7 +1990,12 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
       e.stratum_begin.push_back(k + 1);
       continue;
     }
-    if (k == 1 && e.n_strata == 1) {  // the rest of the run as a device-driven graph, when it qualifies
+    if (k == 1 && e.n_strata == 1) {
+      run_linear(e, max_iters, s, lin);  // linear components, to their fixpoint
+      bool rest = !lin.taken;
+      for (auto& r : e.rels) rest = rest || r.n_recent;
+      if (!rest) break;
+      // the rest of the run as a device-driven graph, when it qualifies
       bool taken = false;
       const int r2 = run_device_loop(e, k, max_iters, s, &taken);
       if (taken) {
@@ -1989,6 +2003,11 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
         break;
       }
     }
+  }
+  if (lin.taken) {
+    k = std::max(k, lin.last);
+    if (lin.max_iter) rc = LOB_E_MAXITER;
+    linear_merge(e, k, lin);
   }
   for (auto& r : e.rels)
     if (r.keys_stale) materialize_keys(e, r, r.bitmap.as<u32>());

@@ -88,6 +88,7 @@ struct RelSt {
   bool in_has_tags = false, in_has_samples = false;
   std::vector<u64> in_chunks_tagged;  // (row_begin, row_end, tagged) triples flattened
   int width[kMaxArity] = {0};
+  u32 maxv[kMaxArity] = {0};  // no value of the column is larger
   std::vector<ViewSt> views;  // [0] = primary (identity permutation)
   DevBuf rkeys, rtags;        // recent (primary layout)
   u64 n_recent = 0;
@@ -110,6 +111,7 @@ struct RelSt {
   // (+)-added into dacc[key] and marked in dtouched instead of being written,
   // sorted and uniqued; the iteration's unique candidates are read out in key order
   bool dense = false;
+  bool finished = false;    // run to its fixpoint by the linear loop: the other loops leave it alone
   DevBuf dacc, dtouched;
   u64 last_cand = 0, last_new = 0, cand_iter = 0;
   // gradient routing of loaded rows
@@ -250,6 +252,7 @@ struct lob_engine {
   int state = 0;  // 0 loading, 1 ran
   int semiring = 0;
   int swidth = 0;
+  u32 max_sample = 0;
   bool ran_diff = false;
   u32 last_iter = 0;
   lob_stats stats{};

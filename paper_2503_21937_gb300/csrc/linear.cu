@@ -1,0 +1,711 @@
+// Linear recursion of tagged programs: every iteration after the first in one
+// cooperative launch.
+//
+// A derived relation whose recursive rules read one derived atom and one input
+// atom -- reach(y) :- reach(x), edge(x,y), the shape of the Pathfinder and grid
+// programs -- spends its time on launches: a 64 x 64 grid takes 187 iterations of
+// about 900 candidates each, and count / scan / partition / emit / read-out /
+// merge as separate kernels cost 45 to 80 us an iteration, whatever the number
+// of facts.  Such a relation needs none of the sorted arrays while it grows,
+// because nothing probes it.  Here it lives in dense arrays over its key space
+// (tag, first-appearance stamp, membership bitmap), an iteration's candidates
+// are (+)-added into an accumulator slot each and listed once when first
+// touched, and one step of the loop takes the list of iteration k:
+//     commit   candidate tag against the stored one (the relation's policy),
+//     expand   if new or improved, probe the input relation and (+)-add the
+//              products as candidates of iteration k + 1,
+// with accumulators and lists of alternating parity, so that a single grid
+// barrier separates the steps and the facts of each iteration are exactly those
+// of Algorithm 1's.  A key is listed once, so its commit has one owner.
+//
+// What bounds it: the chain of dependent accesses of a step (list entry,
+// accumulator, stored tag, offsets, matched fact, membership, accumulator) and
+// its barrier.  Relations of a few thousand keys therefore run in one block with
+// every array but the input relation in shared memory, where a step's barrier is
+// __syncthreads; larger ones in up to one block per SM on arrays in L2.  A
+// step's facts are spread over all warps before a warp takes a second one.
+//
+// Measured (GB300, fixpoint, graph of kernels before -> this): 64 x 64 grid,
+// diff-max-min, 300 iterations 25 -> 1.9 ms (1.5 in the loop, 5 us a step; 15 us
+// a step with its arrays in L2), diff-add-mult, 128 iterations 8.6 -> 1.0 ms;
+// reachability of 512 batched grids, 218 iterations 20 -> 4 ms.
+#include "linear.h"
+
+#include <algorithm>
+#include <cstring>
+
+#include "engine.h"
+#include "pjoin.h"
+#include "scan.cuh"
+
+namespace {
+
+constexpr int kLinThreads = 512;        // arrays in global memory
+constexpr int kLinShThreads = 1024;     // one block, arrays in shared memory
+constexpr u32 kLinShBytes = 210 * 1024; // shared memory those may take
+constexpr int kLinMaxArms = 8;
+constexpr int kLinMaxRels = 8;
+constexpr u64 kLinRelSlots = 1ull << 24;  // keys of one relation (dense arrays)
+constexpr u64 kLinMaxSlots = 1ull << 25;
+constexpr u32 kLinSpin = 1u << 26;     // barrier polls before giving up
+
+enum : int { LS_STOP = 0, LS_ITER, LS_CAND, LS_NEW, LS_ERR, LS_BAR, LS_LIST = 8, LS_FRESH = 12 };
+// LS_LIST + i: length of the list of step i mod 3; LS_FRESH + i * kLinMaxRels +
+// rel: the step's new facts (low half) and improved ones (high half); then per
+// relation |F| and |recent| at the end
+constexpr int LS_FULL = LS_FRESH + 3 * kLinMaxRels, LS_LAST = LS_FULL + kLinMaxRels;
+constexpr int kLinSlots = LS_LAST + kLinMaxRels;
+enum : u64 { LIN_FIXPOINT = 1, LIN_MAXITER = 2 };
+
+struct LinArm {
+  PStep P;
+  int drel, hrel;  // relation indexes within the component
+};
+struct LinArgs {
+  int n_rel, n_arm;
+  u32 slots;
+  u32 base[kLinMaxRels];   // a relation's first slot
+  const LinArm* arms;
+  void* acc[2];            // candidate tags by slot, all zero between uses
+  u32* touched[2];         // slots listed already
+  u32* list[2];
+  void* ftag;
+  u32* fstamp;             // add-mult: iteration of first appearance | clamped << 31
+  u32* fbits;              // membership
+  const u32* start;        // slots recent after iteration k0
+  u64 n_start;
+  u64 fcount[kLinMaxRels];  // |F| after iteration k0
+  u32 k0, max_iters;
+  u64* state;
+  u32* rec;                // add-mult: |recent| after iteration k at [(k - k0 - 1) * n_rel + rel]
+};
+
+LOB_DEV u64 lin_word(const void* p, int w64, u64 i) {
+  return w64 ? reinterpret_cast<const u64*>(p)[i] : (u64)reinterpret_cast<const u32*>(p)[i];
+}
+LOB_DEV u64 lin_pick(const POperand& o, u64 wi, u64 wv) {
+  if (o.word == 2) return o.cval;
+  return ((o.word ? wv : wi) >> o.shift) & (o.width >= 64 ? ~0ull : ((1ull << o.width) - 1ull));
+}
+LOB_DEV bool lin_checks(const PCheck* c, int n, u64 wi, u64 wv) {
+  bool ok = true;
+  for (int q = 0; q < n; q++) ok = ok && ((lin_pick(c[q].a, wi, wv) == lin_pick(c[q].b, wi, wv)) == (c[q].eq != 0));
+  return ok;
+}
+LOB_DEV u64 lin_lower(const void* keys, int key64, u64 n, u64 x) {
+  if (key64) return lower_bound_dev<u64>(reinterpret_cast<const u64*>(keys), 0, n, x);
+  if (x > 0xFFFFFFFFull) return n;
+  return lower_bound_dev<u32>(reinterpret_cast<const u32*>(keys), 0, n, (u32)x);
+}
+// the matches of input word wi in the arm's input relation
+LOB_DEV u32 lin_probe(const PStep& P, u64 wi, u32& lo) {
+  lo = 0;
+  if (P.n_in_checks && !lin_checks(P.in_checks, P.n_in_checks, wi, 0)) return 0;
+  u64 pv = 0;
+  for (int q = 0; q < P.n_prefix; q++) {
+    const u64 x = lin_pick(P.prefix[q].op, wi, 0);
+    if (P.prefix[q].limit_bits < 64 && (x >> P.prefix[q].limit_bits)) return 0;
+    pv |= x << P.prefix[q].shift;
+  }
+  u64 l, h;
+  if (P.index_mode == INDEX_DENSE) {
+    l = P.dense_offs[pv];
+    h = P.dense_offs[pv + 1];
+  } else if (P.index_mode == INDEX_HASH) {
+    hash_find(reinterpret_cast<const HashSlot*>(P.dense_offs), P.hash_bits, pv, l, h);
+  } else if (P.whole_view) {
+    l = 0;
+    h = P.v_n;
+  } else {
+    const u64 klo = pv << P.rest_shift, khi = klo + (1ull << P.rest_shift);
+    l = lin_lower(P.v_keys, P.v_key64, P.v_n, klo);
+    h = khi < klo ? P.v_n : lin_lower(P.v_keys, P.v_key64, P.v_n, khi);
+  }
+  lo = (u32)l;
+  return (u32)(h - l);
+}
+
+// All blocks of the launch, or false when one of them gave up waiting.  The
+// count only grows, so a late block can never see it reset.
+LOB_DEV bool lin_barrier(u64* state, u32& gen) {
+  __shared__ u32 ok;
+  __syncthreads();
+  if (gridDim.x == 1) return true;
+  if (threadIdx.x == 0) {
+    volatile u64* s = state;
+    __threadfence();
+    gen++;
+    atomicAdd(reinterpret_cast<unsigned long long*>(state) + LS_BAR, 1ull);
+    const u64 want = (u64)gen * gridDim.x;
+    u32 n = 0;
+    while (s[LS_BAR] < want && !s[LS_ERR] && n < kLinSpin) n++;
+    if (s[LS_BAR] < want) s[LS_ERR] = 1;
+    __threadfence();
+    ok = s[LS_ERR] == 0;
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+template <class T> LOB_DEV T lin_ld(const T* p) { return *reinterpret_cast<const volatile T*>(p); }
+
+// the loop's arrays, in global or shared memory
+template <class Sem>
+struct LinArrays {
+  typename Sem::Cand* acc[2];
+  u32 *touched[2], *list[2];
+  typename Sem::Stored* ftag;
+  u32 *fstamp, *fbits;
+  u64* state;
+};
+// bytes of the shared form, per slot and fixed (the state block)
+template <class Sem> constexpr u32 lin_slot_bytes() {
+  return 2 * (u32)sizeof(typename Sem::Cand) + (u32)sizeof(typename Sem::Stored) + 4 + 8;
+}
+LOB_HD u32 lin_shared_bytes(u32 slot_bytes, u32 slots) { return slots * slot_bytes + 3 * (slots / 8) + kLinSlots * 8; }
+
+template <class Sem, bool kSh>
+__global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(const __grid_constant__ LinArgs A) {
+  constexpr int kT = kSh ? kLinShThreads : kLinThreads;
+  typedef typename Sem::Stored S;
+  typedef typename Sem::Cand C;
+  __shared__ LinArm arms[kLinMaxArms];
+  __shared__ u32 fresh_sh[2][kLinMaxRels];  // new, improved
+  __shared__ unsigned long long cand_sh;
+  LinArrays<Sem> X;
+  if constexpr (kSh) {
+    extern __shared__ __align__(16) unsigned char sh[];
+    unsigned char* q = sh;
+    const u32 n = A.slots;
+    X.state = reinterpret_cast<u64*>(q); q += kLinSlots * 8;
+    for (int b = 0; b < 2; b++) { X.acc[b] = reinterpret_cast<C*>(q); q += (u64)n * sizeof(C); }
+    X.ftag = reinterpret_cast<S*>(q); q += (u64)n * sizeof(S);
+    X.fstamp = reinterpret_cast<u32*>(q); q += (u64)n * 4;
+    for (int b = 0; b < 2; b++) { X.list[b] = reinterpret_cast<u32*>(q); q += (u64)n * 4; }
+    for (int b = 0; b < 2; b++) { X.touched[b] = reinterpret_cast<u32*>(q); q += n / 8; }
+    X.fbits = reinterpret_cast<u32*>(q);
+    for (u32 i = threadIdx.x; i < n; i += kT) {
+      X.acc[0][i] = X.acc[1][i] = C(0);
+      X.ftag[i] = reinterpret_cast<const S*>(A.ftag)[i];
+      X.fstamp[i] = A.fstamp ? A.fstamp[i] : 0u;
+    }
+    for (u32 i = threadIdx.x; i < n / 32; i += kT) {
+      X.touched[0][i] = X.touched[1][i] = 0u;
+      X.fbits[i] = A.fbits[i];
+    }
+    for (u32 i = threadIdx.x; i < (u32)kLinSlots; i += kT) X.state[i] = 0;
+  } else {
+    for (int b = 0; b < 2; b++) {
+      X.acc[b] = reinterpret_cast<C*>(A.acc[b]);
+      X.touched[b] = A.touched[b];
+      X.list[b] = A.list[b];
+    }
+    X.ftag = reinterpret_cast<S*>(A.ftag);
+    X.fstamp = A.fstamp;
+    X.fbits = A.fbits;
+    X.state = A.state;
+  }
+  for (u32 i = threadIdx.x; i < A.n_arm * sizeof(LinArm) / 4; i += kT)
+    reinterpret_cast<u32*>(arms)[i] = reinterpret_cast<const u32*>(A.arms)[i];
+  if (threadIdx.x == 0) cand_sh = 0;
+  const int lane = threadIdx.x & 31;
+  const u64 warp = (u64)blockIdx.x * (kT / 32) + (threadIdx.x >> 5), nwarps = (u64)gridDim.x * (kT / 32);
+  u64* st = X.state;
+  unsigned long long* ast = reinterpret_cast<unsigned long long*>(st);
+  u32 gen = 0;
+  u64 cand = 0;
+  u64 fcount[kLinMaxRels];
+#pragma unroll
+  for (int r = 0; r < kLinMaxRels; r++) fcount[r] = r < A.n_rel ? A.fcount[r] : 0;
+  // step 0 expands the facts recent after iteration k0; step j > 0 commits the
+  // candidates of iteration k0 + j and expands what is new
+  for (u32 step = 0;; step++) {
+    const u32 k = A.k0 + step;
+    const int par = step & 1, rot = step % 3;
+    const bool commit = step > 0;
+    if (threadIdx.x < 2 * kLinMaxRels) (&fresh_sh[0][0])[threadIdx.x] = 0;
+    __syncthreads();
+    const u32* list = commit ? X.list[par] : A.start;
+    const u64 n = commit ? lin_ld(st + LS_LIST + rot) : A.n_start;
+    u32* out_list = X.list[par ^ 1];
+    const bool expand = k < A.max_iters;
+    const u64 per = min(32ull, (n + nwarps - 1) / nwarps);  // facts a warp takes at a time
+    for (u64 i0 = warp * per; i0 < n; i0 += nwarps * per) {
+      const bool in = lane < (int)per && i0 + lane < n;
+      u32 slot = 0;
+      int rel = -1;
+      S tag{};
+      bool fresh = false;
+      if (in) {
+        slot = commit ? lin_ld(list + i0 + lane) : list[i0 + lane];
+        rel = 0;
+        while (rel + 1 < A.n_rel && slot >= A.base[rel + 1]) rel++;
+        S* f = X.ftag + slot;
+        if (commit) {
+          C* a = X.acc[par] + slot;
+          const C c = lin_ld(a);
+          *reinterpret_cast<volatile C*>(a) = C(0);
+          const u32 bit = 1u << (slot & 31u);
+          atomicAnd(X.touched[par] + (slot >> 5), ~bit);
+          tag = Sem::store(c);
+          const bool present = lin_ld(X.fbits + (slot >> 5)) & bit;
+          if (!present) {
+            fresh = true;
+            if constexpr (std::is_same<Sem, SemAddMult>::value)
+              *reinterpret_cast<volatile u32*>(X.fstamp + slot) = k | (c > 1.0 ? 0x80000000u : 0u);
+            *reinterpret_cast<volatile S*>(f) = tag;
+            atomicOr(X.fbits + (slot >> 5), bit);
+            atomicAdd(&fresh_sh[0][rel], 1u);
+          } else if (Sem::kIdempotent && Sem::better(tag, lin_ld(f))) {
+            fresh = true;
+            *reinterpret_cast<volatile S*>(f) = tag;
+            atomicAdd(&fresh_sh[1][rel], 1u);
+          }
+        } else {
+          tag = lin_ld(f);
+          fresh = true;
+        }
+      }
+      if (!expand) continue;
+      const u64 wi = in ? (u64)slot - A.base[rel] : 0ull;
+      const C ct = Sem::from_stored(tag);
+      for (int a = 0; a < A.n_arm; a++) {
+        const LinArm& arm = arms[a];
+        const PStep& P = arm.P;
+        u32 lo = 0;
+        const u32 c = fresh && arm.drel == rel ? lin_probe(P, wi, lo) : 0u;
+        const u32 inc = warp_inclusive_sum(c);
+        const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+        if (!tot) continue;
+        cand += tot;
+        const u32 ex = inc - c;
+        const u32 hbase = A.base[arm.hrel];
+        for (u32 t0 = 0; t0 < tot; t0 += 32) {
+          const u32 t = t0 + lane;
+          int src = 0;  // the last lane whose outputs start at or before t
+#pragma unroll
+          for (int s = 16; s; s >>= 1) {
+            const u32 x = __shfl_sync(0xFFFFFFFFu, ex, src + s);
+            if (x <= t) src += s;
+          }
+          const u64 wr = __shfl_sync(0xFFFFFFFFu, wi, src);
+          const u32 lr = __shfl_sync(0xFFFFFFFFu, lo, src);
+          const u32 er = __shfl_sync(0xFFFFFFFFu, ex, src);
+          const C tr = __shfl_sync(0xFFFFFFFFu, ct, src);
+          bool add = false;
+          u32 hs = 0;
+          if (t < tot) {
+            const u64 v = (u64)lr + (t - er);
+            const u64 wv = lin_word(P.v_keys, P.v_key64, v);
+            if (lin_checks(P.checks, P.n_checks, wr, wv)) {
+              u64 w = 0;
+              for (int q = 0; q < P.n_out; q++) w |= lin_pick(P.out[q].op, wr, wv) << P.out[q].shift;
+              hs = hbase + (u32)w;
+              const u32 bit = 1u << (hs & 31u);
+              const C prod = Sem::mul(tr, Sem::from_stored(reinterpret_cast<const S*>(P.v_tags)[v]));
+              // A candidate that cannot change the stored tag is dropped here: a
+              // fact that is present stays present, and a tag only grows.  Facts
+              // being committed in this step may be seen or not (a tag not yet
+              // seen reads 0): their own commit of this candidate decides then.
+              bool useless = lin_ld(X.fbits + (hs >> 5)) & bit;
+              if constexpr (Sem::kIdempotent) useless = useless && lin_ld(X.ftag + hs) >= Sem::store(prod);
+              if (!useless) {
+                dense_add<Sem>(X.acc[par ^ 1], hs, prod);
+                u32* tw = X.touched[par ^ 1] + (hs >> 5);
+                if (!(lin_ld(tw) & bit)) add = !(atomicOr(tw, bit) & bit);
+              }
+            }
+          }
+          const u32 m = __ballot_sync(0xFFFFFFFFu, add);
+          if (m) {
+            u64 at = 0;
+            if (lane == 0) at = atomicAdd(ast + LS_LIST + (step + 1) % 3, (unsigned long long)__popc(m));
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
+            if (add) *reinterpret_cast<volatile u32*>(out_list + at + __popc(m & ((1u << lane) - 1u))) = hs;
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < A.n_rel && (fresh_sh[0][threadIdx.x] | fresh_sh[1][threadIdx.x]))
+      atomicAdd(ast + LS_FRESH + rot * kLinMaxRels + threadIdx.x,
+                ((unsigned long long)fresh_sh[1][threadIdx.x] << 32) | fresh_sh[0][threadIdx.x]);
+    // Counters of steps to come.  The list length read in the last step is done
+    // with; the new-fact counts of the last step may still be read by a slow
+    // block, those of the step before may not.
+    if (blockIdx.x == 0 && threadIdx.x <= kLinMaxRels) {
+      if (threadIdx.x == kLinMaxRels) st[LS_LIST + (step + 2) % 3] = 0;
+      else st[LS_FRESH + ((step + 1) % 3) * kLinMaxRels + threadIdx.x] = 0;
+    }
+    if (!lin_barrier(st, gen)) break;
+    if (!commit) continue;
+    u64 total = 0;
+#pragma unroll
+    for (int r = 0; r < kLinMaxRels; r++) {
+      if (r >= A.n_rel) break;
+      const u64 v = lin_ld(st + LS_FRESH + rot * kLinMaxRels + r);
+      const u64 added = v & 0xFFFFFFFFull, improved = v >> 32;
+      fcount[r] += added;
+      total += added + improved;
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (A.rec) A.rec[(u64)(step - 1) * A.n_rel + r] = (u32)added;
+        st[LS_FULL + r] = fcount[r];
+        st[LS_LAST + r] = added + improved;
+      }
+    }
+    const u64 stop = !total ? LIN_FIXPOINT : k >= A.max_iters ? LIN_MAXITER : 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      st[LS_NEW] += total;
+      st[LS_ITER] = k;
+      st[LS_STOP] = stop;
+    }
+    if (stop) break;
+  }
+  // join outputs, summed per warp (every lane holds its warp's count)
+  __syncthreads();
+  if (lane == 0 && cand) atomicAdd(&cand_sh, (unsigned long long)cand);
+  __syncthreads();
+  if (threadIdx.x == 0 && cand_sh) atomicAdd(ast + LS_CAND, cand_sh);
+  if constexpr (kSh) {
+    __syncthreads();
+    for (u32 i = threadIdx.x; i < A.slots; i += kT) {
+      reinterpret_cast<S*>(A.ftag)[i] = X.ftag[i];
+      if (A.fstamp) A.fstamp[i] = X.fstamp[i];
+    }
+    for (u32 i = threadIdx.x; i < A.slots / 32; i += kT) A.fbits[i] = X.fbits[i];
+    for (u32 i = threadIdx.x; i < (u32)kLinSlots; i += kT) A.state[i] = X.state[i];
+  }
+}
+
+// facts present after iteration 1: tag, stamp and membership by slot
+template <class S>
+__global__ void k_lin_init(const void* __restrict__ keys, int key64, const S* __restrict__ tags,
+                           const u32* __restrict__ stamps, u64 n, u32 base, S* __restrict__ ftag, u32* __restrict__ fstamp,
+                           u32* __restrict__ fbits) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const u32 s = base + (u32)load_key(keys, key64, i);
+    ftag[s] = tags[i];
+    if (stamps) fstamp[s] = stamps[i];
+    atomicOr(fbits + (s >> 5), 1u << (s & 31u));
+  }
+}
+__global__ void k_lin_slots(const void* __restrict__ keys, int key64, u64 n, u32 base, u32* __restrict__ out) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = base + (u32)load_key(keys, key64, i);
+}
+// tags and stamps of the sorted keys
+template <class S>
+__global__ void k_lin_collect(const void* __restrict__ keys, int key64, u64 n, u32 base, const S* __restrict__ ftag,
+                              const u32* __restrict__ fstamp, S* __restrict__ tags, u32* __restrict__ stamps) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const u32 s = base + (u32)load_key(keys, key64, i);
+    tags[i] = ftag[s];
+    if (stamps) stamps[i] = fstamp[s];
+  }
+}
+
+// Slots of a relation's key space: one more than its largest possible key, in
+// whole 16-byte pieces of the bitmaps.
+u64 lin_slots(const lob_engine& e, const RelSt& r) {
+  const Layout& L = r.views[0].lay;
+  if (L.bits > 40) return ~0ull >> 8;
+  u64 top = L.swidth ? (u64)e.max_sample << L.sshift : 0ull;
+  for (int j = 0; j < L.arity; j++) top += (u64)r.maxv[j] << L.shift[j];
+  return (top + 128) & ~127ull;
+}
+unsigned lin_grid(u64 n) { return (unsigned)std::max<u64>(1, std::min<u64>((n + 255) / 256, 152ull * 16)); }
+
+struct LinRun {
+  lob_engine& e;
+  std::vector<u32> rels;
+  std::vector<int> index;  // relation id -> index in rels, or -1
+  explicit LinRun(lob_engine& en) : e(en) {}
+  DevBuf arms, acc[2], touched[2], list[2], ftag, fstamp, fbits, start, state, rec;
+  ~LinRun() {
+    for (DevBuf* b : {&arms, &acc[0], &acc[1], &touched[0], &touched[1], &list[0], &list[1], &ftag, &fstamp, &fbits, &start,
+                      &state, &rec})
+      e.release(*b);
+  }
+
+  template <class Sem>
+  void launch(const LinArgs& A, unsigned blocks) {
+    void* args[] = {const_cast<LinArgs*>(&A)};
+    const u32 sh = lin_shared_bytes(lin_slot_bytes<Sem>(), A.slots);
+    if (sh <= kLinShBytes && blocks == 1) {
+      e.check(allow_dynamic_smem(k_linear<Sem, true>, (int)sh), "linear loop");
+      ProfScope ps("linear_loop", 0, e.stream);
+      k_linear<Sem, true><<<1, kLinShThreads, sh, e.stream>>>(A);
+    } else {
+      ProfScope ps("linear_loop", 0, e.stream);
+      e.check(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_linear<Sem, false>), dim3(blocks), dim3(kLinThreads), args, 0,
+                                          e.stream), "linear loop");
+    }
+    e.after_launch("linear loop");
+    e.launches++;
+  }
+  template <class S>
+  void init(const RelSt& R, u32 base) {
+    const ViewSt& V = R.views[0];
+    if (V.n)
+      k_lin_init<S><<<lin_grid(V.n), 256, 0, e.stream>>>(V.keys.p, V.lay.key64, V.tags.as<S>(),
+                                                         fstamp.p ? V.stamps.as<u32>() : nullptr, V.n, base, ftag.as<S>(),
+                                                         fstamp.as<u32>(), fbits.as<u32>());
+    e.after_launch("linear facts");
+    e.launches++;
+  }
+  template <class S>
+  void collect(RelSt& R, u32 base) {
+    ViewSt& V = R.views[0];
+    k_lin_collect<S><<<lin_grid(V.n), 256, 0, e.stream>>>(V.keys.p, V.lay.key64, V.n, base, ftag.as<S>(), fstamp.as<u32>(),
+                                                          V.tags.as<S>(), fstamp.p ? V.stamps.as<u32>() : nullptr);
+    e.after_launch("linear result");
+    e.launches++;
+  }
+};
+
+}  // namespace
+
+// The derived relations whose component (relations that rules connect) is
+// linear: dense, in all their rules at most one derived atom, which is then
+// joined with one input relation by a packed step, and, where views carry
+// stamps, no secondary view to keep.  False when there are none.
+bool linear_component(const lob_engine& e, std::vector<char>& in) {
+  const size_t n = e.rels.size();
+  in.assign(n, 0);
+  if (e.semiring == SR_UNIT || sem_top1(e.semiring) || e.n_strata != 1) return false;
+  std::vector<int> comp(n);
+  for (size_t r = 0; r < n; r++) comp[r] = (int)r;
+  std::vector<char> bad(n, 0);
+  std::vector<int> n_arms(n, 0);
+  auto join = [&](int a, int b) {
+    const int x = comp[a], y = comp[b];
+    for (auto& c : comp)
+      if (c == y) c = x;
+  };
+  for (auto& p : e.plans)
+    for (auto& a : p.ast.body)
+      if (e.rels[a.rel].idb) join((int)p.ast.head.rel, (int)a.rel);
+  for (size_t r = 0; r < n; r++) {
+    const RelSt& R = e.rels[r];
+    if (!R.idb) continue;
+    if (!R.dense || lin_slots(e, R) > kLinRelSlots || (sem_stamps(e.semiring) && R.views.size() > 1)) bad[comp[r]] = 1;
+  }
+  for (auto& p : e.plans) {
+    int derived = 0;
+    for (auto& a : p.ast.body) derived += e.rels[a.rel].idb;
+    if (!derived) continue;
+    const int c = comp[p.ast.head.rel];
+    if (derived > 1 || p.ast.body.size() != 2) bad[c] = 1;
+    for (auto& A : p.arms)
+      if (e.rels[p.ast.body[A.delta].rel].idb) {
+        n_arms[c]++;
+        if (!A.packed.ok || A.steps.size() != 2) bad[c] = 1;
+      }
+  }
+  bool any = false;
+  int rels = 0, arms = 0;
+  u64 slots = 0;
+  for (size_t c = 0; c < n; c++) {
+    if (bad[c] || !n_arms[c]) continue;
+    u64 s = 0;
+    int m = 0;
+    for (size_t r = 0; r < n; r++)
+      if (e.rels[r].idb && comp[r] == (int)c) {
+        s += lin_slots(e, e.rels[r]);
+        m++;
+      }
+    if (rels + m > kLinMaxRels || arms + n_arms[c] > kLinMaxArms || slots + s > kLinMaxSlots) continue;
+    rels += m;
+    arms += n_arms[c];
+    slots += s;
+    for (size_t r = 0; r < n; r++)
+      if (e.rels[r].idb && comp[r] == (int)c) in[r] = any = true;
+  }
+  return any;
+}
+
+void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
+  const u32 k0 = 1;
+  std::vector<char> in;
+  if (!e.opt_driver || k0 >= max_iters || !linear_component(e, in)) return;
+  if (e.opt_driver == 1 && !e.loop_caps.count("linear_history")) {
+    // as for the device-driven graph: the first run of an engine is host-driven
+    e.loop_caps["linear_history"] = 1;
+    return;
+  }
+  LinRun L(e);
+  L.index.assign(e.rels.size(), -1);
+  LinArgs A;
+  std::memset(&A, 0, sizeof(A));
+  u64 slots = 0, recent = 0, probed = 0;
+  for (size_t r = 0; r < e.rels.size(); r++) {
+    if (!in[r]) continue;
+    L.index[r] = A.n_rel;
+    A.base[A.n_rel] = (u32)slots;
+    A.fcount[A.n_rel++] = e.rels[r].views[0].n;
+    slots += lin_slots(e, e.rels[r]);
+    recent += e.rels[r].n_recent;
+    L.rels.push_back((u32)r);
+  }
+  if (!recent) return;
+  std::vector<LinArm> arms;
+  for (auto& p : e.plans)
+    for (auto& Ar : p.arms) {
+      const u32 drel = p.ast.body[Ar.delta].rel;
+      if (L.index[p.ast.head.rel] < 0 || !e.rels[drel].idb) continue;
+      const StepPlan& S = Ar.steps[1];
+      ViewSt& W = e.rels[p.ast.body[S.atom].rel].views[S.view];
+      if (W.n > 0x7FFFFFFull) return;  // 32 rows' outputs stay below 2^32
+      LinArm a;
+      std::memset(&a, 0, sizeof(a));
+      a.P = Ar.packed.steps[0];
+      a.drel = L.index[drel];
+      a.hrel = L.index[p.ast.head.rel];
+      if (!W.n) continue;
+      engine_ensure_index(e, W, S.prefix_len);
+      a.P.v_keys = W.keys.p;
+      a.P.v_key64 = W.lay.key64;
+      a.P.v_tags = W.tags.p;
+      a.P.v_n = W.n;
+      const IndexSt& I = W.index[S.prefix_len];
+      a.P.index_mode = I.mode;
+      a.P.dense_offs = I.offs.as<u64>();
+      a.P.hash_bits = I.hash_bits;
+      probed += W.n;
+      arms.push_back(a);
+    }
+  const int ks = sem_kernel(e.semiring);
+  const int sb = stored_bytes(e.semiring), cb = cand_bytes(e.semiring);
+  const bool stamps = sem_stamps(e.semiring);
+  e.ensure(L.arms, std::max<size_t>(arms.size(), 1) * sizeof(LinArm));
+  if (!arms.empty())
+    e.check(cudaMemcpyAsync(L.arms.p, arms.data(), arms.size() * sizeof(LinArm), cudaMemcpyHostToDevice, e.stream), "arms");
+  for (int b = 0; b < 2; b++) {
+    e.ensure(L.acc[b], slots * cb);
+    e.check(cudaMemsetAsync(L.acc[b].p, 0, slots * cb, e.stream), "accumulators");
+    e.ensure(L.touched[b], slots / 8);
+    e.check(cudaMemsetAsync(L.touched[b].p, 0, slots / 8, e.stream), "accumulators");
+    e.ensure(L.list[b], slots * 4);
+  }
+  e.ensure(L.ftag, slots * sb);
+  e.check(cudaMemsetAsync(L.ftag.p, 0, slots * sb, e.stream), "tags");
+  if (stamps) e.ensure(L.fstamp, slots * 4);
+  e.ensure(L.fbits, slots / 8);
+  e.check(cudaMemsetAsync(L.fbits.p, 0, slots / 8, e.stream), "membership");
+  e.ensure(L.start, recent * 4);
+  e.ensure(L.state, kLinSlots * 8);
+  // an add-mult iteration that is not the last adds a fact, so there are at most
+  // as many as slots; the other semirings' backward passes need no record
+  if (stamps) e.ensure(L.rec, (slots + 1) * A.n_rel * 4);
+  u64 at = 0;
+  for (int q = 0; q < A.n_rel; q++) {
+    RelSt& R = e.rels[L.rels[q]];
+    if (sb == 8) L.init<u64>(R, A.base[q]);
+    else L.init<float>(R, A.base[q]);
+    if (R.n_recent) {
+      k_lin_slots<<<lin_grid(R.n_recent), 256, 0, e.stream>>>(R.rkeys.p, R.views[0].lay.key64, R.n_recent, A.base[q],
+                                                              L.start.as<u32>() + at);
+      e.after_launch("linear facts");
+      e.launches++;
+    }
+    at += R.n_recent;
+  }
+  A.n_arm = (int)arms.size();
+  A.arms = L.arms.as<LinArm>();
+  for (int b = 0; b < 2; b++) {
+    A.acc[b] = L.acc[b].p;
+    A.touched[b] = L.touched[b].as<u32>();
+    A.list[b] = L.list[b].as<u32>();
+  }
+  A.ftag = L.ftag.p;
+  A.fstamp = L.fstamp.as<u32>();
+  A.fbits = L.fbits.as<u32>();
+  A.start = L.start.as<u32>();
+  A.n_start = recent;
+  A.max_iters = max_iters;
+  A.state = L.state.as<u64>();
+  A.rec = L.rec.as<u32>();
+  // A block per 16,384 probed rows: a grid of side 64 has about 200 recent facts
+  // in an iteration, which one block expands in a round or two without a grid
+  // barrier.
+  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(152, probed / 16384));
+  A.k0 = k0;
+  A.slots = (u32)slots;
+  std::vector<u64> h(kLinSlots, 0);
+  e.check(cudaMemsetAsync(L.state.p, 0, kLinSlots * 8, e.stream), "linear state");
+  switch (ks) {
+    case SR_MAX_MIN: L.launch<SemMaxMin>(A, blocks); break;
+    case SR_DIFF_MAX_MIN: L.launch<SemDiffMaxMin>(A, blocks); break;
+    default: L.launch<SemAddMult>(A, blocks); break;
+  }
+  e.check(cudaMemcpyAsync(h.data(), L.state.p, kLinSlots * 8, cudaMemcpyDeviceToHost, e.stream), "linear state");
+  e.sync();
+  if (h[LS_ERR]) throw LobError(LOB_E_TIMEOUT, "a bounded wait of the linear loop gave up; the run's results are invalid");
+  if (h[LS_STOP] != LIN_FIXPOINT && h[LS_STOP] != LIN_MAXITER)
+    throw LobError(LOB_E_CUDA, "internal error: linear loop stopped without a reason");
+  const u32 ran = (u32)h[LS_ITER] - k0;
+  std::vector<u32> rec(stamps ? (u64)ran * A.n_rel : 0);
+  if (stamps)
+    e.check(cudaMemcpyAsync(rec.data(), L.rec.p, rec.size() * 4, cudaMemcpyDeviceToHost, e.stream), "linear record");
+  if (stamps) e.sync();
+  out.first = k0 + 1;
+  out.last = k0 + ran;
+  out.max_iter = h[LS_STOP] == LIN_MAXITER;
+  for (u32 i = 0; i < ran; i++) {  // counts at the start of iteration k0 + 1 + i
+    out.counts.emplace_back();
+    for (int q = 0; q < A.n_rel; q++) {
+      const u64 last = i ? (stamps ? rec[(u64)(i - 1) * A.n_rel + q] : 0) : e.rels[L.rels[q]].n_recent;
+      const u64 full = i ? out.counts[i - 1][q].first + (stamps ? last : 0) : A.fcount[q];
+      out.counts.back().emplace_back(full, last);
+    }
+  }
+  s.graph_launches++;
+  s.device_iterations += ran;
+  s.new_facts += h[LS_NEW];
+  e.cand_emitted += h[LS_CAND];
+  // the relations in key order again
+  for (int q = 0; q < A.n_rel; q++) {
+    RelSt& R = e.rels[L.rels[q]];
+    ViewSt& V = R.views[0];
+    const u64 n = h[LS_FULL + q], nbits = lin_slots(e, R);
+    out.rels.push_back(L.rels[q]);
+    out.n_recent.push_back(h[LS_LAST + q]);
+    R.n_recent = 0;
+    R.finished = true;
+    for (auto& kv : V.index) kv.second.valid = false;
+    for (size_t vi = 1; vi < R.views.size(); vi++) R.views[vi].stale = true;
+    const u32* bits = L.fbits.as<u32>() + A.base[q] / 32;
+    const int kb = V.lay.key64 ? 8 : 4;
+    e.ensure(e.scratch, bits_scratch_bytes(nbits));
+    e.launches += bits_count(bits, nullptr, nbits, e.scratch.p, e.counts.as<u64>() + 1, e.stream);
+    e.after_launch("linear result");
+    e.ensure(V.keys, n * kb);
+    e.ensure(V.tags, n * sb);
+    if (stamps) e.ensure(V.stamps, n * 4);
+    bits_extract(bits, nullptr, nbits, V.lay.key64, V.keys.p, n, e.scratch.p, e.stream);
+    e.after_launch("linear result");
+    e.launches++;
+    V.n = n;
+    if (sb == 8) L.collect<u64>(R, A.base[q]);
+    else L.collect<float>(R, A.base[q]);
+  }
+  out.taken = true;
+}
+
+void linear_merge(lob_engine& e, u32 k, const LinearOut& out) {
+  if (!out.taken) return;
+  const size_t nrel = e.rels.size();
+  while (e.iter_counts.size() < k) {  // iterations only the linear components ran: the rest is at rest
+    e.iter_counts.emplace_back();
+    for (size_t r = 0; r < nrel; r++) e.iter_counts.back().emplace_back(e.rels[r].views[0].n, 0);
+  }
+  for (size_t q = 0; q < out.rels.size(); q++) {
+    const u32 r = out.rels[q];
+    for (u32 it = out.first; it <= k; it++)
+      e.iter_counts[it - 1][r] = it <= out.last ? out.counts[it - out.first][q]
+                                                : std::make_pair((u64)e.rels[r].views[0].n, (u64)0);
+    e.rels[r].n_recent = out.max_iter ? out.n_recent[q] : 0;
+  }
+}
