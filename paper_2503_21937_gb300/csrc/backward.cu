@@ -22,6 +22,7 @@
 #include <cstring>
 
 #include "engine.h"
+#include "linear.h"
 #include "pjoin.h"
 #include "join_common.cuh"
 #include "scan.cuh"
@@ -704,9 +705,23 @@ int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* con
         if (begins_stratum(e->stratum_begin, k + 1)) return 0;
         return k < e->iter_counts.size() ? e->iter_counts[k][rel].second : e->rels[rel].n_recent;
       };
+      // Linear components whose head is needed replay in one launch (linear.cu),
+      // down to iteration 2.  They feed no other component, and what they add to
+      // the inputs' adjoints is read at the end.
+      std::vector<char> linear(nrel, 0);
+      {
+        LinearAdjoints J;
+        for (size_t q = 0; q < nrel; q++) {
+          J.adj.push_back(S.adj[q].as<double>());
+          J.hrow.push_back(S.hrow[q].as<u32>());
+          J.prow.emplace_back();
+          for (auto& b : S.prow[q]) J.prow.back().push_back(b.as<u32>());
+        }
+        if (!linear_backward(*e, J, linear)) linear.assign(nrel, 0);
+      }
       for (u32 k = e->last_iter; k >= 1; k--) {
         for (size_t q = 0; q < nrel; q++) {  // the heads new in iteration k
-          if (!S.hnew[q].p || !needed[q] || !new_in(k, (u32)q)) continue;
+          if (!S.hnew[q].p || !needed[q] || (linear[q] && k > 1) || !new_in(k, (u32)q)) continue;
           RelSt& r = e->rels[q];
           e->check(cudaMemsetAsync(S.hnew[q].p, 0, S.hnew[q].cap, e->stream), "new heads");
           k_mark_new<<<grid_for_n(r.views[0].n), 256, 0, e->stream>>>(r.views[0].keys.p, r.views[0].lay.key64,
@@ -719,6 +734,7 @@ int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* con
           for (auto& A : p.arms) {
             if (p.stratum != stratum) continue;  // the rule did not run in iteration k
             if (!needed[p.ast.head.rel] || !new_in(k, p.ast.head.rel)) continue;  // no adjoint can flow here
+            if (linear[p.ast.head.rel] && k > 1) continue;
             const auto& cnt = e->iter_counts[k - 1];  // (total, recent) per relation at the start of iteration k
             if (!cnt[p.ast.body[A.delta].rel].second) continue;
             bool skip = false;

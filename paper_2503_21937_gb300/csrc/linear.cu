@@ -25,10 +25,9 @@
 // __syncthreads; larger ones in up to one block per SM on arrays in L2.  A
 // step's facts are spread over all warps before a warp takes a second one.
 //
-// Measured (GB300, fixpoint, graph of kernels before -> this): 64 x 64 grid,
-// diff-max-min, 300 iterations 25 -> 1.9 ms (1.5 in the loop, 5 us a step; 15 us
-// a step with its arrays in L2), diff-add-mult, 128 iterations 8.6 -> 1.0 ms;
-// reachability of 512 batched grids, 218 iterations 20 -> 4 ms.
+// Measured (GB300): 64 x 64 grid, diff-add-mult, fixpoint of 128 iterations 8.6
+// -> 1.0 ms; diff-max-min, forward and backward 11.1 -> 1.8 ms.  A step takes 5
+// us (15 with the arrays in L2), an iteration of the graph of kernels 67.
 #include "linear.h"
 
 #include <algorithm>
@@ -377,6 +376,127 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
   }
 }
 
+// ---------------------------------------------------------------------------
+// Backward pass of diff-add-mult over the linear components.  A fact first
+// derived in iteration s is the recent fact of its groundings in iteration s +
+// 1 only, so the facts sorted by stamp are the replay: one step per stamp, from
+// the last to 1, expands the facts of stamp s and takes from each head of stamp
+// s + 1 (whose adjoint is complete) its share, with a grid barrier between the
+// steps.  The replay of one iteration as count / scan / partition / emit with a
+// host wait took 55 us whatever its size; a step takes about 3.
+// ---------------------------------------------------------------------------
+struct LinBwdArm {
+  PStep P;
+  int drel, hrel;
+  const u32* prow;  // probed view row -> primary row (null: the primary view)
+  double* vadj;     // adjoints of the probed relation (null: none needed)
+};
+struct LinBwdRel {
+  const void* keys;
+  int key64;
+  const float* tags;
+  const u32* stamps;
+  const u32* hrow;  // key -> row
+  double* adj;
+  u32 base;         // the relation's first entry number
+};
+struct LinBwdArgs {
+  int n_rel, n_arm;
+  LinBwdRel rel[kLinMaxRels];
+  const LinBwdArm* arms;
+  const u32* entries;  // base + row, by stamp
+  const u32* off;      // a stamp's first entry
+  u32 last;            // iterations of the run
+  u64* state;
+};
+
+__global__ void __launch_bounds__(kLinThreads) k_linear_backward(const __grid_constant__ LinBwdArgs A) {
+  __shared__ LinBwdArm arms[kLinMaxArms];
+  for (u32 i = threadIdx.x; i < A.n_arm * sizeof(LinBwdArm) / 4; i += kLinThreads)
+    reinterpret_cast<u32*>(arms)[i] = reinterpret_cast<const u32*>(A.arms)[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const u64 warp = (u64)blockIdx.x * (kLinThreads / 32) + (threadIdx.x >> 5), nwarps = (u64)gridDim.x * (kLinThreads / 32);
+  u32 gen = 0;
+  for (u32 s = A.last - 1; s >= 1; s--) {
+    const u32 first = A.off[s];
+    const u64 n = A.off[s + 1] - first;
+    if (!n) continue;
+    const u64 per = min(32ull, (n + nwarps - 1) / nwarps);
+    for (u64 i0 = warp * per; i0 < n; i0 += nwarps * per) {
+      const bool in = lane < (int)per && i0 + lane < n;
+      int rel = -1;
+      u32 row = 0;
+      u64 wi = 0;
+      double tag = 0.0;
+      if (in) {
+        const u32 x = A.entries[first + i0 + lane];
+        rel = 0;
+        while (rel + 1 < A.n_rel && x >= A.rel[rel + 1].base) rel++;
+        row = x - A.rel[rel].base;
+        wi = lin_word(A.rel[rel].keys, A.rel[rel].key64, row);
+        tag = (double)A.rel[rel].tags[row];
+      }
+      for (int a = 0; a < A.n_arm; a++) {
+        const LinBwdArm& arm = arms[a];
+        const PStep& P = arm.P;
+        const LinBwdRel& H = A.rel[arm.hrel];
+        double* dadj = A.rel[arm.drel].adj;
+        u32 lo = 0;
+        const u32 c = in && arm.drel == rel ? lin_probe(P, wi, lo) : 0u;
+        const u32 inc = warp_inclusive_sum(c);
+        const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+        const u32 ex = inc - c;
+        for (u32 t0 = 0; t0 < tot; t0 += 32) {
+          const u32 t = t0 + lane;
+          int src = 0;  // the last lane whose outputs start at or before t
+#pragma unroll
+          for (int q = 16; q; q >>= 1) {
+            const u32 x = __shfl_sync(0xFFFFFFFFu, ex, src + q);
+            if (x <= t) src += q;
+          }
+          const u64 wr = __shfl_sync(0xFFFFFFFFu, wi, src);
+          const u32 lr = __shfl_sync(0xFFFFFFFFu, lo, src);
+          const u32 er = __shfl_sync(0xFFFFFFFFu, ex, src);
+          const u32 rr = __shfl_sync(0xFFFFFFFFu, row, src);
+          const double tr = __shfl_sync(0xFFFFFFFFu, tag, src);
+          if (t >= tot) continue;
+          const u64 v = (u64)lr + (t - er);
+          const u64 wv = lin_word(P.v_keys, P.v_key64, v);
+          if (!lin_checks(P.checks, P.n_checks, wr, wv)) continue;
+          u64 w = 0;
+          for (int q = 0; q < P.n_out; q++) w |= lin_pick(P.out[q].op, wr, wv) << P.out[q].shift;
+          const u32 h = H.hrow[w];
+          // not new in iteration s + 1, or its sum was clamped (bit 31)
+          if (h == 0xFFFFFFFFu || H.stamps[h] != s + 1) continue;
+          const double adj = lin_ld(H.adj + h);
+          if (adj == 0.0) continue;
+          atomicAdd(dadj + rr, adj * (double)reinterpret_cast<const float*>(P.v_tags)[v]);
+          if (arm.vadj) atomicAdd(arm.vadj + (arm.prow ? arm.prow[v] : (u32)v), adj * tr);
+        }
+      }
+    }
+    if (!lin_barrier(A.state, gen)) return;
+  }
+}
+
+// facts by stamp: stamps 1 .. last - 1 (later ones are never a recent fact)
+__global__ void k_lin_stamp_count(const u32* __restrict__ stamps, u64 n, u32 last, u32* __restrict__ cnt) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const u32 s = stamps[i] & 0x7FFFFFFFu;
+    if (s >= 1 && s < last) atomicAdd(cnt + s, 1u);
+  }
+}
+__global__ void k_lin_stamp_fill(const u32* __restrict__ stamps, u64 n, u32 last, u32 base, const u32* __restrict__ off,
+                                 u32* __restrict__ used, u32* __restrict__ out) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const u32 s = stamps[i] & 0x7FFFFFFFu;
+    if (s >= 1 && s < last) out[off[s] + atomicAdd(used + s, 1u)] = base + (u32)i;
+  }
+}
+
 // facts present after iteration 1: tag, stamp and membership by slot
 template <class S>
 __global__ void k_lin_init(const void* __restrict__ keys, int key64, const S* __restrict__ tags,
@@ -708,4 +828,105 @@ void linear_merge(lob_engine& e, u32 k, const LinearOut& out) {
                                                 : std::make_pair((u64)e.rels[r].views[0].n, (u64)0);
     e.rels[r].n_recent = out.max_iter ? out.n_recent[q] : 0;
   }
+}
+
+bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in) {
+  if (!e.opt_packed_backward || !linear_component(e, in)) return false;
+  const u32 last = e.last_iter;
+  LinRun L(e);
+  L.index.assign(e.rels.size(), -1);
+  LinBwdArgs A;
+  std::memset(&A, 0, sizeof(A));
+  u64 rows = 0, probed = 0;
+  for (size_t r = 0; r < e.rels.size(); r++) {
+    if (!in[r]) continue;
+    const ViewSt& V = e.rels[r].views[0];
+    if (V.n && !J.hrow[r]) return false;
+    L.index[r] = A.n_rel;
+    LinBwdRel& B = A.rel[A.n_rel++];
+    B.keys = V.keys.p;
+    B.key64 = V.lay.key64;
+    B.tags = V.tags.as<float>();
+    B.stamps = V.stamps.as<u32>();
+    B.hrow = J.hrow[r];
+    B.adj = J.adj[r];
+    B.base = (u32)rows;
+    rows += V.n;
+    L.rels.push_back((u32)r);
+  }
+  if (rows >= 0xFFFFFFFFull) return false;
+  std::vector<LinBwdArm> arms;
+  for (auto& p : e.plans)
+    for (auto& Ar : p.arms) {
+      const u32 drel = p.ast.body[Ar.delta].rel;
+      if (L.index[p.ast.head.rel] < 0 || !e.rels[drel].idb) continue;
+      const StepPlan& S = Ar.steps[1];
+      const u32 vrel = p.ast.body[S.atom].rel;
+      ViewSt& W = e.rels[vrel].views[S.view];
+      if (W.n > 0x7FFFFFFull) return false;
+      if (!W.n) continue;
+      engine_ensure_index(e, W, S.prefix_len);
+      LinBwdArm a;
+      std::memset(&a, 0, sizeof(a));
+      a.P = Ar.packed.steps[0];
+      a.drel = L.index[drel];
+      a.hrel = L.index[p.ast.head.rel];
+      a.P.v_keys = W.keys.p;
+      a.P.v_key64 = W.lay.key64;
+      a.P.v_tags = W.tags.p;
+      a.P.v_n = W.n;
+      const IndexSt& I = W.index[S.prefix_len];
+      a.P.index_mode = I.mode;
+      a.P.dense_offs = I.offs.as<u64>();
+      a.P.hash_bits = I.hash_bits;
+      a.prow = S.view ? J.prow[vrel][S.view] : nullptr;
+      a.vadj = e.rels[vrel].in_has_tags ? J.adj[vrel] : nullptr;
+      probed += W.n;
+      arms.push_back(a);
+    }
+  if (last < 2 || arms.empty() || !rows) return true;  // iterations after the first derived nothing
+  e.ensure(L.arms, arms.size() * sizeof(LinBwdArm));
+  e.check(cudaMemcpyAsync(L.arms.p, arms.data(), arms.size() * sizeof(LinBwdArm), cudaMemcpyHostToDevice, e.stream), "arms");
+  // entries by stamp: counts (scanned in place), fill positions
+  DevBuf &off = L.list[0], &used = L.list[1], &entries = L.start;
+  const u64 ns = (u64)last + 1;
+  e.ensure(off, (ns + 1) * 4);
+  e.ensure(used, ns * 4);
+  e.ensure(entries, rows * 4);
+  e.ensure(L.state, kLinSlots * 8);
+  e.check(cudaMemsetAsync(off.p, 0, (ns + 1) * 4, e.stream), "stamps");
+  e.check(cudaMemsetAsync(used.p, 0, ns * 4, e.stream), "stamps");
+  e.check(cudaMemsetAsync(L.state.p, 0, kLinSlots * 8, e.stream), "stamps");
+  for (int q = 0; q < A.n_rel; q++) {
+    const u64 n = e.rels[L.rels[q]].views[0].n;
+    if (n) k_lin_stamp_count<<<lin_grid(n), 256, 0, e.stream>>>(A.rel[q].stamps, n, last, off.as<u32>());
+  }
+  e.after_launch("stamps");
+  e.ensure(e.scratch, scan_scratch_elems(ns + 1) * 4 + 64);
+  exclusive_scan<u32, u32>(off.as<u32>(), off.as<u32>(), ns + 1, nullptr, e.scratch.as<u32>(), e.stream);
+  e.after_launch("stamps");
+  for (int q = 0; q < A.n_rel; q++) {
+    const u64 n = e.rels[L.rels[q]].views[0].n;
+    if (n)
+      k_lin_stamp_fill<<<lin_grid(n), 256, 0, e.stream>>>(A.rel[q].stamps, n, last, A.rel[q].base, off.as<u32>(),
+                                                         used.as<u32>(), entries.as<u32>());
+  }
+  e.after_launch("stamps");
+  A.n_arm = (int)arms.size();
+  A.arms = L.arms.as<LinBwdArm>();
+  A.entries = entries.as<u32>();
+  A.off = off.as<u32>();
+  A.last = last;
+  A.state = L.state.as<u64>();
+  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(152, probed / 16384));
+  void* args[] = {&A};
+  {
+    ProfScope ps("linear_backward", 0, e.stream);
+    e.check(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_linear_backward), dim3(blocks), dim3(kLinThreads), args, 0,
+                                        e.stream), "linear backward");
+  }
+  e.after_launch("linear backward");
+  if (e.read_u64(L.state.as<u64>() + LS_ERR))
+    throw LobError(LOB_E_TIMEOUT, "a bounded wait of the backward pass gave up; its gradients are invalid");
+  return true;
 }

@@ -27,3 +27,14 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out);
 // The whole run ended in iteration k: writes the components' counts into the
 // engine's per-iteration record.
 void linear_merge(lob_engine& e, u32 k, const LinearOut& out);
+
+// diff-add-mult backward of the linear components' iterations after the first.
+// Device pointers by relation id: adjoints and dense key -> row maps (null: none),
+// and per view its rows' primary rows.  Flags the components' relations; false
+// when there is none to take (the caller replays every iteration).
+struct LinearAdjoints {
+  std::vector<double*> adj;
+  std::vector<u32*> hrow;
+  std::vector<std::vector<u32*>> prow;
+};
+bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in);
