@@ -223,6 +223,26 @@ __global__ void k_mark_new(const void* __restrict__ keys, int key64, const u32* 
     }
 }
 
+// rows by the iteration their fact first appeared in: sort keys, then the keys of
+// the sorted rows and each stamp's first entry
+__global__ void k_stamp_keys(const u32* __restrict__ stamps, u64 n, u32* __restrict__ key, u32* __restrict__ row) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    key[i] = stamps[i] & 0x7FFFFFFFu;
+    row[i] = (u32)i;
+  }
+}
+template <class K>
+__global__ void k_stamp_words(const K* __restrict__ keys, const u32* __restrict__ rows, u64 n, K* __restrict__ out) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = keys[rows[i]];
+}
+__global__ void k_stamp_offsets(const u32* __restrict__ sorted, u64 n, u32 n_stamps, u32* __restrict__ off) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x; s <= n_stamps; s += stride)
+    off[s] = (u32)lower_bound_dev<u32>(sorted, 0, n, (u32)s);
+}
+
 __global__ void k_f32_to_f64(const float* __restrict__ a, u64 n, double* __restrict__ out) {
   const u64 stride = (u64)gridDim.x * blockDim.x;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = (double)a[i];
@@ -275,17 +295,52 @@ unsigned grid_for_n(u64 n) {
 // ---------------------------------------------------------------------------
 namespace {
 
+// A relation's rows and keys in the order of their stamps (key order within one):
+// iteration k's recent facts are one run of it.
+struct ByStamp {
+  bool built = false;
+  DevBuf rows, words;
+  std::vector<u32> off;  // first entry of stamp 0, 1, ..., last + 1
+};
+
 struct BwdState {
+  std::vector<ByStamp> stamped;              // per relation, on first use
   std::vector<DevBuf> adj;                   // per relation, f64, primary view order
   std::vector<DevBuf> hrow;                  // per derived relation with a small key space: dense key -> row
   std::vector<DevBuf> hnew;                  // and its bitmap of the facts new in the iteration being replayed
   std::vector<std::vector<DevBuf>> prow;     // per relation, per view (index 0 unused)
+  // masked last steps: per relation, bitmaps by column order -- of all its facts
+  // (have), and of its facts new in the iteration being replayed (fresh)
+  std::vector<std::vector<MaskSt>> have, fresh;
 };
+
+// the bitmap of `rel` with column order perm in set v, allocated on first use
+MaskSt& bwd_mask(lob_engine& e, std::vector<MaskSt>& v, const RelSt& r, const int* perm, bool* made) {
+  *made = false;
+  for (auto& m : v)
+    if (std::equal(perm, perm + r.arity, m.perm)) return m;
+  MaskSt m;
+  std::copy(perm, perm + r.arity, m.perm);
+  m.lay = mask_layout(e, r, perm);
+  v.push_back(m);
+  e.ensure(v.back().bits, mask_bytes(v.back().lay));
+  e.check(cudaMemsetAsync(v.back().bits.p, 0, mask_bytes(v.back().lay), e.stream), "mask");
+  *made = true;
+  return v.back();
+}
+bool bwd_masked(const lob_engine& e, const ArmPlan& A) { return e.opt_packed_backward && A.packed.ok && A.packed.mask_ok; }
 
 void free_state(lob_engine& e, BwdState& S) {
   for (auto& b : S.adj) e.release(b);
   for (auto& b : S.hrow) e.release(b);
   for (auto& b : S.hnew) e.release(b);
+  for (auto& b : S.stamped) {
+    e.release(b.rows);
+    e.release(b.words);
+  }
+  for (auto* set : {&S.have, &S.fresh})
+    for (auto& v : *set)
+      for (auto& m : v) e.release(m.bits);
   for (auto& v : S.prow)
     for (auto& b : v) e.release(b);
 }
@@ -471,6 +526,44 @@ void replay_arm(lob_engine& e, BwdState& S, const RulePlan& rp, const ArmPlan& A
   }
 }
 
+// The rows of relation D by stamp.  A replay of iteration k that scans all rows
+// for those of stamp k - 1 spreads an iteration of few recent facts over tiles of
+// millions of rows, and a tile's block walks all of its rows: on the batched
+// kinship program the 35 first-step emissions took 65 ms that way, 3 by the run.
+ByStamp& by_stamp(lob_engine& e, BwdState& S, u32 rel) {
+  ByStamp& B = S.stamped[rel];
+  if (B.built) return B;
+  B.built = true;
+  const ViewSt& V = e.rels[rel].views[0];
+  const u64 n = V.n;
+  const int kb = V.lay.key64 ? 8 : 4;
+  const u32 n_stamps = e.last_iter + 1;
+  e.ensure(e.tmp_keys, n * 4);
+  e.ensure(e.tmp_keys2, n * 4);
+  e.ensure(e.tmp_tags, n * 4);
+  e.ensure(B.rows, n * 4);
+  e.ensure(B.words, n * kb);
+  k_stamp_keys<<<grid_for_n(n), 256, 0, e.stream>>>(V.stamps.as<u32>(), n, e.tmp_keys.as<u32>(), e.tmp_tags.as<u32>());
+  e.after_launch("stamps");
+  void* k = e.tmp_keys.p;
+  void* r = e.tmp_tags.p;
+  int bits = 1;
+  while (bits < 32 && (n_stamps >> bits)) bits++;
+  e.ensure(e.scratch, sort_scratch_bytes(n, e.opt_radix_bits));
+  sort_pairs(0, 4, &k, &r, e.tmp_keys2.p, B.rows.p, n, bits, e.opt_radix_bits, e.scratch.p, e.stream);
+  e.after_launch("stamp sort");
+  if (r != B.rows.p) e.check(cudaMemcpyAsync(B.rows.p, r, n * 4, cudaMemcpyDeviceToDevice, e.stream), "stamp rows");
+  if (kb == 8) k_stamp_words<u64><<<grid_for_n(n), 256, 0, e.stream>>>(V.keys.as<u64>(), B.rows.as<u32>(), n, B.words.as<u64>());
+  else k_stamp_words<u32><<<grid_for_n(n), 256, 0, e.stream>>>(V.keys.as<u32>(), B.rows.as<u32>(), n, B.words.as<u32>());
+  e.ensure(e.off, (u64)(n_stamps + 1) * 4);
+  k_stamp_offsets<<<grid_for_n(n_stamps + 1), 256, 0, e.stream>>>(static_cast<const u32*>(k), n, n_stamps, e.off.as<u32>());
+  e.after_launch("stamps");
+  B.off.resize((size_t)n_stamps + 1);
+  e.check(cudaMemcpyAsync(B.off.data(), e.off.p, B.off.size() * 4, cudaMemcpyDeviceToHost, e.stream), "stamps");
+  e.sync();
+  return B;
+}
+
 // The same replay on the packed kernels (pjoin.cu): returns false when the arm
 // is not a packed pipeline of at least one probe, or its head has no dense
 // key map, and the general replay runs instead.
@@ -507,6 +600,17 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
   const void* in_words = DV.keys.p;
   u64 n_in = DV.n;
   int side = 0;
+  // the delta atom: the recent set of iteration k, a run of the rows by stamp
+  // (every fact when k begins a stratum)
+  const bool by_run = !begins_stratum(e.stratum_begin, k) && n_in;
+  if (by_run) {
+    const ByStamp& T = by_stamp(e, S, R.body[A.delta].rel);
+    in_words = T.words.as<char>() + (u64)T.off[k - 1] * (DV.lay.key64 ? 8 : 4);
+    n_in = T.off[k] - T.off[k - 1];
+    B.packed_source = 0;
+    B.n_in_facts = 1;
+    B.in_rows[0] = T.rows.as<u32>() + T.off[k - 1];
+  }
   for (size_t s = 1; s < A.steps.size(); s++) {
     const StepPlan& SP = A.steps[s];
     const bool last = s + 1 == A.steps.size();
@@ -518,7 +622,7 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
     P.in_words = in_words;
     P.in_tags = nullptr;
     P.n_in = n_in;
-    if (s == 1) {  // the delta atom: the recent set of iteration k
+    if (s == 1 && !by_run) {
       P.in_stamp = DV.stamps.as<u32>();
       set_delta_stamps(e, k, P.in_stamp_mode, P.in_stamp_val);
     } else {
@@ -535,6 +639,22 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
     P.index_mode = I.mode;
     P.dense_offs = I.offs.as<u64>();
     P.hash_bits = I.hash_bits;
+    if (last && A.packed.mask_ok && I.mode == INDEX_DENSE) {  // only groundings whose head has an adjoint to give
+      bool made;
+      RelSt& V = e.rels[vrel];
+      PMask M = A.packed.mask;
+      MaskSt& have = bwd_mask(e, S.have[vrel], V, W.perm, &made);
+      if (made) mask_set(V.views[0].lay, V.views[0].perm, have.lay, have.perm, V.views[0].keys.p, V.views[0].n, have.bits.as<u32>(), e.stream);
+      M.vbits = have.bits.as<u32>();
+      M.hbits = bwd_mask(e, S.fresh[hrel], H, A.packed.mask_h, &made).bits.as<u32>();
+      if (made) throw LobError(LOB_E_CUDA, "internal error: mask of the new heads missing");
+      B.last = 1;
+      B.v_prow = SP.view ? S.prow[vrel][SP.view].as<u32>() : nullptr;
+      pjoin_backward_masked(P, B, M, e.stream);
+      e.after_launch("backward masked");
+      e.launches++;
+      return true;
+    }
     const u64 n_blk = pjoin_loc_blocks(n_in);
     e.ensure(e.cnt, n_in * 4);
     e.ensure(e.lo, n_in * 4);
@@ -656,6 +776,9 @@ int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* con
       S.hrow.resize(nrel);
       S.hnew.resize(nrel);
       S.prow.resize(nrel);
+      S.have.resize(nrel);
+      S.stamped.resize(nrel);
+      S.fresh.resize(nrel);
       for (size_t k = 0; k < nrel; k++) {
         RelSt& r = e->rels[k];
         const u64 n = r.views[0].n;
@@ -728,6 +851,18 @@ int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* con
                                                                       r.views[0].stamps.as<u32>(), r.views[0].n, k,
                                                                       S.hnew[q].as<u32>());
           e->after_launch("new heads");
+          for (auto& p : e->plans)
+            for (auto& A : p.arms) {
+              if (p.ast.head.rel != q || !bwd_masked(*e, A)) continue;
+              bool made;
+              bwd_mask(*e, S.fresh[q], r, A.packed.mask_h, &made);
+            }
+          for (auto& m : S.fresh[q]) {
+            e->check(cudaMemsetAsync(m.bits.p, 0, mask_bytes(m.lay), e->stream), "new heads");
+            mask_set_new(r.views[0].lay, r.views[0].perm, m.lay, m.perm, r.views[0].keys.p, r.views[0].n,
+                         r.views[0].stamps.as<u32>(), k, S.adj[q].as<double>(), m.bits.as<u32>(), e->stream);
+            e->after_launch("new heads");
+          }
         }
         const int stratum = stratum_of_iter(e->stratum_begin, k);
         for (auto& p : e->plans)

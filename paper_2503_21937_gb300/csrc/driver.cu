@@ -52,6 +52,7 @@ struct GDesc {
   int rel_dense[kGMaxRels];
   int rel_nviews[kGMaxRels];
   int arm_delta[kGMaxArms], arm_last[kGMaxArms], arm_nbefore[kGMaxArms], arm_head[kGMaxArms];
+  int arm_masked[kGMaxArms];  // the last step is a masked one: it adds its outputs to its slot and uses no tiles
   int arm_before[kGMaxArms][kGMaxBefore];
   // double-buffered groups: per dense relation its primary view, its
   // maintained views (in view-slot order) and its recent set
@@ -104,6 +105,7 @@ __global__ void k_iter_begin(const __grid_constant__ GDesc d, u64* s, u64* rec, 
     u64* A = s + arm_base(d.nrel, a);
     A[0] = active ? D[R_RECENT] : 0;
     // an inactive arm may be skipped by its guard: its step totals read 0
+    if (d.arm_masked[a]) A[1 + d.arm_last[a]] = 0;
     if (!active)
       for (int st = 1; st <= d.arm_last[a]; st++) A[1 + st] = 0;
   }
@@ -147,6 +149,7 @@ __global__ void k_iter_end(const __grid_constant__ GDesc d, u64* s) {
   for (int a = 0; a < d.narm; a++)
     for (int st = 1; st <= d.arm_last[a]; st++) {
       const u64 t = s[arm_base(d.nrel, a) + 1 + st];
+      if (st == d.arm_last[a] && d.arm_masked[a]) continue;
       need_at_most(s, t, d.cap_outputs, d.need_tiles);
       if (st < d.arm_last[a]) need_at_most(s, t, d.cap_bind, d.need_bind);
     }
@@ -308,6 +311,12 @@ void plan_loop(lob_engine& e, GLoop& G, u32 max_iters) {
       G.d.arm_last[a] = (int)A.steps.size() - 1;
       G.d.arm_nbefore[a] = (int)A.before_rels.size();
       G.d.arm_head[a] = (int)p.ast.head.rel;
+      {
+        const StepPlan& S = A.steps.back();
+        ViewSt& W = e.rels[p.ast.body[S.atom].rel].views[S.view];
+        engine_ensure_index(e, W, S.prefix_len);
+        G.d.arm_masked[a] = A.packed.mask_ok && W.index[S.prefix_len].mode == INDEX_DENSE;
+      }
       for (size_t b = 0; b < A.before_rels.size(); b++) G.d.arm_before[a][b] = (int)A.before_rels[b];
     }
   G.d.narm = (int)G.arms.size();
@@ -628,6 +637,17 @@ void capture_iteration(lob_engine& e, GLoop& G, u64* st_dev, u64* rec_dev, cudaS
       P.index_mode = I.mode;
       P.dense_offs = I.offs.as<u64>();
       P.hash_bits = I.hash_bits;
+      if (last && G.d.arm_masked[a]) {
+        PMask M = A.packed.mask;
+        M.vbits = VR.masks[find_mask(VR, W.perm)].bits.as<u32>();
+        M.hbits = H.masks[find_mask(H, A.packed.mask_h)].bits.as<u32>();
+        P.bitmap = H.dtouched.as<u32>();
+        P.acc = H.dacc.p;
+        pjoin_masked(ks, P, M, slot(ab + 1 + (int)s), st);
+        e.check(cudaGetLastError(), "join masked");
+        mark(("loop_arm" + std::to_string(a) + "_masked").c_str());
+        break;
+      }
       const u64 n_blk = pjoin_loc_blocks(n_cap);
       P.loc = e.cnt.as<u32>();
       P.lo32 = e.lo.as<u32>();
@@ -763,6 +783,18 @@ void capture_iteration(lob_engine& e, GLoop& G, u64* st_dev, u64* rec_dev, cudaS
   (void)cb;
   k_iter_end<<<1, 32, 0, st>>>(G.d, st_dev);
   e.check(cudaGetLastError(), "iteration end");
+  // the committed iteration's new facts join the masks of their relations (an
+  // iteration that overflowed commits nothing)
+  for (int r = 0; r < G.d.nrel; r++) {
+    if (!G.d.rel_dense[r]) continue;
+    RelSt& H = e.rels[r];
+    const ViewSt& V = H.views[0];
+    for (auto& m : H.masks) {
+      mask_set(V.lay, V.perm, m.lay, m.perm, nullptr, G.cap_r[r], m.bits.as<u32>(), st, slot(rel_base(r) + R_RECENT),
+               nxt(grecent(r)), slot(S_OVERFLOW));
+      e.check(cudaGetLastError(), "mask");
+    }
+  }
   mark("loop_end");
 }
 

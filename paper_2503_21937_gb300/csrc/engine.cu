@@ -160,6 +160,8 @@ static void release_derived(lob_engine& e) {
                       &r.row_keys, &r.akeys, &r.atags, &r.akeys2, &r.atags2, &r.bitmap, &r.prev_bitmap, &r.dacc,
                       &r.dtouched})
       e.release(*b);
+    for (auto& m : r.masks) e.release(m.bits);
+    r.masks.clear();
     r.extract = r.touched = r.keys_stale = r.dense = r.finished = false;
     r.n_recent = r.n_next = r.n_cand = r.n_acc = 0;
     r.flushed = false;
@@ -567,6 +569,60 @@ static void compile_cross(lob_engine& e, const RuleAst& R, const ArmPlan& A, Pac
   out.cross_ok = true;
 }
 
+Layout mask_layout(const lob_engine& e, const RelSt& r, const int* perm) {
+  Layout L;
+  make_layout(e, r, perm, L);
+  return L;
+}
+int find_mask(const RelSt& r, const int* perm) {
+  for (size_t i = 0; i < r.masks.size(); i++)
+    if (std::equal(perm, perm + r.arity, r.masks[i].perm)) return (int)i;
+  return -1;
+}
+
+// The masked form of an arm's last step (pjoin.h): the probed atom leaves one
+// column free, of at most 6 bits, which is the view's last and occurs once in the
+// head, in a column of at most 6 bits.
+constexpr int kMaskBits = 28;  // largest bitmap: 32 MB, cleared by every run
+static void compile_mask(lob_engine& e, const RuleAst& R, const ArmPlan& A, PackedArm& out) {
+  if (!out.ok || A.steps.size() < 2 || !e.rels[R.body[A.delta].rel].idb) return;
+  const StepPlan& S = A.steps.back();
+  const AtomAst& atom = R.body[S.atom];
+  const ViewSt& W = e.rels[atom.rel].views[S.view];
+  const int last = (int)atom.args.size() - 1;
+  if (S.prefix_len != last || S.act[last].op != OP_BIND || W.lay.width[last] > 6 || W.lay.bits > kMaskBits) return;
+  const u32 z = atom.args[W.perm[last]].v;
+  const RelSt& H = e.rels[R.head.rel];
+  int hcol = -1;
+  for (size_t c = 0; c < R.head.args.size(); c++)
+    if (R.head.args[c].var && R.head.args[c].v == z) {
+      if (hcol >= 0) return;
+      hcol = (int)c;
+    }
+  if (hcol < 0 || H.width[hcol] > 6 || H.views[0].lay.bits > kMaskBits) return;
+  int n = 0;
+  for (int c = 0; c < (int)H.arity; c++)
+    if (c != hcol) out.mask_h[n++] = c;
+  out.mask_h[n] = hcol;
+  const Layout L = mask_layout(e, H, out.mask_h);
+  const PStep& P = out.steps.back();
+  PMask& M = out.mask;
+  M.vw = W.lay.width[last];
+  M.hw = L.width[n];
+  M.n_hf = 0;
+  for (int j = 0; j < n; j++) {
+    PField f = P.out[out.mask_h[j]];
+    f.shift = (uint8_t)(L.shift[j] - M.hw);
+    M.hf[M.n_hf++] = f;
+  }
+  if (L.swidth) {
+    PField f = P.out[H.arity];
+    f.shift = (uint8_t)(L.sshift - M.hw);
+    M.hf[M.n_hf++] = f;
+  }
+  out.mask_ok = true;
+}
+
 // Strata (Sec. 3.1: a RAM program is a sequence of strata; Algorithm 1 runs
 // each to its fixpoint before the next).  Derived relations that depend on one
 // another, directly or through others, form a component; a component's level
@@ -701,6 +757,7 @@ static void prepare_arms(lob_engine& e) {
       // and comparison filters run bytecode: general steps only
       A.packed = e.opt_packed_join && !sem_top1(sem) && !p.ast.computes() ? compile_packed(e, p.ast, A) : PackedArm{};
       if (sem == SR_UNIT) compile_cross(e, p.ast, A, A.packed);
+      if (sem_stamps(sem)) compile_mask(e, p.ast, A, A.packed);
     }
 }
 
@@ -1444,6 +1501,18 @@ static void run_arm_packed(lob_engine& e, const RulePlan& rp, const ArmPlan& A, 
       n_in = total;
       continue;
     }
+    if (last && H.dense && A.packed.mask_ok && I.mode == INDEX_DENSE) {  // only the outputs that can be new facts
+      PMask M = A.packed.mask;
+      M.vbits = V.masks[find_mask(V, W.perm)].bits.as<u32>();
+      M.hbits = H.masks[find_mask(H, A.packed.mask_h)].bits.as<u32>();
+      H.touched = true;
+      P.bitmap = H.dtouched.as<u32>();
+      P.acc = H.dacc.p;
+      pjoin_masked(sem, P, M, e.counts.as<u64>() + 13, e.stream);
+      e.after_launch("join masked");
+      e.launches++;
+      return;
+    }
     const u64 n_blk = pjoin_loc_blocks(n_in);
     e.ensure(e.cnt, n_in * 4);
     e.ensure(e.lo, n_in * 4);
@@ -1868,6 +1937,22 @@ static void choose_dedup_mode(lob_engine& e, RelSt& r) {
   r.extract = delta_cost <= sorted_cost;
 }
 
+static void add_mask(lob_engine& e, RelSt& r, const int* perm) {
+  if (find_mask(r, perm) >= 0) return;
+  MaskSt m;
+  std::copy(perm, perm + r.arity, m.perm);
+  m.lay = mask_layout(e, r, perm);
+  r.masks.push_back(m);
+  MaskSt& M = r.masks.back();
+  e.ensure(M.bits, mask_bytes(M.lay));
+  e.check(cudaMemsetAsync(M.bits.p, 0, mask_bytes(M.lay), e.stream), "mask");
+  const ViewSt& V = r.views[0];
+  if (!V.n) return;
+  mask_set(V.lay, V.perm, M.lay, M.perm, V.keys.p, V.n, M.bits.as<u32>(), e.stream);
+  e.after_launch("mask");
+  e.launches++;
+}
+
 // Dense (+)-accumulation for every derived relation of a tagged run whose key
 // space has at most opt_acc_bits bits (accumulator: 2^bits candidate tags).
 static void enable_dense(lob_engine& e) {
@@ -1884,6 +1969,26 @@ static void enable_dense(lob_engine& e) {
     e.check(cudaMemsetAsync(r.dtouched.p, 0, bm_bytes, e.stream), "dense bitmap");
     r.dense = true;
     r.touched = false;
+  }
+  // bitmaps of the masked last steps into dense heads, equal to the loaded facts
+  for (auto& p : e.plans)
+    for (auto& A : p.arms) {
+      if (!A.packed.mask_ok || !e.rels[p.ast.head.rel].dense) continue;
+      const StepPlan& S = A.steps.back();
+      const u32 vrel = p.ast.body[S.atom].rel;
+      add_mask(e, e.rels[vrel], e.rels[vrel].views[S.view].perm);
+      add_mask(e, e.rels[p.ast.head.rel], A.packed.mask_h);
+    }
+}
+
+// the iteration's new facts of r (the next recent set) join its masks
+static void update_masks(lob_engine& e, RelSt& r) {
+  if (!r.n_next) return;
+  const ViewSt& V = r.views[0];
+  for (auto& m : r.masks) {
+    mask_set(V.lay, V.perm, m.lay, m.perm, r.nkeys.p, r.n_next, m.bits.as<u32>(), e.stream);
+    e.after_launch("mask");
+    e.launches++;
   }
 }
 
@@ -1972,6 +2077,7 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
     u64 total_new = 0;
     for (auto& r : e.rels) {
       dedup_relation(e, r, k);
+      update_masks(e, r);
       total_new += r.n_next;
     }
     for (auto& r : e.rels) {

@@ -77,6 +77,14 @@ struct ViewSt {
   std::map<int, IndexSt> index;  // by prefix length
 };
 
+// Membership bitmap of a relation over its keys with one column last (masked
+// join steps): bit k set <=> the fact with key k in that layout exists.
+struct MaskSt {
+  int perm[kMaxArity] = {0};
+  Layout lay{};
+  DevBuf bits;
+};
+
 struct RelSt {
   std::string name;
   u32 arity = 0;
@@ -111,6 +119,7 @@ struct RelSt {
   // (+)-added into dacc[key] and marked in dtouched instead of being written,
   // sorted and uniqued; the iteration's unique candidates are read out in key order
   bool dense = false;
+  std::vector<MaskSt> masks;  // kept equal to the full relation, iteration by iteration
   bool finished = false;    // run to its fixpoint by the linear loop: the other loops leave it alone
   DevBuf dacc, dtouched;
   u64 last_cand = 0, last_new = 0, cand_iter = 0;
@@ -143,6 +152,11 @@ struct PackedArm {
   // (word 1) and its own key (word 3), for the fused cross-product step
   bool cross_ok = false;
   PStep cross;
+  // the last step's matches and its head keys differ in one column of at most 6
+  // bits: a masked step (pjoin.h).  mask_h: the head columns, that one last.
+  bool mask_ok = false;
+  PMask mask{};
+  int mask_h[kMaxArity] = {0};
 };
 struct ArmPlan {
   int delta = 0;
@@ -287,6 +301,10 @@ struct lob_engine {
 };
 
 void engine_ensure_index(lob_engine& e, ViewSt& v, int prefix);
+// the mask of r with column order perm (its layout; allocated by the caller), or -1
+int find_mask(const RelSt& r, const int* perm);
+Layout mask_layout(const lob_engine& e, const RelSt& r, const int* perm);
+inline u64 mask_bytes(const Layout& L) { return std::max<u64>(16, (1ull << L.bits) / 8); }
 // copy a rule's bytecode programs into step parameters
 void set_rule_code(const RuleAst& R, StepParams& P);
 // device-driven iterations after iteration k (driver.cu)

@@ -984,6 +984,209 @@ __global__ void __launch_bounds__(256) k_pwarp_cross(const __grid_constant__ PSt
   if (lane == 0 && mine) atomicAdd(emitted, (unsigned long long)mine);
 }
 
+// ---------------------------------------------------------------------------
+// Masked last step (see pjoin.h).  A warp takes 32 input rows, a lane each forms
+// its row's mask of matches worth emitting, and the masks' bits are expanded in
+// rounds of 32 (the source row by a search over the scanned bit counts, the match
+// by selecting the row's n-th bit).  A match's view row is the row's first (dense
+// offsets) plus the bits below it, as the bitmap row lists the view's run.
+// In the kinship program of the batched workload 4.3e9 matches reach the last
+// step and most derive heads that are facts already, or, going back, heads that
+// were not new: the general step spends a count, an offset and (forward) an
+// atomic on each, this one a lane's AND on each input row of about 18 matches.
+// ---------------------------------------------------------------------------
+LOB_DEV u64 row_bits(const u32* bm, u64 row, int w) {
+  if (w == 6) return reinterpret_cast<const u64*>(bm)[row];
+  const u64 at = row << w;
+  const u32 n = 1u << w;  // at most 32 bits, within one word
+  return (bm[at >> 5] >> (u32)(at & 31u)) & (n == 32 ? 0xFFFFFFFFu : (1u << n) - 1u);
+}
+// position of the n-th (from 0) set bit of m
+LOB_DEV u32 select_bit(u64 m, u32 n) {
+  u32 x = (u32)m, at = 0;
+  u32 c = __popc(x);
+  if (n >= c) { n -= c; x = (u32)(m >> 32); at = 32; }
+#pragma unroll
+  for (int s = 16; s; s >>= 1) {
+    c = __popc(x & ((1u << s) - 1u));
+    if (n >= c) { n -= c; x >>= s; at += s; }
+  }
+  return at;
+}
+
+// row r's input word, probe key and masks; 0 when the row has no match
+LOB_DEV u64 masked_row(const PStep& P, const PPtrs& Q, const PMask& M, u64 r, u64 n_in, u64& wi, u64& pv, u64& hm) {
+  pv = hm = 0;
+  wi = 0;
+  if (r >= n_in) return 0;
+  wi = load_word(Q.in_words, P.in_w64, r);
+  if (wi == (P.in_w64 ? ~0ull : 0xFFFFFFFFull)) return 0;
+  if (P.in_stamp_mode != STAMP_NONE) {
+    const u32 st = P.in_stamp[r] & 0x7FFFFFFFu;
+    if (P.in_stamp_mode == STAMP_LT ? !(st < P.in_stamp_val) : st != P.in_stamp_val) return 0;
+  }
+  if (P.n_in_checks && !checks_ok(P.in_checks, P.n_in_checks, wi, 0)) return 0;
+  for (int q = 0; q < P.n_prefix; q++) {
+    const u64 x = pick(P.prefix[q].op, wi, 0);
+    if (P.prefix[q].limit_bits < 64 && (x >> P.prefix[q].limit_bits)) return 0;
+    pv |= x << P.prefix[q].shift;
+  }
+  const u64 vm = row_bits(M.vbits, pv, M.vw);
+  if (vm) hm = row_bits(M.hbits, compose(M.hf, M.n_hf, wi, 0), M.hw);
+  return vm;
+}
+
+template <class Sem>
+__global__ void __launch_bounds__(256) k_pmasked(const __grid_constant__ PStep P, const __grid_constant__ PMask M,
+                                                 unsigned long long* emitted) {
+  typedef typename Sem::Stored S;
+  typedef typename Sem::Cand C;
+  const int lane = threadIdx.x & 31;
+  const u64 nwarps = (u64)gridDim.x * (blockDim.x / 32);
+  const u64 n_in = dev_size(P.n_in, P.n_in_dev);
+  const PPtrs Q = resolve_ptrs(P);
+  const u32 vsv = P.stamp_dev ? (u32)*P.stamp_dev + P.v_stamp_val : P.v_stamp_val;
+  u64 mine = 0;
+  for (u64 g = (u64)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); g * 32 < n_in; g += nwarps) {
+    u64 wi, pv, hm;
+    const u64 r = g * 32 + lane;
+    const u64 vm = masked_row(P, Q, M, r, n_in, wi, pv, hm);
+    mine += __popcll(vm);
+    const u64 m = vm & ~hm;
+    const u32 c = __popcll(m);
+    const u32 inc = warp_inclusive_sum(c);
+    const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+    if (!tot) continue;
+    const u32 ex = inc - c;
+    C ct = Sem::one();
+    u64 lo = 0;
+    if (c) {
+      lo = P.dense_offs[pv];
+      ct = P.in_packed ? Sem::from_stored(reinterpret_cast<const S*>(Q.in_tags)[r]) : reinterpret_cast<const C*>(Q.in_tags)[r];
+    }
+    for (u32 t0 = 0; t0 < tot; t0 += 32) {
+      const u32 t = t0 + lane;
+      int src = 0;  // the last lane whose outputs start at or before t
+#pragma unroll
+      for (int step = 16; step; step >>= 1) {
+        const u32 e = __shfl_sync(0xFFFFFFFFu, ex, src + step);
+        if (e <= t) src += step;
+      }
+      const u64 wr = __shfl_sync(0xFFFFFFFFu, wi, src);
+      const u64 mr = __shfl_sync(0xFFFFFFFFu, m, src), vr = __shfl_sync(0xFFFFFFFFu, vm, src);
+      const u64 pr = __shfl_sync(0xFFFFFFFFu, pv, src), lr = __shfl_sync(0xFFFFFFFFu, lo, src);
+      const u32 er = __shfl_sync(0xFFFFFFFFu, ex, src);
+      const C tr = __shfl_sync(0xFFFFFFFFu, ct, src);
+      if (t >= tot) continue;
+      const u32 z = select_bit(mr, t - er);
+      const u64 v = lr + __popcll(vr & ((1ull << z) - 1ull));
+      if (P.v_stamp_mode != STAMP_NONE) {
+        const u32 st = Q.v_stamp[v] & 0x7FFFFFFFu;
+        if (P.v_stamp_mode == STAMP_LT ? st >= vsv : st != vsv) continue;
+      }
+      const u64 wv = (pr << M.vw) | z;
+      if (!checks_ok(P.checks, P.n_checks, wr, wv)) continue;
+      const u64 w = compose(P.out, P.n_out, wr, wv);
+      dense_add<Sem>(P.acc, w, Sem::mul(tr, Sem::from_stored(reinterpret_cast<const S*>(Q.v_tags)[v])));
+      touch_bit(P.bitmap, w);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
+  if (lane == 0 && mine) atomicAdd(emitted, (unsigned long long)mine);
+}
+
+// The backward step: a lane walks the bits of its own row.  The matched facts'
+// shares go out as one FP64 atomic each, the carried facts' as one per row: their
+// sum needs no reduction across lanes, which at this GPU's FP64 rate cost more
+// than the lanes left idle by rows of fewer bits (batched kinship, 1.05e9
+// groundings with an adjoint: 17.8 ms; balanced rounds with an atomic per
+// grounding and carried fact 22.4, with a segmented sum 25.0).
+__global__ void __launch_bounds__(256) k_pbwd_masked(const __grid_constant__ PStep P, const __grid_constant__ PBwd B,
+                                                     const __grid_constant__ PMask M) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  const PPtrs Q = resolve_ptrs(P);
+  const int nf_in = B.packed_source ? 1 : B.n_in_facts;
+  for (u64 r = (u64)blockIdx.x * blockDim.x + threadIdx.x; r < P.n_in; r += stride) {
+    u64 wi, pv, hm;
+    const u64 vm = masked_row(P, Q, M, r, P.n_in, wi, pv, hm);
+    const u64 m = vm & hm;
+    if (!m) continue;
+    const u64 lo = P.dense_offs[pv];
+    u32 rows[kMaxArity];
+    float tags[kMaxArity];
+    double carried = 1.0;
+    for (int q = 0; q < nf_in; q++) {
+      rows[q] = B.packed_source ? (u32)r : B.in_rows[q][r];
+      tags[q] = B.fact_tags[q][rows[q]];
+      carried *= (double)tags[q];
+    }
+    double share = 0.0;
+    for (u64 mm = m; mm; mm &= mm - 1) {
+      const u32 z = __ffsll(mm) - 1;
+      const u64 v = lo + __popcll(vm & ((1ull << z) - 1ull));
+      if (P.v_stamp_mode != STAMP_NONE) {
+        const u32 st = P.v_stamp[v] & 0x7FFFFFFFu;
+        if (P.v_stamp_mode == STAMP_LT ? st >= P.v_stamp_val : st != P.v_stamp_val) continue;
+      }
+      const u64 wv = (pv << M.vw) | z;
+      if (!checks_ok(P.checks, P.n_checks, wi, wv)) continue;
+      const double adj = B.h_adj[B.h_row[compose(P.out, P.n_out, wi, wv)]];
+      const u32 vrow = B.v_prow ? B.v_prow[v] : (u32)v;
+      share += adj * (double)B.fact_tags[nf_in][vrow];
+      if (B.fact_adj[nf_in]) atomicAdd(B.fact_adj[nf_in] + vrow, adj * carried);
+    }
+    if (share == 0.0) continue;
+    for (int q = 0; q < nf_in; q++) {
+      if (!B.fact_adj[q]) continue;
+      double x = share;
+      for (int l = 0; l < nf_in; l++)
+        if (l != q) x *= (double)tags[l];
+      atomicAdd(B.fact_adj[q] + rows[q], x);
+    }
+  }
+}
+
+struct MaskPerm {
+  int from[kMaxArity], to[kMaxArity];
+};
+LOB_DEV void set_mask_bit(const Layout& F, const Layout& T, const MaskPerm& p, u64 k, u32* bits) {
+  u32 rel[kMaxArity];
+#pragma unroll
+  for (int j = 0; j < kMaxArity; j++)
+    if (j < F.arity) rel[p.from[j]] = (u32)field_of(k, F.shift[j], F.width[j]);
+  u64 o = F.swidth ? field_of(k, F.sshift, F.swidth) << T.sshift : 0ull;
+#pragma unroll
+  for (int j = 0; j < kMaxArity; j++)
+    if (j < T.arity) o |= (u64)rel[p.to[j]] << T.shift[j];
+  atomicOr(bits + (o >> 5), 1u << (u32)(o & 31u));
+}
+__global__ void k_mask_set(const __grid_constant__ Layout F, const __grid_constant__ Layout T,
+                           const __grid_constant__ MaskPerm p, const void* keys, u64 n, u32* __restrict__ bits,
+                           const u64* n_dev, void* const* keys_pp, const u64* skip) {
+  if (skip && *skip) return;
+  if (n_dev) n = *n_dev < n ? *n_dev : n;
+  if (keys_pp) keys = keys_pp[0];
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
+    set_mask_bit(F, T, p, load_key(keys, F.key64, i), bits);
+}
+__global__ void k_mask_new(const __grid_constant__ Layout F, const __grid_constant__ Layout T,
+                           const __grid_constant__ MaskPerm p, const void* __restrict__ keys, u64 n,
+                           const u32* __restrict__ stamps, u32 k, const double* __restrict__ adj, u32* __restrict__ bits) {
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
+    if (stamps[i] == k && adj[i] != 0.0) set_mask_bit(F, T, p, load_key(keys, F.key64, i), bits);
+}
+MaskPerm mask_perm(const Layout& F, const int* pf, const int* pt) {
+  MaskPerm p{};
+  for (int j = 0; j < F.arity; j++) {
+    p.from[j] = pf[j];
+    p.to[j] = pt[j];
+  }
+  return p;
+}
+
 unsigned grid_n(u64 n) {
   u64 b = (n + 255) / 256;
   if (b > 152ull * 16) b = 152ull * 16;
@@ -1129,6 +1332,27 @@ void pjoin_warp_cross_bitmap(const PStep& A, const PStep& B, u64* emitted_dev, c
 
 bool pjoin_warp_supported(int sem, const PStep& P) {
   return sem == SR_UNIT && P.n_out >= 1 && P.n_out <= 4 && P.n_checks <= 1;
+}
+
+void pjoin_masked(int sem, const PStep& P, const PMask& M, u64* emitted_dev, cudaStream_t st) {
+  // an input row reads its word, two bitmap rows and, with outputs, its tag
+  ProfScope ps("join_masked", P.n_in * (row_bytes(sem, P.in_w64, P.in_packed) + 16.0), st);
+  if (!P.n_in) return;
+  k_pmasked<SemAddMult><<<grid_n(P.n_in), 256, 0, st>>>(P, M, reinterpret_cast<unsigned long long*>(emitted_dev));
+}
+void pjoin_backward_masked(const PStep& P, const PBwd& B, const PMask& M, cudaStream_t st) {
+  ProfScope ps("bwd_masked", P.n_in * ((P.in_w64 ? 8.0 : 4.0) + 16.0), st);
+  if (P.n_in) k_pbwd_masked<<<grid_n(P.n_in), 256, 0, st>>>(P, B, M);
+}
+void mask_set(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys, u64 n,
+              u32* bits, cudaStream_t st, const u64* n_dev, void* const* keys_pp, const u64* skip_dev) {
+  ProfScope ps("mask_set", n * (from.key64 ? 8.0 : 4.0), st);
+  if (n) k_mask_set<<<grid_n(n), 256, 0, st>>>(from, to, mask_perm(from, perm_from, perm_to), keys, n, bits, n_dev, keys_pp, skip_dev);
+}
+void mask_set_new(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys, u64 n,
+                  const u32* stamps, u32 k, const double* adj, u32* bits, cudaStream_t st) {
+  ProfScope ps("mask_set", n * ((from.key64 ? 8.0 : 4.0) + 12.0), st);
+  if (n) k_mask_new<<<grid_n(n), 256, 0, st>>>(from, to, mask_perm(from, perm_from, perm_to), keys, n, stamps, k, adj, bits);
 }
 
 u64 pjoin_warp_blocks(u64 n_in) { return (n_in + kWarpBlockRows - 1) / kWarpBlockRows; }

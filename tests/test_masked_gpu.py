@@ -1,0 +1,63 @@
+"""Masked last join steps (add-mult semirings: the last probe leaves one column
+of at most 6 bits free) against the oracle and against the general kernels:
+row widths from 1 to 6 bits and just past, filters, transposed and constant
+head columns, samples, old-fact arms, gradients, both iteration drivers."""
+import numpy as np
+import pytest
+
+from paper_2503_21937_gb300 import workloads as W
+from tests.common import compare, engine_run
+
+pytestmark = pytest.mark.gpu
+
+PROGRAMS = {
+    "nonlinear": "p(x,y) :- e(x,y).\np(x,z) :- p(x,y), p(y,z).\n",
+    "transposed": "p(x,y) :- e(x,y).\np(z,x) :- p(x,y), p(y,z), x != z.\n",
+    "constant": "p(x,y) :- e(x,y).\nq(7,z) :- p(x,y), p(y,z).\nq(z,3) :- q(x,y), e(x,z).\n",
+    "three": "p(x,y) :- e(x,y).\np(x,w) :- p(x,y), e(y,z), p(z,w), x != w.\n",
+}
+
+
+def _facts(n, m, seed, scale):
+    s = W.stream(seed)
+    return s.below(m, n), s.below(m, n), (s.prob(m) * scale).astype(np.float32)
+
+
+@pytest.mark.parametrize("name", list(PROGRAMS))
+@pytest.mark.parametrize("n", [2, 3, 7, 15, 31, 33, 62, 63, 64])
+def test_row_widths(name, n):
+    a, b, p = _facts(n, 2 * n + 3, 900 + n, 0.3)
+    for driver in (0, 2):
+        compare(PROGRAMS[name], {"e": ((a, b), p)}, "add_mult", options={"driver": driver})
+
+
+@pytest.mark.parametrize("semiring", ["add_mult", "diff_add_mult"])
+@pytest.mark.parametrize("program", ["kinship", "nonlinear", "three"])
+def test_same_as_the_general_kernels(program, semiring):
+    """Statistics equal, tags within the reordering of FP64 sums rounded once to
+    f32, gradients within 1e-4 (as against the oracle)."""
+    if program == "kinship":
+        B = W.batched_instance(40)
+        f, c = B["fact"], B["comp"]
+        text, rel, grad = W.KIN_PROGRAM, "kin", "fact"
+        inputs = {"fact": (f[:3], f[3], f[4]), "comp": (c[:3], None, c[4])}
+    else:
+        a, b, p = _facts(60, 200, 950, 0.2)
+        sid = (np.arange(200) % 3).astype(np.uint32)
+        text, rel, grad = PROGRAMS[program], "p", "e"
+        inputs = {"e": ((a, b), p, sid), "p": ((b[:9], a[:9]), p[:9], sid[:9])}
+    runs = []
+    for opts in ({"packed_join": 0, "driver": 0}, {"driver": 0}, {"driver": 2}):
+        e, st, got = engine_run(text, inputs, semiring, options=opts, read=[rel])
+        g = np.zeros(len(inputs[grad][0][0]), np.float32)
+        if semiring == "diff_add_mult":
+            e.backward(rel, np.linspace(-1, 1, got[rel].cols.shape[1]).astype(np.float32), {grad: g})
+        e.close()
+        runs.append((st, got[rel], g))
+    (a, ra, ga) = runs[0]
+    for st, r, g in runs[1:]:
+        for k in ("iterations", "derived", "candidates", "new_facts"):
+            assert st[k] == a[k], (k, st[k], a[k])
+        assert np.array_equal(r.cols, ra.cols) and np.array_equal(r.samples, ra.samples)
+        np.testing.assert_allclose(r.tags, ra.tags, rtol=3e-7, atol=0)
+        np.testing.assert_allclose(g, ga, rtol=1e-4, atol=1e-5 * max(1.0, float(np.abs(ga).max())))
