@@ -644,7 +644,7 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
       RelSt& V = e.rels[vrel];
       PMask M = A.packed.mask;
       MaskSt& have = bwd_mask(e, S.have[vrel], V, W.perm, &made);
-      if (made) mask_set(V.views[0].lay, V.views[0].perm, have.lay, have.perm, V.views[0].keys.p, V.views[0].n, have.bits.as<u32>(), e.stream);
+      if (made) mask_set(V.views[0].lay, V.views[0].perm, have.lay, have.perm, V.views[0].keys.p, nullptr, 4, V.views[0].n, have.bits.as<u32>(), nullptr, e.stream);
       M.vbits = have.bits.as<u32>();
       M.hbits = bwd_mask(e, S.fresh[hrel], H, A.packed.mask_h, &made).bits.as<u32>();
       if (made) throw LobError(LOB_E_CUDA, "internal error: mask of the new heads missing");

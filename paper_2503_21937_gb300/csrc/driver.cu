@@ -315,7 +315,7 @@ void plan_loop(lob_engine& e, GLoop& G, u32 max_iters) {
         const StepPlan& S = A.steps.back();
         ViewSt& W = e.rels[p.ast.body[S.atom].rel].views[S.view];
         engine_ensure_index(e, W, S.prefix_len);
-        G.d.arm_masked[a] = A.packed.mask_ok && W.index[S.prefix_len].mode == INDEX_DENSE;
+        G.d.arm_masked[a] = masked_step(e, A, W.index[S.prefix_len]);
       }
       for (size_t b = 0; b < A.before_rels.size(); b++) G.d.arm_before[a][b] = (int)A.before_rels[b];
     }
@@ -641,6 +641,8 @@ void capture_iteration(lob_engine& e, GLoop& G, u64* st_dev, u64* rec_dev, cudaS
         PMask M = A.packed.mask;
         M.vbits = VR.masks[find_mask(VR, W.perm)].bits.as<u32>();
         M.hbits = H.masks[find_mask(H, A.packed.mask_h)].bits.as<u32>();
+        M.vtags = VR.masks[find_mask(VR, W.perm)].tags.p;
+        M.htags = H.masks[find_mask(H, A.packed.mask_h)].tags.p;
         P.bitmap = H.dtouched.as<u32>();
         P.acc = H.dacc.p;
         pjoin_masked(ks, P, M, slot(ab + 1 + (int)s), st);
@@ -790,8 +792,8 @@ void capture_iteration(lob_engine& e, GLoop& G, u64* st_dev, u64* rec_dev, cudaS
     RelSt& H = e.rels[r];
     const ViewSt& V = H.views[0];
     for (auto& m : H.masks) {
-      mask_set(V.lay, V.perm, m.lay, m.perm, nullptr, G.cap_r[r], m.bits.as<u32>(), st, slot(rel_base(r) + R_RECENT),
-               nxt(grecent(r)), slot(S_OVERFLOW));
+      mask_set(V.lay, V.perm, m.lay, m.perm, nullptr, nullptr, sb, G.cap_r[r], m.bits.as<u32>(), m.tags.p, st,
+               slot(rel_base(r) + R_RECENT), nxt(grecent(r)), slot(S_OVERFLOW));
       e.check(cudaGetLastError(), "mask");
     }
   }

@@ -160,7 +160,10 @@ static void release_derived(lob_engine& e) {
                       &r.row_keys, &r.akeys, &r.atags, &r.akeys2, &r.atags2, &r.bitmap, &r.prev_bitmap, &r.dacc,
                       &r.dtouched})
       e.release(*b);
-    for (auto& m : r.masks) e.release(m.bits);
+    for (auto& m : r.masks) {
+      e.release(m.bits);
+      e.release(m.tags);
+    }
     r.masks.clear();
     r.extract = r.touched = r.keys_stale = r.dense = r.finished = false;
     r.n_recent = r.n_next = r.n_cand = r.n_acc = 0;
@@ -583,14 +586,16 @@ int find_mask(const RelSt& r, const int* perm) {
 // The masked form of an arm's last step (pjoin.h): the probed atom leaves one
 // column free, of at most 6 bits, which is the view's last and occurs once in the
 // head, in a column of at most 6 bits.
-constexpr int kMaskBits = 28;  // largest bitmap: 32 MB, cleared by every run
+constexpr int kMaskBits = 28;     // largest bitmap: 32 MB, cleared by every run
+constexpr int kMaskTagBits = 27;  // with tags by key (max-min semirings): up to 1 GB each
 static void compile_mask(lob_engine& e, const RuleAst& R, const ArmPlan& A, PackedArm& out) {
   if (!out.ok || A.steps.size() < 2 || !e.rels[R.body[A.delta].rel].idb) return;
   const StepPlan& S = A.steps.back();
   const AtomAst& atom = R.body[S.atom];
   const ViewSt& W = e.rels[atom.rel].views[S.view];
   const int last = (int)atom.args.size() - 1;
-  if (S.prefix_len != last || S.act[last].op != OP_BIND || W.lay.width[last] > 6 || W.lay.bits > kMaskBits) return;
+  const int max_bits = sem_idempotent(e.semiring) ? kMaskTagBits : kMaskBits;
+  if (S.prefix_len != last || S.act[last].op != OP_BIND || W.lay.width[last] > 6 || W.lay.bits > max_bits) return;
   const u32 z = atom.args[W.perm[last]].v;
   const RelSt& H = e.rels[R.head.rel];
   int hcol = -1;
@@ -599,7 +604,7 @@ static void compile_mask(lob_engine& e, const RuleAst& R, const ArmPlan& A, Pack
       if (hcol >= 0) return;
       hcol = (int)c;
     }
-  if (hcol < 0 || H.width[hcol] > 6 || H.views[0].lay.bits > kMaskBits) return;
+  if (hcol < 0 || H.width[hcol] > 6 || H.views[0].lay.bits > max_bits) return;
   int n = 0;
   for (int c = 0; c < (int)H.arity; c++)
     if (c != hcol) out.mask_h[n++] = c;
@@ -620,6 +625,14 @@ static void compile_mask(lob_engine& e, const RuleAst& R, const ArmPlan& A, Pack
     f.shift = (uint8_t)(L.sshift - M.hw);
     M.hf[M.n_hf++] = f;
   }
+  M.n_of = 0;
+  for (int c = 0; c < P.n_out; c++)
+    if (c != hcol) M.of[M.n_of++] = P.out[c];
+  M.zshift = P.out[hcol].shift;
+  // the step's checks compare the free column, or values of the input word
+  for (int q = 0; q < P.n_checks; q++)
+    for (const POperand& o : {P.checks[q].a, P.checks[q].b})
+      if (o.word == 1 && (o.shift != 0 || o.width != M.vw)) return;
   out.mask_ok = true;
 }
 
@@ -757,7 +770,7 @@ static void prepare_arms(lob_engine& e) {
       // and comparison filters run bytecode: general steps only
       A.packed = e.opt_packed_join && !sem_top1(sem) && !p.ast.computes() ? compile_packed(e, p.ast, A) : PackedArm{};
       if (sem == SR_UNIT) compile_cross(e, p.ast, A, A.packed);
-      if (sem_stamps(sem)) compile_mask(e, p.ast, A, A.packed);
+      if (sem != SR_UNIT) compile_mask(e, p.ast, A, A.packed);
     }
 }
 
@@ -1501,10 +1514,12 @@ static void run_arm_packed(lob_engine& e, const RulePlan& rp, const ArmPlan& A, 
       n_in = total;
       continue;
     }
-    if (last && H.dense && A.packed.mask_ok && I.mode == INDEX_DENSE) {  // only the outputs that can be new facts
+    if (last && H.dense && masked_step(e, A, I)) {  // only the outputs that can be new facts
       PMask M = A.packed.mask;
       M.vbits = V.masks[find_mask(V, W.perm)].bits.as<u32>();
       M.hbits = H.masks[find_mask(H, A.packed.mask_h)].bits.as<u32>();
+      M.vtags = V.masks[find_mask(V, W.perm)].tags.p;
+      M.htags = H.masks[find_mask(H, A.packed.mask_h)].tags.p;
       H.touched = true;
       P.bitmap = H.dtouched.as<u32>();
       P.acc = H.dacc.p;
@@ -1946,9 +1961,11 @@ static void add_mask(lob_engine& e, RelSt& r, const int* perm) {
   MaskSt& M = r.masks.back();
   e.ensure(M.bits, mask_bytes(M.lay));
   e.check(cudaMemsetAsync(M.bits.p, 0, mask_bytes(M.lay), e.stream), "mask");
+  const int sb = stored_bytes(e.semiring);
+  if (sem_idempotent(e.semiring)) e.ensure(M.tags, (1ull << M.lay.bits) * sb);
   const ViewSt& V = r.views[0];
   if (!V.n) return;
-  mask_set(V.lay, V.perm, M.lay, M.perm, V.keys.p, V.n, M.bits.as<u32>(), e.stream);
+  mask_set(V.lay, V.perm, M.lay, M.perm, V.keys.p, V.tags.p, sb, V.n, M.bits.as<u32>(), M.tags.p, e.stream);
   e.after_launch("mask");
   e.launches++;
 }
@@ -1986,7 +2003,8 @@ static void update_masks(lob_engine& e, RelSt& r) {
   if (!r.n_next) return;
   const ViewSt& V = r.views[0];
   for (auto& m : r.masks) {
-    mask_set(V.lay, V.perm, m.lay, m.perm, r.nkeys.p, r.n_next, m.bits.as<u32>(), e.stream);
+    mask_set(V.lay, V.perm, m.lay, m.perm, r.nkeys.p, r.ntags.p, stored_bytes(e.semiring), r.n_next, m.bits.as<u32>(),
+             m.tags.p, e.stream);
     e.after_launch("mask");
     e.launches++;
   }

@@ -83,6 +83,7 @@ struct MaskSt {
   int perm[kMaxArity] = {0};
   Layout lay{};
   DevBuf bits;
+  DevBuf tags;  // max-min semirings: the facts' stored tags by key (only where bits says so)
 };
 
 struct RelSt {
@@ -304,6 +305,9 @@ void engine_ensure_index(lob_engine& e, ViewSt& v, int prefix);
 // the mask of r with column order perm (its layout; allocated by the caller), or -1
 int find_mask(const RelSt& r, const int* perm);
 Layout mask_layout(const lob_engine& e, const RelSt& r, const int* perm);
+// whether the arm's last step, probing the index I, runs as a masked one (add-mult
+// finds the matches' rows through a dense index, max-min reads tags by key)
+inline bool masked_step(const lob_engine& e, const ArmPlan& A, const IndexSt& I);
 inline u64 mask_bytes(const Layout& L) { return std::max<u64>(16, (1ull << L.bits) / 8); }
 // copy a rule's bytecode programs into step parameters
 void set_rule_code(const RuleAst& R, StepParams& P);
@@ -343,4 +347,7 @@ inline bool begins_stratum(const std::vector<u32>& begin, u32 k) {
 }
 inline int sem_kernel(int sem) {
   return sem == SR_DIFF_ADD_MULT ? SR_ADD_MULT : (sem == SR_DIFF_TOP1 ? SR_TOP1 : sem);
+}
+inline bool masked_step(const lob_engine& e, const ArmPlan& A, const IndexSt& I) {
+  return A.packed.mask_ok && (sem_idempotent(e.semiring) || I.mode == INDEX_DENSE);
 }

@@ -1014,26 +1014,47 @@ LOB_DEV u32 select_bit(u64 m, u32 n) {
   return at;
 }
 
-// row r's input word, probe key and masks; 0 when the row has no match
-LOB_DEV u64 masked_row(const PStep& P, const PPtrs& Q, const PMask& M, u64 r, u64 n_in, u64& wi, u64& pv, u64& hm) {
-  pv = hm = 0;
-  wi = 0;
-  if (r >= n_in) return 0;
-  wi = load_word(Q.in_words, P.in_w64, r);
-  if (wi == (P.in_w64 ? ~0ull : 0xFFFFFFFFull)) return 0;
+// An input row of a masked step: its matches (vm), those the step's checks let
+// through (ok), its head row's facts (hm), and the keys the columns extend.
+struct MaskedRow {
+  u64 vm, ok, hm, pv, h, hk;
+};
+LOB_DEV MaskedRow masked_row(const PStep& P, const PPtrs& Q, const PMask& M, u64 r, u64 n_in) {
+  MaskedRow x;
+  x.vm = x.ok = x.hm = x.pv = x.h = x.hk = 0;
+  if (r >= n_in) return x;
+  const u64 wi = load_word(Q.in_words, P.in_w64, r);
+  if (wi == (P.in_w64 ? ~0ull : 0xFFFFFFFFull)) return x;
   if (P.in_stamp_mode != STAMP_NONE) {
     const u32 st = P.in_stamp[r] & 0x7FFFFFFFu;
-    if (P.in_stamp_mode == STAMP_LT ? !(st < P.in_stamp_val) : st != P.in_stamp_val) return 0;
+    if (P.in_stamp_mode == STAMP_LT ? !(st < P.in_stamp_val) : st != P.in_stamp_val) return x;
   }
-  if (P.n_in_checks && !checks_ok(P.in_checks, P.n_in_checks, wi, 0)) return 0;
+  if (P.n_in_checks && !checks_ok(P.in_checks, P.n_in_checks, wi, 0)) return x;
   for (int q = 0; q < P.n_prefix; q++) {
-    const u64 x = pick(P.prefix[q].op, wi, 0);
-    if (P.prefix[q].limit_bits < 64 && (x >> P.prefix[q].limit_bits)) return 0;
-    pv |= x << P.prefix[q].shift;
+    const u64 f = pick(P.prefix[q].op, wi, 0);
+    if (P.prefix[q].limit_bits < 64 && (f >> P.prefix[q].limit_bits)) return x;
+    x.pv |= f << P.prefix[q].shift;
   }
-  const u64 vm = row_bits(M.vbits, pv, M.vw);
-  if (vm) hm = row_bits(M.hbits, compose(M.hf, M.n_hf, wi, 0), M.hw);
-  return vm;
+  x.vm = row_bits(M.vbits, x.pv, M.vw);
+  if (!x.vm) return x;
+  x.ok = x.vm;
+  for (int q = 0; q < P.n_checks; q++) {  // a check on the free column (word 1) is a mask of it
+    const PCheck& c = P.checks[q];
+    const bool eq = c.eq != 0;
+    if (c.a.word == 1 && c.b.word == 1) {
+      if (!eq) x.ok = 0;
+    } else if (c.a.word == 1 || c.b.word == 1) {
+      const u64 y = pick(c.a.word == 1 ? c.b : c.a, wi, 0);
+      const u64 bit = y < 64 ? 1ull << y : 0ull;
+      x.ok &= eq ? bit : ~bit;
+    } else if ((pick(c.a, wi, 0) == pick(c.b, wi, 0)) != eq) {
+      x.ok = 0;
+    }
+  }
+  x.h = compose(M.hf, M.n_hf, wi, 0);
+  x.hk = compose(M.of, M.n_of, wi, 0);
+  x.hm = row_bits(M.hbits, x.h, M.hw);
+  return x;
 }
 
 template <class Sem>
@@ -1048,11 +1069,10 @@ __global__ void __launch_bounds__(256) k_pmasked(const __grid_constant__ PStep P
   const u32 vsv = P.stamp_dev ? (u32)*P.stamp_dev + P.v_stamp_val : P.v_stamp_val;
   u64 mine = 0;
   for (u64 g = (u64)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); g * 32 < n_in; g += nwarps) {
-    u64 wi, pv, hm;
     const u64 r = g * 32 + lane;
-    const u64 vm = masked_row(P, Q, M, r, n_in, wi, pv, hm);
-    mine += __popcll(vm);
-    const u64 m = vm & ~hm;
+    const MaskedRow x = masked_row(P, Q, M, r, n_in);
+    mine += __popcll(x.vm);
+    const u64 m = x.ok & ~x.hm;
     const u32 c = __popcll(m);
     const u32 inc = warp_inclusive_sum(c);
     const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
@@ -1061,7 +1081,7 @@ __global__ void __launch_bounds__(256) k_pmasked(const __grid_constant__ PStep P
     C ct = Sem::one();
     u64 lo = 0;
     if (c) {
-      lo = P.dense_offs[pv];
+      lo = P.dense_offs[x.pv];
       ct = P.in_packed ? Sem::from_stored(reinterpret_cast<const S*>(Q.in_tags)[r]) : reinterpret_cast<const C*>(Q.in_tags)[r];
     }
     for (u32 t0 = 0; t0 < tot; t0 += 32) {
@@ -1072,9 +1092,8 @@ __global__ void __launch_bounds__(256) k_pmasked(const __grid_constant__ PStep P
         const u32 e = __shfl_sync(0xFFFFFFFFu, ex, src + step);
         if (e <= t) src += step;
       }
-      const u64 wr = __shfl_sync(0xFFFFFFFFu, wi, src);
-      const u64 mr = __shfl_sync(0xFFFFFFFFu, m, src), vr = __shfl_sync(0xFFFFFFFFu, vm, src);
-      const u64 pr = __shfl_sync(0xFFFFFFFFu, pv, src), lr = __shfl_sync(0xFFFFFFFFu, lo, src);
+      const u64 mr = __shfl_sync(0xFFFFFFFFu, m, src), vr = __shfl_sync(0xFFFFFFFFu, x.vm, src);
+      const u64 kr = __shfl_sync(0xFFFFFFFFu, x.hk, src), lr = __shfl_sync(0xFFFFFFFFu, lo, src);
       const u32 er = __shfl_sync(0xFFFFFFFFu, ex, src);
       const C tr = __shfl_sync(0xFFFFFFFFu, ct, src);
       if (t >= tot) continue;
@@ -1084,12 +1103,80 @@ __global__ void __launch_bounds__(256) k_pmasked(const __grid_constant__ PStep P
         const u32 st = Q.v_stamp[v] & 0x7FFFFFFFu;
         if (P.v_stamp_mode == STAMP_LT ? st >= vsv : st != vsv) continue;
       }
-      const u64 wv = (pr << M.vw) | z;
-      if (!checks_ok(P.checks, P.n_checks, wr, wv)) continue;
-      const u64 w = compose(P.out, P.n_out, wr, wv);
+      const u64 w = kr | ((u64)z << M.zshift);
       dense_add<Sem>(P.acc, w, Sem::mul(tr, Sem::from_stored(reinterpret_cast<const S*>(Q.v_tags)[v])));
       touch_bit(P.bitmap, w);
     }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
+  if (lane == 0 && mine) atomicAdd(emitted, (unsigned long long)mine);
+}
+
+// max-min semirings: a fact that is present still takes candidates with a larger
+// tag, so every match's product is formed -- but against the stored tags of the
+// head row, and only what beats them goes on.  A warp takes an input row at a
+// time, a lane a column, so the two tag rows are read as consecutive words (two
+// rows at once, for loads in flight); the general step reads an accumulator slot
+// in L2 per match that nothing but this iteration has filled.  Bound by issue:
+// the batched kinship program forms 5.3e9 products in 350 million half rows, 5.7e8
+// of which beat the stored tag (54 -> 35 ms, and the read-out of the accumulator
+// 12 -> 4.5 ms, as it lists fewer heads).  Four half rows in flight from a list
+// of the non-empty ones took 39 ms: latency is not what it waits for.
+template <class Sem>
+__global__ void __launch_bounds__(256) k_pmasked_rows(const __grid_constant__ PStep P, const __grid_constant__ PMask M,
+                                                      unsigned long long* emitted) {
+  typedef typename Sem::Stored S;
+  typedef typename Sem::Cand C;
+  struct Rec { u64 v, h, ok, hm, hk; C t; };
+  __shared__ Rec recs[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u64 nwarps = (u64)gridDim.x * (blockDim.x / 32);
+  const u64 n_in = dev_size(P.n_in, P.n_in_dev);
+  const PPtrs Q = resolve_ptrs(P);
+  const S* vt = reinterpret_cast<const S*>(M.vtags);
+  const S* ht = reinterpret_cast<const S*>(M.htags);
+  u64 mine = 0;
+  for (u64 g = (u64)blockIdx.x * (blockDim.x / 32) + warp; g * 32 < n_in; g += nwarps) {
+    const u64 r = g * 32 + lane;
+    const MaskedRow x = masked_row(P, Q, M, r, n_in);
+    mine += __popcll(x.vm);
+    const u32 act = __ballot_sync(0xFFFFFFFFu, x.ok != 0);
+    const int n_act = __popc(act);
+    if (x.ok) {
+      const C t = P.in_packed ? Sem::from_stored(reinterpret_cast<const S*>(Q.in_tags)[r])
+                              : reinterpret_cast<const C*>(Q.in_tags)[r];
+      recs[warp][__popc(act & ((1u << lane) - 1u))] = Rec{x.pv << M.vw, x.h << M.hw, x.ok, x.hm, x.hk, t};
+    }
+    __syncwarp();
+    for (int i = 0; i < n_act; i += 2) {
+      const Rec y[2] = {recs[warp][i], recs[warp][min(i + 1, n_act - 1)]};
+      const bool two = i + 1 < n_act;
+#pragma unroll
+      for (int base = 0; base < 64; base += 32) {
+        if (base && !((y[0].ok | y[1].ok) >> 32)) break;  // no column past 31
+        const int z = base + lane;
+        S tr[2], fh[2];
+        bool on[2], present[2];
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+          on[j] = (j == 0 || two) && ((y[j].ok >> z) & 1u);
+          present[j] = on[j] && ((y[j].hm >> z) & 1u);
+          if (on[j]) tr[j] = vt[y[j].v + z];
+          if (present[j]) fh[j] = ht[y[j].h + z];
+        }
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+          if (!on[j]) continue;
+          const C c = Sem::mul(y[j].t, Sem::from_stored(tr[j]));
+          if (present[j] && fh[j] >= Sem::store(c)) continue;  // changes nothing
+          const u64 w = y[j].hk | ((u64)z << M.zshift);
+          dense_add<Sem>(P.acc, w, c);
+          touch_bit(P.bitmap, w);
+        }
+      }
+    }
+    __syncwarp();
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
@@ -1100,19 +1187,19 @@ __global__ void __launch_bounds__(256) k_pmasked(const __grid_constant__ PStep P
 // shares go out as one FP64 atomic each, the carried facts' as one per row: their
 // sum needs no reduction across lanes, which at this GPU's FP64 rate cost more
 // than the lanes left idle by rows of fewer bits (batched kinship, 1.05e9
-// groundings with an adjoint: 17.8 ms; balanced rounds with an atomic per
-// grounding and carried fact 22.4, with a segmented sum 25.0).
+// groundings with an adjoint: 17.8 ms, 11.7 since a row's checks became a mask;
+// balanced rounds with an atomic per grounding and carried fact 22.4, with a
+// segmented sum 25.0).
 __global__ void __launch_bounds__(256) k_pbwd_masked(const __grid_constant__ PStep P, const __grid_constant__ PBwd B,
                                                      const __grid_constant__ PMask M) {
   const u64 stride = (u64)gridDim.x * blockDim.x;
   const PPtrs Q = resolve_ptrs(P);
   const int nf_in = B.packed_source ? 1 : B.n_in_facts;
   for (u64 r = (u64)blockIdx.x * blockDim.x + threadIdx.x; r < P.n_in; r += stride) {
-    u64 wi, pv, hm;
-    const u64 vm = masked_row(P, Q, M, r, P.n_in, wi, pv, hm);
-    const u64 m = vm & hm;
+    const MaskedRow x = masked_row(P, Q, M, r, P.n_in);
+    const u64 m = x.ok & x.hm;
     if (!m) continue;
-    const u64 lo = P.dense_offs[pv];
+    const u64 lo = P.dense_offs[x.pv];
     u32 rows[kMaxArity];
     float tags[kMaxArity];
     double carried = 1.0;
@@ -1124,14 +1211,12 @@ __global__ void __launch_bounds__(256) k_pbwd_masked(const __grid_constant__ PSt
     double share = 0.0;
     for (u64 mm = m; mm; mm &= mm - 1) {
       const u32 z = __ffsll(mm) - 1;
-      const u64 v = lo + __popcll(vm & ((1ull << z) - 1ull));
+      const u64 v = lo + __popcll(x.vm & ((1ull << z) - 1ull));
       if (P.v_stamp_mode != STAMP_NONE) {
         const u32 st = P.v_stamp[v] & 0x7FFFFFFFu;
         if (P.v_stamp_mode == STAMP_LT ? st >= P.v_stamp_val : st != P.v_stamp_val) continue;
       }
-      const u64 wv = (pv << M.vw) | z;
-      if (!checks_ok(P.checks, P.n_checks, wi, wv)) continue;
-      const double adj = B.h_adj[B.h_row[compose(P.out, P.n_out, wi, wv)]];
+      const double adj = B.h_adj[B.h_row[x.hk | ((u64)z << M.zshift)]];
       const u32 vrow = B.v_prow ? B.v_prow[v] : (u32)v;
       share += adj * (double)B.fact_tags[nf_in][vrow];
       if (B.fact_adj[nf_in]) atomicAdd(B.fact_adj[nf_in] + vrow, adj * carried);
@@ -1139,10 +1224,10 @@ __global__ void __launch_bounds__(256) k_pbwd_masked(const __grid_constant__ PSt
     if (share == 0.0) continue;
     for (int q = 0; q < nf_in; q++) {
       if (!B.fact_adj[q]) continue;
-      double x = share;
+      double y = share;
       for (int l = 0; l < nf_in; l++)
-        if (l != q) x *= (double)tags[l];
-      atomicAdd(B.fact_adj[q] + rows[q], x);
+        if (l != q) y *= (double)tags[l];
+      atomicAdd(B.fact_adj[q] + rows[q], y);
     }
   }
 }
@@ -1150,7 +1235,7 @@ __global__ void __launch_bounds__(256) k_pbwd_masked(const __grid_constant__ PSt
 struct MaskPerm {
   int from[kMaxArity], to[kMaxArity];
 };
-LOB_DEV void set_mask_bit(const Layout& F, const Layout& T, const MaskPerm& p, u64 k, u32* bits) {
+LOB_DEV u64 set_mask_bit(const Layout& F, const Layout& T, const MaskPerm& p, u64 k, u32* bits) {
   u32 rel[kMaxArity];
 #pragma unroll
   for (int j = 0; j < kMaxArity; j++)
@@ -1160,16 +1245,24 @@ LOB_DEV void set_mask_bit(const Layout& F, const Layout& T, const MaskPerm& p, u
   for (int j = 0; j < kMaxArity; j++)
     if (j < T.arity) o |= (u64)rel[p.to[j]] << T.shift[j];
   atomicOr(bits + (o >> 5), 1u << (u32)(o & 31u));
+  return o;
 }
+template <class S>
 __global__ void k_mask_set(const __grid_constant__ Layout F, const __grid_constant__ Layout T,
-                           const __grid_constant__ MaskPerm p, const void* keys, u64 n, u32* __restrict__ bits,
-                           const u64* n_dev, void* const* keys_pp, const u64* skip) {
+                           const __grid_constant__ MaskPerm p, const void* keys, const S* tags, u64 n,
+                           u32* __restrict__ bits, S* __restrict__ otags, const u64* n_dev, void* const* keys_pp,
+                           const u64* skip) {
   if (skip && *skip) return;
   if (n_dev) n = *n_dev < n ? *n_dev : n;
-  if (keys_pp) keys = keys_pp[0];
+  if (keys_pp) {
+    keys = keys_pp[0];
+    tags = reinterpret_cast<const S*>(keys_pp[1]);
+  }
   const u64 stride = (u64)gridDim.x * blockDim.x;
-  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    set_mask_bit(F, T, p, load_key(keys, F.key64, i), bits);
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const u64 o = set_mask_bit(F, T, p, load_key(keys, F.key64, i), bits);
+    if (otags) otags[o] = tags[i];
+  }
 }
 __global__ void k_mask_new(const __grid_constant__ Layout F, const __grid_constant__ Layout T,
                            const __grid_constant__ MaskPerm p, const void* __restrict__ keys, u64 n,
@@ -1338,16 +1431,27 @@ void pjoin_masked(int sem, const PStep& P, const PMask& M, u64* emitted_dev, cud
   // an input row reads its word, two bitmap rows and, with outputs, its tag
   ProfScope ps("join_masked", P.n_in * (row_bytes(sem, P.in_w64, P.in_packed) + 16.0), st);
   if (!P.n_in) return;
-  k_pmasked<SemAddMult><<<grid_n(P.n_in), 256, 0, st>>>(P, M, reinterpret_cast<unsigned long long*>(emitted_dev));
+  auto* em = reinterpret_cast<unsigned long long*>(emitted_dev);
+  if (sem == SR_MAX_MIN) k_pmasked_rows<SemMaxMin><<<grid_n(P.n_in), 256, 0, st>>>(P, M, em);
+  else if (sem == SR_DIFF_MAX_MIN) k_pmasked_rows<SemDiffMaxMin><<<grid_n(P.n_in), 256, 0, st>>>(P, M, em);
+  else k_pmasked<SemAddMult><<<grid_n(P.n_in), 256, 0, st>>>(P, M, em);
 }
 void pjoin_backward_masked(const PStep& P, const PBwd& B, const PMask& M, cudaStream_t st) {
   ProfScope ps("bwd_masked", P.n_in * ((P.in_w64 ? 8.0 : 4.0) + 16.0), st);
   if (P.n_in) k_pbwd_masked<<<grid_n(P.n_in), 256, 0, st>>>(P, B, M);
 }
-void mask_set(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys, u64 n,
-              u32* bits, cudaStream_t st, const u64* n_dev, void* const* keys_pp, const u64* skip_dev) {
-  ProfScope ps("mask_set", n * (from.key64 ? 8.0 : 4.0), st);
-  if (n) k_mask_set<<<grid_n(n), 256, 0, st>>>(from, to, mask_perm(from, perm_from, perm_to), keys, n, bits, n_dev, keys_pp, skip_dev);
+void mask_set(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys,
+              const void* tags, int tag_bytes, u64 n, u32* bits, void* otags, cudaStream_t st, const u64* n_dev,
+              void* const* keys_pp, const u64* skip_dev) {
+  ProfScope ps("mask_set", n * ((from.key64 ? 8.0 : 4.0) + (otags ? 2.0 * tag_bytes : 0.0)), st);
+  if (!n) return;
+  const MaskPerm p = mask_perm(from, perm_from, perm_to);
+  if (tag_bytes == 8)
+    k_mask_set<u64><<<grid_n(n), 256, 0, st>>>(from, to, p, keys, static_cast<const u64*>(tags), n, bits,
+                                               static_cast<u64*>(otags), n_dev, keys_pp, skip_dev);
+  else
+    k_mask_set<u32><<<grid_n(n), 256, 0, st>>>(from, to, p, keys, static_cast<const u32*>(tags), n, bits,
+                                               static_cast<u32*>(otags), n_dev, keys_pp, skip_dev);
 }
 void mask_set_new(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys, u64 n,
                   const u32* stamps, u32 k, const double* adj, u32* bits, cudaStream_t st) {

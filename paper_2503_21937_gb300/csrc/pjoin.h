@@ -108,7 +108,7 @@ struct PBwd {
 void pjoin_backward_emit(const PStep& P, const PBwd& B, const u64* part, cudaStream_t st);
 bool pjoin_backward_supported(const PStep& P);  // the emission has a kernel for the step's shape
 
-// Masked last step (diff-)add-mult: the view's rows for a probe key and the head
+// Masked last step (add-mult and max-min semirings): the view's rows for a probe key and the head
 // keys an input row can produce differ in one column of at most 6 bits, so each
 // is a 64-bit row of a bitmap: vbits over the view's keys (row = probe key), hbits
 // over the head's keys with that column last (row = the hf fields of the input
@@ -118,19 +118,24 @@ struct PMask {
   const u32* vbits; int vw;  // row width in bits: 2^vw
   const u32* hbits; int hw;
   int n_hf; PField hf[kMaxPFields];
+  // head key = the of fields of the input word | column << zshift
+  int n_of; PField of[kMaxPFields]; int zshift;
+  const void* vtags; const void* htags;  // max-min semirings: stored tags by the same keys
 };
-// (+)-adds the outputs whose head is not in hbits (under the key policy of these
-// semirings a fact that is present takes no more candidates) into P.acc, marks
-// them in P.bitmap, and adds all matches to *emitted_dev.  Dense index only.
+// (+)-adds the outputs that can change a fact into P.acc, marks them in P.bitmap,
+// and adds all matches to *emitted_dev.  add-mult: the heads not in hbits (under
+// its key policy a fact that is present takes no more candidates; dense index
+// only).  max-min: the heads that are absent or whose stored tag is smaller.
 void pjoin_masked(int sem, const PStep& P, const PMask& M, u64* emitted_dev, cudaStream_t st);
 // the last step of a backward replay: only the groundings whose head is in hbits
 void pjoin_backward_masked(const PStep& P, const PBwd& B, const PMask& M, cudaStream_t st);
 // sets the bits of n keys, re-encoded from layout `from` to layout `to`; n_dev: a
-// device-resident count (n its capacity); keys_pp: the keys' pointer in device
-// memory; skip_dev: nothing is done when it holds non-zero
-void mask_set(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys, u64 n,
-              u32* bits, cudaStream_t st, const u64* n_dev = nullptr, void* const* keys_pp = nullptr,
-              const u64* skip_dev = nullptr);
+// device-resident count (n its capacity); keys_pp: the keys' and tags' pointers in
+// device memory; skip_dev: nothing is done when it holds non-zero.  With otags,
+// each key's stored tag (tag_bytes) is written there as well.
+void mask_set(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys,
+              const void* tags, int tag_bytes, u64 n, u32* bits, void* otags, cudaStream_t st, const u64* n_dev = nullptr,
+              void* const* keys_pp = nullptr, const u64* skip_dev = nullptr);
 // the same for the facts first derived, unclamped, in iteration k that have an adjoint
 void mask_set_new(const Layout& from, const int* perm_from, const Layout& to, const int* perm_to, const void* keys, u64 n,
                   const u32* stamps, u32 k, const double* adj, u32* bits, cudaStream_t st);
