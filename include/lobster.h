@@ -386,7 +386,9 @@ int lob_prim_diff_merge(lob_engine* e, int semiring, const void* f_keys, const v
  * calls whose work overlaps on the GPU race: order them (one stream, or
  * events).  A row whose every column is 0xFFFFFFFF is dropped (at arity 1
  * and 2 alike).  The work is
- * queued on cuda_stream (NULL: legacy default stream); the call does not wait. */
+ * queued on cuda_stream (NULL: legacy default stream); the call does not wait.
+ * The sort's blocks wait on one another, with a limit; should a wait give up,
+ * *n_out gets 2^64 - 1 and out_cols is not written. */
 #define LOB_NOALLOC_MAX_ROWS 262144u
 int lob_unique_rows_noalloc(const uint32_t* cols, uint32_t arity, uint64_t n, uint32_t* out_cols, uint64_t* n_out,
                             void* cuda_stream);

@@ -543,6 +543,7 @@ ByStamp& by_stamp(lob_engine& e, BwdState& S, u32 rel) {
   e.ensure(e.tmp_tags, n * 4);
   e.ensure(B.rows, n * 4);
   e.ensure(B.words, n * kb);
+  e.check(cudaMemsetAsync(e.counts.as<u64>() + 15, 0, sizeof(u32), e.stream), "sort error word");
   k_stamp_keys<<<grid_for_n(n), 256, 0, e.stream>>>(V.stamps.as<u32>(), n, e.tmp_keys.as<u32>(), e.tmp_tags.as<u32>());
   e.after_launch("stamps");
   void* k = e.tmp_keys.p;
@@ -550,7 +551,8 @@ ByStamp& by_stamp(lob_engine& e, BwdState& S, u32 rel) {
   int bits = 1;
   while (bits < 32 && (n_stamps >> bits)) bits++;
   e.ensure(e.scratch, sort_scratch_bytes(n, e.opt_radix_bits));
-  sort_pairs(0, 4, &k, &r, e.tmp_keys2.p, B.rows.p, n, bits, e.opt_radix_bits, e.scratch.p, e.stream);
+  sort_pairs(0, 4, &k, &r, e.tmp_keys2.p, B.rows.p, n, bits, e.opt_radix_bits, e.scratch.p, e.stream, nullptr,
+             reinterpret_cast<u32*>(e.counts.as<u64>() + 15));
   e.after_launch("stamp sort");
   if (r != B.rows.p) e.check(cudaMemcpyAsync(B.rows.p, r, n * 4, cudaMemcpyDeviceToDevice, e.stream), "stamp rows");
   if (kb == 8) k_stamp_words<u64><<<grid_for_n(n), 256, 0, e.stream>>>(V.keys.as<u64>(), B.rows.as<u32>(), n, B.words.as<u64>());
@@ -560,7 +562,8 @@ ByStamp& by_stamp(lob_engine& e, BwdState& S, u32 rel) {
   e.after_launch("stamps");
   B.off.resize((size_t)n_stamps + 1);
   e.check(cudaMemcpyAsync(B.off.data(), e.off.p, B.off.size() * 4, cudaMemcpyDeviceToHost, e.stream), "stamps");
-  e.sync();
+  if (e.read_u64(e.counts.as<u64>() + 15) & 0xFFFFFFFFull)
+    throw LobError(LOB_E_TIMEOUT, "a bounded device wait of the sort gave up; the gradients are invalid");
   return B;
 }
 

@@ -794,7 +794,7 @@ static void engine_sort(lob_engine& e, int key64, int pay_bytes, void** keys, vo
     e.launches += sort_onesweep_launches(n, bits, rb);
   } else {
     scratch_at_least(e, sort_scratch_bytes(n, rb));
-    sort_pairs(key64, pay_bytes, keys, pay, ktmp, ptmp, n, bits, rb, e.scratch.p, e.stream);
+    sort_pairs(key64, pay_bytes, keys, pay, ktmp, ptmp, n, bits, rb, e.scratch.p, e.stream, nullptr, sort_err(e));
     e.launches += sort_kernel_launches(n, bits, rb);
   }
 }

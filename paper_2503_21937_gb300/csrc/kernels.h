@@ -36,8 +36,10 @@ size_t sort_scratch_bytes(u64 n, int rb);
 // Stable LSD sort of n (key, payload) pairs on the low `bits` key bits.  keys,
 // pay point at the input and are updated to whichever buffer holds the result
 // (the inputs or ktmp/ptmp).  pay_bytes is 0 (no payload), 4 or 8.
+// err (optional) is set, never cleared, if a bounded device wait of the one-launch
+// form gave up, in which case the output is invalid.
 void sort_pairs(int key64, int pay_bytes, void** keys, void** pay, void* ktmp, void* ptmp, u64 n, int bits, int rb,
-                void* scratch, cudaStream_t st, const u64* n_dev = nullptr);
+                void* scratch, cudaStream_t st, const u64* n_dev = nullptr, u32* err = nullptr);
 int sort_kernel_launches(u64 n, int bits, int rb);
 // Same result with one kernel per digit pass (decoupled look-back); *err is set
 // (never cleared) if a bounded wait gave up, in which case the output is invalid.
