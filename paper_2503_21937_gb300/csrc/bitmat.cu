@@ -55,17 +55,25 @@ constexpr int kStateSlots = B_REL + 3 * kMaxBitRels;
 // ... and, not read back, two list lengths for each of an iteration's products
 constexpr int kMaxLists = 32;
 constexpr int kAllSlots = kStateSlots + 2 * kMaxLists;
+// (the loop in one launch uses the first of those as its barrier words)
+constexpr int kReadSlots = kStateSlots + 1;
 
 enum IndexKind { I_IDENT = 0, I_CSR = 1, I_BITS = 2 };
 
 // A bit matrix.  Row r is empty, whatever its words hold, when cnt[r] (bag[r]
 // when bag is set) is 0.  bag[r]: the derivations row r stands for, duplicates
 // included (a stored relation's is its facts, cnt).
+// What a run's iterations write, read by a launch that spans several of them
+// (kLoop): past L1, which keeps lines of earlier iterations.
+template <bool kLoop, class T> LOB_DEV T ldm(const T* p) {
+  if constexpr (kLoop) return __ldcg(p);
+  else return *p;
+}
 struct BMat {
   const u32* bits;
   const u32* cnt;
   const u64* bag;
-  LOB_DEV u64 weight(u32 r) const { return bag ? bag[r] : (u64)cnt[r]; }
+  template <bool kLoop> LOB_DEV u64 weight(u32 r) const { return bag ? ldm<kLoop>(bag + r) : (u64)ldm<kLoop>(cnt + r); }
 };
 struct BCsr {
   const u32* ptr;
@@ -105,10 +113,11 @@ struct BOp {
   int skip[kMaxChain];
 };
 
+template <bool kLoop>
 LOB_DEV bool op_idle(const BOp& P) {
-  if (P.state[B_DONE]) return true;
+  if (ldm<kLoop>(P.state + B_DONE)) return true;
   for (int i = 0; i < P.n_skip; i++)
-    if (P.state[rel_slot(P.skip[i], 0)] == P.state[rel_slot(P.skip[i], 1)]) return true;
+    if (ldm<kLoop>(P.state + rel_slot(P.skip[i], 0)) == ldm<kLoop>(P.state + rel_slot(P.skip[i], 1))) return true;
   return false;
 }
 
@@ -132,6 +141,7 @@ LOB_DEV void diag4(uint4& a, int diag, u32 r, u32 w) {
 
 // The words [w, w + 4) of result row r go where the product's result goes;
 // returns the new facts among them (commit).
+template <bool kLoop>
 LOB_DEV u32 put4(const BOp& P, u32 r, u32 w, uint4 a) {
   const u64 at = ((u64)r * P.words + w) / 4;
   if (P.out) {
@@ -142,19 +152,19 @@ LOB_DEV u32 put4(const BOp& P, u32 r, u32 w, uint4 a) {
   if (!P.commit) {
     if (any4(a)) {
       uint4* N = reinterpret_cast<uint4*>(P.acc) + at;
-      or4(a, *N);
+      or4(a, ldm<kLoop>(N));
       *N = a;
       P.aflag[r] = 1;
     }
     return 0;
   }
-  if (P.aflag && P.aflag[r]) {
+  if (P.aflag && ldm<kLoop>(P.aflag + r)) {
     uint4* N = reinterpret_cast<uint4*>(P.acc) + at;
-    or4(a, *N);
+    or4(a, ldm<kLoop>(N));
     *N = make_uint4(0, 0, 0, 0);
   }
   uint4* F = reinterpret_cast<uint4*>(P.full) + at;
-  uint4 f = *F;
+  uint4 f = ldm<kLoop>(F);
   a.x &= ~f.x; a.y &= ~f.y; a.z &= ~f.z; a.w &= ~f.w;
   reinterpret_cast<uint4*>(P.next)[at] = a;
   if (any4(a)) {
@@ -232,17 +242,18 @@ LOB_DEV Lanes split_lanes(u32 words, u32 chunk) {
 }
 
 // acc |= the words of the n operand rows listed in shared memory
+template <bool kLoop>
 LOB_DEV void gather_list(const BMat& M, u32 words, const Lanes& L, const u32* list, int n, uint4& acc) {
   if (!L.in) return;
   const uint4* base = reinterpret_cast<const uint4*>(M.bits + L.w);
   const u64 stride = words / 4;
   int k = L.sub;
   for (; k + 3 * L.n_sub < n; k += 4 * L.n_sub) {  // four rows in flight
-    const uint4 a = base[list[k] * stride], b = base[list[k + L.n_sub] * stride];
-    const uint4 c = base[list[k + 2 * L.n_sub] * stride], d = base[list[k + 3 * L.n_sub] * stride];
+    const uint4 a = ldm<kLoop>(base + list[k] * stride), b = ldm<kLoop>(base + list[k + L.n_sub] * stride);
+    const uint4 c = ldm<kLoop>(base + list[k + 2 * L.n_sub] * stride), d = ldm<kLoop>(base + list[k + 3 * L.n_sub] * stride);
     or4(acc, a); or4(acc, b); or4(acc, c); or4(acc, d);
   }
-  for (; k < n; k += L.n_sub) or4(acc, base[list[k] * stride]);
+  for (; k < n; k += L.n_sub) or4(acc, ldm<kLoop>(base + list[k] * stride));
 }
 
 LOB_DEV void or_groups(const Lanes& L, uint4& a) {
@@ -256,9 +267,10 @@ LOB_DEV void or_groups(const Lanes& L, uint4& a) {
 
 // add one warp's batch of up to 32 candidate operand rows (idx, valid) to its
 // list, reading them once the list holds 32 or more; n entries are pending
+template <bool kLoop>
 LOB_DEV void push_batch(const BMat& M, u32 words, const Lanes& L, u32* list, int& n, u32 idx, bool valid, bool count,
                         u64& bag, u64& read, uint4& acc, bool& any) {
-  const u64 wgt = valid ? M.weight(idx) : 0ull;
+  const u64 wgt = valid ? M.weight<kLoop>(idx) : 0ull;
   const bool act = wgt != 0;
   if (count) bag += wgt;
   const u32 m = __ballot_sync(0xFFFFFFFFu, act);
@@ -269,15 +281,16 @@ LOB_DEV void push_batch(const BMat& M, u32 words, const Lanes& L, u32* list, int
   n += __popc(m);
   __syncwarp();
   if (n >= kListCap - 32) {
-    gather_list(M, words, L, list, n, acc);
+    gather_list<kLoop>(M, words, L, list, n, acc);
     if (lane == 0) read += (u64)n * (u64)min(128u, words);
     n = 0;
     __syncwarp();
   }
 }
+template <bool kLoop>
 LOB_DEV void flush_list(const BMat& M, u32 words, const Lanes& L, u32* list, int& n, u64& read, uint4& acc) {
   if (n) {
-    gather_list(M, words, L, list, n, acc);
+    gather_list<kLoop>(M, words, L, list, n, acc);
     if ((threadIdx.x & 31) == 0) read += (u64)n * (u64)min(128u, words);
   }
   n = 0;
@@ -285,12 +298,13 @@ LOB_DEV void flush_list(const BMat& M, u32 words, const Lanes& L, u32* list, int
 }
 
 // store a task's combined words; row r of a temporary always gets its weight
+template <bool kLoop>
 LOB_DEV u32 finish_task(const BOp& P, const Lanes& L, u32 r, bool count, const uint4& acc, bool any, u64 bag) {
   if (P.out && count && (threadIdx.x & 31) == 0) P.obag[r] = any ? bag : 0ull;
-  const bool flagged = P.commit && P.aflag && P.aflag[r];
+  const bool flagged = P.commit && P.aflag && ldm<kLoop>(P.aflag + r);
   if (!any && !flagged) return 0;
   u32 fresh = 0;
-  if (L.in && L.sub == 0) fresh = put4(P, r, L.w, acc);
+  if (L.in && L.sub == 0) fresh = put4<kLoop>(P, r, L.w, acc);
   if (P.commit) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
@@ -316,7 +330,7 @@ LOB_DEV u64 warp_total(u64 v) {
 // x chunks of a 50,000-value matrix takes 100 us where the list takes 5.
 template <int IK>
 __global__ void __launch_bounds__(256) k_bit_active(const __grid_constant__ BOp P, int operand_bits) {
-  if (op_idle(P)) return;
+  if (op_idle<false>(P)) return;
   const int lane = threadIdx.x & 31;
   const u64 nwarps = (u64)gridDim.x * 8;
   u64 cand = 0;
@@ -327,7 +341,7 @@ __global__ void __launch_bounds__(256) k_bit_active(const __grid_constant__ BOp 
     u64 bag = 0;
     u32 len = 0;
     if constexpr (IK == I_BITS) {
-      live = live && P.ib.weight(r) != 0;
+      live = live && P.ib.weight<false>(r) != 0;
     } else {
       u32 j0 = 0;
       if constexpr (IK == I_CSR) {
@@ -340,12 +354,12 @@ __global__ void __launch_bounds__(256) k_bit_active(const __grid_constant__ BOp 
       }
       if (operand_bits) {
         if (len <= 32)
-          for (u32 j = 0; j < len; j++) bag += P.mb.weight(IK == I_CSR ? P.ic.col[j0 + j] : r);
+          for (u32 j = 0; j < len; j++) bag += P.mb.weight<false>(IK == I_CSR ? P.ic.col[j0 + j] : r);
         for (u32 m = __ballot_sync(0xFFFFFFFFu, len > 32); m; m &= m - 1) {
           const int src = __ffs(m) - 1;
           const u32 a = __shfl_sync(0xFFFFFFFFu, j0, src), n = __shfl_sync(0xFFFFFFFFu, len, src);
           u64 b = 0;
-          for (u32 j = lane; j < n; j += 32) b += P.mb.weight(P.ic.col[a + j]);
+          for (u32 j = lane; j < n; j += 32) b += P.mb.weight<false>(P.ic.col[a + j]);
           b = warp_total(b);
           if (lane == src) bag = b;
         }
@@ -374,13 +388,13 @@ __global__ void __launch_bounds__(256) k_bit_active(const __grid_constant__ BOp 
   block_totals(P, cand, 0, 0);
 }
 
-template <int IK>
-__global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp P) {
+template <int IK, bool kLoop>
+LOB_DEV void gather_rows(const BOp& P) {
   __shared__ u32 lists[kGatherWarps][kListCap];
   __shared__ uint4 part[kGatherWarps][32];
   __shared__ u64 pbag[kGatherWarps];
   __shared__ u32 pany[kGatherWarps];
-  if (op_idle(P)) return;
+  if (op_idle<kLoop>(P)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 chunks = (P.words + 127) / 128;
   u32* list = lists[warp];
@@ -401,21 +415,21 @@ __global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp 
       bool any = false;
       if (!P.need || P.need[r]) {
         if constexpr (IK == I_IDENT) {
-          push_batch(P.mb, P.words, L, list, n, r, lane == 0, count, bag, read, acc, any);
+          push_batch<kLoop>(P.mb, P.words, L, list, n, r, lane == 0, count, bag, read, acc, any);
         } else {
           const u32 j0 = P.ic.ptr[r], j1 = P.ic.ptr[r + 1];
           if (j1 - j0 > kHeavyRow && !P.list) continue;  // below, by whole blocks
           for (u32 j = j0; j < j1; j += 32) {
             const bool v = j + lane < j1;
-            push_batch(P.mb, P.words, L, list, n, v ? P.ic.col[j + lane] : 0u, v, count, bag, read, acc, any);
+            push_batch<kLoop>(P.mb, P.words, L, list, n, v ? P.ic.col[j + lane] : 0u, v, count, bag, read, acc, any);
           }
         }
-        flush_list(P.mb, P.words, L, list, n, read, acc);
+        flush_list<kLoop>(P.mb, P.words, L, list, n, read, acc);
         or_groups(L, acc);
       }
       bag = warp_total(bag);
       if (lane == 0) cand += bag;
-      fresh += finish_task(P, L, r, count, acc, any, bag);
+      fresh += finish_task<kLoop>(P, L, r, count, acc, any, bag);
     }
   }
   if constexpr (IK != I_IDENT) {
@@ -432,29 +446,29 @@ __global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp 
       int n = 0;
       bool any = false;
       bool live = !P.need || P.need[r];
-      if constexpr (IK == I_BITS) live = live && P.ib.weight(r) != 0;
+      if constexpr (IK == I_BITS) live = live && P.ib.weight<kLoop>(r) != 0;
       if (!live) {  // the same for the whole block
-        if (warp == 0) fresh += finish_task(P, L, r, count, acc, false, 0);
+        if (warp == 0) fresh += finish_task<kLoop>(P, L, r, count, acc, false, 0);
         continue;
       }
       if constexpr (IK == I_CSR) {
         const u32 j0 = P.ic.ptr[r], j1 = P.ic.ptr[r + 1];
         for (u32 j = j0 + warp * 32; j < j1; j += 256) {
           const bool v = j + lane < j1;
-          push_batch(P.mb, P.words, L, list, n, v ? P.ic.col[j + lane] : 0u, v, count, bag, read, acc, any);
+          push_batch<kLoop>(P.mb, P.words, L, list, n, v ? P.ic.col[j + lane] : 0u, v, count, bag, read, acc, any);
         }
       } else {
         const u32* row = P.ib.bits + (u64)r * P.words;
         for (u32 w0 = warp * 32; w0 < P.words; w0 += 256) {
-          const u32 mine = w0 + lane < P.words ? row[w0 + lane] : 0u;
+          const u32 mine = w0 + lane < P.words ? ldm<kLoop>(row + w0 + lane) : 0u;
           for (u32 m = __ballot_sync(0xFFFFFFFFu, mine != 0u); m; m &= m - 1) {
             const int src = __ffs(m) - 1;
             const u32 word = __shfl_sync(0xFFFFFFFFu, mine, src);
-            push_batch(P.mb, P.words, L, list, n, (w0 + src) * 32 + lane, (word >> lane) & 1u, count, bag, read, acc, any);
+            push_batch<kLoop>(P.mb, P.words, L, list, n, (w0 + src) * 32 + lane, (word >> lane) & 1u, count, bag, read, acc, any);
           }
         }
       }
-      flush_list(P.mb, P.words, L, list, n, read, acc);
+      flush_list<kLoop>(P.mb, P.words, L, list, n, read, acc);
       or_groups(L, acc);
       bag = warp_total(bag);
       part[warp][lane] = acc;
@@ -470,13 +484,15 @@ __global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp 
           any = any || pany[v];
         }
         if (lane == 0) cand += bag;
-        fresh += finish_task(P, L, r, count, acc, any, bag);
+        fresh += finish_task<kLoop>(P, L, r, count, acc, any, bag);
       }
       __syncthreads();  // part is rewritten by the next task
     }
   }
   block_totals(P, cand, read, fresh);
 }
+template <int IK>
+__global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp P) { gather_rows<IK, false>(P); }
 
 // ---------------------------------------------------------------------------
 // scatter: row r of the result = the union of the compressed operand rows
@@ -509,11 +525,11 @@ LOB_DEV void set_row_bits(const BCsr& M, u32* row, u32 y, bool valid, u64& bag) 
   }
 }
 
-template <int IK>
-__global__ void __launch_bounds__(256) k_bit_scatter(const __grid_constant__ BOp P) {
+template <int IK, bool kLoop>
+LOB_DEV void scatter_rows(const BOp& P) {
   extern __shared__ __align__(16) u32 row[];
   __shared__ u64 sm[256 / 32 + 1];
-  if (op_idle(P)) return;
+  if (op_idle<kLoop>(P)) return;
   u64 cand = 0, read = 0, fresh_all = 0;
   const u32 n_rows = P.list ? (u32)P.n_list[0] : P.rows;
   for (u32 q = blockIdx.x; q < n_rows; q += gridDim.x) {
@@ -521,14 +537,14 @@ __global__ void __launch_bounds__(256) k_bit_scatter(const __grid_constant__ BOp
     bool live = !P.need || P.need[r];
     u32 j0 = 0, j1 = 0;
     if constexpr (IK == I_BITS) {
-      live = live && P.ib.weight(r) != 0;
+      live = live && P.ib.weight<kLoop>(r) != 0;
     } else {
       const BCsr& C = IK == I_CSR ? P.ic : P.mc;
       j0 = C.ptr[r];
       j1 = C.ptr[r + 1];
       live = live && j1 > j0;
     }
-    const bool flagged = P.commit && P.aflag && P.aflag[r];
+    const bool flagged = P.commit && P.aflag && ldm<kLoop>(P.aflag + r);
     if (!live && !flagged) {
       if (P.out && threadIdx.x == 0) P.obag[r] = 0;
       continue;
@@ -552,7 +568,7 @@ __global__ void __launch_bounds__(256) k_bit_scatter(const __grid_constant__ BOp
         const u32* src = P.ib.bits + (u64)r * P.words;
         for (u32 w0 = 0; w0 < P.words; w0 += 256) {
           const u32 w = w0 + threadIdx.x;
-          u32 m = w < P.words ? src[w] : 0u;
+          u32 m = w < P.words ? ldm<kLoop>(src + w) : 0u;
           while (__any_sync(0xFFFFFFFFu, m != 0u)) {
             const u32 y = w * 32 + (m ? (u32)__ffs(m) - 1 : 0u);
             set_row_bits(P.mc, row, y, m != 0u, bag);
@@ -568,7 +584,7 @@ __global__ void __launch_bounds__(256) k_bit_scatter(const __grid_constant__ BOp
     if (P.out && threadIdx.x == 0) P.obag[r] = tot;
     u32 fresh = 0;
     if (!P.out || tot)
-      for (u32 w = threadIdx.x * 4; w < P.words; w += 1024) fresh += put4(P, r, w, *reinterpret_cast<const uint4*>(row + w));
+      for (u32 w = threadIdx.x * 4; w < P.words; w += 1024) fresh += put4<kLoop>(P, r, w, *reinterpret_cast<const uint4*>(row + w));
     if (P.commit) {
 #pragma unroll
       for (int o = 16; o; o >>= 1) fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
@@ -581,19 +597,22 @@ __global__ void __launch_bounds__(256) k_bit_scatter(const __grid_constant__ BOp
   }
   block_totals(P, cand, read, fresh_all);
 }
+template <int IK>
+__global__ void __launch_bounds__(256) k_bit_scatter(const __grid_constant__ BOp P) { scatter_rows<IK, false>(P); }
 
 // D' = N & ~F, F |= D' of the rows some product added to; N is cleared
-__global__ void __launch_bounds__(256) k_bit_commit(const __grid_constant__ BOp P) {
-  if (P.state[B_DONE]) return;
+template <bool kLoop>
+LOB_DEV void commit_rows(const BOp& P) {
+  if (ldm<kLoop>(P.state + B_DONE)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 chunks = (P.words + 127) / 128;
   const u64 tasks = (u64)P.rows * chunks, nwarps = (u64)gridDim.x * kGatherWarps;
   u64 fresh_all = 0, read = 0;
   for (u64 t = (u64)blockIdx.x * kGatherWarps + warp; t < tasks; t += nwarps) {
     const u32 r = (u32)(t / chunks);
-    if (!P.aflag[r]) continue;
+    if (!ldm<kLoop>(P.aflag + r)) continue;
     const u32 w = (u32)(t % chunks) * 128 + lane * 4;
-    u32 fresh = w < P.words ? put4(P, r, w, make_uint4(0, 0, 0, 0)) : 0u;
+    u32 fresh = w < P.words ? put4<kLoop>(P, r, w, make_uint4(0, 0, 0, 0)) : 0u;
 #pragma unroll
     for (int o = 16; o; o >>= 1) fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
     if (lane == 0) {
@@ -604,6 +623,7 @@ __global__ void __launch_bounds__(256) k_bit_commit(const __grid_constant__ BOp 
   }
   block_totals(P, 0, read, fresh_all);
 }
+__global__ void __launch_bounds__(256) k_bit_commit(const __grid_constant__ BOp P) { commit_rows<false>(P); }
 
 struct BEnd {
   u32 rows;
@@ -618,10 +638,10 @@ struct BEnd {
 // End of an iteration: sizes, the stop decision, cleared row counts and flags.
 // Only block 0 writes the state; a block that sees the new done flag skips
 // clearing what no later iteration reads.
-__global__ void __launch_bounds__(256) k_bit_end(const __grid_constant__ BEnd E) {
+template <bool kLoop>
+LOB_DEV void end_iteration(const BEnd& E) {
   u64* s = E.state;
   const u64 stride = (u64)gridDim.x * blockDim.x;
-  if (s[B_DONE]) return;
   for (int i = 0; i < E.n_rel; i++)
     for (u64 q = (u64)blockIdx.x * blockDim.x + threadIdx.x; q < E.rows; q += stride) {
       E.old_cnt[i][q] = 0;
@@ -632,17 +652,23 @@ __global__ void __launch_bounds__(256) k_bit_end(const __grid_constant__ BEnd E)
   u64 total = 0;
   for (int i = 0; i < E.n_rel; i++) {
     const int r = E.rel[i];
-    const u64 n = s[rel_slot(r, 2)];
-    s[rel_slot(r, 0)] += n;
+    const u64 n = ldm<kLoop>(s + rel_slot(r, 2));
+    s[rel_slot(r, 0)] = ldm<kLoop>(s + rel_slot(r, 0)) + n;
     s[rel_slot(r, 1)] = n;
     s[rel_slot(r, 2)] = 0;
     total += n;
   }
-  for (int i = 0; i < 2 * kMaxLists; i++) s[kStateSlots + i] = 0;
-  s[B_NEW] += total;
-  s[B_ITER] += 1;
+  if constexpr (!kLoop)
+    for (int i = 0; i < 2 * kMaxLists; i++) s[kStateSlots + i] = 0;
+  s[B_NEW] = ldm<kLoop>(s + B_NEW) + total;
+  const u64 it = ldm<kLoop>(s + B_ITER) + 1;
+  s[B_ITER] = it;
   if (!total) s[B_DONE] = 1;
-  else if (s[B_ITER] >= E.max_iters) s[B_DONE] = 2;
+  else if (it >= E.max_iters) s[B_DONE] = 2;
+}
+__global__ void __launch_bounds__(256) k_bit_end(const __grid_constant__ BEnd E) {
+  if (E.state[B_DONE]) return;
+  end_iteration<false>(E);
 }
 
 // ---------------------------------------------------------------------------
@@ -650,23 +676,32 @@ __global__ void __launch_bounds__(256) k_bit_end(const __grid_constant__ BEnd E)
 // 32 x 32 squares by ballots, and the block stores 32-byte pieces of 256 result
 // rows.  With `full`, the same bits are ORed into a second matrix (F' follows D').
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_bit_transpose(BMat src, u32 rows, u32 words, u32* __restrict__ dst,
-                                                       u32* __restrict__ dcnt, u32* __restrict__ full,
-                                                       u32* __restrict__ fcnt, const u64* state) {
+struct BTrans {
+  BMat src;
+  u32 rows, words;
+  u32 *dst, *dcnt, *full, *fcnt;
+  const u64* state;
+};
+template <bool kLoop>
+LOB_DEV void transpose_rows(const BTrans& X) {
+  const BMat& src = X.src;
+  const u32 rows = X.rows, words = X.words;
+  u32 *dst = X.dst, *dcnt = X.dcnt, *full = X.full, *fcnt = X.fcnt;
+  const u64* state = X.state;
   __shared__ u32 tile[256][9];  // result row within the block, its 8 words (+1: no bank conflicts)
-  if (state && state[B_DONE]) return;
+  if (state && ldm<kLoop>(state + B_DONE)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 bw = (words + 7) / 8;
   const u64 tiles = (u64)((rows + 255) / 256) * bw;
   for (u64 t = blockIdx.x; t < tiles; t += gridDim.x) {
     const u32 r0 = (u32)(t / bw) * 256, w0 = (u32)(t % bw) * 8;
     const u32 r = r0 + warp * 32 + lane;
-    const bool live = r < rows && src.weight(r) != 0;
+    const bool live = r < rows && src.weight<kLoop>(r) != 0;
     u32 x[8];
 #pragma unroll
     for (int j = 0; j < 8; j += 4) {
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (live && w0 + j < words) v = *reinterpret_cast<const uint4*>(src.bits + (u64)r * words + w0 + j);
+      if (live && w0 + j < words) v = ldm<kLoop>(reinterpret_cast<const uint4*>(src.bits + (u64)r * words + w0 + j));
       x[j] = v.x; x[j + 1] = v.y; x[j + 2] = v.z; x[j + 3] = v.w;
     }
 #pragma unroll
@@ -699,7 +734,7 @@ __global__ void __launch_bounds__(256) k_bit_transpose(BMat src, u32 rows, u32 w
           reinterpret_cast<uint4*>(dst)[at] = v;
           if (full && any4(v)) {
             uint4* f = reinterpret_cast<uint4*>(full) + at;
-            or4(v, *f);
+            or4(v, ldm<kLoop>(f));
             *f = v;
           }
         }
@@ -707,6 +742,97 @@ __global__ void __launch_bounds__(256) k_bit_transpose(BMat src, u32 rows, u32 w
       if (c && fcnt) atomicAdd(fcnt + orow, c);
     }
     __syncthreads();
+  }
+}
+__global__ void __launch_bounds__(256) k_bit_transpose(const __grid_constant__ BTrans X) { transpose_rows<false>(X); }
+
+// ---------------------------------------------------------------------------
+// The whole run in one cooperative launch, for matrices of at most kLoopTasks
+// tasks (rows x 128-word chunks).  A closure over 1,000 nodes takes 15 iterations of two
+// kernels that do a microsecond's work each, plus the iterations queued past the
+// fixpoint: the steps of an iteration, described in global memory, run one after
+// another with a grid barrier between them, and the loop ends where the state says
+// so.  One block per eight tasks of a step, up to four per SM.
+// Measured (GB300, whole passes): closure of 67 nodes 554 -> 425 us, of 1,000
+// nodes 609 -> 491 us; points-to over 2,681 values, whose products fill the GPU by
+// themselves, 2.96 -> 3.33 ms, so the line lies at 2,048 tasks.
+// ---------------------------------------------------------------------------
+enum StepKind { K_GATHER, K_SCATTER, K_COMMIT, K_TRANSPOSE };
+struct BStep {
+  int kind, ik;
+  BOp P;
+  BTrans X;
+};
+struct BLoop {
+  const BStep* steps;
+  int first[4];   // steps of: the first iteration, those on recent buffer 1, on buffer 0
+  BEnd end[2];    // by recent buffer
+  const BStep* after;  // transposes that follow an iteration's end, by the buffer it wrote
+  int after_first[3];
+  u64* state;
+  u32* bar;       // arrivals, give-up flag
+};
+constexpr u64 kLoopTasks = 2048;
+constexpr u32 kLoopSpin = 1u << 26;  // barrier polls before a block gives up
+
+LOB_DEV bool loop_barrier(u32* bar, u32& gen) {
+  __shared__ u32 ok;
+  __syncthreads();
+  if (gridDim.x == 1) return true;
+  if (threadIdx.x == 0) {
+    volatile u32* b = bar;
+    __threadfence();
+    gen++;
+    atomicAdd(bar, 1u);
+    const u32 want = gen * gridDim.x;
+    u32 n = 0;
+    while ((int)(b[0] - want) < 0 && !b[1] && n < kLoopSpin) n++;
+    if ((int)(b[0] - want) < 0) b[1] = 1;
+    __threadfence();
+    ok = b[1] == 0;
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+LOB_DEV void run_step(const BStep& S) {
+  if (S.kind == K_GATHER) {
+    if (S.ik == I_IDENT) gather_rows<I_IDENT, true>(S.P);
+    else if (S.ik == I_CSR) gather_rows<I_CSR, true>(S.P);
+    else gather_rows<I_BITS, true>(S.P);
+  } else if (S.kind == K_SCATTER) {
+    if (S.ik == I_IDENT) scatter_rows<I_IDENT, true>(S.P);
+    else if (S.ik == I_CSR) scatter_rows<I_CSR, true>(S.P);
+    else scatter_rows<I_BITS, true>(S.P);
+  } else if (S.kind == K_COMMIT) {
+    commit_rows<true>(S.P);
+  } else {
+    transpose_rows<true>(S.X);
+  }
+}
+
+__global__ void __launch_bounds__(256, 4) k_bit_loop(const __grid_constant__ BLoop L) {
+  __shared__ BStep step;
+  u32 gen = 0;
+  for (u32 it = 1;; it++) {
+    const int cur = (it - 1) & 1, list = it == 1 ? 0 : (cur ? 1 : 2);
+    for (int i = L.first[list]; i < L.first[list + 1]; i++) {
+      for (u32 q = threadIdx.x; q < sizeof(BStep) / 4; q += blockDim.x)
+        reinterpret_cast<u32*>(&step)[q] = reinterpret_cast<const u32*>(L.steps + i)[q];
+      __syncthreads();
+      run_step(step);
+      if (!loop_barrier(L.bar, gen)) return;
+    }
+    end_iteration<true>(L.end[cur]);
+    if (!loop_barrier(L.bar, gen)) return;
+    if (ldm<true>(L.state + B_DONE)) return;
+    for (int i = L.after_first[cur ^ 1]; i < L.after_first[(cur ^ 1) + 1]; i++) {
+      for (u32 q = threadIdx.x; q < sizeof(BStep) / 4; q += blockDim.x)
+        reinterpret_cast<u32*>(&step)[q] = reinterpret_cast<const u32*>(L.after + i)[q];
+      __syncthreads();
+      run_step(step);
+      if (!loop_barrier(L.bar, gen)) return;
+    }
   }
 }
 
@@ -1224,9 +1350,23 @@ struct Run {
   }
 
   int n_lists = 0;  // products of the current iteration that listed their rows
+  std::vector<BStep>* record = nullptr;  // the loop's steps are being collected, not launched
+  void add_step(int kind, int ik, const BOp* P, const BTrans* X) {
+    BStep S;
+    std::memset(&S, 0, sizeof(S));
+    S.kind = kind;
+    S.ik = ik;
+    if (P) S.P = *P;
+    if (X) S.X = *X;
+    record->push_back(S);
+  }
 
   void product(BOp P, int ik, bool bits) {
     const u32 chunks = (P.words + 127) / 128;
+    if (record) {
+      add_step(bits ? K_GATHER : K_SCATTER, ik, &P, nullptr);
+      return;
+    }
     profile_before();
     if (listed() && n_lists < kMaxLists) {
       P.list = B.list.as<u32>();
@@ -1262,23 +1402,54 @@ struct Run {
     profile_after();
   }
 
+  void transpose(const BTrans& X) {
+    {
+      ProfScope ps("bit_transpose", 2.0 * mat_bytes(), e.stream);
+      const u64 tiles = (u64)((B.rows + 255) / 256) * ((B.words + 7) / 8);
+      k_bit_transpose<<<block_grid(tiles), 256, 0, e.stream>>>(X);
+    }
+    launch_check("bit transpose");
+  }
+
   void transpose_recent(int cur, u64* state) {
     for (size_t r = 0; r < e.rels.size(); r++) {
       BitRel& R = B.rel[r];
       if (!e.rels[r].idb || !R.need_t) continue;
-      BMat m{};
-      m.bits = R.recent[cur].as<u32>();
-      m.cnt = R.rcnt[cur].as<u32>();
-      ProfScope ps("bit_transpose", 2.0 * mat_bytes(), e.stream);
-      const u64 tiles = (u64)((B.rows + 255) / 256) * ((B.words + 7) / 8);
-      k_bit_transpose<<<block_grid(tiles), 256, 0, e.stream>>>(m, B.rows, B.words, R.trecent.as<u32>(), R.trcnt.as<u32>(),
-                                                               R.tfull.as<u32>(), R.tfcnt.as<u32>(), state);
-      launch_check("bit transpose");
+      BTrans X{};
+      X.src.bits = R.recent[cur].as<u32>();
+      X.src.cnt = R.rcnt[cur].as<u32>();
+      X.rows = B.rows;
+      X.words = B.words;
+      X.dst = R.trecent.as<u32>();
+      X.dcnt = R.trcnt.as<u32>();
+      X.full = R.tfull.as<u32>();
+      X.fcnt = R.tfcnt.as<u32>();
+      X.state = state;
+      if (record) add_step(K_TRANSPOSE, 0, nullptr, &X);
+      else transpose(X);
     }
   }
 
-  // one iteration (k >= 1) on recent buffers `cur`; its results go to cur ^ 1
-  void iteration(u32 k, u32 max_iters, int cur) {
+  BEnd end_of(u32 max_iters, int cur) {
+    BEnd E{};
+    E.rows = B.rows;
+    E.max_iters = max_iters;
+    E.state = B.state.as<u64>();
+    for (size_t r = 0; r < e.rels.size(); r++) {
+      if (!e.rels[r].idb) continue;
+      const int i = E.n_rel++;
+      BitRel& R = B.rel[r];
+      E.rel[i] = (int)r;
+      E.old_cnt[i] = R.rcnt[cur].as<u32>();
+      E.aflag[i] = R.aflag.as<u32>();
+      E.tcnt[i] = R.need_t ? R.trcnt.as<u32>() : nullptr;
+    }
+    return E;
+  }
+
+  // the products of one iteration (k >= 1) on recent buffers `cur`; their results
+  // go to cur ^ 1
+  void products(u32 k, int cur) {
     // the arms of this iteration: in the first, every loaded fact is recent, so
     // the arm of each rule's first atom covers the rule; later only derived
     // atoms have recent facts
@@ -1312,6 +1483,10 @@ struct Run {
         P.state = B.state.as<u64>();
         set_head(P, (u32)r, cur, true);
         const u32 chunks = (P.words + 127) / 128;
+        if (record) {
+          add_step(K_COMMIT, 0, &P, nullptr);
+          continue;
+        }
         profile_before();
         {
           ProfScope ps("bit_commit", 0, e.stream);
@@ -1321,19 +1496,11 @@ struct Run {
         profile_after();
       }
     }
-    BEnd E{};
-    E.rows = B.rows;
-    E.max_iters = max_iters;
-    E.state = B.state.as<u64>();
-    for (size_t r = 0; r < e.rels.size(); r++) {
-      if (!e.rels[r].idb) continue;
-      const int i = E.n_rel++;
-      BitRel& R = B.rel[r];
-      E.rel[i] = (int)r;
-      E.old_cnt[i] = R.rcnt[cur].as<u32>();
-      E.aflag[i] = R.aflag.as<u32>();
-      E.tcnt[i] = R.need_t ? R.trcnt.as<u32>() : nullptr;
-    }
+  }
+
+  void iteration(u32 k, u32 max_iters, int cur) {
+    products(k, cur);
+    const BEnd E = end_of(max_iters, cur);
     k_bit_end<<<std::min(elem_grid(B.rows), 152u), 256, 0, e.stream>>>(E);
     launch_check("bit end");
     transpose_recent(cur ^ 1, B.state.as<u64>());
@@ -1392,17 +1559,72 @@ struct Run {
       e.sync();  // h goes out of scope with the run; the copy is from pageable memory
       transpose_recent(0, nullptr);
     }
+    if ((u64)B.rows * ((B.words + 127) / 128) <= kLoopTasks && !g_prof) {
+      loop_launch(max_iters);
+      read_state();
+      return done(k, new_facts, rc);
+    }
     // Iterations are queued in groups without waiting: one that follows the
     // fixpoint sees the done flag and does nothing (about 2 us a launch), which
     // is cheaper than a host wait per iteration (about 10 us).
-    u64* s = e.pinned;
     u32 queued = 0;
     for (u32 group = 4;; group = std::min(16u, group * 2)) {
       for (u32 i = 0; i < group && queued < max_iters; i++, queued++) iteration(queued + 1, max_iters, (int)(queued & 1));
-      e.check(cudaMemcpyAsync(s, B.state.p, kStateSlots * 8, cudaMemcpyDeviceToHost, e.stream), "bit state");
-      e.sync();
-      if (s[B_DONE] || queued >= max_iters) break;
+      read_state();
+      if (e.pinned[B_DONE] || queued >= max_iters) break;
     }
+    return done(k, new_facts, rc);
+  }
+
+  void read_state() {
+    e.check(cudaMemcpyAsync(e.pinned, B.state.p, kReadSlots * 8, cudaMemcpyDeviceToHost, e.stream), "bit state");
+    e.sync();
+    if (e.pinned[kStateSlots] >> 32)
+      throw LobError(LOB_E_TIMEOUT, "a bounded wait of the bit-matrix loop gave up; the run's results are invalid");
+  }
+
+  // the first iteration's steps, then those of later ones by recent buffer, and the
+  // transposes after them
+  void loop_launch(u32 max_iters) {
+    std::vector<BStep> steps, after;
+    BLoop L;
+    std::memset(&L, 0, sizeof(L));
+    record = &steps;
+    for (int i = 0; i < 3; i++) {
+      L.first[i] = (int)steps.size();
+      products(i == 0 ? 1 : 2, i == 1 ? 1 : 0);
+    }
+    L.first[3] = (int)steps.size();
+    record = &after;
+    for (int b = 0; b < 2; b++) {
+      L.after_first[b] = (int)after.size();
+      transpose_recent(b, B.state.as<u64>());
+    }
+    L.after_first[2] = (int)after.size();
+    record = nullptr;
+    const size_t n_steps = steps.size();
+    steps.insert(steps.end(), after.begin(), after.end());
+    e.ensure(B.steps, std::max<size_t>(steps.size(), 1) * sizeof(BStep));
+    e.check(cudaMemcpyAsync(B.steps.p, steps.data(), steps.size() * sizeof(BStep), cudaMemcpyHostToDevice, e.stream), "steps");
+    L.steps = B.steps.as<BStep>();
+    L.after = B.steps.as<BStep>() + n_steps;
+    for (int b = 0; b < 2; b++) L.end[b] = end_of(max_iters, b);
+    L.state = B.state.as<u64>();
+    L.bar = reinterpret_cast<u32*>(B.state.as<u64>() + kStateSlots);
+    const u64 tasks = (u64)B.rows * ((B.words + 127) / 128);
+    const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>((tasks + kGatherWarps - 1) / kGatherWarps, 4ull * e.sms));
+    const size_t sm = (size_t)B.words * 4;
+    void* args[] = {&L};
+    {
+      ProfScope ps("bit_loop", 0, e.stream);
+      e.check(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_bit_loop), dim3(blocks), dim3(256), args, sm, e.stream),
+              "bit loop");
+    }
+    launch_check("bit loop");
+  }
+
+  bool done(u32& k, u64& new_facts, int* rc) {
+    const u64* s = e.pinned;
     *rc = s[B_DONE] == 1 ? LOB_OK : LOB_E_MAXITER;
     k = (u32)s[B_ITER];
     new_facts = s[B_NEW];
@@ -1420,16 +1642,13 @@ struct Run {
       BitRel& R = B.rel[r];
       if (!e.rels[r].idb) continue;
       if (B.transposed) {
-        BMat m{};
-        m.bits = R.full.as<u32>();
-        m.cnt = R.fcnt.as<u32>();
-        {
-          ProfScope ps("bit_transpose", 2.0 * mat_bytes(), e.stream);
-          const u64 tiles = (u64)((B.rows + 255) / 256) * ((B.words + 7) / 8);
-          k_bit_transpose<<<block_grid(tiles), 256, 0, e.stream>>>(m, B.rows, B.words, R.recent[0].as<u32>(), nullptr,
-                                                                   nullptr, nullptr, nullptr);
-        }
-        launch_check("bit transpose");
+        BTrans X{};
+        X.src.bits = R.full.as<u32>();
+        X.src.cnt = R.fcnt.as<u32>();
+        X.rows = B.rows;
+        X.words = B.words;
+        X.dst = R.recent[0].as<u32>();
+        transpose(X);
         std::swap(R.full, R.recent[0]);
         {
           ProfScope ps("bit_counts", (double)mat_bytes(), e.stream);
@@ -1475,7 +1694,7 @@ bool bit_run(lob_engine& e, u32 max_iters, u32& k, u64& new_facts, int* rc) {
 void bit_release(lob_engine& e) {
   if (!e.bit) return;
   BitRun& B = *e.bit;
-  for (DevBuf* b : {&B.pres, &B.pref, &B.dict, &B.state, &B.list, &B.hlist, &B.temp[0], &B.temp[1], &B.tbag[0], &B.tbag[1]}) e.release(*b);
+  for (DevBuf* b : {&B.pres, &B.pref, &B.dict, &B.state, &B.steps, &B.list, &B.hlist, &B.temp[0], &B.temp[1], &B.tbag[0], &B.tbag[1]}) e.release(*b);
   for (BitRel& R : B.rel) {
     for (DevBuf* b : {&R.full, &R.fcnt, &R.recent[0], &R.recent[1], &R.rcnt[0], &R.rcnt[1], &R.acc, &R.aflag, &R.trecent,
                       &R.trcnt, &R.tfull, &R.tfcnt, &R.off})

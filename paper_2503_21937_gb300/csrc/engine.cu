@@ -2191,7 +2191,8 @@ int lob_create(lob_engine** out, const lob_alloc* alloc, void* cuda_stream) {
   if (!out) return LOB_E_ARG;
   *out = nullptr;
   lob_engine* e = new lob_engine();
-  if (cudaGetDevice(&e->device) != cudaSuccess) {
+  if (cudaGetDevice(&e->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&e->sms, cudaDevAttrMultiProcessorCount, e->device) != cudaSuccess) {
     cudaGetLastError();
     g_create_err = "no CUDA device";
     delete e;

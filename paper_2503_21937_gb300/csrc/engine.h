@@ -221,12 +221,13 @@ struct BitRun {
   bool transposed = false;  // stored transposed while the run lasts
   bool mapped = false;      // values are renumbered (dict: code -> value)
   u32 rows = 0, words = 0;
-  DevBuf pres, pref, dict, state, list, hlist, temp[2], tbag[2];
+  DevBuf pres, pref, dict, state, steps, list, hlist, temp[2], tbag[2];
   std::vector<BitRel> rel;
 };
 
 struct lob_engine {
   int device = 0;
+  int sms = 1;  // multiprocessors: blocks of a cooperative launch that are resident together
   cudaStream_t stream = nullptr;
   cudaMemPool_t pool = nullptr;  // engine-owned pool; freed blocks stay reserved for reuse
   lob_alloc alloc{};

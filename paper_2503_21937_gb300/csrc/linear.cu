@@ -750,7 +750,7 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   // A block per 16,384 probed rows: a grid of side 64 has about 200 recent facts
   // in an iteration, which one block expands in a round or two without a grid
   // barrier.
-  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(152, probed / 16384));
+  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(e.sms, probed / 16384));
   A.k0 = k0;
   A.slots = (u32)slots;
   std::vector<u64> h(kLinSlots, 0);
@@ -918,7 +918,7 @@ bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& 
   A.off = off.as<u32>();
   A.last = last;
   A.state = L.state.as<u64>();
-  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(152, probed / 16384));
+  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(e.sms, probed / 16384));
   void* args[] = {&A};
   {
     ProfScope ps("linear_backward", 0, e.stream);
