@@ -1176,10 +1176,10 @@ struct Run {
     const BitRel& R = B.rel[l.rel];
     const BitCsr& C = R.csr[l.inv];
     BCsr c{};
-    c.ptr = C.ptr.as<u32>();
+    c.ptr = C.ptr;
     c.col = C.col.as<u32>();
-    c.heavy = C.heavy.as<u32>();
-    c.n_heavy = C.heavy.as<u32>() + C.heavy_cap;
+    c.heavy = C.heavy;
+    c.n_heavy = C.heavy + C.heavy_cap;
     return c;
   }
   void build_csr(const Link& l) {
@@ -1190,25 +1190,24 @@ struct Run {
     const u64 D = B.rows;
     C.heavy_cap = (u32)(K.n / kHeavyRow + 1);
     // lengths (their scan: ptr), fill positions, column flags, heavy rows and their number
-    e.ensure(C.ptr, (D + 1) * 4);
-    e.ensure(C.used, D * 4);
-    e.ensure(C.colflag, D * 4);
+    const u64 words = (D + 1) + D + D + C.heavy_cap + 1;
+    e.ensure(C.zeroed, words * 4);
     e.ensure(C.col, std::max<u64>(K.n, 1) * 4);
-    e.ensure(C.heavy, ((u64)C.heavy_cap + 1) * 4);
-    e.check(cudaMemsetAsync(C.ptr.p, 0, (D + 1) * 4, e.stream), "rows");
-    e.check(cudaMemsetAsync(C.used.p, 0, D * 4, e.stream), "rows");
-    e.check(cudaMemsetAsync(C.colflag.p, 0, D * 4, e.stream), "rows");
-    e.check(cudaMemsetAsync(C.heavy.p, 0, ((u64)C.heavy_cap + 1) * 4, e.stream), "rows");
+    e.check(cudaMemsetAsync(C.zeroed.p, 0, words * 4, e.stream), "rows");
+    C.ptr = C.zeroed.as<u32>();
+    C.used = C.ptr + D + 1;
+    C.colflag = C.used + D;
+    C.heavy = C.colflag + D;
     if (!K.n) return;
     ProfScope ps("bit_rows", K.n * (K.key64 ? 8.0 : 4.0) * 2.0 + K.n * 4.0 + D * 12.0, e.stream);
-    k_csr_count<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), l.inv, C.ptr.as<u32>(), C.colflag.as<u32>());
+    k_csr_count<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), l.inv, C.ptr, C.colflag);
     launch_check("rows");
     e.ensure(e.scratch, scan_scratch_elems(D + 1) * 4 + 64);
-    exclusive_scan<u32, u32>(C.ptr.as<u32>(), C.ptr.as<u32>(), D + 1, nullptr, e.scratch.as<u32>(), e.stream);
+    exclusive_scan<u32, u32>(C.ptr, C.ptr, D + 1, nullptr, e.scratch.as<u32>(), e.stream);
     e.after_launch("rows");
     e.launches += scan_launches(D + 1);
-    k_csr_fill<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), l.inv, C.ptr.as<u32>(), C.used.as<u32>(), C.col.as<u32>(),
-                                                     C.heavy.as<u32>(), C.heavy.as<u32>() + C.heavy_cap);
+    k_csr_fill<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), l.inv, C.ptr, C.used, C.col.as<u32>(),
+                                                     C.heavy, C.heavy + C.heavy_cap);
     launch_check("rows");
   }
 
@@ -1221,28 +1220,30 @@ struct Run {
       if (!e.rels[r].idb) continue;
       e.ensure(R.full, mb);
       e.check(cudaMemsetAsync(R.full.p, 0, mb, e.stream), "bit matrix");
-      e.ensure(R.fcnt, D * 4);
-      for (int b = 0; b < 2; b++) {
-        e.ensure(R.recent[b], mb);
-        e.ensure(R.rcnt[b], D * 4);
-        e.check(cudaMemsetAsync(R.rcnt[b].p, 0, D * 4, e.stream), "bit matrix");
-      }
-      e.check(cudaMemsetAsync(R.fcnt.p, 0, D * 4, e.stream), "bit matrix");
+      for (int b = 0; b < 2; b++) e.ensure(R.recent[b], mb);
+      // row counts of F, D, D' (and the transposed copies), flags: cleared as one
+      const int n_counts = 3 + (accumulates[r] ? 1 : 0) + (R.need_t ? (linear ? 1 : 2) : 0);
+      e.ensure(R.counts, n_counts * D * 4);
+      e.check(cudaMemsetAsync(R.counts.p, 0, n_counts * D * 4, e.stream), "bit matrix");
+      u32* c = R.counts.as<u32>();
+      R.fcnt = c;
+      R.rcnt[0] = c + D;
+      R.rcnt[1] = c + 2 * D;
+      c += 3 * D;
       if (accumulates[r]) {
         e.ensure(R.acc, mb);
-        e.ensure(R.aflag, D * 4);
         e.check(cudaMemsetAsync(R.acc.p, 0, mb, e.stream), "bit matrix");
-        e.check(cudaMemsetAsync(R.aflag.p, 0, D * 4, e.stream), "bit matrix");
+        R.aflag = c;
+        c += D;
       }
       if (R.need_t) {
         e.ensure(R.trecent, mb);
-        e.ensure(R.trcnt, D * 4);
-        e.check(cudaMemsetAsync(R.trcnt.p, 0, D * 4, e.stream), "bit matrix");
+        R.trcnt = c;
+        c += D;
         if (!linear) {
           e.ensure(R.tfull, mb);
-          e.ensure(R.tfcnt, D * 4);
           e.check(cudaMemsetAsync(R.tfull.p, 0, mb, e.stream), "bit matrix");
-          e.check(cudaMemsetAsync(R.tfcnt.p, 0, D * 4, e.stream), "bit matrix");
+          R.tfcnt = c;
         }
       }
     }
@@ -1269,9 +1270,8 @@ struct Run {
     BMat m{};
     const bool st = stored_way(l);
     const DevBuf& bits = recent ? (st ? R.recent[cur] : R.trecent) : (st ? R.full : R.tfull);
-    const DevBuf& cnt = recent ? (st ? R.rcnt[cur] : R.trcnt) : (st ? R.fcnt : R.tfcnt);
     m.bits = bits.as<u32>();
-    m.cnt = cnt.as<u32>();
+    m.cnt = recent ? (st ? R.rcnt[cur] : R.trcnt) : (st ? R.fcnt : R.tfcnt);
     return m;
   }
 
@@ -1324,7 +1324,7 @@ struct Run {
         P.out = B.temp[t].as<u32>();
         P.obag = B.tbag[t].as<u64>();
         // rows that the next index matrix never lists need not be formed
-        if (!e.rels[L[i - 1].rel].idb) P.need = B.rel[L[i - 1].rel].csr[L[i - 1].inv].colflag.as<u32>();
+        if (!e.rels[L[i - 1].rel].idb) P.need = B.rel[L[i - 1].rel].csr[L[i - 1].inv].colflag;
       } else {
         set_head(P, C.head, cur, commit);
         P.diag = C.diag;
@@ -1340,12 +1340,12 @@ struct Run {
   void set_head(BOp& P, u32 head, int cur, bool commit) {
     BitRel& H = B.rel[head];
     P.acc = H.acc.as<u32>();
-    P.aflag = H.aflag.as<u32>();
+    P.aflag = H.aflag;
     P.commit = commit;
     P.full = H.full.as<u32>();
     P.next = H.recent[cur ^ 1].as<u32>();
-    P.ncnt = H.rcnt[cur ^ 1].as<u32>();
-    P.fcnt = H.fcnt.as<u32>();
+    P.ncnt = H.rcnt[cur ^ 1];
+    P.fcnt = H.fcnt;
     P.n_new = B.state.as<u64>() + rel_slot((int)head, 2);
   }
 
@@ -1417,13 +1417,13 @@ struct Run {
       if (!e.rels[r].idb || !R.need_t) continue;
       BTrans X{};
       X.src.bits = R.recent[cur].as<u32>();
-      X.src.cnt = R.rcnt[cur].as<u32>();
+      X.src.cnt = R.rcnt[cur];
       X.rows = B.rows;
       X.words = B.words;
       X.dst = R.trecent.as<u32>();
-      X.dcnt = R.trcnt.as<u32>();
+      X.dcnt = R.trcnt;
       X.full = R.tfull.as<u32>();
-      X.fcnt = R.tfcnt.as<u32>();
+      X.fcnt = R.tfcnt;
       X.state = state;
       if (record) add_step(K_TRANSPOSE, 0, nullptr, &X);
       else transpose(X);
@@ -1440,9 +1440,9 @@ struct Run {
       const int i = E.n_rel++;
       BitRel& R = B.rel[r];
       E.rel[i] = (int)r;
-      E.old_cnt[i] = R.rcnt[cur].as<u32>();
-      E.aflag[i] = R.aflag.as<u32>();
-      E.tcnt[i] = R.need_t ? R.trcnt.as<u32>() : nullptr;
+      E.old_cnt[i] = R.rcnt[cur];
+      E.aflag[i] = R.aflag;
+      E.tcnt[i] = R.need_t ? R.trcnt : nullptr;
     }
     return E;
   }
@@ -1550,7 +1550,7 @@ struct Run {
       const KeyCols K = key_cols(e.rels[r]);
       e.check(cudaMemsetAsync(R.recent[0].p, 0, mat_bytes(), e.stream), "bit matrix");
       k_set_facts<<<elem_grid(K.n), 256, 0, e.stream>>>(K, codes(), B.transposed, B.words, R.full.as<u32>(),
-                                                        R.recent[0].as<u32>(), R.rcnt[0].as<u32>(), R.fcnt.as<u32>());
+                                                        R.recent[0].as<u32>(), R.rcnt[0], R.fcnt);
       launch_check("bit facts");
       h[rel_slot((int)r, 0)] = h[rel_slot((int)r, 1)] = K.n;
     }
@@ -1644,7 +1644,7 @@ struct Run {
       if (B.transposed) {
         BTrans X{};
         X.src.bits = R.full.as<u32>();
-        X.src.cnt = R.fcnt.as<u32>();
+        X.src.cnt = R.fcnt;
         X.rows = B.rows;
         X.words = B.words;
         X.dst = R.recent[0].as<u32>();
@@ -1652,18 +1652,16 @@ struct Run {
         std::swap(R.full, R.recent[0]);
         {
           ProfScope ps("bit_counts", (double)mat_bytes(), e.stream);
-          k_row_counts<<<warp_grid(D), 256, 0, e.stream>>>(R.full.as<u32>(), B.rows, B.words, R.fcnt.as<u32>());
+          k_row_counts<<<warp_grid(D), 256, 0, e.stream>>>(R.full.as<u32>(), B.rows, B.words, R.fcnt);
         }
         launch_check("bit counts");
       }
       e.ensure(R.off, (D + 1) * 8);
       e.ensure(e.scratch, scan_scratch_elems(D) * 8 + 64);
-      exclusive_scan<u32, u64>(R.fcnt.as<u32>(), R.off.as<u64>(), D, R.off.as<u64>() + D, e.scratch.as<u64>(), e.stream);
+      exclusive_scan<u32, u64>(R.fcnt, R.off.as<u64>(), D, R.off.as<u64>() + D, e.scratch.as<u64>(), e.stream);
       e.after_launch("bit offsets");
       e.launches += scan_launches(D);
-      for (DevBuf* b : {&R.recent[0], &R.recent[1], &R.rcnt[0], &R.rcnt[1], &R.acc, &R.aflag, &R.trecent, &R.trcnt, &R.tfull,
-                        &R.tfcnt})
-        e.release(*b);
+      for (DevBuf* b : {&R.recent[0], &R.recent[1], &R.counts, &R.acc, &R.trecent, &R.tfull}) e.release(*b);
     }
     for (int i = 0; i < 2; i++) {
       e.release(B.temp[i]);
@@ -1696,11 +1694,9 @@ void bit_release(lob_engine& e) {
   BitRun& B = *e.bit;
   for (DevBuf* b : {&B.pres, &B.pref, &B.dict, &B.state, &B.steps, &B.list, &B.hlist, &B.temp[0], &B.temp[1], &B.tbag[0], &B.tbag[1]}) e.release(*b);
   for (BitRel& R : B.rel) {
-    for (DevBuf* b : {&R.full, &R.fcnt, &R.recent[0], &R.recent[1], &R.rcnt[0], &R.rcnt[1], &R.acc, &R.aflag, &R.trecent,
-                      &R.trcnt, &R.tfull, &R.tfcnt, &R.off})
-      e.release(*b);
+    for (DevBuf* b : {&R.full, &R.recent[0], &R.recent[1], &R.counts, &R.acc, &R.trecent, &R.tfull, &R.off}) e.release(*b);
     for (BitCsr& C : R.csr)
-      for (DevBuf* b : {&C.ptr, &C.used, &C.colflag, &C.col, &C.heavy}) e.release(*b);
+      for (DevBuf* b : {&C.zeroed, &C.col}) e.release(*b);
   }
   e.bit.reset();
 }

@@ -92,14 +92,30 @@ void lob_engine::after_launch(const char* what) {
   if (opt_sync_check) check(cudaStreamSynchronize(stream), what);
 }
 
+// the size a block of the engine's pool is made with: small ones by powers of two
+static size_t block_bytes(size_t bytes) {
+  if (bytes > kSmallBlock) return bytes;
+  size_t c = 256;
+  while (c < bytes) c <<= 1;
+  return c;
+}
+
 void* lob_engine::dalloc(size_t bytes) {
   if (!bytes) return nullptr;
   void* p = nullptr;
   if (custom_alloc) {
     p = alloc.alloc(bytes, stream, alloc.ctx);
-  } else if (cudaMallocFromPoolAsync(&p, bytes, pool, stream) != cudaSuccess) {
-    cudaGetLastError();
-    p = nullptr;
+  } else {
+    const size_t want = block_bytes(bytes);
+    auto it = small_free.find(want);
+    if (it != small_free.end() && !it->second.empty()) {
+      p = it->second.back();
+      it->second.pop_back();
+      small_bytes -= want;
+    } else if (cudaMallocFromPoolAsync(&p, want, pool, stream) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
   }
   if (!p) throw LobError(LOB_E_OOM, "device allocation of " + std::to_string(bytes) + " bytes failed");
   live_bytes += bytes;
@@ -109,8 +125,17 @@ void* lob_engine::dalloc(size_t bytes) {
 
 void lob_engine::dfree(void* p, size_t bytes) {
   if (!p) return;
-  if (custom_alloc) alloc.release(p, bytes, stream, alloc.ctx);
-  else cudaFreeAsync(p, stream);
+  if (custom_alloc) {
+    alloc.release(p, bytes, stream, alloc.ctx);
+  } else {
+    const size_t made = block_bytes(bytes);
+    if (made <= kSmallBlock && small_bytes + made <= kSmallKept) {
+      small_free[made].push_back(p);
+      small_bytes += made;
+    } else {
+      cudaFreeAsync(p, stream);
+    }
+  }
   live_bytes -= bytes;
 }
 
@@ -685,24 +710,15 @@ static void prepare(lob_engine& e, int sem) {
   e.semiring = sem;
   // column widths: bitlen(max + 1) of the loaded values, so that no field ever
   // holds its all-ones value (the all-ones key marks dropped candidates)
-  u32* dmax = reinterpret_cast<u32*>(e.counts.p) + 32;
   bool any_samples = false;
   u32 max_sample = 0;
   for (auto& r : e.rels) {
     for (u32 c = 0; c < r.arity; c++) {
-      u32 m = 0;
-      if (r.n_in) {
-        reduce_max_u32(r.in_cols[0].as<u32>() + (u64)c * r.in_cap, r.n_in, dmax, e.stream);
-        e.after_launch("column max");
-        m = (u32)(e.read_u64(reinterpret_cast<u64*>(dmax)) & 0xFFFFFFFFull);
-      }
-      r.width[c] = r.n_in ? std::max(1, bitlen((u64)m + 1)) : 1;
-      r.maxv[c] = m;
+      r.maxv[c] = r.n_in ? r.in_max[c] : 0;
+      r.width[c] = r.n_in ? std::max(1, bitlen((u64)r.maxv[c] + 1)) : 1;
     }
     if (r.in_has_samples && r.n_in) {
-      reduce_max_u32(r.in_samples.as<u32>(), r.n_in, dmax, e.stream);
-      e.after_launch("sample max");
-      max_sample = std::max(max_sample, (u32)(e.read_u64(reinterpret_cast<u64*>(dmax)) & 0xFFFFFFFFull));
+      max_sample = std::max(max_sample, r.in_max_sample);
       any_samples = true;
     }
   }
@@ -936,13 +952,31 @@ static void load_facts(lob_engine& e) {
     a.otags = V.tags.p;
     a.ostamp = stamps ? V.stamps.as<u32>() : nullptr;
     a.row_factor = sem == SR_DIFF_ADD_MULT ? r.row_factor.as<float>() : nullptr;
-    a.count_dev = e.counts.as<u64>();
+    const size_t slot = kRowSlot + (&r - &e.rels[0]) % kRowSlots;
+    a.count_dev = e.counts.as<u64>() + slot;
     scratch_at_least(e, unique_scratch_bytes(n));
     load_unique(a, e.scratch.p, e.stream);
     e.after_launch("load unique");
     e.launches += 2 + scan_launches((n + 4095) / 4096);
-    V.n = e.read_u64(e.counts.as<u64>());
-    // recent = all loaded facts (Algorithm 1 starts with stable empty, recent = F_T)
+    if (e.rels.size() > (size_t)kRowSlots) V.n = e.read_u64(e.counts.as<u64>() + slot);
+  }
+  if (e.rels.size() <= (size_t)kRowSlots) {  // the row counts of all relations with one wait
+    e.check(cudaMemcpyAsync(e.pinned, e.counts.as<u64>() + kRowSlot, e.rels.size() * sizeof(u64), cudaMemcpyDeviceToHost,
+                            e.stream), "row counts");
+    e.sync();
+    for (size_t k = 0; k < e.rels.size(); k++)
+      if (e.rels[k].n_in) e.rels[k].views[0].n = e.pinned[k];
+  }
+  if (sem_top1(sem)) top1_setup(e, id_base);
+}
+
+// recent = all loaded facts (Algorithm 1 starts with stable empty, recent = F_T)
+static void load_recent(lob_engine& e) {
+  const int sb = stored_bytes(e.semiring);
+  for (auto& r : e.rels) {
+    const ViewSt& V = r.views[0];
+    if (!r.n_in) continue;
+    const int kb = V.lay.key64 ? 8 : 4;
     e.ensure(r.rkeys, V.n * kb);
     e.check(cudaMemcpyAsync(r.rkeys.p, V.keys.p, V.n * kb, cudaMemcpyDeviceToDevice, e.stream), "recent keys");
     if (sb) {
@@ -951,7 +985,6 @@ static void load_facts(lob_engine& e) {
     }
     r.n_recent = V.n;
   }
-  if (sem_top1(sem)) top1_setup(e, id_base);
 }
 
 // the secondary views of the loaded facts
@@ -2035,16 +2068,9 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   e.peak_bytes = e.live_bytes;
   e.launches = 0;
   const u64 syncs0 = e.host_syncs;
-  struct RunEvents {  // destroyed on every exit, the error paths included
-    cudaEvent_t a = nullptr, b = nullptr;
-    ~RunEvents() {
-      if (a) cudaEventDestroy(a);
-      if (b) cudaEventDestroy(b);
-    }
-  } ev;
-  e.check(cudaEventCreate(&ev.a), "event");
-  e.check(cudaEventCreate(&ev.b), "event");
-  cudaEvent_t ev0 = ev.a, ev1 = ev.b;
+  if (!e.run_begin) e.check(cudaEventCreate(&e.run_begin), "event");
+  if (!e.run_end) e.check(cudaEventCreate(&e.run_end), "event");
+  cudaEvent_t ev0 = e.run_begin, ev1 = e.run_end;
   e.check(cudaEventRecord(ev0, e.stream), "event");
   e.iter_counts.clear();
   e.cand_emitted = 0;
@@ -2065,6 +2091,7 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   const bool bit_done = bits && bit_run(e, max_iters, k, (u64&)s.new_facts, &rc);
   if (!bit_done) {
     if (bits) prepare_arms(e);
+    load_recent(e);
     load_views(e);
   }
   enable_dense(e);
@@ -2135,11 +2162,12 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   }
   for (auto& r : e.rels)
     if (r.keys_stale) materialize_keys(e, r, r.bitmap.as<u32>());
-  e.cand_emitted += e.read_u64(e.counts.as<u64>() + 13);  // outputs of bitmap-only warp steps
+  e.check(cudaMemcpyAsync(e.pinned, e.counts.as<u64>() + 13, 3 * sizeof(u64), cudaMemcpyDeviceToHost, e.stream), "run status");
   e.check(cudaEventRecord(ev1, e.stream), "event");
   e.sync();
   e.prof.flush();
-  if (e.read_u64(e.counts.as<u64>() + 15) & 0xFFFFFFFFull)
+  e.cand_emitted += e.pinned[0];  // outputs of the steps that count them on the device
+  if (e.pinned[2] & 0xFFFFFFFFull)
     throw LobError(LOB_E_TIMEOUT, "a bounded device wait of the sort gave up; the run's results are invalid");
   float ms = 0;
   cudaEventElapsedTime(&ms, ev0, ev1);
@@ -2225,7 +2253,7 @@ int lob_create(lob_engine** out, const lob_alloc* alloc, void* cuda_stream) {
       return LOB_E_CUDA;
     }
   }
-  if (cudaMallocHost(&e->pinned, 64 * sizeof(u64)) != cudaSuccess) {
+  if (cudaMallocHost(&e->pinned, kPinnedSlots * sizeof(u64)) != cudaSuccess) {
     cudaGetLastError();
     g_create_err = "pinned host allocation failed";
     if (e->pool) cudaMemPoolDestroy(e->pool);
@@ -2235,7 +2263,7 @@ int lob_create(lob_engine** out, const lob_alloc* alloc, void* cuda_stream) {
   int rc = guarded(e, [&] {
     // status and count words: every flag a kernel may set starts cleared, so a
     // flag read back reports the call that set it, never an allocator's leftovers
-    e->ensure(e->counts, 64 * sizeof(u64) + 256);
+    e->ensure(e->counts, (kRowSlot + kRowSlots) * sizeof(u64));
     e->check(cudaMemsetAsync(e->counts.p, 0, e->counts.cap, e->stream), "clear status words");
     e->sync();
     return LOB_OK;
@@ -2257,9 +2285,13 @@ void lob_destroy(lob_engine* e) {
     cudaSetDevice(e->device);
     e->release_all();
     e->release(e->counts);
+    for (auto& c : e->small_free)
+      for (void* p : c.second) cudaFreeAsync(p, e->stream);
     cudaStreamSynchronize(e->stream);
   } catch (...) {
   }
+  if (e->run_begin) cudaEventDestroy(e->run_begin);
+  if (e->run_end) cudaEventDestroy(e->run_end);
   if (e->pool) cudaMemPoolDestroy(e->pool);
   if (e->capture_stream) cudaStreamDestroy(e->capture_stream);
   if (e->capture_stream2) cudaStreamDestroy(e->capture_stream2);
@@ -2356,15 +2388,20 @@ int lob_load_relation(lob_engine* e, uint32_t rel, const uint32_t* cols, const f
       else
         e->check(cudaMemsetAsync(r.in_samples.as<u32>() + r.n_in, 0, n * 4, e->stream), "samples");
     }
-    if (mem == LOB_MEM_HOST) e->sync();  // the caller may reuse its host buffers on return
-    // values must leave the all-ones code free
-    u32* dmax = e->counts.as<u32>() + 32;
-    for (u32 c = 0; c < r.arity; c++) {
-      reduce_max_u32(r.in_cols[0].as<u32>() + (u64)c * r.in_cap + r.n_in, n, dmax, e->stream);
-      e->after_launch("column max");
-      if ((u32)(e->read_u64(reinterpret_cast<u64*>(dmax)) & 0xFFFFFFFFull) == 0xFFFFFFFFu)
-        throw LobError(LOB_E_ARG, "column value 0xFFFFFFFF is reserved");
-    }
+    // The largest values, of every column and the sample ids at once: they must
+    // leave the all-ones code free, and the run lays its keys out by them.  The
+    // wait also means that the caller may reuse its buffers on return.
+    u32* dmax = reinterpret_cast<u32*>(e->counts.as<u64>() + kMaxSlot);
+    reduce_max_cols(r.in_cols[0].as<u32>() + r.n_in, r.in_cap, (int)r.arity,
+                    r.in_has_samples ? r.in_samples.as<u32>() + r.n_in : nullptr, n, dmax, e->stream);
+    e->after_launch("column max");
+    e->check(cudaMemcpyAsync(e->pinned, dmax, (kMaxArity + 1) * sizeof(u32), cudaMemcpyDeviceToHost, e->stream), "column max");
+    e->sync();
+    const u32* top = reinterpret_cast<const u32*>(e->pinned);
+    for (u32 c = 0; c < r.arity; c++)
+      if (top[c] == 0xFFFFFFFFu) throw LobError(LOB_E_ARG, "column value 0xFFFFFFFF is reserved");
+    for (u32 c = 0; c < r.arity; c++) r.in_max[c] = std::max(r.in_max[c], top[c]);
+    if (r.in_has_samples) r.in_max_sample = std::max(r.in_max_sample, top[kMaxArity]);
     r.n_in += n;
     return LOB_OK;
   });
@@ -2760,6 +2797,8 @@ int lob_reset(lob_engine* e) {
       e->release(r.in_samples);
       r.n_in = r.in_cap = 0;
       r.in_has_tags = r.in_has_samples = false;
+      for (auto& m : r.in_max) m = 0;
+      r.in_max_sample = 0;
     }
     e->state = 0;
     e->ran_diff = false;

@@ -96,6 +96,8 @@ struct RelSt {
   u64 n_in = 0, in_cap = 0;
   bool in_has_tags = false, in_has_samples = false;
   std::vector<u64> in_chunks_tagged;  // (row_begin, row_end, tagged) triples flattened
+  u32 in_max[kMaxArity] = {0};  // largest loaded value of each column, and sample id
+  u32 in_max_sample = 0;
   int width[kMaxArity] = {0};
   u32 maxv[kMaxArity] = {0};  // no value of the column is larger
   std::vector<ViewSt> views;  // [0] = primary (identity permutation)
@@ -205,7 +207,8 @@ struct EngineProfiler : KernelProfiler {
 // values occur as columns, the long rows and (last word) their number
 struct BitCsr {
   bool built = false;
-  DevBuf ptr, col, used, colflag, heavy;
+  DevBuf zeroed, col;  // zeroed: everything but the columns
+  u32 *ptr = nullptr, *used = nullptr, *colflag = nullptr, *heavy = nullptr;
   u32 heavy_cap = 0;
 };
 // a derived relation: F, the two recent sets' buffers, the accumulator of an
@@ -213,7 +216,8 @@ struct BitCsr {
 // row counts -- and the final row offsets
 struct BitRel {
   bool need_t = false;
-  DevBuf full, fcnt, recent[2], rcnt[2], acc, aflag, trecent, trcnt, tfull, tfcnt, off;
+  DevBuf full, recent[2], acc, trecent, tfull, off, counts;  // counts: the row counts and flags
+  u32 *fcnt = nullptr, *rcnt[2] = {nullptr, nullptr}, *aflag = nullptr, *trcnt = nullptr, *tfcnt = nullptr;
   BitCsr csr[2];  // an input relation read forwards / backwards
 };
 struct BitRun {
@@ -224,6 +228,12 @@ struct BitRun {
   DevBuf pres, pref, dict, state, steps, list, hlist, temp[2], tbag[2];
   std::vector<BitRel> rel;
 };
+
+constexpr int kPinnedSlots = 256;
+constexpr size_t kSmallBlock = 1 << 20, kSmallKept = 64 << 20;
+// status words of e.counts: 64 of the steps, the column maxima (u32, from word 32
+// of the block that follows), then one row count per loaded relation
+constexpr int kCountSlots = 64, kMaxSlot = kCountSlots, kRowSlot = kMaxSlot + 8, kRowSlots = 128;
 
 struct lob_engine {
   int device = 0;
@@ -281,7 +291,13 @@ struct lob_engine {
   // iterations that begin a stratum after the first (every fact recent)
   int n_strata = 1;
   std::vector<u32> stratum_begin;
-  u64* pinned = nullptr;           // host readback slots
+  u64* pinned = nullptr;           // host readback slots (kPinnedSlots)
+  cudaEvent_t run_begin = nullptr, run_end = nullptr;  // time a run
+  // Blocks of up to kSmallBlock bytes given back to the engine's own pool stay
+  // here, by size class, for the next request on the stream (kSmallKept bytes at
+  // most): a run makes some 40 of them, and each trip to the pool costs about 1.5 us.
+  std::map<size_t, std::vector<void*>> small_free;
+  size_t small_bytes = 0;
   // top-1-proofs: the proof arena (u32 words), its tail and error word
   // (top1_state[0], [1]) and the probability of every input-fact id
   DevBuf arena, top1_state, top1_prob;

@@ -255,7 +255,10 @@ __global__ void k_read_rows(Layout L, Perm perm, const void* __restrict__ keys, 
   }
 }
 
-__global__ void k_reduce_max(const u32* __restrict__ a, u64 n, u32* __restrict__ out) {
+__global__ void k_reduce_max(const u32* __restrict__ cols, u64 stride_c, int arity, const u32* __restrict__ samples, u64 n,
+                             u32* __restrict__ out) {
+  const u32* a = (int)blockIdx.y < arity ? cols + blockIdx.y * stride_c : samples;
+  out += (int)blockIdx.y < arity ? (int)blockIdx.y : kMaxArity;
   const u64 stride = (u64)gridDim.x * blockDim.x;
   u32 m = 0;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) m = max(m, a[i]);
@@ -423,7 +426,7 @@ void bitmap_set_keys(const void* keys, int key64, u64 n, u32* bitmap, cudaStream
   if (n) k_bitmap_set<<<grid_for(n), 256, 0, st>>>(keys, key64, n, bitmap);
 }
 
-void reduce_max_u32(const u32* a, u64 n, u32* out_dev, cudaStream_t st) {
-  cudaMemsetAsync(out_dev, 0, sizeof(u32), st);
-  if (n) k_reduce_max<<<grid_for(n), 256, 0, st>>>(a, n, out_dev);
+void reduce_max_cols(const u32* cols, u64 stride, int arity, const u32* samples, u64 n, u32* out_dev, cudaStream_t st) {
+  cudaMemsetAsync(out_dev, 0, (kMaxArity + 1) * sizeof(u32), st);
+  if (n) k_reduce_max<<<dim3(grid_for(n), arity + (samples ? 1 : 0)), 256, 0, st>>>(cols, stride, arity, samples, n, out_dev);
 }

@@ -227,7 +227,9 @@ void pack_rows(const Layout& L, const u32* cols, u64 stride, const u32* samples,
                cudaStream_t st);
 void read_rows(int sem, const Layout& L, const int* perm, const void* keys, const void* tags, u64 n, u32* cols,
                u64 stride, float* otags, u32* samples, cudaStream_t st);
-void reduce_max_u32(const u32* a, u64 n, u32* out_dev, cudaStream_t st);
+// out_dev[c] = the largest of column c's n values (0 <= c < arity, columns `stride`
+// apart), out_dev[kMaxArity] that of the sample ids (null: 0)
+void reduce_max_cols(const u32* cols, u64 stride, int arity, const u32* samples, u64 n, u32* out_dev, cudaStream_t st);
 void gather_cand_tags(int sem, const void* stored, const u64* idx, u64 n, void* out, cudaStream_t st);
 
 // top-1-proofs (top1.cu).  The arena: word 0 the empty proof, words 1 + 2i and
