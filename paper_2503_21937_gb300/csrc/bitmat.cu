@@ -52,11 +52,20 @@ constexpr u64 kMaxValue = 1ull << 28;     // largest id the renumbering's presen
 enum : int { B_DONE = 0, B_ITER, B_NEW, B_CAND, B_WORDS, B_REL = 8 };
 LOB_HD int rel_slot(int r, int f) { return B_REL + 3 * r + f; }
 constexpr int kStateSlots = B_REL + 3 * kMaxBitRels;
-// ... and, not read back, two list lengths for each of an iteration's products
+// ... and, not read back, three list lengths for each of an iteration's products
 constexpr int kMaxLists = 32;
-constexpr int kAllSlots = kStateSlots + 2 * kMaxLists;
+constexpr int kAllSlots = kStateSlots + 3 * kMaxLists;
 // (the loop in one launch uses the first of those as its barrier words)
 constexpr int kReadSlots = kStateSlots + 1;
+
+// set bits a warp of a scatter lists before it sets their columns (at least the
+// 1,024 of one batch of words)
+constexpr int kBitList = 1024;
+// k_bit_gather_wide: chunks of a task, and the most entries of a row it takes (the
+// rows of 512 entries that the other form takes would keep one warp for four
+// chunks: closure of the power-law graph 0.86 -> 1.48 ms)
+constexpr int kWide = 4;
+constexpr u32 kWideRow = 8;
 
 enum IndexKind { I_IDENT = 0, I_CSR = 1, I_BITS = 2 };
 
@@ -88,12 +97,14 @@ struct BOp {
   BMat ib;
   BCsr mc;             // operand U
   BMat mb;
+  const u32* filled;   // scatter by bits: the operand rows that are not empty, as bits
   const u32* need;     // rows of the result that a later product reads (null: all)
   // listed form: only the result rows some index entry gives anything to, as
   // k_bit_active found them (long compressed rows apart); null: every row
   u32* list;
   u32* hlist;
-  u64* n_list;         // [0] rows listed, [1] long rows listed
+  u32* slist;          // (or null) rows of few entries, for k_bit_gather_wide
+  u64* n_list;         // rows listed in list, hlist, slist
   // result: a temporary (out, obag) ...
   u32* out;
   u64* obag;
@@ -164,6 +175,10 @@ LOB_DEV u32 put4(const BOp& P, u32 r, u32 w, uint4 a) {
     *N = make_uint4(0, 0, 0, 0);
   }
   uint4* F = reinterpret_cast<uint4*>(P.full) + at;
+  if (!any4(a)) {  // nothing derived here: F stays unread
+    reinterpret_cast<uint4*>(P.next)[at] = a;
+    return 0;
+  }
   uint4 f = ldm<kLoop>(F);
   a.x &= ~f.x; a.y &= ~f.y; a.z &= ~f.z; a.w &= ~f.w;
   reinterpret_cast<uint4*>(P.next)[at] = a;
@@ -373,17 +388,19 @@ __global__ void __launch_bounds__(256) k_bit_active(const __grid_constant__ BOp 
     cand += bag;
     live = live || (in && P.commit && P.aflag && P.aflag[r]);
     const bool heavy = live && IK == I_CSR && operand_bits && len > kHeavyRow;
-    const u32 ml = __ballot_sync(0xFFFFFFFFu, live && !heavy), mh = __ballot_sync(0xFFFFFFFFu, heavy);
-    u32 at = 0, hat = 0;
-    if (lane == 0) {
-      if (ml) at = (u32)atomicAdd(reinterpret_cast<unsigned long long*>(P.n_list), (unsigned long long)__popc(ml));
-      if (mh) hat = (u32)atomicAdd(reinterpret_cast<unsigned long long*>(P.n_list) + 1, (unsigned long long)__popc(mh));
-    }
-    at = __shfl_sync(0xFFFFFFFFu, at, 0);
-    hat = __shfl_sync(0xFFFFFFFFu, hat, 0);
+    const bool brief = live && P.slist && len <= kWideRow;
+    const int which = heavy ? 1 : brief ? 2 : 0;
     const u32 below = (1u << lane) - 1u;
-    if (heavy) P.hlist[hat + __popc(mh & below)] = r;
-    else if (live) P.list[at + __popc(ml & below)] = r;
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const u32 m = __ballot_sync(0xFFFFFFFFu, live && which == q);
+      if (!m) continue;
+      u32 at = 0;
+      if (lane == 0) at = (u32)atomicAdd(reinterpret_cast<unsigned long long*>(P.n_list) + q, (unsigned long long)__popc(m));
+      at = __shfl_sync(0xFFFFFFFFu, at, 0);
+      u32* to = q == 0 ? P.list : q == 1 ? P.hlist : P.slist;
+      if (live && which == q) to[at + __popc(m & below)] = r;
+    }
   }
   block_totals(P, cand, 0, 0);
 }
@@ -494,6 +511,91 @@ LOB_DEV void gather_rows(const BOp& P) {
 template <int IK>
 __global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp P) { gather_rows<IK, false>(P); }
 
+// The same for the rows of few entries of wide matrices (compressed index, listed
+// apart): a warp takes four chunks of a row, so that what it waits for on the way to
+// the first word -- list, offsets, column, weight, one after another -- is paid
+// once, and the words of two operand rows and of F come eight and four loads at a
+// time.  Same generation on the 50,000-node tree, whose rows list one operand row:
+// the gathers of a run 3.2 -> 2.2 ms.
+__global__ void __launch_bounds__(256) k_bit_gather_wide(const __grid_constant__ BOp P) {
+  if (op_idle<false>(P)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 groups = (P.words + kWide * 128 - 1) / (kWide * 128);
+  const u64 stride = P.words / 4;
+  u64 read = 0, fresh_all = 0;
+  const u64 tasks = P.n_list[2] * groups, nwarps = (u64)gridDim.x * kGatherWarps;
+  for (u64 t = (u64)blockIdx.x * kGatherWarps + warp; t < tasks; t += nwarps) {
+    const u32 r = P.slist[t / groups], w0 = (u32)(t % groups) * (kWide * 128) + lane * 4;
+    const u32 j0 = P.ic.ptr[r], j1 = P.ic.ptr[r + 1];
+    const uint4* base = reinterpret_cast<const uint4*>(P.mb.bits + w0);
+    uint4 acc[kWide];
+#pragma unroll
+    for (int c = 0; c < kWide; c++) acc[c] = make_uint4(0, 0, 0, 0);
+    for (u32 j = j0; j < j1; j += 32) {
+      const u32 idx = j + lane < j1 ? P.ic.col[j + lane] : 0u;
+      u32 m = __ballot_sync(0xFFFFFFFFu, j + lane < j1 && P.mb.weight<false>(idx) != 0);
+      if (lane == 0) read += (u64)__popc(m) * min(P.words - (w0 & ~127u), (u32)kWide * 128);
+      while (m) {
+        const u32 a = __shfl_sync(0xFFFFFFFFu, idx, __ffs(m) - 1);
+        m &= m - 1;
+        const u32 b = m ? __shfl_sync(0xFFFFFFFFu, idx, __ffs(m) - 1) : a;
+        m &= m - 1;
+        uint4 x[kWide], y[kWide];
+#pragma unroll
+        for (int c = 0; c < kWide; c++)
+          if (w0 + c * 128 < P.words) {
+            x[c] = base[a * stride + c * 32];
+            y[c] = base[b * stride + c * 32];
+          }
+#pragma unroll
+        for (int c = 0; c < kWide; c++)
+          if (w0 + c * 128 < P.words) {
+            or4(acc[c], x[c]);
+            or4(acc[c], y[c]);
+          }
+      }
+    }
+    u32 fresh = 0;
+    if (P.commit && !(P.aflag && P.aflag[r])) {
+      uint4* F = reinterpret_cast<uint4*>(P.full + (u64)r * P.words + w0);
+      uint4* D = reinterpret_cast<uint4*>(P.next + (u64)r * P.words + w0);
+      uint4 f[kWide];
+#pragma unroll
+      for (int c = 0; c < kWide; c++) {
+        diag4(acc[c], P.diag, r, w0 + c * 128);
+        if (w0 + c * 128 < P.words && any4(acc[c])) f[c] = F[c * 32];
+      }
+#pragma unroll
+      for (int c = 0; c < kWide; c++) {
+        if (w0 + c * 128 >= P.words) continue;
+        uint4 a = acc[c];
+        if (any4(a)) {
+          a.x &= ~f[c].x; a.y &= ~f[c].y; a.z &= ~f[c].z; a.w &= ~f[c].w;
+          if (any4(a)) {
+            or4(f[c], a);
+            F[c * 32] = f[c];
+            fresh += popc4(a);
+          }
+        }
+        D[c * 32] = a;
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < kWide; c++)
+        if (w0 + c * 128 < P.words) fresh += put4<false>(P, r, w0 + c * 128, acc[c]);
+    }
+    if (P.commit) {
+#pragma unroll
+      for (int o = 16; o; o >>= 1) fresh += __shfl_xor_sync(0xFFFFFFFFu, fresh, o);
+      if (lane == 0) {
+        count_new(P, r, fresh);
+        fresh_all += fresh;
+      }
+    }
+  }
+  block_totals(P, 0, read, fresh_all);
+}
+
 // ---------------------------------------------------------------------------
 // scatter: row r of the result = the union of the compressed operand rows
 // listed in row r of the index matrix (identity: operand row r itself), built
@@ -501,26 +603,44 @@ __global__ void __launch_bounds__(256) k_bit_gather(const __grid_constant__ BOp 
 // derivation, where the global ones of the general path go to L2; rows of up
 // to 92,000 values take 11.5 KB, so 8 blocks an SM stay resident.
 // ---------------------------------------------------------------------------
-LOB_DEV void set_row_bits(const BCsr& M, u32* row, u32 y, bool valid, u64& bag) {
-  u32 j0 = 0, j1 = 0;
-  if (valid) {
-    j0 = M.ptr[y];
-    j1 = M.ptr[y + 1];
-    bag += j1 - j0;
-  }
-  const bool big = j1 - j0 > 16;
-  if (!big)
-    for (u32 j = j0; j < j1; j++) {
-      const u32 c = M.col[j];
-      atomicOr(row + (c >> 5), 1u << (c & 31u));
-    }
+// The columns of n operand rows, named by a warp's list (`base` added to each
+// entry), are set in `row`; four of them per lane and step, so that their loads
+// overlap.
+template <class T>
+LOB_DEV void set_list(const BCsr& M, u32* row, const T* list, u32 n, u32 base, u64& bag) {
+  constexpr int kAt = 4;
   const int lane = threadIdx.x & 31;
-  for (u32 m = __ballot_sync(0xFFFFFFFFu, big); m; m &= m - 1) {  // long rows: the whole warp
-    const int src = __ffs(m) - 1;
-    const u32 a = __shfl_sync(0xFFFFFFFFu, j0, src), b = __shfl_sync(0xFFFFFFFFu, j1, src);
-    for (u32 j = a + lane; j < b; j += 32) {
-      const u32 c = M.col[j];
-      atomicOr(row + (c >> 5), 1u << (c & 31u));
+  for (u32 i0 = 0; i0 < n; i0 += 32 * kAt) {
+    u32 j[kAt], e[kAt], c[kAt];
+#pragma unroll
+    for (int q = 0; q < kAt; q++) {
+      const u32 i = i0 + q * 32 + lane;
+      const u32 y = i < n ? base + list[i] : 0u;
+      j[q] = i < n ? M.ptr[y] : 0u;
+      e[q] = i < n ? M.ptr[y + 1] : 0u;
+    }
+#pragma unroll
+    for (int q = 0; q < kAt; q++) {
+      c[q] = j[q] < e[q] ? M.col[j[q]] : 0u;
+      bag += e[q] - j[q];
+    }
+#pragma unroll
+    for (int q = 0; q < kAt; q++) {
+      if (j[q] < e[q]) atomicOr(row + (c[q] >> 5), 1u << (c[q] & 31u));
+      const bool big = e[q] - j[q] > 16;
+      if (!big)
+        for (u32 k = j[q] + 1; k < e[q]; k++) {
+          const u32 x = M.col[k];
+          atomicOr(row + (x >> 5), 1u << (x & 31u));
+        }
+      for (u32 m = __ballot_sync(0xFFFFFFFFu, big); m; m &= m - 1) {  // long rows: the whole warp
+        const int src = __ffs(m) - 1;
+        const u32 a = __shfl_sync(0xFFFFFFFFu, j[q], src), b = __shfl_sync(0xFFFFFFFFu, e[q], src);
+        for (u32 k = a + lane; k < b; k += 32) {
+          const u32 x = M.col[k];
+          atomicOr(row + (x >> 5), 1u << (x & 31u));
+        }
+      }
     }
   }
 }
@@ -560,21 +680,37 @@ LOB_DEV void scatter_rows(const BOp& P) {
           bag++;
         }
       } else if constexpr (IK == I_CSR) {
-        for (u32 j = j0; j < j1; j += 256) {
-          const bool v = j + threadIdx.x < j1;
-          set_row_bits(P.mc, row, v ? P.ic.col[j + threadIdx.x] : 0u, v, bag);
-        }
+        const u32 per = (j1 - j0 + 7) / 8, a = j0 + (threadIdx.x >> 5) * per;
+        if (a < j1) set_list(P.mc, row, P.ic.col + a, min(per, j1 - a), 0, bag);
       } else {
+        // A warp lists the bits of its share of the row -- those whose operand row
+        // holds something -- and then sets their columns, evenly over its lanes.  (A
+        // lane walking its own word's bits waits for two loads per bit, and for the
+        // lane with the most bits: 4.8 ms on the 50,000-node tree, 4.2 without the
+        // empty operand rows.)
+        __shared__ uint16_t lists[8][kBitList];
+        uint16_t* list = lists[threadIdx.x >> 5];
+        const int lane = threadIdx.x & 31;
         const u32* src = P.ib.bits + (u64)r * P.words;
-        for (u32 w0 = 0; w0 < P.words; w0 += 256) {
-          const u32 w = w0 + threadIdx.x;
-          u32 m = w < P.words ? ldm<kLoop>(src + w) : 0u;
-          while (__any_sync(0xFFFFFFFFu, m != 0u)) {
-            const u32 y = w * 32 + (m ? (u32)__ffs(m) - 1 : 0u);
-            set_row_bits(P.mc, row, y, m != 0u, bag);
-            m &= m - 1;
+        const u32 share = (P.words + 7) / 8, first = (threadIdx.x >> 5) * share, end = min(P.words, first + share);
+        u32 n = 0;
+        for (u32 w0 = first; w0 < end; w0 += 32) {
+          const u32 w = w0 + lane;
+          u32 m = w < end ? ldm<kLoop>(src + w) & P.filled[w] : 0u;
+          const u32 inc = warp_inclusive_sum((u32)__popc(m));
+          const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
+          if (n + tot > (u32)kBitList) {
+            __syncwarp();
+            set_list(P.mc, row, list, n, first * 32, bag);
+            __syncwarp();
+            n = 0;
           }
+          u32 at = n + inc - __popc(m);
+          for (; m; m &= m - 1) list[at++] = (uint16_t)((w - first) * 32 + (u32)__ffs(m) - 1);
+          n += tot;
         }
+        __syncwarp();
+        set_list(P.mc, row, list, n, first * 32, bag);
         read += threadIdx.x == 0 ? P.words : 0;
       }
     }
@@ -659,7 +795,7 @@ LOB_DEV void end_iteration(const BEnd& E) {
     total += n;
   }
   if constexpr (!kLoop)
-    for (int i = 0; i < 2 * kMaxLists; i++) s[kStateSlots + i] = 0;
+    for (int i = 0; i < 3 * kMaxLists; i++) s[kStateSlots + i] = 0;
   s[B_NEW] = ldm<kLoop>(s + B_NEW) + total;
   const u64 it = ldm<kLoop>(s + B_ITER) + 1;
   s[B_ITER] = it;
@@ -895,6 +1031,15 @@ __global__ void k_csr_fill(KeyCols K, Codes code, int inv, const u32* __restrict
     if (q == kHeavyRow) heavy[atomicAdd(n_heavy, 1u)] = r;  // one entry of a longer row gets here
   }
 }
+// bit r of the result: row r holds something; a warp a word
+__global__ void __launch_bounds__(256) k_filled_rows(const u32* __restrict__ ptr, u32 rows, u32 words, u32* __restrict__ out) {
+  const u32 lane = threadIdx.x & 31;
+  for (u32 w = blockIdx.x * 8 + (threadIdx.x >> 5); w < words; w += gridDim.x * 8) {
+    const u32 r = w * 32 + lane;
+    const u32 x = __ballot_sync(0xFFFFFFFFu, r < rows && ptr[r] != ptr[r + 1]);
+    if (lane == 0) out[w] = x;
+  }
+}
 // facts loaded into a derived relation: F and D start with them
 __global__ void k_set_facts(KeyCols K, Codes code, int inv, u32 words, u32* full, u32* recent, u32* cnt, u32* fcnt) {
   const u64 stride = (u64)gridDim.x * blockDim.x;
@@ -924,14 +1069,32 @@ __global__ void __launch_bounds__(256) k_row_counts(const u32* __restrict__ bits
   }
 }
 
+// A warp stores n consecutive words: up to the next 16-byte boundary one by one,
+// then four a lane (value / four: the word, the four words, from an offset on).
+template <class F, class G>
+LOB_DEV void store_run(u32* __restrict__ p, u32 n, int lane, F&& value, G&& four) {
+  const u32 head = min(n, (u32)(0 - (reinterpret_cast<uintptr_t>(p) >> 2)) & 3u);
+  const u32 quads = (n - head) / 4;
+  for (u32 q = lane; q < quads; q += 32) {
+    const u32 s = head + 4 * q;
+    *reinterpret_cast<uint4*>(p + s) = four(s);
+  }
+  const u32 rest = n - 4 * quads;  // at most six
+  if ((u32)lane < rest) {
+    const u32 s = (u32)lane < head ? (u32)lane : 4 * quads + (u32)lane;
+    p[s] = value(s);
+  }
+}
+
 // Read-out: a warp walks a row 32 words at a time; a scan of the words' bit
 // counts places each lane's columns in the warp's shared-memory stage, and the
-// warp stores the batch's rows of every output column to consecutive addresses.
+// warp stores the batch's rows of every output column to consecutive addresses,
+// 16 bytes a lane.
 __global__ void __launch_bounds__(256) k_bit_read(const u32* __restrict__ bits, u32 rows, u32 words,
                                                   const u64* __restrict__ off, const u32* __restrict__ dict,
                                                   u32* __restrict__ c0, u32* __restrict__ c1, float* __restrict__ tags,
                                                   u32* __restrict__ samples) {
-  __shared__ u32 stages[8][1024];
+  __shared__ __align__(16) u32 stages[8][1024 + 4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   u32* stage = stages[warp];
   const u64 nwarps = (u64)gridDim.x * 8;
@@ -948,17 +1111,24 @@ __global__ void __launch_bounds__(256) k_bit_read(const u32* __restrict__ bits, 
       const u32 inc = warp_inclusive_sum(c);
       const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
       if (!tot) continue;
-      u32 pos = inc - c;
+      // staged at the offset the destination has within 16 bytes
+      const u32 skew = (u32)(reinterpret_cast<uintptr_t>(c1 + base) >> 2) & 3u;
+      u32 pos = inc - c + skew;
       const u32 kw = (w0 + lane) * 32;
       for (u32 m = m0; m; m &= m - 1) stage[pos++] = kw + (u32)__ffs(m) - 1;
       __syncwarp();
-      for (u32 q = lane; q < tot; q += 32) {
-        const u32 y = stage[q];
-        c0[base + q] = x;
-        c1[base + q] = dict ? dict[y] : y;
-        if (tags) tags[base + q] = 1.0f;
-        if (samples) samples[base + q] = 0u;
-      }
+      store_run(c0 + base, tot, lane, [&](u32) { return x; }, [&](u32) { return make_uint4(x, x, x, x); });
+      store_run(c1 + base, tot, lane, [&](u32 s) { return dict ? dict[stage[s + skew]] : stage[s + skew]; },
+                [&](u32 s) {
+                  uint4 y = *reinterpret_cast<const uint4*>(stage + s + skew);
+                  return dict ? make_uint4(dict[y.x], dict[y.y], dict[y.z], dict[y.w]) : y;
+                });
+      const u32 one = __float_as_uint(1.0f);
+      if (tags)
+        store_run(reinterpret_cast<u32*>(tags) + base, tot, lane, [&](u32) { return one; },
+                  [&](u32) { return make_uint4(one, one, one, one); });
+      if (samples)
+        store_run(samples + base, tot, lane, [&](u32) { return 0u; }, [&](u32) { return make_uint4(0, 0, 0, 0); });
       __syncwarp();
       base += tot;
     }
@@ -1139,7 +1309,11 @@ struct Run {
       e.after_launch("values");
       e.launches += scan_launches(nw);
       D = std::max<u64>(1, e.read_u64(e.counts.as<u64>() + 1) & 0xFFFFFFFFull);
-      B.mapped = true;
+      u64 top = 0;
+      for (size_t r = 0; r < e.rels.size(); r++)
+        if (used[r])
+          for (int c = 0; c < 2; c++) top = std::max<u64>(top, e.rels[r].maxv[c]);
+      B.mapped = D != top + 1;  // else every value up to the largest occurs: it is its own code
     }
     B.rows = (u32)D;
     B.words = (u32)((D + 127) / 128 * 4);
@@ -1211,6 +1385,14 @@ struct Run {
     launch_check("rows");
   }
 
+  void build_filled(const Link& l) {
+    BitCsr& C = B.rel[l.rel].csr[l.inv];
+    if (C.filled.p) return;
+    e.ensure(C.filled, (u64)B.words * 4);
+    k_filled_rows<<<warp_grid(B.words), 256, 0, e.stream>>>(C.ptr, B.rows, B.words, C.filled.as<u32>());
+    launch_check("rows");
+  }
+
   u64 mat_bytes() const { return (u64)B.rows * B.words * 4; }
 
   void allocate() {
@@ -1256,6 +1438,7 @@ struct Run {
     if (listed()) {
       e.ensure(B.list, D * 4);
       e.ensure(B.hlist, D * 4);
+      e.ensure(B.slist, D * 4);
     }
   }
 
@@ -1329,6 +1512,9 @@ struct Run {
         set_head(P, C.head, cur, commit);
         P.diag = C.diag;
       }
+      if (!bits && ik == I_BITS) {
+        P.filled = B.rel[L[m - 1].rel].csr[L[m - 1].inv].filled.as<u32>();
+      }
       product(P, ik, bits);
       cur_m = BMat{};
       cur_m.bits = P.out;
@@ -1371,7 +1557,8 @@ struct Run {
     if (listed() && n_lists < kMaxLists) {
       P.list = B.list.as<u32>();
       P.hlist = B.hlist.as<u32>();
-      P.n_list = B.state.as<u64>() + kStateSlots + 2 * n_lists++;
+      if (bits && ik == I_CSR && P.words > kWide * 128) P.slist = B.slist.as<u32>();
+      P.n_list = B.state.as<u64>() + kStateSlots + 3 * n_lists++;
       {
         ProfScope ps("bit_active", P.rows * 12.0, e.stream);
         const unsigned g = warp_grid((P.rows + 31) / 32);
@@ -1385,8 +1572,13 @@ struct Run {
       {
         ProfScope ps("bit_gather", 0, e.stream);
         if (ik == I_IDENT) k_bit_gather<I_IDENT><<<warp_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
-        else if (ik == I_CSR) k_bit_gather<I_CSR><<<warp_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
-        else k_bit_gather<I_BITS><<<block_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
+        else if (ik == I_CSR) {
+          if (P.slist) {
+            k_bit_gather_wide<<<warp_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
+            e.launches++;
+          }
+          k_bit_gather<I_CSR><<<warp_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
+        } else k_bit_gather<I_BITS><<<block_grid((u64)P.rows * chunks), 256, 0, e.stream>>>(P);
       }
       launch_check("bit gather");
     } else {
@@ -1539,8 +1731,14 @@ struct Run {
     if (!domain()) return false;
     allocate();
     for (auto& C : chains)
-      for (auto& l : C.links)
-        if (!e.rels[l.rel].idb) build_csr(oriented(l));
+      for (size_t i = 0; i < C.links.size(); i++) {
+        const Link l = oriented(C.links[i]);
+        if (e.rels[l.rel].idb) continue;
+        build_csr(l);
+        // the operand of a scatter by bits: which of its rows hold something
+        const size_t n = C.links.size(), before = B.transposed ? i + 1 : i - 1;
+        if (n > 1 && i == (B.transposed ? 0 : n - 1) && e.rels[C.links[before].rel].idb) build_filled(l);
+      }
     std::vector<u64> h(kStateSlots, 0);
     bool loaded = false;
     for (size_t r = 0; r < e.rels.size(); r++) {
@@ -1692,11 +1890,11 @@ bool bit_run(lob_engine& e, u32 max_iters, u32& k, u64& new_facts, int* rc) {
 void bit_release(lob_engine& e) {
   if (!e.bit) return;
   BitRun& B = *e.bit;
-  for (DevBuf* b : {&B.pres, &B.pref, &B.dict, &B.state, &B.steps, &B.list, &B.hlist, &B.temp[0], &B.temp[1], &B.tbag[0], &B.tbag[1]}) e.release(*b);
+  for (DevBuf* b : {&B.pres, &B.pref, &B.dict, &B.state, &B.steps, &B.list, &B.hlist, &B.slist, &B.temp[0], &B.temp[1], &B.tbag[0], &B.tbag[1]}) e.release(*b);
   for (BitRel& R : B.rel) {
     for (DevBuf* b : {&R.full, &R.recent[0], &R.recent[1], &R.counts, &R.acc, &R.trecent, &R.tfull, &R.off}) e.release(*b);
     for (BitCsr& C : R.csr)
-      for (DevBuf* b : {&C.zeroed, &C.col}) e.release(*b);
+      for (DevBuf* b : {&C.zeroed, &C.col, &C.filled}) e.release(*b);
   }
   e.bit.reset();
 }

@@ -207,7 +207,7 @@ struct EngineProfiler : KernelProfiler {
 // values occur as columns, the long rows and (last word) their number
 struct BitCsr {
   bool built = false;
-  DevBuf zeroed, col;  // zeroed: everything but the columns
+  DevBuf zeroed, col, filled;  // zeroed: everything but the columns; filled: the non-empty rows, as bits
   u32 *ptr = nullptr, *used = nullptr, *colflag = nullptr, *heavy = nullptr;
   u32 heavy_cap = 0;
 };
@@ -225,7 +225,7 @@ struct BitRun {
   bool transposed = false;  // stored transposed while the run lasts
   bool mapped = false;      // values are renumbered (dict: code -> value)
   u32 rows = 0, words = 0;
-  DevBuf pres, pref, dict, state, steps, list, hlist, temp[2], tbag[2];
+  DevBuf pres, pref, dict, state, steps, list, hlist, slist, temp[2], tbag[2];
   std::vector<BitRel> rel;
 };
 

@@ -62,12 +62,13 @@ def test_facts_loaded_into_derived_relations(name):
     same_as_general(PROGRAMS[name], inputs)
 
 
+@pytest.mark.parametrize("n", [12000, 17000])
 @pytest.mark.parametrize("name", ["left", "right", "same_generation", "two_rules"])
-def test_listed_rows_and_long_rows(name):
-    """Matrices beyond the listing threshold (12,000 values), rows of more than
-    512 entries in both directions (a hub), most rows idle in most iterations."""
+def test_listed_rows_and_long_rows(name, n):
+    """Matrices beyond the listing threshold (12,000 values) and the one for wide
+    rows (17,000), rows of more than 512 entries in both directions (a hub), most
+    rows idle in most iterations."""
     s = W.stream(7300)
-    n = 12000
     parent, child, _ = W.random_tree(n, seed_index=7301)
     hub = np.full(700, 5, np.uint32)
     leaf = s.below(700, n)
