@@ -84,7 +84,8 @@ typedef struct lob_stats {
   uint64_t host_syncs;      /* times the host waited for the GPU during the run */
   uint32_t device_iterations; /* iterations run by the device-driven loop (option "driver") */
   uint32_t graph_launches;  /* launches of that loop's graph (1 unless a buffer had to grow) */
-  uint64_t proof_words;     /* top-1-proofs: u32 words of the proof arena in use at the end */
+  uint64_t proof_words;     /* top-1-proofs: u32 words of the proof arena in use at the end
+                               (linear components form only the unions that can win) */
   uint32_t strata;          /* strata run one after another (1: one loop over every rule) */
   uint32_t reserved;
 } lob_stats;

@@ -227,7 +227,7 @@ LOB_DEV void dense_add(void* acc, u64 key, typename Sem::Cand t) {
     int* a = reinterpret_cast<int*>(acc) + key;
     const int v = __float_as_int(t);
     if (*reinterpret_cast<volatile int*>(a) < v) atomicMax(a, v);
-  } else if constexpr (std::is_same<Sem, SemDiffMaxMin>::value) {
+  } else if constexpr (std::is_same<Sem, SemDiffMaxMin>::value || std::is_same<Sem, SemTop1>::value) {
     unsigned long long* a = reinterpret_cast<unsigned long long*>(acc) + key;
     if (*reinterpret_cast<volatile unsigned long long*>(a) < t) atomicMax(a, (unsigned long long)t);
   }

@@ -782,9 +782,11 @@ static void prepare_arms(lob_engine& e) {
     }
   for (auto& p : e.plans)
     for (auto& A : p.arms) {
-      // top-1-proofs joins form unions of proofs, and computed head arguments
-      // and comparison filters run bytecode: general steps only
-      A.packed = e.opt_packed_join && !sem_top1(sem) && !p.ast.computes() ? compile_packed(e, p.ast, A) : PackedArm{};
+      // computed head arguments and comparison filters run bytecode: general
+      // steps only; so are top-1-proofs joins outside the linear loop
+      A.packed = e.opt_packed_join && !p.ast.computes() ? compile_packed(e, p.ast, A) : PackedArm{};
+      A.packed.linear_only = A.packed.ok && sem_top1(sem);
+      if (A.packed.linear_only) A.packed.ok = false;
       if (sem == SR_UNIT) compile_cross(e, p.ast, A, A.packed);
       if (sem != SR_UNIT) compile_mask(e, p.ast, A, A.packed);
     }
@@ -865,7 +867,7 @@ static void top1_setup(lob_engine& e, u64 n_ids) {
   e.launches += 3;
 }
 
-static Top1Arena top1_desc(lob_engine& e) {
+Top1Arena top1_desc(lob_engine& e) {
   Top1Arena A{};
   A.words = e.arena.as<u32>();
   A.tail = e.top1_state.as<unsigned long long>();
@@ -876,26 +878,30 @@ static Top1Arena top1_desc(lob_engine& e) {
   return A;
 }
 
-// After a top-1-proofs join emission: a union longer than the proof cap is an
-// error; when the arena ran out, it grows (keeping the proofs before this
-// step) and the step runs again from the same tail.  Emission is idempotent:
-// every output has a fixed position.
+// After kernels that formed unions: a union longer than the proof cap is an
+// error; when the arena ran out, it grows (keeping the proofs before them), the
+// tail goes back to where it was, and false is returned: they run again.
+bool top1_settle(lob_engine& e) {
+  e.check(cudaMemcpyAsync(e.pinned, e.top1_state.p, 16, cudaMemcpyDeviceToHost, e.stream), "proof arena state");
+  e.sync();
+  const u64 tail = e.pinned[0];
+  if (e.pinned[1] & 1)
+    throw LobError(LOB_E_CAPACITY, "top-1-proofs: a proof is longer than the proof cap (option proof_cap)");
+  if (tail <= e.arena_cap) {
+    e.arena_tail = tail;
+    return true;
+  }
+  if (e.arena_cap >= kArenaMaxWords) throw LobError(LOB_E_CAPACITY, "top-1-proofs: the proof arena needs 2^32 words");
+  const u64 want = std::min(kArenaMaxWords, std::max(2 * e.arena_cap, tail + tail / 2));
+  e.ensure(e.arena, want * 4, true);
+  e.arena_cap = std::min<u64>(kArenaMaxWords, e.arena.cap / 4);
+  set_u64_dev(e.top1_state.as<unsigned long long>(), e.arena_tail, e.stream);
+  return false;
+}
+
+// A join emission is idempotent: every output has a fixed position.
 static void top1_after_emit(lob_engine& e, int sem, StepParams& P, const u64* part) {
-  for (;;) {
-    e.check(cudaMemcpyAsync(e.pinned, e.top1_state.p, 16, cudaMemcpyDeviceToHost, e.stream), "proof arena state");
-    e.sync();
-    const u64 tail = e.pinned[0];
-    if (e.pinned[1] & 1)
-      throw LobError(LOB_E_CAPACITY, "top-1-proofs: a proof is longer than the proof cap (option proof_cap)");
-    if (tail <= e.arena_cap) {
-      e.arena_tail = tail;
-      return;
-    }
-    if (e.arena_cap >= kArenaMaxWords) throw LobError(LOB_E_CAPACITY, "top-1-proofs: the proof arena needs 2^32 words");
-    const u64 want = std::min(kArenaMaxWords, std::max(2 * e.arena_cap, tail + tail / 2));
-    e.ensure(e.arena, want * 4, true);
-    e.arena_cap = std::min<u64>(kArenaMaxWords, e.arena.cap / 4);
-    set_u64_dev(e.top1_state.as<unsigned long long>(), e.arena_tail, e.stream);
+  while (!top1_settle(e)) {
     P.top1 = top1_desc(e);
     join_emit(sem, P, part, e.stream);
     e.after_launch("join emit (proof arena grown)");

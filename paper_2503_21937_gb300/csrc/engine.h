@@ -149,6 +149,9 @@ struct StepPlan {
 // the single projection) a PStep template whose pointers are filled per launch.
 struct PackedArm {
   bool ok = false;
+  // top-1-proofs: the steps are compiled, but only the linear loop runs them
+  // (ok stays false: joins form unions of proofs elsewhere)
+  bool linear_only = false;
   std::vector<PStep> steps;
   // two probes where the second is keyed by the delta row alone: the second
   // probe compiled against the delta row (word 0), the first probe's key

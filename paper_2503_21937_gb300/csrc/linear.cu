@@ -26,7 +26,8 @@
 // step's facts are spread over all warps before a warp takes a second one.
 //
 // Measured (GB300): 64 x 64 grid, diff-add-mult, fixpoint of 128 iterations 8.6
-// -> 1.0 ms; diff-max-min, forward and backward 11.1 -> 1.8 ms.  A step takes 5
+// -> 1.0 ms; diff-max-min, forward and backward 11.1 -> 1.8 ms; top-1-proofs over 64
+// grids of side 16, forward and backward 9.1 -> 2.0 ms.  A step takes 5
 // us (15 with the arrays in L2), an iteration of the graph of kernels 67.
 #include "linear.h"
 
@@ -48,13 +49,15 @@ constexpr u64 kLinRelSlots = 1ull << 24;  // keys of one relation (dense arrays)
 constexpr u64 kLinMaxSlots = 1ull << 25;
 constexpr u32 kLinSpin = 1u << 26;     // barrier polls before giving up
 
-enum : int { LS_STOP = 0, LS_ITER, LS_CAND, LS_NEW, LS_ERR, LS_BAR, LS_LIST = 8, LS_FRESH = 12 };
+// LS_FULLARENA: top-1-proofs, one more than the first step that found the proof
+// arena full
+enum : int { LS_STOP = 0, LS_ITER, LS_CAND, LS_NEW, LS_ERR, LS_BAR, LS_FULLARENA, LS_LIST = 8, LS_FRESH = 12 };
 // LS_LIST + i: length of the list of step i mod 3; LS_FRESH + i * kLinMaxRels +
 // rel: the step's new facts (low half) and improved ones (high half); then per
 // relation |F| and |recent| at the end
 constexpr int LS_FULL = LS_FRESH + 3 * kLinMaxRels, LS_LAST = LS_FULL + kLinMaxRels;
 constexpr int kLinSlots = LS_LAST + kLinMaxRels;
-enum : u64 { LIN_FIXPOINT = 1, LIN_MAXITER = 2 };
+enum : u64 { LIN_FIXPOINT = 1, LIN_MAXITER = 2, LIN_ARENA = 3 };
 
 struct LinArm {
   PStep P;
@@ -76,6 +79,7 @@ struct LinArgs {
   u64 fcount[kLinMaxRels];  // |F| after iteration k0
   u32 k0, max_iters;
   u64* state;
+  Top1Arena top1;          // top-1-proofs
   u32* rec;                // add-mult: |recent| after iteration k at [(k - k0 - 1) * n_rel + rel]
 };
 
@@ -163,11 +167,119 @@ template <class Sem> constexpr u32 lin_slot_bytes() {
 }
 LOB_HD u32 lin_shared_bytes(u32 slot_bytes, u32 slots) { return slots * slot_bytes + 3 * (slots / 8) + kLinSlots * 8; }
 
+// ---------------------------------------------------------------------------
+// top-1-proofs: (x) of a derived fact's proof and an input fact's, which is one
+// id or empty.  Candidates that cannot win are not formed (a stored proof only
+// gets likelier): the proof {p_1 .. p_n} and one more fact x has probability at
+// most p max(1, p_x), and about p p_x once x is known not to be among them.  A
+// union with a fact of the proof is the proof itself.  What is left reads the
+// proof in eight lanes, four candidates a warp, and forms the product as
+// top1_union does: ascending ids, FP64, rounded once.  Bound by the chain of
+// loads (tag, length, ids, probabilities) and the FP64 products.  64 grids of side
+// 16, 44 iterations of 3,500 candidates: the general steps took 190 us an
+// iteration (53 of them for unions by single threads), a step here takes 20.
+// ---------------------------------------------------------------------------
+constexpr float kTopSlack = 1.000001f;  // f32 rounding of p, of p_x and of their product, with room to spare
+// probability bits of a candidate that cannot beat `best` (bits; ~0: nothing there)
+LOB_DEV bool top_loses(u32 p, u32 px, bool together, u32 best) {
+  if (p > 0x7F800000u || px > 0x7F800000u || best > 0x7F800000u) return false;  // a sign, a NaN, nothing to beat
+  const float fp = __uint_as_float(p), fx = __uint_as_float(px);
+  const float u = together ? fp * fx : fp * fmaxf(fx, 1.0f);
+  return fp >= 1e-30f && u >= 1e-30f && u * kTopSlack <= __uint_as_float(best);
+}
+// One union for each group of eight lanes with live set (all lanes of the warp
+// call).  Returns its tag to the whole group, 0 when it is dropped.
+LOB_DEV u64 top_union(const Top1Arena& T, bool live, u64 a, u64 b, u32 best, unsigned long long* full, u32 step) {
+  const int lane = threadIdx.x & 31, g0 = lane & 24, l8 = lane & 7;
+  const u32 ra = (u32)a, rb = (u32)b;
+  u64 out = 0;
+  u32 la = live ? __ldcg(T.words + ra) : 0u;
+  if (live && la == 0) out = b;  // the empty proof is the identity
+  else if (live && (rb == 0 || ra == rb)) out = a;
+  bool work = live && !out;
+  if (!work) la = 0;
+  const u32 x = (rb - 1) >> 1, px = (u32)(b >> 32);
+  const u32 lmax = __reduce_max_sync(0xFFFFFFFFu, la);
+  u32 below = 0, id0[4];
+  bool has = false;
+#pragma unroll
+  for (int c = 0; c < 4; c++) {
+    const u32 i = 8 * c + l8;
+    id0[c] = i < la ? __ldcg(T.words + ra + 1 + i) : 0xFFFFFFFFu;
+    below += id0[c] < x;
+    has = has || (i < la && id0[c] == x);
+  }
+  for (u32 i = 32 + l8; i < lmax + l8; i += 8) {
+    const u32 id = i < la ? __ldcg(T.words + ra + 1 + i) : 0xFFFFFFFFu;
+    below += id < x;
+    has = has || (i < la && id == x);
+  }
+  has = (__ballot_sync(0xFFFFFFFFu, has) >> g0) & 0xFFu;
+#pragma unroll
+  for (int o = 4; o; o >>= 1) below += __shfl_xor_sync(0xFFFFFFFFu, below, o);
+  if (work && has) {
+    out = a;
+    work = false;
+  }
+  if (out && best != ~0u && (u32)(out >> 32) <= best) out = 0;
+  if (work && la + 1 > T.proof_cap) {
+    if (l8 == 0) atomicOr(T.err, 1u);
+    work = false;
+  }
+  if (work && top_loses((u32)(a >> 32), px, true, best)) work = false;
+  if (!__any_sync(0xFFFFFFFFu, work)) return out;
+  double p = 1.0;
+  const double fx = (double)__uint_as_float(px);
+  if (!work) la = 0;
+  const u32 pmax = __reduce_max_sync(0xFFFFFFFFu, la);
+  for (u32 i0 = 0; i0 < pmax; i0 += 8) {
+    const u32 i = i0 + l8;
+    u32 id = i0 < 32 ? id0[0] : 0u;
+    if (i0 == 8) id = id0[1];
+    if (i0 == 16) id = id0[2];
+    if (i0 == 24) id = id0[3];
+    if (i0 >= 32 && i < la) id = __ldcg(T.words + ra + 1 + i);
+    const float pr = i < la ? __ldg(T.prob + id) : 1.0f;
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      const float q = __shfl_sync(0xFFFFFFFFu, pr, g0 + j);
+      if (i0 + j == below) p *= fx;
+      if (i0 + j < la) p *= (double)q;
+    }
+  }
+  if (below >= ((pmax + 7) & ~7u)) p *= fx;
+  const u32 bits = __float_as_uint((float)p);
+  if (best != ~0u && bits <= best) work = false;
+  unsigned long long at = 0;
+  const u32 need = la + 2;
+  if (work && l8 == 0) at = atomicAdd(T.tail, (unsigned long long)need);
+  at = __shfl_sync(0xFFFFFFFFu, at, g0);
+  if (work && at + need > T.cap) {
+    if (l8 == 0) atomicCAS(full, 0ull, (unsigned long long)step + 1);
+    work = false;
+  }
+  if (!work) return out;
+  u32* w = T.words + at;
+  if (l8 == 0) {
+    w[0] = la + 1;
+    w[1 + below] = x;
+  }
+#pragma unroll
+  for (int c = 0; c < 4; c++)
+    if (8 * c + l8 < la) w[1 + 8 * c + l8 + (id0[c] > x)] = id0[c];
+  for (u32 i = 32 + l8; i < la; i += 8) {
+    const u32 id = __ldcg(T.words + ra + 1 + i);
+    w[1 + i + (id > x)] = id;
+  }
+  return ((u64)bits << 32) | at;
+}
+
 template <class Sem, bool kSh>
 __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(const __grid_constant__ LinArgs A) {
   constexpr int kT = kSh ? kLinShThreads : kLinThreads;
   typedef typename Sem::Stored S;
   typedef typename Sem::Cand C;
+  constexpr bool kTop1 = std::is_same<Sem, SemTop1>::value;
   __shared__ LinArm arms[kLinMaxArms];
   __shared__ u32 fresh_sh[2][kLinMaxRels];  // new, improved
   __shared__ unsigned long long cand_sh;
@@ -268,6 +380,8 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
       if (!expand) continue;
       const u64 wi = in ? (u64)slot - A.base[rel] : 0ull;
       const C ct = Sem::from_stored(tag);
+      u32 plen = 0;  // top-1-proofs: the length of the fact's proof
+      if constexpr (kTop1) plen = fresh ? __ldcg(A.top1.words + (u32)tag) : 0u;
       for (int a = 0; a < A.n_arm; a++) {
         const LinArm& arm = arms[a];
         const PStep& P = arm.P;
@@ -293,7 +407,49 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
           const C tr = __shfl_sync(0xFFFFFFFFu, ct, src);
           bool add = false;
           u32 hs = 0;
-          if (t < tot) {
+          if constexpr (kTop1) {
+            u64 edge = 0;
+            u32 best = ~0u;
+            bool want = false;
+            const u32 len = __shfl_sync(0xFFFFFFFFu, plen, src);
+            if (t < tot) {
+              const u64 v = (u64)lr + (t - er);
+              const u64 wv = lin_word(P.v_keys, P.v_key64, v);
+              if (lin_checks(P.checks, P.n_checks, wr, wv)) {
+                u64 w = 0;
+                for (int q = 0; q < P.n_out; q++) w |= lin_pick(P.out[q].op, wr, wv) << P.out[q].shift;
+                hs = hbase + (u32)w;
+                edge = reinterpret_cast<const S*>(P.v_tags)[v];
+                // the likelier of the stored proof and the candidate there already
+                const u64 c = lin_ld(X.acc[par ^ 1] + hs);
+                if (c) best = (u32)(c >> 32);
+                if (lin_ld(X.fbits + (hs >> 5)) & (1u << (hs & 31u))) {
+                  const u32 f = (u32)(lin_ld(X.ftag + hs) >> 32);
+                  best = best == ~0u ? f : max(best, f);
+                }
+                want = len >= A.top1.proof_cap || !top_loses((u32)(tr >> 32), (u32)(edge >> 32), false, best);
+              }
+            }
+            u64 made = 0;
+            for (u32 todo = __ballot_sync(0xFFFFFFFFu, want); todo;) {
+              u32 m = todo;
+              for (int q = 0; q < (lane >> 3); q++) m &= m - 1;
+              const int of = m ? __ffs(m) - 1 : 0;
+              const u64 ta = __shfl_sync(0xFFFFFFFFu, (u64)tr, of), te = __shfl_sync(0xFFFFFFFFu, edge, of);
+              const u32 tb = __shfl_sync(0xFFFFFFFFu, best, of);
+              const u64 u = top_union(A.top1, m != 0, ta, te, tb, ast + LS_FULLARENA, step);
+              const int mine = __popc(todo & ((1u << lane) - 1u));
+              const u64 back = __shfl_sync(0xFFFFFFFFu, u, (mine & 3) * 8);
+              if (((todo >> lane) & 1u) && mine < 4) made = back;
+              for (int q = 0; q < 4; q++) todo &= todo - 1;
+            }
+            if (made) {
+              dense_add<Sem>(X.acc[par ^ 1], hs, made);
+              const u32 bit = 1u << (hs & 31u);
+              u32* tw = X.touched[par ^ 1] + (hs >> 5);
+              if (!(lin_ld(tw) & bit)) add = !(atomicOr(tw, bit) & bit);
+            }
+          } else if (t < tot) {
             const u64 v = (u64)lr + (t - er);
             const u64 wv = lin_word(P.v_keys, P.v_key64, v);
             if (lin_checks(P.checks, P.n_checks, wr, wv)) {
@@ -337,6 +493,13 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
       else st[LS_FRESH + ((step + 1) % 3) * kLinMaxRels + threadIdx.x] = 0;
     }
     if (!lin_barrier(st, gen)) break;
+    if constexpr (kTop1) {  // a faster block's next step may have found it full already
+      const u64 f = lin_ld(st + LS_FULLARENA);
+      if (f && f <= step + 1) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) st[LS_STOP] = LIN_ARENA;
+        break;
+      }
+    }
     if (!commit) continue;
     u64 total = 0;
 #pragma unroll
@@ -594,7 +757,9 @@ struct LinRun {
 bool linear_component(const lob_engine& e, std::vector<char>& in) {
   const size_t n = e.rels.size();
   in.assign(n, 0);
-  if (e.semiring == SR_UNIT || sem_top1(e.semiring) || e.n_strata != 1) return false;
+  if (e.semiring == SR_UNIT || e.n_strata != 1) return false;
+  // top-1-proofs runs keep no dense accumulators outside this loop
+  const bool top1 = sem_top1(e.semiring);
   std::vector<int> comp(n);
   for (size_t r = 0; r < n; r++) comp[r] = (int)r;
   std::vector<char> bad(n, 0);
@@ -610,7 +775,8 @@ bool linear_component(const lob_engine& e, std::vector<char>& in) {
   for (size_t r = 0; r < n; r++) {
     const RelSt& R = e.rels[r];
     if (!R.idb) continue;
-    if (!R.dense || lin_slots(e, R) > kLinRelSlots || (sem_stamps(e.semiring) && R.views.size() > 1)) bad[comp[r]] = 1;
+    const bool dense = top1 ? e.opt_acc_dense && R.views[0].lay.bits <= e.opt_acc_bits : R.dense;
+    if (!dense || lin_slots(e, R) > kLinRelSlots || (sem_stamps(e.semiring) && R.views.size() > 1)) bad[comp[r]] = 1;
   }
   for (auto& p : e.plans) {
     int derived = 0;
@@ -621,7 +787,7 @@ bool linear_component(const lob_engine& e, std::vector<char>& in) {
     for (auto& A : p.arms)
       if (e.rels[p.ast.body[A.delta].rel].idb) {
         n_arms[c]++;
-        if (!A.packed.ok || A.steps.size() != 2) bad[c] = 1;
+        if (!(top1 ? A.packed.linear_only : A.packed.ok) || A.steps.size() != 2) bad[c] = 1;
       }
   }
   bool any = false;
@@ -698,22 +864,18 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
     }
   const int ks = sem_kernel(e.semiring);
   const int sb = stored_bytes(e.semiring), cb = cand_bytes(e.semiring);
-  const bool stamps = sem_stamps(e.semiring);
+  const bool stamps = sem_stamps(e.semiring), top1 = sem_top1(e.semiring);
   e.ensure(L.arms, std::max<size_t>(arms.size(), 1) * sizeof(LinArm));
   if (!arms.empty())
     e.check(cudaMemcpyAsync(L.arms.p, arms.data(), arms.size() * sizeof(LinArm), cudaMemcpyHostToDevice, e.stream), "arms");
   for (int b = 0; b < 2; b++) {
     e.ensure(L.acc[b], slots * cb);
-    e.check(cudaMemsetAsync(L.acc[b].p, 0, slots * cb, e.stream), "accumulators");
     e.ensure(L.touched[b], slots / 8);
-    e.check(cudaMemsetAsync(L.touched[b].p, 0, slots / 8, e.stream), "accumulators");
     e.ensure(L.list[b], slots * 4);
   }
   e.ensure(L.ftag, slots * sb);
-  e.check(cudaMemsetAsync(L.ftag.p, 0, slots * sb, e.stream), "tags");
   if (stamps) e.ensure(L.fstamp, slots * 4);
   e.ensure(L.fbits, slots / 8);
-  e.check(cudaMemsetAsync(L.fbits.p, 0, slots / 8, e.stream), "membership");
   e.ensure(L.start, recent * 4);
   e.ensure(L.state, kLinSlots * 8);
   // an add-mult iteration that is not the last adds a fact, so there are at most
@@ -721,9 +883,7 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   if (stamps) e.ensure(L.rec, (slots + 1) * A.n_rel * 4);
   u64 at = 0;
   for (int q = 0; q < A.n_rel; q++) {
-    RelSt& R = e.rels[L.rels[q]];
-    if (sb == 8) L.init<u64>(R, A.base[q]);
-    else L.init<float>(R, A.base[q]);
+    const RelSt& R = e.rels[L.rels[q]];
     if (R.n_recent) {
       k_lin_slots<<<lin_grid(R.n_recent), 256, 0, e.stream>>>(R.rkeys.p, R.views[0].lay.key64, R.n_recent, A.base[q],
                                                               L.start.as<u32>() + at);
@@ -749,17 +909,34 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   A.rec = L.rec.as<u32>();
   // A block per 16,384 probed rows: a grid of side 64 has about 200 recent facts
   // in an iteration, which one block expands in a round or two without a grid
-  // barrier.
-  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(e.sms, probed / 16384));
+  // barrier.  Unions of proofs are worth more blocks: the loop over 64 grids of
+  // side 16 (65,000 rows) takes 1.61 / 1.19 / 0.98 / 0.90 / 0.87 ms with a block
+  // per 4,096 / 2,048 / 1,024 / 512 / 256 rows.
+  const u64 share = top1 ? 512 : 16384;
+  const unsigned blocks = (unsigned)std::max<u64>(1, std::min<u64>(e.sms, probed / share));
   A.k0 = k0;
   A.slots = (u32)slots;
   std::vector<u64> h(kLinSlots, 0);
-  e.check(cudaMemsetAsync(L.state.p, 0, kLinSlots * 8, e.stream), "linear state");
-  switch (ks) {
-    case SR_MAX_MIN: L.launch<SemMaxMin>(A, blocks); break;
-    case SR_DIFF_MAX_MIN: L.launch<SemDiffMaxMin>(A, blocks); break;
-    default: L.launch<SemAddMult>(A, blocks); break;
-  }
+  do {  // again when the proof arena ran out: the loop changes only arrays of its own
+    for (int b = 0; b < 2; b++) {
+      e.check(cudaMemsetAsync(L.acc[b].p, 0, slots * cb, e.stream), "accumulators");
+      e.check(cudaMemsetAsync(L.touched[b].p, 0, slots / 8, e.stream), "accumulators");
+    }
+    e.check(cudaMemsetAsync(L.ftag.p, 0, slots * sb, e.stream), "tags");
+    e.check(cudaMemsetAsync(L.fbits.p, 0, slots / 8, e.stream), "membership");
+    e.check(cudaMemsetAsync(L.state.p, 0, kLinSlots * 8, e.stream), "linear state");
+    for (int q = 0; q < A.n_rel; q++) {
+      if (sb == 8) L.init<u64>(e.rels[L.rels[q]], A.base[q]);
+      else L.init<float>(e.rels[L.rels[q]], A.base[q]);
+    }
+    if (top1) A.top1 = top1_desc(e);
+    switch (ks) {
+      case SR_MAX_MIN: L.launch<SemMaxMin>(A, blocks); break;
+      case SR_DIFF_MAX_MIN: L.launch<SemDiffMaxMin>(A, blocks); break;
+      case SR_TOP1: L.launch<SemTop1>(A, blocks); break;
+      default: L.launch<SemAddMult>(A, blocks); break;
+    }
+  } while (top1 && !top1_settle(e));
   e.check(cudaMemcpyAsync(h.data(), L.state.p, kLinSlots * 8, cudaMemcpyDeviceToHost, e.stream), "linear state");
   e.sync();
   if (h[LS_ERR]) throw LobError(LOB_E_TIMEOUT, "a bounded wait of the linear loop gave up; the run's results are invalid");

@@ -28,6 +28,12 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out);
 // engine's per-iteration record.
 void linear_merge(lob_engine& e, u32 k, const LinearOut& out);
 
+// top-1-proofs: the run's proof arena, and what follows kernels that append to it
+// (engine.cu)
+struct Top1Arena;
+Top1Arena top1_desc(lob_engine& e);
+bool top1_settle(lob_engine& e);
+
 // diff-add-mult backward of the linear components' iterations after the first.
 // Device pointers by relation id: adjoints and dense key -> row maps (null: none),
 // and per view its rows' primary rows.  Flags the components' relations; false

@@ -92,3 +92,53 @@ def test_several_blocks_and_a_hub(semiring):
     p = (s.prob(len(src)) * 0.2).astype(np.float32)
     inputs = {"edge": ((src, dst), p), "start": ((np.array([7, 11], np.uint32),),)}
     both(W.REACH_PROGRAM, inputs, semiring, ["reach"], "edge" if semiring.startswith("diff") else None)
+
+
+def _proofs(program, inputs, rels, options):
+    e, st, got = engine_run(program, inputs, "diff_top1_proofs", options=options, read=rels)
+    out = [(got[r].cols, got[r].samples, got[r].tags, [list(p) for p in e.proofs(r)]) for r in rels]
+    e.close()
+    return st, out
+
+
+@pytest.mark.parametrize("program,rels", [(W.REACH_PROGRAM, ["reach"]), (TURNS, ["a", "b"]), (W.TC_PROGRAM, ["path"])])
+@pytest.mark.parametrize("n,m,words,lo,hi", [(6, 9, 1 << 22, 0.0, 1.0), (40, 150, 1 << 22, 0.0, 1.0), (40, 150, 64, 0.5, 1.0),
+                                             (300, 7000, 1 << 22, 0.9, 1.0), (64, 63, 1 << 22, 0.9, 1.0),
+                                             (64, 63, 256, 0.0, 0.01), (12, 30, 1 << 22, 1.0, 1.3)])
+def test_proofs_of_linear_components(program, rels, n, m, words, lo, hi):
+    """The likeliest proof of every fact (driver 2) against the general steps
+    (driver 0): tags bit for bit, the same proofs, iterations and candidates.
+    m = n - 1: a chain, proofs of up to 63 facts; a small arena runs out and the
+    loop runs again; tags that underflow, tags of 0, probabilities above 1."""
+    s = W.stream(810 + n)
+    src, dst = (np.arange(m, dtype=np.uint32), np.arange(1, m + 1, dtype=np.uint32)) if m == n - 1 else (s.below(m, n), s.below(m, n))
+    p = (lo + (hi - lo) * s.prob(m)).astype(np.float32)
+    if lo == 0.0:
+        p[::7] = 0.0
+    inputs = {"edge": ((src, dst), p), "start": ((np.array([0, 3], np.uint32),), np.array([0.5, 0.75], np.float32))}
+    if program is W.TC_PROGRAM:
+        inputs.pop("start")
+        if m > 1000:
+            return
+    (a, ga), (b, gb) = (_proofs(program, inputs, rels, {"driver": d, "proof_arena_words": words}) for d in (2, 0))
+    assert a["device_iterations"] > 0 and b["device_iterations"] == 0
+    for k in ("iterations", "derived", "candidates", "new_facts"):
+        assert a[k] == b[k], (k, a[k], b[k])
+    for x, y in zip(ga, gb):
+        assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
+        assert np.array_equal(x[2].view(np.uint32), y[2].view(np.uint32))
+        likely = x[2] > 0.0  # proofs of probability 0 tie; the others have distinct probabilities
+        assert [q for q, t in zip(x[3], likely) if t] == [q for q, t in zip(y[3], likely) if t]
+
+
+@pytest.mark.parametrize("driver", [0, 2])
+def test_proof_cap_in_the_linear_loop(driver):
+    """A chain of nine facts below 0.5: a cap of seven is an error, of eight is not."""
+    from paper_2503_21937_gb300 import LobsterError
+    a, b = W.ktree_chain(9)
+    inputs = {"edge": ((a, b), np.full(8, 0.5, np.float32)), "start": ((np.array([0], np.uint32),),)}
+    with pytest.raises(LobsterError) as ei:
+        engine_run(W.REACH_PROGRAM, inputs, "top1_proofs", options={"driver": driver, "proof_cap": 7})
+    assert ei.value.code == -9
+    _, st, got = engine_run(W.REACH_PROGRAM, inputs, "top1_proofs", options={"driver": driver, "proof_cap": 8})
+    assert got["reach"].tags.tolist() == [0.5 ** k for k in range(9)]
