@@ -1114,69 +1114,171 @@ __global__ void __launch_bounds__(256) k_pmasked(const __grid_constant__ PStep P
 }
 
 // max-min semirings: a fact that is present still takes candidates with a larger
-// tag, so every match's product is formed -- but against the stored tags of the
-// head row, and only what beats them goes on.  A warp takes an input row at a
-// time, a lane a column, so the two tag rows are read as consecutive words (two
-// rows at once, for loads in flight); the general step reads an accumulator slot
-// in L2 per match that nothing but this iteration has filled.  Bound by issue:
-// the batched kinship program forms 5.3e9 products in 350 million half rows, 5.7e8
-// of which beat the stored tag (54 -> 35 ms, and the read-out of the accumulator
-// 12 -> 4.5 ms, as it lists fewer heads).  Four half rows in flight from a list
-// of the non-empty ones took 39 ms: latency is not what it waits for.
+// tag, so every match's product is formed, but only the best one of a head can
+// matter, and only if it beats the stored tag.  A block takes a tile of input rows
+// and groups them by head row in shared memory (hash table, counting sort); a warp
+// takes up to 32 rows of one head row, a lane a column: a row then costs one load
+// of the matched tags, a minimum and a maximum in registers, and the head row's
+// tags, the comparison and the accumulator are reached once for all of them.  Bound
+// by the integer pipe: 64-bit minima and maxima, about 45 instructions an input
+// row of 28 matches.  The batched kinship program (5.3e9 products of 4e8 rows, 1.5e9
+// of them in one launch): a row at a time against the stored tags of its head took
+// 33 ms; grouped, tiles of 2,048 rows and two blocks an SM 27, of 4,096 and one 24.
+constexpr int kMTile = 4096, kMTable = 2 * kMTile, kMThreads2 = 1024, kMRows = kMTile / kMThreads2;
+template <class C>
+struct MaskedSmem {
+  struct alignas(16) Row { C t; u32 v; };
+  Row row[kMTile];
+  u64 ok[kMTile];
+  u32 h[kMTile], hk[kMTile];
+  u32 items[kMTile];                 // first row | rows << 16
+  u32 key[kMTable], cnt[kMTable];
+  u32 sums[kMThreads2 / 32 + 1];
+};
+// the order of accumulator slots (dense_add): f32 tags compare as integers there
+LOB_DEV float slot_lowest(float) { return __int_as_float((int)0x80000000); }
+LOB_DEV u64 slot_lowest(u64) { return 0; }
+LOB_DEV float slot_max(float a, float b) { return __int_as_float(max(__float_as_int(a), __float_as_int(b))); }
+LOB_DEV u64 slot_max(u64 a, u64 b) { return a > b ? a : b; }
+
+// best products of a run of rows, a lane the columns lane and (kHalves 2) lane + 32
+template <class Sem, int kHalves>
+LOB_DEV void masked_rows_best(const MaskedSmem<typename Sem::Cand>& X, const typename Sem::Stored* __restrict__ vt, u32 first,
+                              u32 len, typename Sem::Cand* best) {
+  typedef typename Sem::Cand C;
+  const int lane = threadIdx.x & 31;
+  const u32 bit = 1u << lane;
+  const typename Sem::Stored* base = vt + lane;
+  auto rows = [&](u32 p, auto n) {
+    constexpr int kN = decltype(n)::value;
+    C x[kN][kHalves], tr[kN];
+#pragma unroll
+    for (int j = 0; j < kN; j++) {
+      const u64 ok = X.ok[p + j];
+      const auto row = X.row[p + j];
+      tr[j] = row.t;
+#pragma unroll
+      for (int q = 0; q < kHalves; q++) {
+        x[j][q] = slot_lowest(C());  // no product is smaller
+        if ((q ? (u32)(ok >> 32) : (u32)ok) & bit) x[j][q] = Sem::from_stored(base[row.v + 32 * q]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kN; j++)
+#pragma unroll
+      for (int q = 0; q < kHalves; q++) best[q] = slot_max(best[q], Sem::mul(tr[j], x[j][q]));
+  };
+  u32 i = 0;
+  for (; i + 4 <= len; i += 4) rows(first + i, std::integral_constant<int, 4>());
+  for (; i < len; i++) rows(first + i, std::integral_constant<int, 1>());
+}
+
 template <class Sem>
-__global__ void __launch_bounds__(256) k_pmasked_rows(const __grid_constant__ PStep P, const __grid_constant__ PMask M,
-                                                      unsigned long long* emitted) {
+__global__ void __launch_bounds__(kMThreads2, 1) k_pmasked_rows(const __grid_constant__ PStep P,
+                                                                const __grid_constant__ PMask M,
+                                                                unsigned long long* emitted) {
   typedef typename Sem::Stored S;
   typedef typename Sem::Cand C;
-  struct Rec { u64 v, h, ok, hm, hk; C t; };
-  __shared__ Rec recs[8][32];
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MaskedSmem<C>& X = *reinterpret_cast<MaskedSmem<C>*>(smem_raw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const u64 nwarps = (u64)gridDim.x * (blockDim.x / 32);
   const u64 n_in = dev_size(P.n_in, P.n_in_dev);
   const PPtrs Q = resolve_ptrs(P);
   const S* vt = reinterpret_cast<const S*>(M.vtags);
   const S* ht = reinterpret_cast<const S*>(M.htags);
+  // tiles of equal size, as many as whole waves of the grid, of 256 rows at least
+  const u64 waves = (n_in + (u64)kMTile * gridDim.x - 1) / ((u64)kMTile * gridDim.x);
+  const u64 tile = waves ? max((u64)256, (n_in + waves * gridDim.x - 1) / (waves * gridDim.x)) : 256;
   u64 mine = 0;
-  for (u64 g = (u64)blockIdx.x * (blockDim.x / 32) + warp; g * 32 < n_in; g += nwarps) {
-    const u64 r = g * 32 + lane;
-    const MaskedRow x = masked_row(P, Q, M, r, n_in);
-    mine += __popcll(x.vm);
-    const u32 act = __ballot_sync(0xFFFFFFFFu, x.ok != 0);
-    const int n_act = __popc(act);
-    if (x.ok) {
-      const C t = P.in_packed ? Sem::from_stored(reinterpret_cast<const S*>(Q.in_tags)[r])
-                              : reinterpret_cast<const C*>(Q.in_tags)[r];
-      recs[warp][__popc(act & ((1u << lane) - 1u))] = Rec{x.pv << M.vw, x.h << M.hw, x.ok, x.hm, x.hk, t};
+  for (u64 t0 = blockIdx.x * tile; t0 < n_in; t0 += gridDim.x * tile) {
+    const u64 t1 = min(n_in, t0 + tile);
+    for (int i = threadIdx.x; i < kMTable; i += kMThreads2) {
+      X.key[i] = 0xFFFFFFFFu;
+      X.cnt[i] = 0;
     }
-    __syncwarp();
-    for (int i = 0; i < n_act; i += 2) {
-      const Rec y[2] = {recs[warp][i], recs[warp][min(i + 1, n_act - 1)]};
-      const bool two = i + 1 < n_act;
+    __syncthreads();
+    u64 ok[kMRows];
+    C tag[kMRows];
+    u32 v[kMRows], h[kMRows], hk[kMRows], at[kMRows];
 #pragma unroll
-      for (int base = 0; base < 64; base += 32) {
-        if (base && !((y[0].ok | y[1].ok) >> 32)) break;  // no column past 31
-        const int z = base + lane;
-        S tr[2], fh[2];
-        bool on[2], present[2];
+    for (int j = 0; j < kMRows; j++) {
+      const u64 r = t0 + j * kMThreads2 + threadIdx.x;
+      const MaskedRow x = masked_row(P, Q, M, r, t1);
+      mine += __popcll(x.vm);
+      ok[j] = x.ok;
+      if (!x.ok) continue;
+      tag[j] = P.in_packed ? Sem::from_stored(reinterpret_cast<const S*>(Q.in_tags)[r])
+                           : reinterpret_cast<const C*>(Q.in_tags)[r];
+      v[j] = (u32)(x.pv << M.vw);
+      h[j] = (u32)x.h;
+      hk[j] = (u32)x.hk;
+      u32 s = (h[j] * 0x9E3779B1u) >> 16 & (kMTable - 1);
+      for (;;) {  // twice as many slots as rows: an empty one is found
+        const u32 o = atomicCAS(&X.key[s], 0xFFFFFFFFu, h[j]);
+        if (o == 0xFFFFFFFFu || o == h[j]) break;
+        s = (s + 1) & (kMTable - 1);
+      }
+      at[j] = s | atomicAdd(&X.cnt[s], 1u) << 16;
+    }
+    __syncthreads();
+    // rows and items before each slot, packed in one word
+    constexpr int kPer = kMTable / kMThreads2;
+    u32 c[kPer], sum = 0;
 #pragma unroll
-        for (int j = 0; j < 2; j++) {
-          on[j] = (j == 0 || two) && ((y[j].ok >> z) & 1u);
-          present[j] = on[j] && ((y[j].hm >> z) & 1u);
-          if (on[j]) tr[j] = vt[y[j].v + z];
-          if (present[j]) fh[j] = ht[y[j].h + z];
-        }
+    for (int q = 0; q < kPer; q++) {
+      const u32 n = X.cnt[threadIdx.x * kPer + q];
+      c[q] = n;
+      sum += n | ((n + 31) >> 5) << 16;
+    }
+    const u32 inc = warp_inclusive_sum(sum);
+    if (lane == 31) X.sums[warp] = inc;
+    __syncthreads();
+    u32 before = inc - sum, n_items = 0;
+    for (int w = 0; w < kMThreads2 / 32; w++) {
+      const u32 x = X.sums[w];
+      if (w < warp) before += x;
+      n_items += x >> 16;
+    }
 #pragma unroll
-        for (int j = 0; j < 2; j++) {
-          if (!on[j]) continue;
-          const C c = Sem::mul(y[j].t, Sem::from_stored(tr[j]));
-          if (present[j] && fh[j] >= Sem::store(c)) continue;  // changes nothing
-          const u64 w = y[j].hk | ((u64)z << M.zshift);
-          dense_add<Sem>(P.acc, w, c);
-          touch_bit(P.bitmap, w);
-        }
+    for (int q = 0; q < kPer; q++) {
+      const u32 off = before & 0xFFFFu;
+      u32 it = before >> 16;
+      X.cnt[threadIdx.x * kPer + q] = off;
+      for (u32 d = 0; d < c[q]; d += 32) X.items[it++] = (off + d) | min(32u, c[q] - d) << 16;
+      before += c[q] | ((c[q] + 31) >> 5) << 16;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kMRows; j++) {
+      if (!ok[j]) continue;
+      const u32 p = X.cnt[at[j] & 0xFFFFu] + (at[j] >> 16);
+      X.ok[p] = ok[j];
+      X.row[p] = {tag[j], v[j]};
+      X.h[p] = h[j];
+      X.hk[p] = hk[j];
+    }
+    __syncthreads();
+    for (u32 it = warp; it < n_items; it += kMThreads2 / 32) {
+      const u32 first = X.items[it] & 0xFFFFu, len = X.items[it] >> 16;
+      const u64 hr = X.h[first];
+      const u64 key = X.hk[first];
+      const u64 hm = row_bits(M.hbits, hr, M.hw);
+      const u64 mok = lane < (int)len ? X.ok[first + lane] : 0ull;
+      const u32 any0 = __reduce_or_sync(0xFFFFFFFFu, (u32)mok), any1 = __reduce_or_sync(0xFFFFFFFFu, (u32)(mok >> 32));
+      C best[2] = {slot_lowest(C()), slot_lowest(C())};
+      if (any1) masked_rows_best<Sem, 2>(X, vt, first, len, best);
+      else masked_rows_best<Sem, 1>(X, vt, first, len, best);
+#pragma unroll
+      for (int half = 0; half < 2; half++) {
+        const int z = 32 * half + lane;
+        if (!(((half ? any1 : any0) >> lane) & 1u)) continue;
+        if (((hm >> z) & 1u) && ht[(hr << M.hw) + z] >= Sem::store(best[half])) continue;  // changes nothing
+        const u64 w = key | ((u64)z << M.zshift);
+        dense_add<Sem>(P.acc, w, best[half]);
+        touch_bit(P.bitmap, w);
       }
     }
-    __syncwarp();
+    __syncthreads();
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) mine += __shfl_xor_sync(0xFFFFFFFFu, mine, o);
@@ -1427,13 +1529,20 @@ bool pjoin_warp_supported(int sem, const PStep& P) {
   return sem == SR_UNIT && P.n_out >= 1 && P.n_out <= 4 && P.n_checks <= 1;
 }
 
+template <class Sem>
+static void launch_masked_rows(const PStep& P, const PMask& M, unsigned long long* em, cudaStream_t st) {
+  constexpr int kSm = (int)sizeof(MaskedSmem<typename Sem::Cand>);
+  allow_dynamic_smem(k_pmasked_rows<Sem>, kSm);
+  const unsigned g = (unsigned)std::max<u64>(1, std::min<u64>((P.n_in + 255) / 256, 152ull));
+  k_pmasked_rows<Sem><<<g, kMThreads2, kSm, st>>>(P, M, em);
+}
 void pjoin_masked(int sem, const PStep& P, const PMask& M, u64* emitted_dev, cudaStream_t st) {
   // an input row reads its word, two bitmap rows and, with outputs, its tag
   ProfScope ps("join_masked", P.n_in * (row_bytes(sem, P.in_w64, P.in_packed) + 16.0), st);
   if (!P.n_in) return;
   auto* em = reinterpret_cast<unsigned long long*>(emitted_dev);
-  if (sem == SR_MAX_MIN) k_pmasked_rows<SemMaxMin><<<grid_n(P.n_in), 256, 0, st>>>(P, M, em);
-  else if (sem == SR_DIFF_MAX_MIN) k_pmasked_rows<SemDiffMaxMin><<<grid_n(P.n_in), 256, 0, st>>>(P, M, em);
+  if (sem == SR_MAX_MIN) launch_masked_rows<SemMaxMin>(P, M, em, st);
+  else if (sem == SR_DIFF_MAX_MIN) launch_masked_rows<SemDiffMaxMin>(P, M, em, st);
   else k_pmasked<SemAddMult><<<grid_n(P.n_in), 256, 0, st>>>(P, M, em);
 }
 void pjoin_backward_masked(const PStep& P, const PBwd& B, const PMask& M, cudaStream_t st) {

@@ -63,3 +63,27 @@ def test_same_as_the_general_kernels(program, semiring):
         assert np.array_equal(r.cols, ra.cols) and np.array_equal(r.samples, ra.samples)
         np.testing.assert_allclose(r.tags, ra.tags, rtol=3e-7 if "add" in semiring else 0, atol=0)
         np.testing.assert_allclose(g, ga, rtol=1e-4, atol=1e-5 * max(1.0, float(np.abs(ga).max())))
+
+
+@pytest.mark.parametrize("semiring", ["max_min", "diff_max_min"])
+@pytest.mark.parametrize("rows", [1, 33, 255, 257, 152 * 256 + 1, 152 * 4096 - 1, 152 * 4096 + 41])
+def test_rows_grouped_by_head(rows, semiring):
+    """Input rows just past the smallest tiles, one wave of full tiles and two
+    waves; heads of 64 rows (two items) and of one."""
+    s = W.stream(960)
+    i = np.arange(rows, dtype=np.uint32)
+    a = (i // 64, i % 64)
+    if rows > 64:
+        a[0][-3:], a[1][-3:] = rows + np.arange(3), 5  # heads of a single row
+    b = (s.below(700, 64), s.below(700, 50))
+    inputs = {"a": (a, s.prob(rows)), "b": (b, s.prob(700))}
+    text = "q(x,z) :- a(x,y), b(y,z), y != z.\n"
+    got = []
+    for opts in ({"packed_join": 0}, {}):
+        e, st, g = engine_run(text, inputs, semiring, options=opts, read=["q"])
+        e.close()
+        got.append((st, g["q"]))
+    (x, p), (y, q) = got
+    for k in ("iterations", "derived", "candidates", "new_facts"):
+        assert x[k] == y[k], (k, x[k], y[k])
+    assert np.array_equal(p.cols, q.cols) and np.array_equal(p.tags, q.tags)
