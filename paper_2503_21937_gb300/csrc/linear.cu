@@ -26,9 +26,12 @@
 // step's facts are spread over all warps before a warp takes a second one.
 //
 // Measured (GB300): 64 x 64 grid, diff-add-mult, fixpoint of 128 iterations 8.6
-// -> 1.0 ms; diff-max-min, forward and backward 11.1 -> 1.8 ms; top-1-proofs over 64
-// grids of side 16, forward and backward 9.1 -> 2.0 ms.  A step takes 5
-// us (15 with the arrays in L2), an iteration of the graph of kernels 67.
+// -> 0.76 ms; diff-max-min, forward and backward 13.5 -> 1.7 ms; top-1-proofs over 64
+// grids of side 16, forward and backward 9.1 -> 2.0 ms.  A step takes 4 us (12 with the
+// arrays in L2), an iteration of the graph of kernels 67.  In shared memory a step
+// has one barrier, the arrays of either parity are one array (an indexed pair of
+// pointers would be generic ones: a step took 5.1 us), new facts are counted per
+// warp, and a match's key and tag are loaded together.
 #include "linear.h"
 
 #include <algorithm>
@@ -68,9 +71,10 @@ struct LinArgs {
   u32 slots;
   u32 base[kLinMaxRels];   // a relation's first slot
   const LinArm* arms;
-  void* acc[2];            // candidate tags by slot, all zero between uses
-  u32* touched[2];         // slots listed already
-  u32* list[2];
+  // of either parity, one after the other:
+  void* acc;               // candidate tags by slot, all zero between uses
+  u32* touched;            // slots listed already
+  u32* list;
   void* ftag;
   u32* fstamp;             // add-mult: iteration of first appearance | clamped << 31
   u32* fbits;              // membership
@@ -129,23 +133,25 @@ LOB_DEV u32 lin_probe(const PStep& P, u64 wi, u32& lo) {
 }
 
 // All blocks of the launch, or false when one of them gave up waiting.  The
-// count only grows, so a late block can never see it reset.
+// count only grows, so a late block can never see it reset.  Thread 0's own writes
+// before the call, and its warp's before a __syncwarp, are among those ordered.
+LOB_DEV bool lin_barrier_warp0(u64* state, u32& gen) {
+  volatile u64* s = state;
+  __threadfence();
+  gen++;
+  atomicAdd(reinterpret_cast<unsigned long long*>(state) + LS_BAR, 1ull);
+  const u64 want = (u64)gen * gridDim.x;
+  u32 n = 0;
+  while (s[LS_BAR] < want && !s[LS_ERR] && n < kLinSpin) n++;
+  if (s[LS_BAR] < want) s[LS_ERR] = 1;
+  __threadfence();
+  return s[LS_ERR] == 0;
+}
 LOB_DEV bool lin_barrier(u64* state, u32& gen) {
   __shared__ u32 ok;
   __syncthreads();
   if (gridDim.x == 1) return true;
-  if (threadIdx.x == 0) {
-    volatile u64* s = state;
-    __threadfence();
-    gen++;
-    atomicAdd(reinterpret_cast<unsigned long long*>(state) + LS_BAR, 1ull);
-    const u64 want = (u64)gen * gridDim.x;
-    u32 n = 0;
-    while (s[LS_BAR] < want && !s[LS_ERR] && n < kLinSpin) n++;
-    if (s[LS_BAR] < want) s[LS_ERR] = 1;
-    __threadfence();
-    ok = s[LS_ERR] == 0;
-  }
+  if (threadIdx.x == 0) ok = lin_barrier_warp0(state, gen);
   __syncthreads();
   return ok != 0;
 }
@@ -155,8 +161,8 @@ template <class T> LOB_DEV T lin_ld(const T* p) { return *reinterpret_cast<const
 // the loop's arrays, in global or shared memory
 template <class Sem>
 struct LinArrays {
-  typename Sem::Cand* acc[2];
-  u32 *touched[2], *list[2];
+  typename Sem::Cand* acc;
+  u32 *touched, *list;
   typename Sem::Stored* ftag;
   u32 *fstamp, *fbits;
   u64* state;
@@ -281,7 +287,8 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
   typedef typename Sem::Cand C;
   constexpr bool kTop1 = std::is_same<Sem, SemTop1>::value;
   __shared__ LinArm arms[kLinMaxArms];
-  __shared__ u32 fresh_sh[2][kLinMaxRels];  // new, improved
+  __shared__ u32 fresh_sh[2][2][kLinMaxRels];  // by parity: new, improved (several blocks)
+  __shared__ u32 go;
   __shared__ unsigned long long cand_sh;
   LinArrays<Sem> X;
   if constexpr (kSh) {
@@ -289,28 +296,26 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
     unsigned char* q = sh;
     const u32 n = A.slots;
     X.state = reinterpret_cast<u64*>(q); q += kLinSlots * 8;
-    for (int b = 0; b < 2; b++) { X.acc[b] = reinterpret_cast<C*>(q); q += (u64)n * sizeof(C); }
+    X.acc = reinterpret_cast<C*>(q); q += 2 * (u64)n * sizeof(C);
     X.ftag = reinterpret_cast<S*>(q); q += (u64)n * sizeof(S);
     X.fstamp = reinterpret_cast<u32*>(q); q += (u64)n * 4;
-    for (int b = 0; b < 2; b++) { X.list[b] = reinterpret_cast<u32*>(q); q += (u64)n * 4; }
-    for (int b = 0; b < 2; b++) { X.touched[b] = reinterpret_cast<u32*>(q); q += n / 8; }
+    X.list = reinterpret_cast<u32*>(q); q += 2 * (u64)n * 4;
+    X.touched = reinterpret_cast<u32*>(q); q += 2 * (n / 8);
     X.fbits = reinterpret_cast<u32*>(q);
     for (u32 i = threadIdx.x; i < n; i += kT) {
-      X.acc[0][i] = X.acc[1][i] = C(0);
+      X.acc[i] = X.acc[n + i] = C(0);
       X.ftag[i] = reinterpret_cast<const S*>(A.ftag)[i];
       X.fstamp[i] = A.fstamp ? A.fstamp[i] : 0u;
     }
     for (u32 i = threadIdx.x; i < n / 32; i += kT) {
-      X.touched[0][i] = X.touched[1][i] = 0u;
+      X.touched[i] = X.touched[n / 32 + i] = 0u;
       X.fbits[i] = A.fbits[i];
     }
     for (u32 i = threadIdx.x; i < (u32)kLinSlots; i += kT) X.state[i] = 0;
   } else {
-    for (int b = 0; b < 2; b++) {
-      X.acc[b] = reinterpret_cast<C*>(A.acc[b]);
-      X.touched[b] = A.touched[b];
-      X.list[b] = A.list[b];
-    }
+    X.acc = reinterpret_cast<C*>(A.acc);
+    X.touched = A.touched;
+    X.list = A.list;
     X.ftag = reinterpret_cast<S*>(A.ftag);
     X.fstamp = A.fstamp;
     X.fbits = A.fbits;
@@ -319,58 +324,76 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
   for (u32 i = threadIdx.x; i < A.n_arm * sizeof(LinArm) / 4; i += kT)
     reinterpret_cast<u32*>(arms)[i] = reinterpret_cast<const u32*>(A.arms)[i];
   if (threadIdx.x == 0) cand_sh = 0;
+  if (threadIdx.x < 4 * kLinMaxRels) (&fresh_sh[0][0][0])[threadIdx.x] = 0;
+  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const u64 warp = (u64)blockIdx.x * (kT / 32) + (threadIdx.x >> 5), nwarps = (u64)gridDim.x * (kT / 32);
+  const u32 warp = blockIdx.x * (kT / 32) + (threadIdx.x >> 5), nwarps = gridDim.x * (kT / 32);
   u64* st = X.state;
   unsigned long long* ast = reinterpret_cast<unsigned long long*>(st);
+  // the last warp, least likely to hold facts, keeps the counters
+  const bool keeper = blockIdx.x == 0 && (threadIdx.x >> 5) == kT / 32 - 1;
   u32 gen = 0;
-  u64 cand = 0;
+  u64 cand = 0, new_facts = 0;
   u64 fcount[kLinMaxRels];
 #pragma unroll
   for (int r = 0; r < kLinMaxRels; r++) fcount[r] = r < A.n_rel ? A.fcount[r] : 0;
   // step 0 expands the facts recent after iteration k0; step j > 0 commits the
   // candidates of iteration k0 + j and expands what is new
-  for (u32 step = 0;; step++) {
+  u32 rot = 0, rot1 = 1, rot2 = 2;  // step, step + 1, step + 2 mod 3
+  for (u32 step = 0;; step++, rot = rot1, rot1 = rot2, rot2 = rot == 0 ? 2 : rot - 1) {
     const u32 k = A.k0 + step;
-    const int par = step & 1, rot = step % 3;
+    const int par = step & 1;
     const bool commit = step > 0;
-    if (threadIdx.x < 2 * kLinMaxRels) (&fresh_sh[0][0])[threadIdx.x] = 0;
-    __syncthreads();
-    const u32* list = commit ? X.list[par] : A.start;
-    const u64 n = commit ? lin_ld(st + LS_LIST + rot) : A.n_start;
-    u32* out_list = X.list[par ^ 1];
+    // this step's arrays, and those of the next
+    C *acc = X.acc + (par ? A.slots : 0u), *next_acc = X.acc + (par ? 0u : A.slots);
+    u32 *touched = X.touched + (par ? A.slots / 32 : 0u), *next_touched = X.touched + (par ? 0u : A.slots / 32);
+    const u32* list = X.list + (par ? A.slots : 0u);
+    u32* out_list = X.list + (par ? 0u : A.slots);
+    const u32 n = commit ? (u32)lin_ld(st + LS_LIST + rot) : (u32)A.n_start;
+    // Counters of steps to come.  The list length read in the last step is done
+    // with; the new-fact counts of the last step may still be read by a slow
+    // warp, those of the step before may not.
+    if (keeper && lane <= kLinMaxRels) {
+      if (lane == kLinMaxRels) st[LS_LIST + rot2] = 0;
+      else st[LS_FRESH + rot1 * kLinMaxRels + lane] = 0;
+    }
+    u32 n_fresh = 0, n_better = 0;  // one relation: this warp's new and improved facts
     const bool expand = k < A.max_iters;
-    const u64 per = min(32ull, (n + nwarps - 1) / nwarps);  // facts a warp takes at a time
-    for (u64 i0 = warp * per; i0 < n; i0 += nwarps * per) {
+    const u32 per = min(32u, (n + nwarps - 1) / nwarps);  // facts a warp takes at a time
+    for (u32 i0 = warp * per; i0 < n; i0 += nwarps * per) {
       const bool in = lane < (int)per && i0 + lane < n;
       u32 slot = 0;
       int rel = -1;
       S tag{};
       bool fresh = false;
       if (in) {
-        slot = commit ? lin_ld(list + i0 + lane) : list[i0 + lane];
+        slot = commit ? lin_ld(list + i0 + lane) : A.start[i0 + lane];
         rel = 0;
         while (rel + 1 < A.n_rel && slot >= A.base[rel + 1]) rel++;
         S* f = X.ftag + slot;
         if (commit) {
-          C* a = X.acc[par] + slot;
-          const C c = lin_ld(a);
-          *reinterpret_cast<volatile C*>(a) = C(0);
+          C* a = acc + slot;
           const u32 bit = 1u << (slot & 31u);
-          atomicAnd(X.touched[par] + (slot >> 5), ~bit);
-          tag = Sem::store(c);
+          const C c = lin_ld(a);
           const bool present = lin_ld(X.fbits + (slot >> 5)) & bit;
+          S old{};
+          if constexpr (Sem::kIdempotent) old = lin_ld(f);  // not written yet: 0
+          *reinterpret_cast<volatile C*>(a) = C(0);
+          atomicAnd(touched + (slot >> 5), ~bit);
+          tag = Sem::store(c);
           if (!present) {
             fresh = true;
             if constexpr (std::is_same<Sem, SemAddMult>::value)
               *reinterpret_cast<volatile u32*>(X.fstamp + slot) = k | (c > 1.0 ? 0x80000000u : 0u);
             *reinterpret_cast<volatile S*>(f) = tag;
             atomicOr(X.fbits + (slot >> 5), bit);
-            atomicAdd(&fresh_sh[0][rel], 1u);
-          } else if (Sem::kIdempotent && Sem::better(tag, lin_ld(f))) {
+            if (A.n_rel == 1) n_fresh++;
+            else atomicAdd(kSh ? reinterpret_cast<u32*>(st + LS_FRESH + rot * kLinMaxRels + rel) : &fresh_sh[par][0][rel], 1u);
+          } else if (Sem::kIdempotent && Sem::better(tag, old)) {
             fresh = true;
             *reinterpret_cast<volatile S*>(f) = tag;
-            atomicAdd(&fresh_sh[1][rel], 1u);
+            if (A.n_rel == 1) n_better++;
+            else atomicAdd(kSh ? reinterpret_cast<u32*>(st + LS_FRESH + rot * kLinMaxRels + rel) + 1 : &fresh_sh[par][1][rel], 1u);
           }
         } else {
           tag = lin_ld(f);
@@ -415,13 +438,13 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
             if (t < tot) {
               const u64 v = (u64)lr + (t - er);
               const u64 wv = lin_word(P.v_keys, P.v_key64, v);
+              edge = reinterpret_cast<const S*>(P.v_tags)[v];
               if (lin_checks(P.checks, P.n_checks, wr, wv)) {
                 u64 w = 0;
                 for (int q = 0; q < P.n_out; q++) w |= lin_pick(P.out[q].op, wr, wv) << P.out[q].shift;
                 hs = hbase + (u32)w;
-                edge = reinterpret_cast<const S*>(P.v_tags)[v];
                 // the likelier of the stored proof and the candidate there already
-                const u64 c = lin_ld(X.acc[par ^ 1] + hs);
+                const u64 c = lin_ld(next_acc + hs);
                 if (c) best = (u32)(c >> 32);
                 if (lin_ld(X.fbits + (hs >> 5)) & (1u << (hs & 31u))) {
                   const u32 f = (u32)(lin_ld(X.ftag + hs) >> 32);
@@ -444,20 +467,21 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
               for (int q = 0; q < 4; q++) todo &= todo - 1;
             }
             if (made) {
-              dense_add<Sem>(X.acc[par ^ 1], hs, made);
+              dense_add<Sem>(next_acc, hs, made);
               const u32 bit = 1u << (hs & 31u);
-              u32* tw = X.touched[par ^ 1] + (hs >> 5);
+              u32* tw = next_touched + (hs >> 5);
               if (!(lin_ld(tw) & bit)) add = !(atomicOr(tw, bit) & bit);
             }
           } else if (t < tot) {
             const u64 v = (u64)lr + (t - er);
             const u64 wv = lin_word(P.v_keys, P.v_key64, v);
+            const S vtag = reinterpret_cast<const S*>(P.v_tags)[v];  // both loads in flight at once
             if (lin_checks(P.checks, P.n_checks, wr, wv)) {
               u64 w = 0;
               for (int q = 0; q < P.n_out; q++) w |= lin_pick(P.out[q].op, wr, wv) << P.out[q].shift;
               hs = hbase + (u32)w;
               const u32 bit = 1u << (hs & 31u);
-              const C prod = Sem::mul(tr, Sem::from_stored(reinterpret_cast<const S*>(P.v_tags)[v]));
+              const C prod = Sem::mul(tr, Sem::from_stored(vtag));
               // A candidate that cannot change the stored tag is dropped here: a
               // fact that is present stays present, and a tag only grows.  Facts
               // being committed in this step may be seen or not (a tag not yet
@@ -465,8 +489,8 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
               bool useless = lin_ld(X.fbits + (hs >> 5)) & bit;
               if constexpr (Sem::kIdempotent) useless = useless && lin_ld(X.ftag + hs) >= Sem::store(prod);
               if (!useless) {
-                dense_add<Sem>(X.acc[par ^ 1], hs, prod);
-                u32* tw = X.touched[par ^ 1] + (hs >> 5);
+                dense_add<Sem>(next_acc, hs, prod);
+                u32* tw = next_touched + (hs >> 5);
                 if (!(lin_ld(tw) & bit)) add = !(atomicOr(tw, bit) & bit);
               }
             }
@@ -474,29 +498,41 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
           const u32 m = __ballot_sync(0xFFFFFFFFu, add);
           if (m) {
             u64 at = 0;
-            if (lane == 0) at = atomicAdd(ast + LS_LIST + (step + 1) % 3, (unsigned long long)__popc(m));
+            if (lane == 0) at = atomicAdd(ast + LS_LIST + rot1, (unsigned long long)__popc(m));
             at = __shfl_sync(0xFFFFFFFFu, at, 0);
             if (add) *reinterpret_cast<volatile u32*>(out_list + at + __popc(m & ((1u << lane) - 1u))) = hs;
           }
         }
       }
     }
-    __syncthreads();
-    if (threadIdx.x < A.n_rel && (fresh_sh[0][threadIdx.x] | fresh_sh[1][threadIdx.x]))
-      atomicAdd(ast + LS_FRESH + rot * kLinMaxRels + threadIdx.x,
-                ((unsigned long long)fresh_sh[1][threadIdx.x] << 32) | fresh_sh[0][threadIdx.x]);
-    // Counters of steps to come.  The list length read in the last step is done
-    // with; the new-fact counts of the last step may still be read by a slow
-    // block, those of the step before may not.
-    if (blockIdx.x == 0 && threadIdx.x <= kLinMaxRels) {
-      if (threadIdx.x == kLinMaxRels) st[LS_LIST + (step + 2) % 3] = 0;
-      else st[LS_FRESH + ((step + 1) % 3) * kLinMaxRels + threadIdx.x] = 0;
+    if (A.n_rel == 1) {
+      n_fresh = __reduce_add_sync(0xFFFFFFFFu, n_fresh);
+      n_better = __reduce_add_sync(0xFFFFFFFFu, n_better);
+      if (lane == 0 && (n_fresh | n_better)) {
+        u32* to = kSh ? reinterpret_cast<u32*>(st + LS_FRESH + rot * kLinMaxRels) : &fresh_sh[par][0][0];
+        if (n_fresh) atomicAdd(to, n_fresh);
+        if (n_better) atomicAdd(kSh ? to + 1 : &fresh_sh[par][1][0], n_better);
+      }
     }
-    if (!lin_barrier(st, gen)) break;
+    __syncthreads();
+    if constexpr (!kSh) {
+      if (threadIdx.x < 32) {
+        if (lane < A.n_rel && (fresh_sh[par][0][lane] | fresh_sh[par][1][lane])) {
+          atomicAdd(ast + LS_FRESH + rot * kLinMaxRels + lane,
+                    ((unsigned long long)fresh_sh[par][1][lane] << 32) | fresh_sh[par][0][lane]);
+          fresh_sh[par][0][lane] = fresh_sh[par][1][lane] = 0;
+          __threadfence();
+        }
+        __syncwarp();
+        if (lane == 0) go = gridDim.x == 1 || lin_barrier_warp0(st, gen);
+      }
+      __syncthreads();
+      if (!go) break;
+    }
     if constexpr (kTop1) {  // a faster block's next step may have found it full already
       const u64 f = lin_ld(st + LS_FULLARENA);
       if (f && f <= step + 1) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) st[LS_STOP] = LIN_ARENA;
+        if (keeper && lane == 0) st[LS_STOP] = LIN_ARENA;
         break;
       }
     }
@@ -509,19 +545,22 @@ __global__ void __launch_bounds__(kSh ? kLinShThreads : kLinThreads) k_linear(co
       const u64 added = v & 0xFFFFFFFFull, improved = v >> 32;
       fcount[r] += added;
       total += added + improved;
-      if (blockIdx.x == 0 && threadIdx.x == 0) {
+      if (keeper && lane == 0) {
         if (A.rec) A.rec[(u64)(step - 1) * A.n_rel + r] = (u32)added;
-        st[LS_FULL + r] = fcount[r];
+        st[LS_FULL + r] = fcount[r];  // (read by the host, after the last step)
         st[LS_LAST + r] = added + improved;
       }
     }
     const u64 stop = !total ? LIN_FIXPOINT : k >= A.max_iters ? LIN_MAXITER : 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      st[LS_NEW] += total;
-      st[LS_ITER] = k;
-      st[LS_STOP] = stop;
+    new_facts += total;
+    if (stop) {
+      if (keeper && lane == 0) {
+        st[LS_NEW] = new_facts;
+        st[LS_ITER] = k;
+        st[LS_STOP] = stop;
+      }
+      break;
     }
-    if (stop) break;
   }
   // join outputs, summed per warp (every lane holds its warp's count)
   __syncthreads();
@@ -705,9 +744,9 @@ struct LinRun {
   std::vector<u32> rels;
   std::vector<int> index;  // relation id -> index in rels, or -1
   explicit LinRun(lob_engine& en) : e(en) {}
-  DevBuf arms, acc[2], touched[2], list[2], ftag, fstamp, fbits, start, state, rec;
+  DevBuf arms, acc, touched, list, used, ftag, fstamp, fbits, start, state, rec;
   ~LinRun() {
-    for (DevBuf* b : {&arms, &acc[0], &acc[1], &touched[0], &touched[1], &list[0], &list[1], &ftag, &fstamp, &fbits, &start,
+    for (DevBuf* b : {&arms, &acc, &touched, &list, &used, &ftag, &fstamp, &fbits, &start,
                       &state, &rec})
       e.release(*b);
   }
@@ -868,11 +907,9 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   e.ensure(L.arms, std::max<size_t>(arms.size(), 1) * sizeof(LinArm));
   if (!arms.empty())
     e.check(cudaMemcpyAsync(L.arms.p, arms.data(), arms.size() * sizeof(LinArm), cudaMemcpyHostToDevice, e.stream), "arms");
-  for (int b = 0; b < 2; b++) {
-    e.ensure(L.acc[b], slots * cb);
-    e.ensure(L.touched[b], slots / 8);
-    e.ensure(L.list[b], slots * 4);
-  }
+  e.ensure(L.acc, 2 * slots * cb);
+  e.ensure(L.touched, 2 * (slots / 8));
+  e.ensure(L.list, 2 * slots * 4);
   e.ensure(L.ftag, slots * sb);
   if (stamps) e.ensure(L.fstamp, slots * 4);
   e.ensure(L.fbits, slots / 8);
@@ -894,11 +931,9 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   }
   A.n_arm = (int)arms.size();
   A.arms = L.arms.as<LinArm>();
-  for (int b = 0; b < 2; b++) {
-    A.acc[b] = L.acc[b].p;
-    A.touched[b] = L.touched[b].as<u32>();
-    A.list[b] = L.list[b].as<u32>();
-  }
+  A.acc = L.acc.p;
+  A.touched = L.touched.as<u32>();
+  A.list = L.list.as<u32>();
   A.ftag = L.ftag.p;
   A.fstamp = L.fstamp.as<u32>();
   A.fbits = L.fbits.as<u32>();
@@ -918,10 +953,8 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   A.slots = (u32)slots;
   std::vector<u64> h(kLinSlots, 0);
   do {  // again when the proof arena ran out: the loop changes only arrays of its own
-    for (int b = 0; b < 2; b++) {
-      e.check(cudaMemsetAsync(L.acc[b].p, 0, slots * cb, e.stream), "accumulators");
-      e.check(cudaMemsetAsync(L.touched[b].p, 0, slots / 8, e.stream), "accumulators");
-    }
+    e.check(cudaMemsetAsync(L.acc.p, 0, 2 * slots * cb, e.stream), "accumulators");
+    e.check(cudaMemsetAsync(L.touched.p, 0, 2 * (slots / 8), e.stream), "accumulators");
     e.check(cudaMemsetAsync(L.ftag.p, 0, slots * sb, e.stream), "tags");
     e.check(cudaMemsetAsync(L.fbits.p, 0, slots / 8, e.stream), "membership");
     e.check(cudaMemsetAsync(L.state.p, 0, kLinSlots * 8, e.stream), "linear state");
@@ -1065,7 +1098,7 @@ bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& 
   e.ensure(L.arms, arms.size() * sizeof(LinBwdArm));
   e.check(cudaMemcpyAsync(L.arms.p, arms.data(), arms.size() * sizeof(LinBwdArm), cudaMemcpyHostToDevice, e.stream), "arms");
   // entries by stamp: counts (scanned in place), fill positions
-  DevBuf &off = L.list[0], &used = L.list[1], &entries = L.start;
+  DevBuf &off = L.list, &used = L.used, &entries = L.start;
   const u64 ns = (u64)last + 1;
   e.ensure(off, (ns + 1) * 4);
   e.ensure(used, ns * 4);
