@@ -180,6 +180,7 @@ __global__ void k_bitmap_set(const void* __restrict__ keys, int key64, u64 n, u3
   const u64 stride = (u64)gridDim.x * blockDim.x;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const u64 k = load_key(keys, key64, i);
+    if (k == invalid_of(key64)) continue;  // a row that a filter dropped
     atomicOr(bm + (k >> 5), 1u << (u32)(k & 31u));
   }
 }
