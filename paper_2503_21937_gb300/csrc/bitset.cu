@@ -139,14 +139,17 @@ __global__ void __launch_bounds__(256) k_bits_extract(const u32* __restrict__ a,
 // result of Sec. 3.2's sort + unique<(+)> over the candidate tuples, without
 // materialising or sorting the candidates.  Each read slot is reset to 0 and
 // each bitmap word cleared, ready for the next iteration.  Same tiling as
-// k_bits_extract; the warp stages keys and tags side by side.
+// k_bits_extract; a warp stages keys until 1,024 are full, and then reads their
+// slots, consecutive lanes neighbouring keys and four loads in flight a lane.  A lane
+// reading its own word's slots one after another, batch by batch, waited for each:
+// the read-outs of a batched kinship run took 4.4 ms and take 0.9 (26 iterations of
+// 6.1e6 facts), those of 1e6 facts in 22 bits 46 and now 17 us.
 template <class K, class C>
 __global__ void __launch_bounds__(256) k_dense_extract(u32* __restrict__ a, u64 nwords, u64 ntiles,
                                                        const u64* __restrict__ tile_off, C* __restrict__ acc,
                                                        K* __restrict__ out, C* __restrict__ otags, u64 cap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C* tstage = reinterpret_cast<C*>(smem_raw) + (threadIdx.x >> 5) * 1024;
-  K* stage = reinterpret_cast<K*>(reinterpret_cast<C*>(smem_raw) + 8 * 1024) + (threadIdx.x >> 5) * 1024;
+  K* stage = reinterpret_cast<K*>(smem_raw) + (threadIdx.x >> 5) * 1024;
   __shared__ u64 wbase[256 / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (u64 t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -165,6 +168,33 @@ __global__ void __launch_bounds__(256) k_dense_extract(u32* __restrict__ a, u64 
     u64 base = tile_off[t];
     for (int v = 0; v < warp; v++) base += wbase[v];
     __syncthreads();
+    u32 filled = 0;  // keys staged
+    auto flush = [&]() {
+      __syncwarp();
+      for (u32 q0 = lane; q0 < filled; q0 += 128) {
+        K k[4];
+        C v[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          if (q0 + 32 * j < filled) {
+            k[j] = stage[q0 + 32 * j];
+            v[j] = acc[k[j]];
+          }
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+          if (q0 + 32 * j < filled) {
+            acc[k[j]] = C(0);
+            const u64 o = base + q0 + 32 * j;
+            if (o < cap) {  // beyond the output's capacity only the resets happen
+              out[o] = k[j];
+              otags[o] = v[j];
+            }
+          }
+      }
+      __syncwarp();
+      base += filled;
+      filled = 0;
+    };
 #pragma unroll
     for (int i = 0; i < kBatches; i++) {
       const u32 m0 = x[i];
@@ -172,24 +202,14 @@ __global__ void __launch_bounds__(256) k_dense_extract(u32* __restrict__ a, u64 
       const u32 inc = warp_inclusive_sum(cnt);
       const u32 tot = __shfl_sync(0xFFFFFFFFu, inc, 31);
       if (!tot) continue;
-      u32 pos = inc - cnt;
+      if (filled + tot > 1024) flush();
+      u32 pos = filled + inc - cnt;
       const u64 kw = (wf + (u64)i * 32 + lane) << 5;
-      for (u32 m = m0; m; m &= m - 1) {
-        const u64 key = kw | (u64)(__ffs(m) - 1);
-        tstage[pos] = acc[key];
-        acc[key] = C(0);
-        stage[pos++] = (K)key;
-      }
-      __syncwarp();
-      for (u32 q = lane; q < tot; q += 32) {
-        if (base + q >= cap) break;  // beyond the output's capacity: only the resets happen
-        out[base + q] = stage[q];
-        otags[base + q] = tstage[q];
-      }
-      __syncwarp();
-      base += tot;
+      for (u32 m = m0; m; m &= m - 1) stage[pos++] = (K)(kw | (u64)(__ffs(m) - 1));
+      filled += tot;
       if (m0) a[wf + (u64)i * 32 + lane] = 0u;
     }
+    flush();
   }
 }
 
@@ -257,7 +277,7 @@ template <class K, class C>
 void dense_extract_t(u32* a, u64 nbits, void* acc, void* out, void* otags, void* scratch, cudaStream_t st, u64 cap) {
   const u64 nw = bit_words(nbits), nt = bit_tiles(nbits);
   const u64* tile_off = reinterpret_cast<const u64*>(scratch) + nt;
-  const int smem = 8 * 1024 * (int)(sizeof(K) + sizeof(C));
+  const int smem = 8 * 1024 * (int)sizeof(K);
   allow_dynamic_smem(k_dense_extract<K, C>, smem);
   k_dense_extract<K, C><<<bit_grid(nt), 256, smem, st>>>(a, nw, nt, tile_off, reinterpret_cast<C*>(acc),
                                                          reinterpret_cast<K*>(out), reinterpret_cast<C*>(otags), cap);
