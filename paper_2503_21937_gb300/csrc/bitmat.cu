@@ -27,9 +27,9 @@
 //
 // Measured (GB300, fixpoint only, general path before -> bit matrices): closure
 // of the 20,000-node / 100,000-edge power-law graph 11.9 -> 1.5 ms; same
-// generation on a 50,000-node tree 22.6 -> 8.8 ms; points-to on 400,000
+// generation on a 50,000-node tree 22.6 -> 6.1 ms; points-to on 400,000
 // statements (8.7e9 derivations of 1.8e6 facts, 36-bit keys: sorted before)
-// 418 -> 2.9 ms; closure of 1,000 nodes / 3,000 edges 0.99 -> 0.45 ms.
+// 418 -> 2.4 ms; closure of 1,000 nodes / 3,000 edges 0.99 -> 0.27 ms.
 #include "bitmat.h"
 
 #include <algorithm>
@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(256) k_bit_active(const __grid_constant__ BOp 
       }
       if (operand_bits) {
         if (len <= 32)
-          for (u32 j = 0; j < len; j += 8) {  // eight entries' loads in flight (one at a time: 33 us a list of 20,000 rows, now 24)
+          // eight entries' loads in flight (one at a time: 33 us a list of 20,000 rows, so 24)
+          for (u32 j = 0; j < len; j += 8) {
             u32 x[8];
 #pragma unroll
             for (int q = 0; q < 8; q++)
@@ -1095,16 +1096,18 @@ LOB_DEV void store_run(u32* __restrict__ p, u32 n, int lane, F&& value, G&& four
 }
 
 // Read-out: a warp walks a row 32 words at a time; a scan of the words' bit
-// counts places each lane's columns in the warp's shared-memory stage, and the
-// warp stores the batch's rows of every output column to consecutive addresses,
-// 16 bytes a lane.
+// counts places each lane's columns in the warp's shared-memory stage (16 bits each,
+// counted from the batch's first), and the warp stores them to consecutive
+// addresses, 16 bytes a lane; the columns that are the same for the whole row are
+// stored in one run before.  Bound by the chain of a batch (scan, stage, store):
+// 7.5e8 pairs in 3.0 ms, 2.0 TB/s; with every column a batch at a time 3.4.
 __global__ void __launch_bounds__(256) k_bit_read(const u32* __restrict__ bits, u32 rows, u32 words,
                                                   const u64* __restrict__ off, const u32* __restrict__ dict,
                                                   u32* __restrict__ c0, u32* __restrict__ c1, float* __restrict__ tags,
                                                   u32* __restrict__ samples) {
-  __shared__ __align__(16) u32 stages[8][1024 + 4];
+  __shared__ __align__(16) uint16_t stages[8][1024 + 8];  // columns from the batch's first on
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  u32* stage = stages[warp];
+  uint16_t* stage = stages[warp];
   const u64 nwarps = (u64)gridDim.x * 8;
   for (u64 r = (u64)blockIdx.x * 8 + warp; r < rows; r += nwarps) {
     u64 base = off[r];
@@ -1112,6 +1115,14 @@ __global__ void __launch_bounds__(256) k_bit_read(const u32* __restrict__ bits, 
     const u32 x = dict ? dict[r] : (u32)r;
     const u32* row = bits + r * words;
     u32 nextw = lane < words ? row[lane] : 0u;
+    // what is the same for the whole row in one run
+    const u32 n_row = (u32)(off[r + 1] - base), one = __float_as_uint(1.0f);
+    store_run(c0 + base, n_row, lane, [&](u32) { return x; }, [&](u32) { return make_uint4(x, x, x, x); });
+    if (tags)
+      store_run(reinterpret_cast<u32*>(tags) + base, n_row, lane, [&](u32) { return one; },
+                [&](u32) { return make_uint4(one, one, one, one); });
+    if (samples)
+      store_run(samples + base, n_row, lane, [&](u32) { return 0u; }, [&](u32) { return make_uint4(0, 0, 0, 0); });
     for (u32 w0 = 0; w0 < words; w0 += 32) {
       const u32 m0 = nextw;
       nextw = w0 + 32 + lane < words ? row[w0 + 32 + lane] : 0u;
@@ -1122,21 +1133,15 @@ __global__ void __launch_bounds__(256) k_bit_read(const u32* __restrict__ bits, 
       // staged at the offset the destination has within 16 bytes
       const u32 skew = (u32)(reinterpret_cast<uintptr_t>(c1 + base) >> 2) & 3u;
       u32 pos = inc - c + skew;
-      const u32 kw = (w0 + lane) * 32;
-      for (u32 m = m0; m; m &= m - 1) stage[pos++] = kw + (u32)__ffs(m) - 1;
+      for (u32 m = m0; m; m &= m - 1) stage[pos++] = (uint16_t)(lane * 32 + __ffs(m) - 1);
       __syncwarp();
-      store_run(c0 + base, tot, lane, [&](u32) { return x; }, [&](u32) { return make_uint4(x, x, x, x); });
-      store_run(c1 + base, tot, lane, [&](u32 s) { return dict ? dict[stage[s + skew]] : stage[s + skew]; },
+      const u32 k0 = w0 * 32;
+      store_run(c1 + base, tot, lane, [&](u32 s) { return dict ? dict[k0 + stage[s + skew]] : k0 + stage[s + skew]; },
                 [&](u32 s) {
-                  uint4 y = *reinterpret_cast<const uint4*>(stage + s + skew);
+                  const ushort4 z = *reinterpret_cast<const ushort4*>(stage + s + skew);
+                  const uint4 y = make_uint4(k0 + z.x, k0 + z.y, k0 + z.z, k0 + z.w);
                   return dict ? make_uint4(dict[y.x], dict[y.y], dict[y.z], dict[y.w]) : y;
                 });
-      const u32 one = __float_as_uint(1.0f);
-      if (tags)
-        store_run(reinterpret_cast<u32*>(tags) + base, tot, lane, [&](u32) { return one; },
-                  [&](u32) { return make_uint4(one, one, one, one); });
-      if (samples)
-        store_run(samples + base, tot, lane, [&](u32) { return 0u; }, [&](u32) { return make_uint4(0, 0, 0, 0); });
       __syncwarp();
       base += tot;
     }
