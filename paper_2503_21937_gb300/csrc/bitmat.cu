@@ -1446,6 +1446,11 @@ struct Run {
       e.ensure(B.temp[i], mb);
       e.ensure(B.tbag[i], D * 8);
     }
+    // what finish() needs is taken here as well: a request refused after the
+    // iterations would throw their work away
+    for (size_t r = 0; r < e.rels.size(); r++)
+      if (e.rels[r].idb) e.ensure(B.rel[r].off, (D + 1) * 8);
+    e.ensure(e.scratch, scan_scratch_elems(D) * 8 + 64);
     e.ensure(B.state, kAllSlots * 8);
     e.check(cudaMemsetAsync(B.state.p, 0, kAllSlots * 8, e.stream), "bit state");
     if (listed()) {
@@ -1834,15 +1839,18 @@ struct Run {
     launch_check("bit loop");
   }
 
+  // The run's results become the engine's only after the last step that can fail:
+  // until then the relations hold their loaded facts, which the general path starts
+  // from when this one gives up.
   bool done(u32& k, u64& new_facts, int* rc) {
-    const u64* s = e.pinned;
+    const std::vector<u64> s(e.pinned, e.pinned + kStateSlots);
+    finish();
     *rc = s[B_DONE] == 1 ? LOB_OK : LOB_E_MAXITER;
     k = (u32)s[B_ITER];
     new_facts = s[B_NEW];
     e.cand_emitted = s[B_CAND];
     for (size_t r = 0; r < e.rels.size(); r++)
       if (e.rels[r].idb) e.rels[r].views[0].n = s[rel_slot((int)r, 0)];
-    finish();
     return true;
   }
 
@@ -1867,8 +1875,6 @@ struct Run {
         }
         launch_check("bit counts");
       }
-      e.ensure(R.off, (D + 1) * 8);
-      e.ensure(e.scratch, scan_scratch_elems(D) * 8 + 64);
       exclusive_scan<u32, u64>(R.fcnt, R.off.as<u64>(), D, R.off.as<u64>() + D, e.scratch.as<u64>(), e.stream);
       e.after_launch("bit offsets");
       e.launches += scan_launches(D);
