@@ -384,8 +384,8 @@ int lob_prim_diff_merge(lob_engine* e, int semiring, const void* f_keys, const v
  * NULL when n is 0; *n_out then gets 0).  The first call on a device
  * looks up the scratch array's device address; make that first call before
  * any stream capture.  All calls on a device share the scratch array, so
- * calls whose work overlaps on the GPU race: order them (one stream, or
- * events).  A row whose every column is 0xFFFFFFFF is dropped (at arity 1
+ * calls whose work overlaps on the GPU race and get wrong rows: order them (one
+ * stream, or events).  Later calls are not affected.  A row whose every column is 0xFFFFFFFF is dropped (at arity 1
  * and 2 alike).  The work is
  * queued on cuda_stream (NULL: legacy default stream); the call does not wait.
  * The sort's blocks wait on one another, with a limit; should a wait give up,

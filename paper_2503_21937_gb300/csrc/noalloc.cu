@@ -12,10 +12,12 @@
 //
 // The scratch array is shared by every call on a device and keeps whatever the
 // last call left in it.  Everything a call reads from it is written earlier in
-// the same call (keys, digit counts, the blocks' maxima and row counts), except
-// the barrier words, which the last block of a call leaves at zero.  Two calls whose work overlaps on
-// the GPU (for example on two streams at once) race on the array; callers must
-// order them.
+// the same call: keys, digit counts, the blocks' maxima and row counts, and the
+// barrier words, which a memset before the launch clears (about 2 us).  Two calls
+// whose work overlaps on the GPU (for example on two streams at once) race on the
+// array, and callers must order them; should they not, those two results are wrong
+// and no later call's.  The calls of a process take turns at kHeads sets of barrier
+// words, so that one of the two cannot clear what the other's blocks wait for.
 //
 // One cooperative launch does it all: the columns' largest values (a barrier), keys
 // packed into as few bits as those need, the radix passes over them
@@ -24,6 +26,7 @@
 // 8 bits of key.  Pack, 40 sort launches, three for the distinct rows and unpack
 // took 219 us for 100,003 rows of two columns; one launch takes 53.
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "../../include/lobster.h"
@@ -34,17 +37,18 @@ namespace {
 
 constexpr u64 kMaxRows = LOB_NOALLOC_MAX_ROWS;
 constexpr u64 kKeyBytes = kMaxRows * sizeof(u64);
-// barrier words and digit counts, then per block its columns' maxima and row count
-constexpr u64 kSortWords = kFHead + 2 * 256 * (u64)kFTiles;
-constexpr u64 kScratchBytes = 2 * kKeyBytes + kSortWords * 4 + 4 * kFTiles * 4;
+// digit counts, then per block its columns' maxima and row count; barrier words
+constexpr u64 kCountWords = fused_count_words(kFTiles) + 4 * kFTiles;
+constexpr u32 kHeads = 64;
+constexpr u64 kScratchBytes = 2 * kKeyBytes + kCountWords * 4 + (u64)kHeads * kFHead * 4;
 static_assert(kScratchBytes <= 4600000, "scratch budget");
 static_assert(512ull * kFItems * kFTiles >= kMaxRows, "the largest batch fits the launch");
 
-// zero in the library image; the barrier words are zero again after every call
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mutex;
+std::atomic<u32> g_calls{0};
 unsigned char* g_scratch_ptr[kMaxDevices] = {nullptr};
 
 // Host code must not use g_noalloc_scratch directly: on the host that name is
@@ -74,13 +78,13 @@ LOB_DEV int bit_count(u32 x) { return 32 - __clz(x); }
 
 template <int NT>
 __global__ void __launch_bounds__(NT, 1) k_unique_rows(const u32* __restrict__ cols, u32 arity, u64 n, u32* __restrict__ out,
-                                                       u64* __restrict__ n_out, u64* keys_a, u64* keys_b, u32* scratch) {
+                                                       u64* __restrict__ n_out, u64* keys_a, u64* keys_b, u32* counts, u32* head) {
   typedef FusedSmem<u64, NoPay, NT> Smem;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem& S = *reinterpret_cast<Smem*>(smem_raw);
   __shared__ u32 red[2][NT / 32];
   __shared__ u64 sm64[NT / 32 + 1];
-  u32* per_block = scratch + kSortWords;
+  u32* per_block = counts + fused_count_words(kFTiles);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   FusedTile<u64, NoPay, NT> T;
   T.place(n);
@@ -108,7 +112,7 @@ __global__ void __launch_bounds__(NT, 1) k_unique_rows(const u32* __restrict__ c
   for (int w = 0; w < NT / 32; w++) { m0 = max(m0, red[0][w]); m1 = max(m1, red[1][w]); }
   if (gridDim.x > 1) {
     if (threadIdx.x == 0) { per_block[2 * blockIdx.x] = m0; per_block[2 * blockIdx.x + 1] = m1; }
-    good = fused_barrier(scratch, gen);
+    good = fused_barrier(head, gen);
     m0 = m1 = 0;
     for (u32 b = lane; b < gridDim.x; b += 32) {
       m0 = max(m0, __ldcg(per_block + 2 * b));
@@ -128,13 +132,13 @@ __global__ void __launch_bounds__(NT, 1) k_unique_rows(const u32* __restrict__ c
       keys_a[T.at(r)] = T.k[r];
     }
   // (a pass's count barrier comes before anything reads the keys of another block)
-  good = good && fused_passes(T, S, n, bits, scratch, gen);
+  good = good && fused_passes(T, S, n, bits, head, counts, gen);
   // distinct keys: those that differ from the one before; a row of all ones is dropped
   if (good) {
 #pragma unroll
     for (int r = 0; r < kFItems; r++)
       if (T.valid(r)) S.keys[T.wofs + r * 32 + lane] = T.k[r];
-    if (gridDim.x > 1 && bits == 0) good = fused_barrier(scratch, gen);  // no pass had one
+    if (gridDim.x > 1 && bits == 0) good = fused_barrier(head, gen);  // no pass had one
     __syncthreads();
   }
   u32 heads[kFItems], mine = 0;
@@ -157,15 +161,15 @@ __global__ void __launch_bounds__(NT, 1) k_unique_rows(const u32* __restrict__ c
   const u64 wbase = block_exclusive_sum<u64>(lane == 0 ? (u64)mine : 0ull, sm64, &tile_count);
   u64 pos = __shfl_sync(0xFFFFFFFFu, wbase, 0), all = tile_count;
   if (gridDim.x > 1) {
-    u32* counts = per_block + 2 * kFTiles;
+    u32* rows = per_block + 2 * kFTiles;
     if (good) {
-      if (threadIdx.x == 0) counts[blockIdx.x] = (u32)tile_count;
-      good = fused_barrier(scratch, gen);
+      if (threadIdx.x == 0) rows[blockIdx.x] = (u32)tile_count;
+      good = fused_barrier(head, gen);
     }
     u64 before = 0;
     all = 0;
     for (u32 b = lane; b < gridDim.x; b += 32) {
-      const u32 c = good ? __ldcg(counts + b) : 0u;
+      const u32 c = good ? __ldcg(rows + b) : 0u;
       all += c;
       if (b < blockIdx.x) before += c;
     }
@@ -188,13 +192,9 @@ __global__ void __launch_bounds__(NT, 1) k_unique_rows(const u32* __restrict__ c
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *n_out = all;
   }
-  if (gridDim.x > 1 && threadIdx.x == 0) {  // the last block to leave clears the barrier words for the next call
+  if (gridDim.x > 1 && threadIdx.x == 0) {  // the last block to leave: did some block give up?
     __threadfence();
-    if (atomicAdd(scratch + 2, 1u) + 1 == gridDim.x) {
-      if (scratch[1]) *n_out = ~0ull;  // some block gave up
-      scratch[0] = scratch[1] = scratch[2] = 0;
-      __threadfence();
-    }
+    if (atomicAdd(head + 2, 1u) + 1 == gridDim.x && *reinterpret_cast<volatile u32*>(head + 1)) *n_out = ~0ull;
   }
 }
 
@@ -202,15 +202,18 @@ template <int NT>
 cudaError_t launch_unique_rows(const u32* cols, u32 arity, u64 n, u32* out, u64* n_out, unsigned char* s, cudaStream_t st) {
   u64* a = reinterpret_cast<u64*>(s);
   u64* b = reinterpret_cast<u64*>(s + kKeyBytes);
-  u32* scratch = reinterpret_cast<u32*>(s + 2 * kKeyBytes);
+  u32* counts = reinterpret_cast<u32*>(s + 2 * kKeyBytes);
+  u32* head = counts + kCountWords + kFHead * (g_calls.fetch_add(1, std::memory_order_relaxed) % kHeads);
   constexpr int kSm = (int)sizeof(FusedSmem<u64, NoPay, NT>);
   if (kSm > 48 * 1024) allow_dynamic_smem(k_unique_rows<NT>, kSm);
   const unsigned tiles = (unsigned)std::max<u64>(1, (n + NT * kFItems - 1) / (NT * kFItems));
   if (tiles == 1) {
-    k_unique_rows<NT><<<1, NT, kSm, st>>>(cols, arity, n, out, n_out, a, b, scratch);
+    k_unique_rows<NT><<<1, NT, kSm, st>>>(cols, arity, n, out, n_out, a, b, counts, head);
     return cudaGetLastError();
   }
-  void* args[] = {&cols, &arity, &n, &out, &n_out, &a, &b, &scratch};
+  const cudaError_t cleared = cudaMemsetAsync(head, 0, kFHead * sizeof(u32), st);
+  if (cleared != cudaSuccess) return cleared;
+  void* args[] = {&cols, &arity, &n, &out, &n_out, &a, &b, &counts, &head};
   return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k_unique_rows<NT>), dim3(tiles), dim3(NT), args, kSm, st);
 }
 

@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(NT, 1) k_sort_fused(const K* keys, const P* pa
   T.dst_p = ptmp;
   T.reload();
   u32 gen = 0;
-  if (!fused_passes(T, S, n, bits, scratch, gen) && err && threadIdx.x == 0) *err = 1;
+  if (!fused_passes(T, S, n, bits, scratch, scratch + kFHead, gen) && err && threadIdx.x == 0) *err = 1;
   if (gridDim.x > 1 && T.src_k == ktmp) return;
 #pragma unroll
   for (int r = 0; r < kFItems; r++)

@@ -23,11 +23,13 @@ struct NoPay {};
 constexpr int kFItems = 8;    // keys per thread
 constexpr int kFTiles = 64;   // blocks of a launch at most
 constexpr u32 kFSpin = 1u << 26;  // barrier polls before a block gives up
-// fused scratch, in u32 words: barrier arrivals, give-up flag, blocks that left,
-// padding, then the tiles' digit counts, two passes' worth (a block may still add
-// up one pass's when another counts the next)
+// fused scratch, in u32 words: a head (barrier arrivals, give-up flag, blocks that
+// left, padding), zero when a launch of several blocks starts, and the tiles' digit
+// counts, two passes' worth (a block may still add up one pass's when another counts
+// the next)
 constexpr u32 kFHead = 16;
-LOB_HD u64 fused_scratch_words(u64 tiles) { return kFHead + 2 * 256 * tiles; }
+LOB_HD constexpr u64 fused_count_words(u64 tiles) { return 2 * 256 * tiles; }
+LOB_HD u64 fused_scratch_words(u64 tiles) { return kFHead + fused_count_words(tiles); }
 
 // Lanes of this warp holding the same RB-bit digit (and a valid key): the
 // intersection over the digit's bits of the ballot of lanes agreeing on that bit.
@@ -107,7 +109,8 @@ struct FusedTile {
 // Sorts by the low `bits` bits; afterwards every block's tile is in registers, and
 // (unless the launch has one tile) in src_k / src_p.  False when a barrier gave up.
 template <class K, class P, int NT>
-LOB_DEV bool fused_passes(FusedTile<K, P, NT>& T, FusedSmem<K, P, NT>& S, u64 n, int bits, u32* scratch, u32& gen) {
+LOB_DEV bool fused_passes(FusedTile<K, P, NT>& T, FusedSmem<K, P, NT>& S, u64 n, int bits, u32* head, u32* counts,
+                          u32& gen) {
   constexpr bool kPay = FusedTile<K, P, NT>::kPay;
   constexpr int kWarps = NT / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -143,9 +146,9 @@ LOB_DEV bool fused_passes(FusedTile<K, P, NT>& T, FusedSmem<K, P, NT>& S, u64 n,
     }
     u32 before = 0, total = mine;  // of the tiles before this one, of all tiles
     if (tiles > 1) {
-      u32* cnt = scratch + kFHead + (u64)(pass & 1) * 256 * tiles;
+      u32* cnt = counts + (u64)(pass & 1) * 256 * tiles;
       if (threadIdx.x < 256) cnt[blockIdx.x * 256 + threadIdx.x] = mine;
-      if (!fused_barrier(scratch, gen)) return false;
+      if (!fused_barrier(head, gen)) return false;
       if (threadIdx.x < 256) {
         total = 0;
 #pragma unroll 16
@@ -199,7 +202,7 @@ LOB_DEV bool fused_passes(FusedTile<K, P, NT>& T, FusedSmem<K, P, NT>& S, u64 n,
     }
     { K* t = T.src_k; T.src_k = T.dst_k; T.dst_k = t; }
     { P* t = T.src_p; T.src_p = T.dst_p; T.dst_p = t; }
-    if (!fused_barrier(scratch, gen)) return false;
+    if (!fused_barrier(head, gen)) return false;
     T.reload();
   }
   return true;

@@ -68,3 +68,32 @@ def test_noalloc_in_a_captured_graph():
         want = np.unique(r, axis=1)
         assert int(n_out.item()) == want.shape[1]
         assert np.array_equal(out[:, : want.shape[1]].cpu().numpy().view(np.uint32), want)
+
+
+def test_each_noalloc_call_clears_its_barrier_words():
+    """A call whose blocks wait on one another starts with a memset node (64 bytes of
+    zeros) in the captured graph: it trusts nothing that an earlier call left.  (Calls
+    that overlap, which could leave words behind, are not run.)"""
+    import ctypes
+    import torch
+    from paper_2503_21937_gb300 import lobster
+    cols = _dev(np.stack([W.stream(8200).below(50000, 3000)] * 2))
+    out, n_out = torch.zeros_like(cols), torch.zeros(1, dtype=torch.int64, device="cuda")
+    assert lobster.unique_rows_noalloc(cols, out, n_out) == 0
+    torch.cuda.synchronize()
+    if not hasattr(torch.cuda.CUDAGraph, "raw_cuda_graph"):
+        pytest.skip("this torch does not give the captured graph")
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        assert lobster.unique_rows_noalloc(cols, out, n_out) == 0
+    cu = ctypes.CDLL("libcuda.so.1")
+    h, n = ctypes.c_void_p(g.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert cu.cuGraphGetNodes(h, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(h, nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for node in nodes:
+        t = ctypes.c_int(-1)
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(t)) == 0
+        kinds.append(t.value)
+    assert sorted(kinds) == [0, 2], kinds  # one kernel, one memset
