@@ -35,7 +35,8 @@ typedef struct lob_engine lob_engine;
 #define LOB_E_PARSE (-2)        /* rule text does not parse */
 #define LOB_E_UNKNOWN_REL (-3)  /* relation id or name not declared */
 #define LOB_E_UNSAFE_RULE (-4)  /* head or filter variable not bound by a body atom */
-#define LOB_E_OOM (-5)          /* device allocation failed; engine state is unchanged */
+#define LOB_E_OOM (-5)          /* device allocation failed; engine state is unchanged (a run or a backward pass
+                                   that was refused memory it only is faster with has tried without it) */
 #define LOB_E_MAXITER (-6)      /* max_iters reached before the fixpoint; state is kept and readable */
 #define LOB_E_TIMEOUT (-7)      /* a bounded device wait gave up; results of the run are invalid */
 #define LOB_E_CUDA (-8)         /* a CUDA runtime call failed */

@@ -304,6 +304,9 @@ struct ByStamp {
 };
 
 struct BwdState {
+  // extra: the pass has used memory that it could do without (rows by stamp, masks,
+  // the linear components' launch); lean: it uses none of them
+  bool extra = false, lean = false;
   std::vector<ByStamp> stamped;              // per relation, on first use
   std::vector<DevBuf> adj;                   // per relation, f64, primary view order
   std::vector<DevBuf> hrow;                  // per derived relation with a small key space: dense key -> row
@@ -315,10 +318,11 @@ struct BwdState {
 };
 
 // the bitmap of `rel` with column order perm in set v, allocated on first use
-MaskSt& bwd_mask(lob_engine& e, std::vector<MaskSt>& v, const RelSt& r, const int* perm, bool* made) {
+MaskSt& bwd_mask(lob_engine& e, BwdState& S, std::vector<MaskSt>& v, const RelSt& r, const int* perm, bool* made) {
   *made = false;
   for (auto& m : v)
     if (std::equal(perm, perm + r.arity, m.perm)) return m;
+  S.extra = true;
   MaskSt m;
   std::copy(perm, perm + r.arity, m.perm);
   m.lay = mask_layout(e, r, perm);
@@ -328,7 +332,9 @@ MaskSt& bwd_mask(lob_engine& e, std::vector<MaskSt>& v, const RelSt& r, const in
   *made = true;
   return v.back();
 }
-bool bwd_masked(const lob_engine& e, const ArmPlan& A) { return e.opt_packed_backward && A.packed.ok && A.packed.mask_ok; }
+bool bwd_masked(const lob_engine& e, const BwdState& S, const ArmPlan& A) {
+  return e.opt_packed_backward && !S.lean && A.packed.ok && A.packed.mask_ok;
+}
 
 void free_state(lob_engine& e, BwdState& S) {
   for (auto& b : S.adj) e.release(b);
@@ -533,7 +539,7 @@ void replay_arm(lob_engine& e, BwdState& S, const RulePlan& rp, const ArmPlan& A
 ByStamp& by_stamp(lob_engine& e, BwdState& S, u32 rel) {
   ByStamp& B = S.stamped[rel];
   if (B.built) return B;
-  B.built = true;
+  B.built = S.extra = true;
   const ViewSt& V = e.rels[rel].views[0];
   const u64 n = V.n;
   const int kb = V.lay.key64 ? 8 : 4;
@@ -605,7 +611,7 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
   int side = 0;
   // the delta atom: the recent set of iteration k, a run of the rows by stamp
   // (every fact when k begins a stratum)
-  const bool by_run = !begins_stratum(e.stratum_begin, k) && n_in;
+  const bool by_run = !S.lean && !begins_stratum(e.stratum_begin, k) && n_in;
   if (by_run) {
     const ByStamp& T = by_stamp(e, S, R.body[A.delta].rel);
     in_words = T.words.as<char>() + (u64)T.off[k - 1] * (DV.lay.key64 ? 8 : 4);
@@ -642,14 +648,14 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
     P.index_mode = I.mode;
     P.dense_offs = I.offs.as<u64>();
     P.hash_bits = I.hash_bits;
-    if (last && A.packed.mask_ok && I.mode == INDEX_DENSE) {  // only groundings whose head has an adjoint to give
+    if (last && bwd_masked(e, S, A) && I.mode == INDEX_DENSE) {  // only groundings whose head has an adjoint to give
       bool made;
       RelSt& V = e.rels[vrel];
       PMask M = A.packed.mask;
-      MaskSt& have = bwd_mask(e, S.have[vrel], V, W.perm, &made);
+      MaskSt& have = bwd_mask(e, S, S.have[vrel], V, W.perm, &made);
       if (made) mask_set(V.views[0].lay, V.views[0].perm, have.lay, have.perm, V.views[0].keys.p, nullptr, 4, V.views[0].n, have.bits.as<u32>(), nullptr, e.stream);
       M.vbits = have.bits.as<u32>();
-      M.hbits = bwd_mask(e, S.fresh[hrel], H, A.packed.mask_h, &made).bits.as<u32>();
+      M.hbits = bwd_mask(e, S, S.fresh[hrel], H, A.packed.mask_h, &made).bits.as<u32>();
       if (made) throw LobError(LOB_E_CUDA, "internal error: mask of the new heads missing");
       B.last = 1;
       B.v_prow = SP.view ? S.prow[vrel][SP.view].as<u32>() : nullptr;
@@ -711,6 +717,126 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
   return true;
 }
 
+// The adjoints of a diff-add-mult run, and from them the inputs' gradients.
+void add_mult_backward(lob_engine* e, BwdState& S, u32 out_rel, const float* gdev, u64 n_out, const std::vector<float*>& gin) {
+  const size_t nrel = e->rels.size();
+  S.adj.resize(nrel);
+  S.hrow.resize(nrel);
+  S.hnew.resize(nrel);
+  S.prow.resize(nrel);
+  S.have.resize(nrel);
+  S.stamped.resize(nrel);
+  S.fresh.resize(nrel);
+  for (size_t k = 0; k < nrel; k++) {
+    RelSt& r = e->rels[k];
+    const u64 n = r.views[0].n;
+    const Layout& L = r.views[0].lay;
+    if (r.idb && n && L.bits <= e->opt_acc_bits) {  // heads are found by one load instead of a binary search
+      const u64 slots = 1ull << L.bits;
+      e->ensure(S.hrow[k], slots * 4);
+      e->check(cudaMemsetAsync(S.hrow[k].p, 0xFF, slots * 4, e->stream), "head rows");
+      k_dense_rows<<<grid_for_n(n), 256, 0, e->stream>>>(r.views[0].keys.p, L.key64, n, S.hrow[k].as<u32>());
+      e->after_launch("head rows");
+      e->ensure(S.hnew[k], std::max<u64>(16, slots / 8));
+    }
+    e->ensure(S.adj[k], std::max<u64>(n, 1) * 8);
+    e->check(cudaMemsetAsync(S.adj[k].p, 0, std::max<u64>(n, 1) * 8, e->stream), "adjoint init");
+    if (n > 0xFFFFFFFFull) throw LobError(LOB_E_ARG, "backward supports relations below 2^32 facts");
+    S.prow[k].resize(r.views.size());
+    for (size_t vi = 1; vi < r.views.size(); vi++) {
+      ViewSt& W = r.views[vi];
+      if (!W.n) continue;
+      const int kb = r.views[0].lay.key64 ? 8 : 4;
+      e->ensure(e->tmp_keys, W.n * kb);
+      repack_keys(W.lay, W.perm, r.views[0].lay, r.views[0].perm, W.keys.p, e->tmp_keys.p, W.n, e->stream);
+      e->ensure(S.prow[k][vi], W.n * 4);
+      k_locate<<<grid_for_n(W.n), 256, 0, e->stream>>>(r.views[0].keys.p, r.views[0].lay.key64, r.views[0].n,
+                                                         e->tmp_keys.p, W.n, S.prow[k][vi].as<u32>());
+      e->after_launch("view rows");
+    }
+  }
+  if (n_out) {
+    k_f32_to_f64<<<grid_for_n(n_out), 256, 0, e->stream>>>(gdev, n_out, S.adj[out_rel].as<double>());
+    e->after_launch("adjoint seed");
+  }
+  // Only relations out_rel depends on carry adjoints: rules with another
+  // head contribute nothing and are not replayed.
+  std::vector<char> needed(nrel, 0);
+  needed[out_rel] = 1;
+  for (bool grew = true; grew;) {
+    grew = false;
+    for (auto& p : e->plans)
+      if (needed[p.ast.head.rel])
+        for (auto& a : p.ast.body)
+          if (!needed[a.rel]) needed[a.rel] = grew = true;
+  }
+  // facts first derived in iteration k (the recent set at the start of k + 1,
+  // unless k + 1 began a stratum: then iteration k, its stratum's last, found none)
+  auto new_in = [&](u32 k, u32 rel) -> u64 {
+    if (begins_stratum(e->stratum_begin, k + 1)) return 0;
+    return k < e->iter_counts.size() ? e->iter_counts[k][rel].second : e->rels[rel].n_recent;
+  };
+  // Linear components whose head is needed replay in one launch (linear.cu),
+  // down to iteration 2.  They feed no other component, and what they add to
+  // the inputs' adjoints is read at the end.
+  std::vector<char> linear(nrel, 0);
+  {
+    LinearAdjoints J;
+    for (size_t q = 0; q < nrel; q++) {
+      J.adj.push_back(S.adj[q].as<double>());
+      J.hrow.push_back(S.hrow[q].as<u32>());
+      J.prow.emplace_back();
+      for (auto& b : S.prow[q]) J.prow.back().push_back(b.as<u32>());
+    }
+    if (S.lean || !linear_backward(*e, J, linear, S.extra)) linear.assign(nrel, 0);
+  }
+  for (u32 k = e->last_iter; k >= 1; k--) {
+    for (size_t q = 0; q < nrel; q++) {  // the heads new in iteration k
+      if (!S.hnew[q].p || !needed[q] || (linear[q] && k > 1) || !new_in(k, (u32)q)) continue;
+      RelSt& r = e->rels[q];
+      e->check(cudaMemsetAsync(S.hnew[q].p, 0, S.hnew[q].cap, e->stream), "new heads");
+      k_mark_new<<<grid_for_n(r.views[0].n), 256, 0, e->stream>>>(r.views[0].keys.p, r.views[0].lay.key64,
+                                                                  r.views[0].stamps.as<u32>(), r.views[0].n, k,
+                                                                  S.hnew[q].as<u32>());
+      e->after_launch("new heads");
+      for (auto& p : e->plans)
+        for (auto& A : p.arms) {
+          if (p.ast.head.rel != q || !bwd_masked(*e, S, A)) continue;
+          bool made;
+          bwd_mask(*e, S, S.fresh[q], r, A.packed.mask_h, &made);
+        }
+      for (auto& m : S.fresh[q]) {
+        e->check(cudaMemsetAsync(m.bits.p, 0, mask_bytes(m.lay), e->stream), "new heads");
+        mask_set_new(r.views[0].lay, r.views[0].perm, m.lay, m.perm, r.views[0].keys.p, r.views[0].n,
+                     r.views[0].stamps.as<u32>(), k, S.adj[q].as<double>(), m.bits.as<u32>(), e->stream);
+        e->after_launch("new heads");
+      }
+    }
+    const int stratum = stratum_of_iter(e->stratum_begin, k);
+    for (auto& p : e->plans)
+      for (auto& A : p.arms) {
+        if (p.stratum != stratum) continue;  // the rule did not run in iteration k
+        if (!needed[p.ast.head.rel] || !new_in(k, p.ast.head.rel)) continue;  // no adjoint can flow here
+        if (linear[p.ast.head.rel] && k > 1) continue;
+        const auto& cnt = e->iter_counts[k - 1];  // (total, recent) per relation at the start of iteration k
+        if (!cnt[p.ast.body[A.delta].rel].second) continue;
+        bool skip = false;
+        for (u32 b : A.before_rels)
+          if (cnt[b].first == cnt[b].second) { skip = true; break; }
+        if (skip) continue;
+        if (!replay_arm_packed(*e, S, p, A, k)) replay_arm(*e, S, p, A, k);
+      }
+  }
+  for (size_t k = 0; k < nrel; k++) {
+    RelSt& r = e->rels[k];
+    if (!gin[k] || !r.n_in || !r.views[0].n) continue;
+    k_bwd_inputs<<<grid_for_n(r.n_in), 256, 0, e->stream>>>(r.views[0].keys.p, r.views[0].lay.key64, r.views[0].n,
+                                                             r.row_keys.p, r.row_factor.as<float>(),
+                                                             S.adj[k].as<double>(), r.n_in, gin[k]);
+    e->after_launch("input gradients");
+  }
+}
+
 }  // namespace
 
 int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* const* grad_inputs, int mem) {
@@ -722,8 +848,17 @@ int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* con
   const u64 n_out = O.views[0].n;
   if (n_out && !grad_tags) throw LobError(LOB_E_ARG, "null grad_tags");
   const size_t nrel = e->rels.size();
+  bool lean = false;
   // device views of the caller's buffers
-  DevBuf g, gin_all;
+  struct Held {  // given back on every exit
+    lob_engine* e;
+    DevBuf g, gin_all;
+    ~Held() {
+      e->release(g);
+      e->release(gin_all);
+    }
+  } held{e, {}, {}};
+  DevBuf &g = held.g, &gin_all = held.gin_all;
   std::vector<float*> gin(nrel, nullptr);
   const float* gdev = grad_tags;
   if (mem == LOB_MEM_HOST) {
@@ -773,128 +908,27 @@ int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* con
     top1_grad_scatter(O.views[0].tags.as<u64>(), gdev, n_out, e->arena.as<u32>(), e->top1_prob.as<float>(), T, e->stream);
     e->after_launch("top-1-proofs backward");
   } else {
-    BwdState S;
-    try {
-      S.adj.resize(nrel);
-      S.hrow.resize(nrel);
-      S.hnew.resize(nrel);
-      S.prow.resize(nrel);
-      S.have.resize(nrel);
-      S.stamped.resize(nrel);
-      S.fresh.resize(nrel);
-      for (size_t k = 0; k < nrel; k++) {
-        RelSt& r = e->rels[k];
-        const u64 n = r.views[0].n;
-        const Layout& L = r.views[0].lay;
-        if (r.idb && n && L.bits <= e->opt_acc_bits) {  // heads are found by one load instead of a binary search
-          const u64 slots = 1ull << L.bits;
-          e->ensure(S.hrow[k], slots * 4);
-          e->check(cudaMemsetAsync(S.hrow[k].p, 0xFF, slots * 4, e->stream), "head rows");
-          k_dense_rows<<<grid_for_n(n), 256, 0, e->stream>>>(r.views[0].keys.p, L.key64, n, S.hrow[k].as<u32>());
-          e->after_launch("head rows");
-          e->ensure(S.hnew[k], std::max<u64>(16, slots / 8));
+    // As a run does (run_fixpoint), a pass that is refused memory while it holds some
+    // that it could do without starts again without; the gradients of the inputs are
+    // added to at its very end.
+    for (bool again = true; again;) {
+      BwdState S;
+      S.lean = lean;
+      again = false;
+      try {
+        add_mult_backward(e, S, out_rel, gdev, n_out, gin);
+      } catch (const LobError& x) {
+        if (x.code != LOB_E_OOM || !S.extra) {
+          free_state(*e, S);
+          throw;
         }
-        e->ensure(S.adj[k], std::max<u64>(n, 1) * 8);
-        e->check(cudaMemsetAsync(S.adj[k].p, 0, std::max<u64>(n, 1) * 8, e->stream), "adjoint init");
-        if (n > 0xFFFFFFFFull) throw LobError(LOB_E_ARG, "backward supports relations below 2^32 facts");
-        S.prow[k].resize(r.views.size());
-        for (size_t vi = 1; vi < r.views.size(); vi++) {
-          ViewSt& W = r.views[vi];
-          if (!W.n) continue;
-          const int kb = r.views[0].lay.key64 ? 8 : 4;
-          e->ensure(e->tmp_keys, W.n * kb);
-          repack_keys(W.lay, W.perm, r.views[0].lay, r.views[0].perm, W.keys.p, e->tmp_keys.p, W.n, e->stream);
-          e->ensure(S.prow[k][vi], W.n * 4);
-          k_locate<<<grid_for_n(W.n), 256, 0, e->stream>>>(r.views[0].keys.p, r.views[0].lay.key64, r.views[0].n,
-                                                             e->tmp_keys.p, W.n, S.prow[k][vi].as<u32>());
-          e->after_launch("view rows");
-        }
+        again = lean = true;
+      } catch (...) {
+        free_state(*e, S);
+        throw;
       }
-      if (n_out) {
-        k_f32_to_f64<<<grid_for_n(n_out), 256, 0, e->stream>>>(gdev, n_out, S.adj[out_rel].as<double>());
-        e->after_launch("adjoint seed");
-      }
-      // Only relations out_rel depends on carry adjoints: rules with another
-      // head contribute nothing and are not replayed.
-      std::vector<char> needed(nrel, 0);
-      needed[out_rel] = 1;
-      for (bool grew = true; grew;) {
-        grew = false;
-        for (auto& p : e->plans)
-          if (needed[p.ast.head.rel])
-            for (auto& a : p.ast.body)
-              if (!needed[a.rel]) needed[a.rel] = grew = true;
-      }
-      // facts first derived in iteration k (the recent set at the start of k + 1,
-      // unless k + 1 began a stratum: then iteration k, its stratum's last, found none)
-      auto new_in = [&](u32 k, u32 rel) -> u64 {
-        if (begins_stratum(e->stratum_begin, k + 1)) return 0;
-        return k < e->iter_counts.size() ? e->iter_counts[k][rel].second : e->rels[rel].n_recent;
-      };
-      // Linear components whose head is needed replay in one launch (linear.cu),
-      // down to iteration 2.  They feed no other component, and what they add to
-      // the inputs' adjoints is read at the end.
-      std::vector<char> linear(nrel, 0);
-      {
-        LinearAdjoints J;
-        for (size_t q = 0; q < nrel; q++) {
-          J.adj.push_back(S.adj[q].as<double>());
-          J.hrow.push_back(S.hrow[q].as<u32>());
-          J.prow.emplace_back();
-          for (auto& b : S.prow[q]) J.prow.back().push_back(b.as<u32>());
-        }
-        if (!linear_backward(*e, J, linear)) linear.assign(nrel, 0);
-      }
-      for (u32 k = e->last_iter; k >= 1; k--) {
-        for (size_t q = 0; q < nrel; q++) {  // the heads new in iteration k
-          if (!S.hnew[q].p || !needed[q] || (linear[q] && k > 1) || !new_in(k, (u32)q)) continue;
-          RelSt& r = e->rels[q];
-          e->check(cudaMemsetAsync(S.hnew[q].p, 0, S.hnew[q].cap, e->stream), "new heads");
-          k_mark_new<<<grid_for_n(r.views[0].n), 256, 0, e->stream>>>(r.views[0].keys.p, r.views[0].lay.key64,
-                                                                      r.views[0].stamps.as<u32>(), r.views[0].n, k,
-                                                                      S.hnew[q].as<u32>());
-          e->after_launch("new heads");
-          for (auto& p : e->plans)
-            for (auto& A : p.arms) {
-              if (p.ast.head.rel != q || !bwd_masked(*e, A)) continue;
-              bool made;
-              bwd_mask(*e, S.fresh[q], r, A.packed.mask_h, &made);
-            }
-          for (auto& m : S.fresh[q]) {
-            e->check(cudaMemsetAsync(m.bits.p, 0, mask_bytes(m.lay), e->stream), "new heads");
-            mask_set_new(r.views[0].lay, r.views[0].perm, m.lay, m.perm, r.views[0].keys.p, r.views[0].n,
-                         r.views[0].stamps.as<u32>(), k, S.adj[q].as<double>(), m.bits.as<u32>(), e->stream);
-            e->after_launch("new heads");
-          }
-        }
-        const int stratum = stratum_of_iter(e->stratum_begin, k);
-        for (auto& p : e->plans)
-          for (auto& A : p.arms) {
-            if (p.stratum != stratum) continue;  // the rule did not run in iteration k
-            if (!needed[p.ast.head.rel] || !new_in(k, p.ast.head.rel)) continue;  // no adjoint can flow here
-            if (linear[p.ast.head.rel] && k > 1) continue;
-            const auto& cnt = e->iter_counts[k - 1];  // (total, recent) per relation at the start of iteration k
-            if (!cnt[p.ast.body[A.delta].rel].second) continue;
-            bool skip = false;
-            for (u32 b : A.before_rels)
-              if (cnt[b].first == cnt[b].second) { skip = true; break; }
-            if (skip) continue;
-            if (!replay_arm_packed(*e, S, p, A, k)) replay_arm(*e, S, p, A, k);
-          }
-      }
-      for (size_t k = 0; k < nrel; k++) {
-        RelSt& r = e->rels[k];
-        if (!gin[k] || !r.n_in || !r.views[0].n) continue;
-        k_bwd_inputs<<<grid_for_n(r.n_in), 256, 0, e->stream>>>(r.views[0].keys.p, r.views[0].lay.key64, r.views[0].n,
-                                                                 r.row_keys.p, r.row_factor.as<float>(),
-                                                                 S.adj[k].as<double>(), r.n_in, gin[k]);
-        e->after_launch("input gradients");
-      }
-    } catch (...) {
       free_state(*e, S);
-      throw;
     }
-    free_state(*e, S);
   }
   if (mem == LOB_MEM_HOST) {
     for (size_t k = 0; k < nrel; k++)
@@ -903,7 +937,5 @@ int backward_impl(lob_engine* e, u32 out_rel, const float* grad_tags, float* con
                  "grad inputs out");
   }
   e->sync();
-  e->release(g);
-  e->release(gin_all);
   return LOB_OK;
 }

@@ -830,15 +830,22 @@ struct GraphHolder {
 // *taken when the loop cannot take this run (the host loop continues).
 int run_device_loop(lob_engine& e, u32& k, u32 max_iters, lob_stats& s, bool* taken) {
   *taken = false;
-  if (!loop_eligible(e) || k >= max_iters) return LOB_OK;
+  if (e.lean || !loop_eligible(e) || k >= max_iters) return LOB_OK;
   if (e.opt_driver == 1 && !e.loop_caps.count("history")) {
     // this run stays host-driven and records the sizes the loop will plan with
     e.loop_caps["history"] = 1;
     return LOB_OK;
   }
-  *taken = true;
+  *taken = e.extra = true;
   g_cap_floor = (u64)e.opt_loop_cap_floor;
   GLoop G;
+  struct Buffers {  // given back on every exit
+    lob_engine& e;
+    GLoop& G;
+    ~Buffers() {
+      for (DevBuf* b : {&G.times, &G.state, &G.rec, &G.tab, &G.res}) e.release(*b);
+    }
+  } buffers{e, G};
   plan_loop(e, G, max_iters);
   initial_caps(e, G);
   u32 rec_cap = std::min<u32>(max_iters, std::max<u32>(k + 256, 1024));
@@ -1051,11 +1058,6 @@ int run_device_loop(lob_engine& e, u32& k, u32 max_iters, lob_stats& s, bool* ta
       a.launches += s.device_iterations;
       a.ms += t[1 + i] / 1e6;
     }
-    e.release(G.times);
   }
-  e.release(G.state);
-  e.release(G.rec);
-  e.release(G.tab);
-  e.release(G.res);
   return rc;
 }

@@ -816,6 +816,8 @@ static void prepare(lob_engine& e, int sem) {
     for (u32 c = 0; c < r.arity; c++) bits += r.width[c];
     any_computed = any_computed && bits <= 64;
   }
+  any_computed = any_computed && !e.lean;
+  e.extra = e.extra || any_computed;
   for (int round = 0; any_computed && round < 3; round++) {
     for (size_t i = 0; i < e.rules.size(); i++)
       for (size_t c = 0; c < e.rules[i].head_prog.size(); c++)
@@ -862,7 +864,8 @@ static void prepare_arms(lob_engine& e) {
       A.packed.linear_only = A.packed.ok && sem_top1(sem);
       if (A.packed.linear_only) A.packed.ok = false;
       if (sem == SR_UNIT) compile_cross(e, p.ast, A, A.packed);
-      if (sem != SR_UNIT) compile_mask(e, p.ast, A, A.packed);
+      if (sem != SR_UNIT && !e.lean) compile_mask(e, p.ast, A, A.packed);
+      e.extra = e.extra || A.packed.mask_ok;
     }
 }
 
@@ -2142,7 +2145,7 @@ static void all_recent(lob_engine& e) {
   }
 }
 
-static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
+static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   if (e.state != 0) throw LobError(LOB_E_STATE, "run_to_fixpoint was already called; call lob_reset first");
   if (sem < 0 || sem > 6) throw LobError(LOB_E_ARG, "unknown semiring id");
   e.peak_bytes = e.live_bytes;
@@ -2267,6 +2270,19 @@ static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   e.ran_diff = sem == SR_DIFF_MAX_MIN || sem == SR_DIFF_ADD_MULT || sem == SR_DIFF_TOP1;
   if (st) *st = s;
   return rc;
+}
+
+// Memory that only makes a run faster must not make it fail: one that is refused
+// memory while it has such a use for it starts again, from the loaded facts, without.
+static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
+  e.lean = e.extra = false;
+  try {
+    return run_attempt(e, sem, max_iters, st);
+  } catch (const LobError& x) {
+    if (x.code != LOB_E_OOM || !e.extra) throw;
+  }
+  e.lean = true;
+  return run_attempt(e, sem, max_iters, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -283,6 +283,11 @@ struct lob_engine {
   int swidth = 0;
   u32 max_sample = 0;
   bool ran_diff = false;
+  // extra: the run holds, or plans to hold, memory that it could do without (masks,
+  // the linear loop's arrays, the device-driven loop's second buffers, accumulators
+  // over bounded computed columns).  lean: it
+  // was refused memory that way and runs again without them (run_fixpoint).
+  bool extra = false, lean = false;
   u32 last_iter = 0;
   lob_stats stats{};
   // scratch and transient buffers

@@ -854,7 +854,7 @@ bool linear_component(const lob_engine& e, std::vector<char>& in) {
 void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   const u32 k0 = 1;
   std::vector<char> in;
-  if (!e.opt_driver || k0 >= max_iters || !linear_component(e, in)) return;
+  if (!e.opt_driver || e.lean || k0 >= max_iters || !linear_component(e, in)) return;
   if (e.opt_driver == 1 && !e.loop_caps.count("linear_history")) {
     // as for the device-driven graph: the first run of an engine is host-driven
     e.loop_caps["linear_history"] = 1;
@@ -904,6 +904,7 @@ void run_linear(lob_engine& e, u32 max_iters, lob_stats& s, LinearOut& out) {
   const int ks = sem_kernel(e.semiring);
   const int sb = stored_bytes(e.semiring), cb = cand_bytes(e.semiring);
   const bool stamps = sem_stamps(e.semiring), top1 = sem_top1(e.semiring);
+  e.extra = true;
   e.ensure(L.arms, std::max<size_t>(arms.size(), 1) * sizeof(LinArm));
   if (!arms.empty())
     e.check(cudaMemcpyAsync(L.arms.p, arms.data(), arms.size() * sizeof(LinArm), cudaMemcpyHostToDevice, e.stream), "arms");
@@ -1040,7 +1041,7 @@ void linear_merge(lob_engine& e, u32 k, const LinearOut& out) {
   }
 }
 
-bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in) {
+bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in, bool& extra) {
   if (!e.opt_packed_backward || !linear_component(e, in)) return false;
   const u32 last = e.last_iter;
   LinRun L(e);
@@ -1095,6 +1096,7 @@ bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& 
       arms.push_back(a);
     }
   if (last < 2 || arms.empty() || !rows) return true;  // iterations after the first derived nothing
+  extra = true;
   e.ensure(L.arms, arms.size() * sizeof(LinBwdArm));
   e.check(cudaMemcpyAsync(L.arms.p, arms.data(), arms.size() * sizeof(LinBwdArm), cudaMemcpyHostToDevice, e.stream), "arms");
   // entries by stamp: counts (scanned in place), fill positions

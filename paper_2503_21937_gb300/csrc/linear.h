@@ -37,10 +37,11 @@ bool top1_settle(lob_engine& e);
 // diff-add-mult backward of the linear components' iterations after the first.
 // Device pointers by relation id: adjoints and dense key -> row maps (null: none),
 // and per view its rows' primary rows.  Flags the components' relations; false
-// when there is none to take (the caller replays every iteration).
+// when there is none to take (the caller replays every iteration).  extra is set
+// once memory is asked for.
 struct LinearAdjoints {
   std::vector<double*> adj;
   std::vector<u32*> hrow;
   std::vector<std::vector<u32*>> prow;
 };
-bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in);
+bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in, bool& extra);

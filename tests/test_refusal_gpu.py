@@ -85,3 +85,95 @@ def test_bit_matrices_with_a_request_refused(program, n, loaded):
         e.close()
         assert not A.live
     assert at > 12  # the run made at least that many requests
+
+
+HOPS = "hop(x,y,1) :- edge(x,y).\nhop(x,z,d + 1) :- hop(x,y,d), edge(y,z), d < 4.\n"
+
+
+def _tagged(kind):
+    s = W.stream(7600)
+    if kind == "kinship":  # masked last steps
+        n, r, a, b, p = W.kinship_instance(s)
+        return W.KIN_PROGRAM, {"fact": ((r, a, b), p), "comp": (W.composition_table(),)}, "kin", "fact"
+    if kind == "grid":  # a linear component
+        g = W.grid_reach_instance(9, sub=761)
+        return W.REACH_PROGRAM, {"edge": (g["edge"][:2], g["edge"][2]), "start": (g["start"],)}, "reach", "edge"
+    src, dst = W.erdos_renyi(40, 90, seed_index=762)  # a computed column of few bits
+    return HOPS, {"edge": ((src, dst), s.prob(90))}, "hop", "edge"
+
+
+@pytest.mark.parametrize("kind,semiring,options", [
+    ("kinship", "max_min", {"driver": 0}), ("kinship", "diff_add_mult", {"driver": 0}), ("kinship", "diff_max_min", {"driver": 2}),
+    ("grid", "max_min", {"driver": 2}), ("grid", "diff_add_mult", {"driver": 2}),
+    ("grid", "diff_top1_proofs", {"driver": 2, "proof_arena_words": 256}), ("hops", "max_min", {"driver": 0})])
+def test_tagged_runs_with_a_request_refused(kind, semiring, options):
+    """Every single request of a run refused in turn.  Once the run has a use for
+    memory that it could do without, the refusal costs it only that; before, it is an
+    LOB_E_OOM after which the engine runs again.  Tags are compared with those of a
+    run that lost nothing (add-mult: FP64 sums in another order, rounded once)."""
+    from paper_2503_21937_gb300 import LobsterError
+    program, inputs, rel, _ = _tagged(kind)
+    want, lost, kept, at = None, [], [], 0
+    while True:
+        A = Refusing()
+        e = loaded_engine(program, inputs, options, A)
+        A.arm(at)
+        try:
+            e.run(semiring)
+            if A.refused:
+                kept.append(at)
+        except LobsterError as x:
+            assert x.code == -5
+            lost.append(at)
+            A.armed = False
+            e.run(semiring)
+        refused, A.armed = A.refused, False
+        r = e.read(rel)
+        e.close()
+        assert not A.live
+        if want is None:  # the first run loses nothing
+            assert not refused
+            want = r
+        assert np.array_equal(r.cols, want.cols), at
+        np.testing.assert_allclose(r.tags, want.tags, rtol=3e-7 if "add" in semiring else 0, atol=0)
+        if at and not refused:
+            break
+        at += 1
+    assert len(kept) > 5 and (not lost or max(lost) < min(kept)), (lost, kept)
+    if kind != "grid":
+        assert not lost
+
+
+@pytest.mark.parametrize("kind", ["kinship", "grid"])
+def test_backward_with_a_request_refused(kind):
+    """Every single request of an add-mult backward pass refused in turn: the pass
+    ends without what it could do without, or with LOB_E_OOM and the gradients as
+    they were.  Gradients within the order of their FP64 sums, rounded to f32."""
+    from paper_2503_21937_gb300 import LobsterError
+    program, inputs, rel, grad = _tagged(kind)
+    A = Refusing()
+    e = loaded_engine(program, inputs, {"driver": 2}, A)
+    e.run("diff_add_mult")
+    seed = np.linspace(-1, 1, e.size(rel)).astype(np.float32)
+    want, lost, kept, at = None, [], [], 0
+    while True:
+        g = np.zeros(len(inputs[grad][1]), np.float32)
+        A.arm(at)
+        try:
+            e.backward(rel, seed, {grad: g})
+            if A.refused:
+                kept.append(at)
+        except LobsterError as x:
+            assert x.code == -5 and not g.any()
+            lost.append(at)
+            A.armed = False
+            e.backward(rel, seed, {grad: g})
+        refused, A.armed = A.refused, False
+        want = g if want is None else want
+        np.testing.assert_allclose(g, want, rtol=1e-6, atol=1e-6 * float(np.abs(want).max()))
+        if at and not refused:
+            break
+        at += 1
+    e.close()
+    assert not A.live
+    assert len(kept) > 2 and max(lost) < min(kept), (lost, kept)
