@@ -788,7 +788,7 @@ void add_mult_backward(lob_engine* e, BwdState& S, u32 out_rel, const float* gde
       J.prow.emplace_back();
       for (auto& b : S.prow[q]) J.prow.back().push_back(b.as<u32>());
     }
-    if (S.lean || !linear_backward(*e, J, linear, S.extra)) linear.assign(nrel, 0);
+    if (S.lean || !linear_backward(*e, J, needed, linear, S.extra)) linear.assign(nrel, 0);
   }
   for (u32 k = e->last_iter; k >= 1; k--) {
     for (size_t q = 0; q < nrel; q++) {  // the heads new in iteration k

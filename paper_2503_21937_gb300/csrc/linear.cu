@@ -1041,8 +1041,14 @@ void linear_merge(lob_engine& e, u32 k, const LinearOut& out) {
   }
 }
 
-bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in, bool& extra) {
+bool linear_backward(lob_engine& e, const LinearAdjoints& J, const std::vector<char>& needed, std::vector<char>& in,
+                     bool& extra) {
   if (!e.opt_packed_backward || !linear_component(e, in)) return false;
+  // a rule's head is needed only if its body is, so what is needed of a component
+  // takes its adjoints from needed heads alone
+  bool any = false;
+  for (size_t r = 0; r < in.size(); r++) any = (in[r] = in[r] && needed[r]) || any;
+  if (!any) return false;
   const u32 last = e.last_iter;
   LinRun L(e);
   L.index.assign(e.rels.size(), -1);

@@ -36,7 +36,8 @@ bool top1_settle(lob_engine& e);
 
 // diff-add-mult backward of the linear components' iterations after the first.
 // Device pointers by relation id: adjoints and dense key -> row maps (null: none),
-// and per view its rows' primary rows.  Flags the components' relations; false
+// and per view its rows' primary rows.  needed: relations that carry adjoints; a
+// component with none of them is left out.  Flags the components' relations; false
 // when there is none to take (the caller replays every iteration).  extra is set
 // once memory is asked for.
 struct LinearAdjoints {
@@ -44,4 +45,5 @@ struct LinearAdjoints {
   std::vector<u32*> hrow;
   std::vector<std::vector<u32*>> prow;
 };
-bool linear_backward(lob_engine& e, const LinearAdjoints& J, std::vector<char>& in, bool& extra);
+bool linear_backward(lob_engine& e, const LinearAdjoints& J, const std::vector<char>& needed, std::vector<char>& in,
+                     bool& extra);

@@ -142,3 +142,30 @@ def test_proof_cap_in_the_linear_loop(driver):
     assert ei.value.code == -9
     _, st, got = engine_run(W.REACH_PROGRAM, inputs, "top1_proofs", options={"driver": driver, "proof_cap": 8})
     assert got["reach"].tags.tolist() == [0.5 ** k for k in range(9)]
+
+
+def test_backward_replays_only_what_the_output_depends_on():
+    """Two components that share no rule: the backward pass of one leaves the other's
+    launch out, and gives the same gradients as in a program of its own."""
+    s = W.stream(805)
+    src, dst, p = s.below(60, 30), s.below(60, 30), (s.prob(60) * 0.3).astype(np.float32)
+    inputs = {"edge": ((src, dst), p), "start": ((src[:1],),)}
+    e, _, got = engine_run(TAILED, inputs, "diff_add_mult", options={"driver": 2}, read=["reach", "pair"])
+    e.set_option("profile", 1)
+
+    def backward(en, rel):
+        g = np.zeros(len(src), np.float32)
+        en.profile_reset()
+        en.backward(rel, np.linspace(-1, 1, en.size(rel)).astype(np.float32), {"edge": g})
+        return g, en.profile()
+
+    g, kernels = backward(e, "pair")
+    assert "linear_backward" not in kernels
+    assert "linear_backward" in backward(e, "reach")[1]
+    e.close()
+    pair = TAILED[len(W.REACH_PROGRAM):]
+    e, _, _ = engine_run(pair, {"edge": inputs["edge"]}, "diff_add_mult", options={"driver": 2}, read=[])
+    want = np.zeros(len(src), np.float32)
+    e.backward("pair", np.linspace(-1, 1, e.size("pair")).astype(np.float32), {"edge": want})
+    e.close()
+    np.testing.assert_allclose(g, want, rtol=1e-6, atol=1e-6 * float(np.abs(want).max()))
