@@ -610,8 +610,9 @@ bool replay_arm_packed(lob_engine& e, BwdState& S, const RulePlan& rp, const Arm
   u64 n_in = DV.n;
   int side = 0;
   // the delta atom: the recent set of iteration k, a run of the rows by stamp
-  // (every fact when k begins a stratum)
-  const bool by_run = !S.lean && !begins_stratum(e.stratum_begin, k) && n_in;
+  // (where every fact is recent -- an input relation, the start of a stratum -- the
+  // rows as they are)
+  const bool by_run = !S.lean && !begins_stratum(e.stratum_begin, k) && e.iter_counts[k - 1][R.body[A.delta].rel].second < n_in;
   if (by_run) {
     const ByStamp& T = by_stamp(e, S, R.body[A.delta].rel);
     in_words = T.words.as<char>() + (u64)T.off[k - 1] * (DV.lay.key64 ? 8 : 4);

@@ -146,7 +146,8 @@ def test_proof_cap_in_the_linear_loop(driver):
 
 def test_backward_replays_only_what_the_output_depends_on():
     """Two components that share no rule: the backward pass of one leaves the other's
-    launch out, and gives the same gradients as in a program of its own."""
+    launch out, and gives the same gradients as in a program of its own.  An arm over
+    an input relation, all of whose facts are recent, sorts nothing by stamp."""
     s = W.stream(805)
     src, dst, p = s.below(60, 30), s.below(60, 30), (s.prob(60) * 0.3).astype(np.float32)
     inputs = {"edge": ((src, dst), p), "start": ((src[:1],),)}
@@ -169,3 +170,8 @@ def test_backward_replays_only_what_the_output_depends_on():
     e.backward("pair", np.linspace(-1, 1, e.size("pair")).astype(np.float32), {"edge": want})
     e.close()
     np.testing.assert_allclose(g, want, rtol=1e-6, atol=1e-6 * float(np.abs(want).max()))
+    e, _, _ = engine_run("two(x,z) :- edge(x,y), edge(y,z).\n", {"edge": inputs["edge"]}, "diff_add_mult", read=[])
+    e.set_option("profile", 1)
+    g, kernels = backward(e, "two")
+    assert g.any() and "radix_sort" not in kernels, kernels
+    e.close()
