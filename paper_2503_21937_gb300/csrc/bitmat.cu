@@ -34,6 +34,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <numeric>
 
 #include "engine.h"
 #include "scan.cuh"
@@ -43,7 +44,7 @@ namespace {
 constexpr int kMaxChain = 4;       // body atoms of a chain rule
 constexpr int kMaxBitRels = 16;    // relations the state block holds sizes of
 constexpr u32 kHeavyRow = 512;     // compressed rows longer than this are gathered by a whole block
-constexpr u64 kMatrixBytes = 1ull << 30;  // largest bit matrix (92,000 values): beyond it sparse facts cost too much
+constexpr u64 kMatrixBytes = 1ull << 30;  // largest bit matrix (92,000 values)
 constexpr u64 kMaxValue = 1ull << 28;     // largest id the renumbering's presence bitmap covers
 
 // state block: done flag (1 fixpoint, 2 max_iters), iterations run, new facts
@@ -1149,6 +1150,71 @@ __global__ void __launch_bounds__(256) k_bit_read(const u32* __restrict__ bits, 
 }
 
 // ---------------------------------------------------------------------------
+// Does a run fill its matrices?  They cost n^2 / 8 bytes each to clear, scan and
+// read out whatever they hold, so on many values with few facts the general path,
+// whose cost goes with the facts, is the faster one.  For a program of one linear
+// recursive rule, head = L head R with L and R products of input relations, and base
+// rules of sum B, iteration k + 1 makes at most sum(L^k B R^k) derivations, in rows
+// where L^k 1 is not zero: both are counted for kWalkSteps iterations by vectors of n
+// floats -- (L^T)^k 1, R^k 1, L^k 1, each a pass over the facts.  Operations that
+// depend on each other follow in launches of their own, about 3 us each.
+// ---------------------------------------------------------------------------
+constexpr int kWalkSteps = 16, kWalkOps = 8;
+struct WalkOp {      // y[column] += x[row] (or the other way, back) over a link's facts;
+  KeyCols K;         // with sum: *sum += x[row] z[column]
+  int inv, back;
+  const float *x, *z;
+  float* y;
+  double* sum;
+};
+struct WalkOps {
+  WalkOp op[kWalkOps];
+  Codes code;
+};
+__global__ void __launch_bounds__(256) k_bit_walks(const __grid_constant__ WalkOps W) {
+  const WalkOp& P = W.op[blockIdx.y];
+  const u64 stride = (u64)gridDim.x * blockDim.x;
+  const u64 n = (P.K.n + 31) & ~31ull;  // whole warps
+  double sum = 0.0;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const bool in = i < P.K.n;
+    const u64 k = load_key(P.K.keys, P.K.key64, in ? i : P.K.n - 1);
+    const u32 r = W.code((u32)field_of(k, P.K.shift[P.inv], P.K.width[P.inv]));
+    const u32 c = W.code((u32)field_of(k, P.K.shift[P.inv ^ 1], P.K.width[P.inv ^ 1]));
+    float v = in ? P.x[P.back ? c : r] : 0.0f;
+    if (P.sum) {
+      const float z = P.z[c];
+      if (v != 0.0f && z != 0.0f) sum += (double)v * (double)z;  // (no infinity times 0)
+      continue;
+    }
+    const u32 to = P.back ? r : c;
+    int same;
+    __match_all_sync(0xFFFFFFFFu, to, &same);
+    if (same) {  // a hub's facts: one atomic a warp
+#pragma unroll
+      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+      if (threadIdx.x & 31) v = 0.0f;
+    }
+    if (v != 0.0f) atomicAdd(P.y + to, v);
+  }
+  if (!P.sum) return;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+  if ((threadIdx.x & 31) == 0 && sum != 0.0) atomicAdd(P.sum, sum);
+}
+
+struct WalkRows {
+  const float* x[kWalkSteps + 1];
+};
+__global__ void __launch_bounds__(256) k_bit_walk_rows(const __grid_constant__ WalkRows W, u32 n, double* out) {
+  const u32 stride = gridDim.x * blockDim.x;
+  u32 c = 0;
+  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) c += W.x[blockIdx.y][i] != 0.0f;
+  c = __reduce_add_sync(0xFFFFFFFFu, c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(out + blockIdx.y, (double)c);
+}
+
+// ---------------------------------------------------------------------------
 // planning
 // ---------------------------------------------------------------------------
 struct Link {
@@ -1331,6 +1397,7 @@ struct Run {
     B.rows = (u32)D;
     B.words = (u32)((D + 127) / 128 * 4);
     if ((u64)B.rows * B.words * 4 > kMatrixBytes) return false;
+    if (!fills()) return false;
     if (B.mapped) {
       const u64 nw = (1ull << width) / 32;
       e.ensure(B.dict, (u64)B.rows * 4);
@@ -1347,6 +1414,156 @@ struct Run {
       c.pref = B.pref.as<u32>();
     }
     return c;
+  }
+
+  // Up to kSureRows values (a matrix is as large as L2 then) the matrices are taken as
+  // they are; up to kSureRows2 when a rule joins derived relations (an index row is
+  // scanned once for every 128 words of the result).  Beyond, a program whose
+  // derivations can be counted (k_bit_walks) runs on matrices when they exceed a 256th
+  // of the pairs or still grow, or when the time estimated for them is the lower one;
+  // any other one starts on the general path, which gives up in favour of the matrices
+  // when an iteration is about to derive a 32nd of the pairs (bit_watch).
+  // Measured (GB300, whole passes in ms, general path / bit matrices).  Left-recursive
+  // closure: a random tree of 20,000 nodes 1.6 / 1.1, 35,000 1.9 / 2.2, 90,000 2.7 / 9.1;
+  // disjoint edges 0.42 / 0.49, 0.59 / 0.71, 0.38 / 2.4; 0.9 random edges a node 35,000 6.2
+  // / 2.6, 90,000 7.3 / 4.5; 60,000 of them on 50,000 nodes (2.5e8 facts) 72 / 11.
+  // Right-recursive: trees 35,000 1.9 / 1.1, 90,000 2.6 / 2.0; chains of 40 35,000 4.9 /
+  // 3.6, 50,000 5.0 / 5.9, 90,000 7.0 / 14.  Same generation: trees of 200 nodes 35,000 2.0
+  // / 1.9, 50,000 2.2 / 2.8, 90,000 3.0 / 6.5; one tree of 50,000 (9.1e8 facts) 29 / 9.7.
+  // p.p closure: trees 12,000 1.6 / 1.2, 20,000 1.7 / 2.1, 90,000 3.4 / 55; chains 10,000
+  // 2.1 / 2.1, 14,000 2.1 / 3.7, 90,000 4.2 / 275; 24,000 random edges on 20,000 nodes
+  // 641 / 22.  The general path with the walks before it takes 0.1 ms more than alone.
+  static constexpr u32 kSureRows = 32768, kSureRows2 = 12288;
+  bool fills() {
+    if (e.bit_force || B.rows <= (linear ? kSureRows : kSureRows2)) return true;
+    e.bit_watch = B.rows;
+    const Chain* rec = nullptr;
+    size_t bases = 0;
+    for (const Chain& C : chains) {
+      const bool derived = std::any_of(C.links.begin(), C.links.end(), [&](const Link& l) { return e.rels[l.rel].idb; });
+      if (C.head != chains[0].head || (derived && rec)) return false;
+      if (derived) rec = &C;
+      else bases++;
+    }
+    if (!linear || bases > 4) return false;
+    return many_walks(rec);
+  }
+  bool many_walks(const Chain* rec) {
+    const u32 head = chains[0].head;
+    const int steps = rec ? kWalkSteps : 0;
+    std::vector<std::vector<Link>> base;
+    for (const Chain& C : chains)
+      if (&C != rec) base.push_back(C.links);
+    if (e.rels[head].views[0].n) base.push_back({Link{head, 0, 0}});
+    std::vector<Link> left, right;
+    for (bool past = false; rec && left.size() + right.size() + 1 < rec->links.size();) {
+      const Link& l = rec->links[left.size() + right.size() + past];
+      if (l.rel == head) past = true;
+      else (past ? right : left).push_back(l);
+    }
+    size_t inner = 0;
+    for (auto& b : base) inner += b.size() - 1;
+    const std::vector<Link>& row_links = B.transposed ? right : left;  // of the matrices as stored
+    const u64 n = (B.rows + 31) & ~31u;
+    const u64 vectors = 1 + steps * (left.size() + right.size() + row_links.size()) + (steps + 1) * inner;
+    const u64 pad = 128;  // floats: the derivations and live rows of each step
+    e.ensure(e.scratch, (pad + vectors * n) * 4);
+    e.check(cudaMemsetAsync(e.scratch.p, 0, (pad + vectors * n) * 4, e.stream), "walks");
+    double* sums = e.scratch.as<double>();
+    float* next = e.scratch.as<float>() + pad;
+    struct Vec { const float* p; int at; };  // a vector, and the launch before which it is complete
+    std::vector<std::vector<WalkOp>> launches;
+    const auto put = [&](int at, WalkOp op) {
+      if ((int)launches.size() <= at) launches.resize(at + 1);
+      launches[at].push_back(op);
+    };
+    const auto apply = [&](const Link& l, Vec v, int back) {
+      WalkOp op{key_cols(e.rels[l.rel]), l.inv, back, v.p, nullptr, next, nullptr};
+      if (op.K.n) put(v.at, op);
+      next += n;
+      return Vec{op.y, v.at + 1};
+    };
+    const Vec ones{next, 0};
+    fill_f32(next, B.rows, 1.0f, e.stream);
+    next += n;
+    Vec a = ones, b = ones, live = ones;
+    WalkRows rows{};
+    std::vector<double> s(2 * (kWalkSteps + 1));
+    size_t done = 0;
+    int ran = 0, live_done = 0;
+    const double many = (double)B.rows * B.rows / 256.0;
+    for (int k = 0; k <= steps; k++) {
+      if (k) {
+        for (const Link& l : left) a = apply(l, a, 0);
+        for (size_t i = right.size(); i--;) b = apply(right[i], b, 1);
+        if (B.transposed)
+          for (const Link& l : right) live = apply(l, live, 0);
+        else
+          for (size_t i = left.size(); i--;) live = apply(left[i], live, 1);
+      }
+      rows.x[k] = live.p;
+      for (auto& links : base) {
+        Vec c = a;
+        for (size_t i = 0; i + 1 < links.size(); i++) c = apply(links[i], c, 0);
+        WalkOp op{key_cols(e.rels[links.back().rel]), links.back().inv, 0, c.p, b.p, nullptr, sums + k};
+        if (op.K.n) put(std::max(c.at, b.at), op);
+      }
+      if (k != 5 && k != steps) continue;
+      // the first few steps alone may show the end, or that there are many
+      for (; done < launches.size(); done++)
+        for (size_t q = 0; q < launches[done].size(); q += kWalkOps) {
+          WalkOps W{};
+          W.code = codes();
+          const unsigned m = (unsigned)std::min<size_t>(kWalkOps, launches[done].size() - q);
+          u64 most = 0;
+          for (unsigned i = 0; i < m; i++) {
+            W.op[i] = launches[done][q + i];
+            most = std::max(most, W.op[i].K.n);
+          }
+          ProfScope ps("bit_walks", 0, e.stream);
+          k_bit_walks<<<dim3(elem_grid(most), m), 256, 0, e.stream>>>(W);
+          launch_check("walks");
+        }
+      WalkRows fresh{};
+      std::copy(rows.x + live_done, rows.x + k + 1, fresh.x);
+      k_bit_walk_rows<<<dim3(elem_grid(n) / 4 + 1, k + 1 - live_done), 256, 0, e.stream>>>(fresh, (u32)n,
+                                                                                       sums + kWalkSteps + 1 + live_done);
+      launch_check("walks");
+      live_done = k + 1;
+      e.check(cudaMemcpyAsync(e.pinned, sums, s.size() * 8, cudaMemcpyDeviceToHost, e.stream), "walks");
+      e.sync();
+      std::memcpy(s.data(), e.pinned, s.size() * 8);
+      ran = k;
+      if (s[k] == 0.0 || !(std::accumulate(s.begin(), s.begin() + k + 1, 0.0) <= many)) break;
+      a.at = b.at = live.at = (int)done;  // what follows goes to launches of its own
+    }
+    // iterations, derivations and live rows to the end; past the last step as if their
+    // decline over the last four went on to zero, 64 steps at most
+    double its = 0, total = 0, touched = 0;
+    for (int k = 0; k <= ran; k++) {
+      its += k == 0 || s[k] > 0.0;
+      total += s[k];
+      touched += std::min(s[k], s[kWalkSteps + 1 + k]);
+    }
+    if (!(total <= many)) return true;
+    if (ran > 4 && s[ran] > 0.0) {
+      if (s[ran] > 1.1 * s[ran - 4]) return true;
+      const double fall = (s[ran - 4] - s[ran]) / 4;
+      const double tail = s[ran] < 64.0 * fall ? s[ran] / fall : 64.0;
+      its += tail;
+      total += s[ran] * tail / 2;
+      touched += std::min(s[ran], s[kWalkSteps + 1 + ran]) * tail / 2;
+    }
+    // Seconds.  Matrices: clearing, scanning, reading out (and turning back), launches,
+    // and each live row read and written by each product.  The general path: its
+    // launches and host waits, its derivations, and for keys of 32 bits a filter's
+    // clearing, which spares it a sort in every iteration.
+    const double row = B.words * 4.0 / 6.8e12;  // a row's time at the copy rate
+    const double products = rec ? rec->links.size() - 1.0 : 1.0;
+    const double on_bits = (B.transposed ? 13.0 : 7.5) * B.rows * row + (3.0 + products) * touched * row +
+                           its * (15e-6 + 18e-6 * products);
+    const double general = (B.rows > 65536 ? its * 160e-6 : 200e-6 + its * 120e-6) + total * 50e-12;
+    return on_bits < general;
   }
 
   // a link as the stored orientation reads it
@@ -1891,6 +2108,7 @@ struct Run {
 
 bool bit_run(lob_engine& e, u32 max_iters, u32& k, u64& new_facts, int* rc) {
   e.bit.reset(new BitRun());
+  e.bit_watch = 0;
   try {
     Run R(e);
     if (R.run(max_iters, k, new_facts, rc)) {
@@ -1904,6 +2122,21 @@ bool bit_run(lob_engine& e, u32 max_iters, u32& k, u64& new_facts, int* rc) {
   }
   bit_release(e);
   return false;
+}
+
+bool bit_blow_up(const lob_engine& e) {
+  const double n = (double)e.bit_watch;
+  double next = 0.0;
+  for (auto& p : e.plans)
+    for (auto& A : p.arms) {
+      const auto& body = p.ast.body;
+      if (!e.rels[body[A.delta].rel].idb) continue;
+      double d = (double)e.rels[body[A.delta].rel].n_recent;
+      for (size_t i = 0; i < body.size(); i++)
+        if ((int)i != A.delta) d *= (double)e.rels[body[i].rel].views[0].n / n;
+      next += d;
+    }
+  return next > n * n / 32.0;
 }
 
 void bit_release(lob_engine& e) {

@@ -2145,6 +2145,8 @@ static void all_recent(lob_engine& e) {
   }
 }
 
+struct ToBitMatrices {};  // thrown by a run that had better start again on them
+
 static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   if (e.state != 0) throw LobError(LOB_E_STATE, "run_to_fixpoint was already called; call lob_reset first");
   if (sem < 0 || sem > 6) throw LobError(LOB_E_ARG, "unknown semiring id");
@@ -2165,6 +2167,7 @@ static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   // a chain program under the unit semiring runs on bit matrices and needs
   // neither arms nor secondary views
   const bool bits = max_iters > 0 && bit_eligible(e);
+  e.bit_watch = 0;
   if (!bits) prepare_arms(e);
   load_facts(e);
   lob_stats s{};
@@ -2224,6 +2227,7 @@ static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
       e.stratum_begin.push_back(k + 1);
       continue;
     }
+    if (e.bit_watch && bit_blow_up(e)) throw ToBitMatrices();
     if (k == 1 && e.n_strata == 1) {
       run_linear(e, max_iters, s, lin);  // linear components, to their fixpoint
       bool rest = !lin.taken;
@@ -2274,15 +2278,19 @@ static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
 
 // Memory that only makes a run faster must not make it fail: one that is refused
 // memory while it has such a use for it starts again, from the loaded facts, without.
+// So does one whose facts turn out to be many after all (bit_blow_up).
 static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
-  e.lean = e.extra = false;
-  try {
-    return run_attempt(e, sem, max_iters, st);
-  } catch (const LobError& x) {
-    if (x.code != LOB_E_OOM || !e.extra) throw;
+  for (e.lean = e.bit_force = false;;) {
+    e.extra = false;
+    try {
+      return run_attempt(e, sem, max_iters, st);
+    } catch (const LobError& x) {
+      if (x.code != LOB_E_OOM || !e.extra || e.lean) throw;
+      e.lean = true;
+    } catch (const ToBitMatrices&) {
+      e.bit_force = true;
+    }
   }
-  e.lean = true;
-  return run_attempt(e, sem, max_iters, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -288,6 +288,10 @@ struct lob_engine {
   // over bounded computed columns).  lean: it
   // was refused memory that way and runs again without them (run_fixpoint).
   bool extra = false, lean = false;
+  // bit_watch: the values of a program that bit matrices were not taken for as its
+  // facts seemed few (else 0); bit_force: they were not, and it runs on them
+  u32 bit_watch = 0;
+  bool bit_force = false;
   u32 last_iter = 0;
   lob_stats stats{};
   // scratch and transient buffers

@@ -98,3 +98,56 @@ def test_points_to_and_iteration_limit():
         got.append(e.read("path").cols)
         e.close()
     assert np.array_equal(got[0], got[1])
+
+
+def _profiled(program, inputs, on):
+    e, st, _ = engine_run(program, inputs, options={"bit_matrix": on, "profile": 1}, read=[])
+    kernels = e.profile()
+    e.close()
+    return st, {k for k in kernels if k.startswith(("bit_gather", "bit_scatter"))}, \
+        {k for k in kernels if k.startswith(("join", "pwarp", "cross"))}
+
+
+def _forest(n, chain, seed):
+    """Trees (or chains) of 40 nodes over n nodes."""
+    i = np.arange(n, dtype=np.uint32)
+    k = i[i % 40 != 0]
+    up = np.ones(len(k), np.uint32) if chain else (k % 40) - W.stream(seed).below(len(k), k % 40)
+    return k - up, k
+
+
+@pytest.mark.parametrize("name,n,chain", [("left", 60000, True), ("left", 80001, False), ("right", 70001, True),
+                                          ("nonlinear", 12640, True), ("same_generation", 80001, False),
+                                          ("two_rules", 33840, False), ("loops", 60000, False)])
+def test_sparse_programs_keep_the_general_path(name, n, chain):
+    """Few facts over many values: no product of matrices is formed, and the relations
+    and statistics are those of bit_matrix = 0."""
+    inputs = {"edge": (_forest(n, chain, 7600),)}
+    assert not _profiled(PROGRAMS[name], inputs, 1)[1]
+    same_as_general(PROGRAMS[name], inputs)
+
+
+@pytest.mark.parametrize("name,n,m", [("left", 45000, 54000), ("right", 60000, 70000), ("same_generation", 50001, 0),
+                                      ("left", 70000, 60000)])
+def test_programs_run_on_matrices_from_the_start(name, n, m):
+    """Many facts over many values, or few in few rows and many iterations, as the
+    count of walks tells: matrices only."""
+    edges = W.erdos_renyi(n, m, seed_index=7601) if m else W.random_tree(n, seed_index=7602)[:2]
+    st, bits, joins = _profiled(PROGRAMS[name], {"edge": (edges,)}, 1)
+    assert bits and not joins
+    want, none, _ = _profiled(PROGRAMS[name], {"edge": (edges,)}, 0)
+    assert not none and all(st[k] == want[k] for k in ("iterations", "derived", "candidates", "new_facts"))
+
+
+@pytest.mark.parametrize("name,n", [("nonlinear", 14000), ("mutual", 40000)])
+def test_programs_that_turn_out_dense_start_again_on_matrices(name, n):
+    """Programs whose walks are not counted: general until they are about to derive a
+    32nd of the pairs.  The closure's pairs are those of the left-recursive rule."""
+    inputs = {"edge": (W.erdos_renyi(n, int(1.3 * n), seed_index=7603),)}
+    st, bits, joins = _profiled(PROGRAMS[name], inputs, 1)
+    assert bits and joins
+    if name == "nonlinear":
+        assert st["derived"] == _profiled(PROGRAMS["left"], inputs, 1)[0]["derived"]
+    else:
+        want = _profiled(PROGRAMS[name], inputs, 0)[0]
+        assert all(st[k] == want[k] for k in ("iterations", "derived", "candidates", "new_facts"))
