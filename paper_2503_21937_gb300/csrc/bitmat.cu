@@ -45,6 +45,7 @@ constexpr int kMaxChain = 4;       // body atoms of a chain rule
 constexpr int kMaxBitRels = 16;    // relations the state block holds sizes of
 constexpr u32 kHeavyRow = 512;     // compressed rows longer than this are gathered by a whole block
 constexpr u64 kMatrixBytes = 1ull << 30;  // largest bit matrix (92,000 values)
+constexpr u64 kRunBytes = 8ull << 30;     // all matrices of a run: two to six a derived relation, two temporaries
 constexpr u64 kMaxValue = 1ull << 28;     // largest id the renumbering's presence bitmap covers
 
 // state block: done flag (1 fixpoint, 2 max_iters), iterations run, new facts
@@ -1397,7 +1398,12 @@ struct Run {
     B.rows = (u32)D;
     B.words = (u32)((D + 127) / 128 * 4);
     if ((u64)B.rows * B.words * 4 > kMatrixBytes) return false;
-    if (!fills()) return false;
+    // A matrix per derived relation for F, D and D', one for N where an iteration has
+    // several products, transposed copies where it is read both ways; the temporaries.
+    u64 matrices = n_temp;
+    for (size_t r = 0; r < e.rels.size(); r++)
+      if (e.rels[r].idb) matrices += 3 + accumulates[r] + (B.rel[r].need_t ? (linear ? 1 : 2) : 0);
+    if (matrices * mat_bytes() > kRunBytes || !fills()) return false;
     if (B.mapped) {
       const u64 nw = (1ull << width) / 32;
       e.ensure(B.dict, (u64)B.rows * 4);
