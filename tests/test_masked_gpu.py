@@ -87,3 +87,31 @@ def test_rows_grouped_by_head(rows, semiring):
     for k in ("iterations", "derived", "candidates", "new_facts"):
         assert x[k] == y[k], (k, x[k], y[k])
     assert np.array_equal(p.cols, q.cols) and np.array_equal(p.tags, q.tags)
+
+
+@pytest.mark.parametrize("semiring", ["max_min", "diff_max_min"])
+@pytest.mark.parametrize("rows", [1, 33, 255, 257, 152 * 256 + 1, 152 * 4096 - 1, 152 * 4096 + 41])
+def test_rows_of_a_derived_relation_grouped_by_head(rows, semiring):
+    """The masked step with exactly `rows` input rows: the delta atom is derived, so
+    that the step of iteration 2 is a masked one (a rule over input relations alone,
+    as in the test before, never is), and the loop in one launch is off.  Rows just
+    past the smallest tiles, one wave of full tiles and two waves; heads of 64 rows
+    (two items) and of one."""
+    s = W.stream(961)
+    i = np.arange(rows, dtype=np.uint32)
+    a = (i // 64, i % 64)
+    if rows > 64:
+        a[0][-3:], a[1][-3:] = rows + np.arange(3), 5  # heads of a single row
+    b = (s.below(700, 64), s.below(700, 50))
+    inputs = {"a": (a, s.prob(rows)), "b": (b, s.prob(700))}
+    text = "p(x,y) :- a(x,y).\nq(x,z) :- p(x,y), b(y,z), y != z.\n"
+    got = []
+    for opts in ({"packed_join": 0, "driver": 0}, {"driver": 0, "profile": 1}):
+        e, st, g = engine_run(text, inputs, semiring, options=opts, read=["q"])
+        got.append((st, g["q"], e.profile()))
+        e.close()
+    (x, p, _), (y, q, kernels) = got
+    assert kernels["join_masked"]["launches"] == 1
+    for k in ("iterations", "derived", "candidates", "new_facts"):
+        assert x[k] == y[k], (k, x[k], y[k])
+    assert np.array_equal(p.cols, q.cols) and np.array_equal(p.tags, q.tags)
