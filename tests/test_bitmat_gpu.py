@@ -163,3 +163,46 @@ def test_matrices_are_bounded_in_all():
     assert st["peak_bytes"] < 4 << 30
     assert e.size("r0") == len(i)
     e.close()
+
+
+POINTS_TO = ("pt(p,q) :- addr(p,q).\npt(p,q) :- assign(p,r), pt(r,q).\npt(p,q) :- load(p,r), pt(r,s), pt(s,q).\n"
+             "pt(r,q) :- store(p,s), pt(p,r), pt(s,q).\n")
+
+
+@pytest.mark.parametrize("n", [4200, 5000, 12200])
+@pytest.mark.parametrize("name", ["nonlinear", "four_atoms", "loops", "points_to"])
+def test_products_of_derived_relations_over_many_values(name, n):
+    """Rules that join derived relations over more than 4,096 values (several chunks of
+    a row) and over listed matrices (12,200): index rows in bits over temporaries,
+    transposed full sets, skipped arms, rows that no later product reads."""
+    s = W.stream(7700 + n)
+    if name == "points_to":
+        stmt = lambda m: (s.below(m, n), s.below(m, n))
+        inputs = {"addr": ((s.below(n, n), s.below(n, n)),), "assign": (stmt(n // 3),), "load": (stmt(n // 20),),
+                  "store": (stmt(n // 20),)}
+        program = POINTS_TO
+    else:
+        parent, child, _ = W.random_tree(n, seed_index=7701)
+        hub, leaf = np.full(560, 5, np.uint32), s.below(560, n)
+        inputs = {"edge": ((np.concatenate([parent, hub]), np.concatenate([child, leaf])),)}
+        program = PROGRAMS[name]
+    e, _, _ = engine_run(program, inputs, options={"profile": 1}, read=[])
+    assert "bit_gather" in e.profile()
+    e.close()
+    if name != "four_atoms":
+        same_as_general(program, inputs)
+        return
+    # (on 12,200 values the general path would need 393 GB for the bindings of a step)
+    import torch
+    edge = torch.zeros((n, n), device="cuda")
+    edge[tuple(torch.from_numpy(c.astype(np.int64)).cuda() for c in inputs["edge"][0])] = 1.0
+    path, size = edge, -1
+    while int(path.sum(dtype=torch.float64)) != size:
+        size = int(path.sum(dtype=torch.float64))
+        step = edge
+        for m in (path.T, edge, path):
+            step = ((step @ m) > 0).float()
+        path = torch.maximum(path, step)
+    e, st, got = engine_run(program, inputs, read=["path"])
+    e.close()
+    assert np.array_equal(got["path"].cols.astype(np.int64), torch.nonzero(path).T.cpu().numpy())
