@@ -2278,15 +2278,18 @@ static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
 
 // Memory that only makes a run faster must not make it fail: one that is refused
 // memory while it has such a use for it starts again, from the loaded facts, without.
-// So does one whose facts turn out to be many after all (bit_blow_up).
+// So does one whose facts turn out to be many after all (bit_blow_up), or a join of
+// which is too large for the general path (a hub's), on the bit matrices it left out.
 static int run_fixpoint(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
+  e.bit_watch = 0;
   for (e.lean = e.bit_force = false;;) {
     e.extra = false;
     try {
       return run_attempt(e, sem, max_iters, st);
     } catch (const LobError& x) {
-      if (x.code != LOB_E_OOM || !e.extra || e.lean) throw;
-      e.lean = true;
+      if (e.bit_watch && (x.code == LOB_E_OOM || x.code == LOB_E_ARG)) e.bit_force = true;
+      else if (x.code == LOB_E_OOM && e.extra && !e.lean) e.lean = true;
+      else throw;
     } catch (const ToBitMatrices&) {
       e.bit_force = true;
     }
