@@ -48,9 +48,9 @@ def load_peaks():
 
 
 def kernel_source_hash(unit: str = "pjoin.cu"):
-    """Hash of the translation unit that holds the join emission kernels and
-    of every local header it includes (recursively): the sources the ncu
-    counters in profiles/ were taken on."""
+    """Hash of the translation unit that holds a kernel class (the join emission
+    kernels, bitmat.cu's products) and of every local header it includes
+    (recursively): the sources the ncu counters in profiles/ were taken on."""
     import re
     d = os.path.join(ROOT, "paper_2503_21937_gb300", "csrc")
     seen, todo = set(), [unit]
@@ -68,23 +68,24 @@ def kernel_source_hash(unit: str = "pjoin.cu"):
     return h.hexdigest()[:16]
 
 
-def ncu_traffic(kernel: str, outputs_per_launch: float):
+def ncu_traffic(kernel: str, outputs_per_launch: float, bytes_per_launch: float):
     """DRAM bytes per launch of `kernel` at the benchmark's size, from the
-    committed ncu summary: DRAM bytes per join output measured on the small
-    profile cases (one kernel, a few launches), times this workload's join
-    outputs per launch.  None when the summary was taken on other kernel sources."""
+    committed ncu summary: DRAM bytes per join output (the emission kernels) or
+    per algorithmic byte (the bit-matrix products) measured on the small profile
+    cases, times this workload's join outputs or algorithmic bytes per launch.
+    None when the summary was taken on other kernel sources."""
     path = os.path.join(ROOT, "profiles", "ncu_traffic.json")
     try:
         with open(path) as f:
             t = json.load(f)
     except Exception:
         return None
-    if t.get("source_hash") != kernel_source_hash():
-        return None
     k = t.get("kernels", {}).get(kernel)
-    if k is None or not outputs_per_launch:
+    if k is None or k["source_hash"] != kernel_source_hash(k["unit"]):
         return None
-    return k["dram_bytes_per_output"] * outputs_per_launch
+    if "dram_bytes_per_algorithmic_byte" in k:
+        return k["dram_bytes_per_algorithmic_byte"] * bytes_per_launch
+    return k["dram_bytes_per_output"] * outputs_per_launch if outputs_per_launch else None
 
 
 # ---------------------------------------------------------------------------
@@ -501,6 +502,8 @@ def profile_case(name, options=()):
         e.program(W.SG_PROGRAM)
         e.load("parent", torch.from_numpy(np.stack([parent, child]).astype(np.int32)).cuda())
         print(json.dumps({"case": name, **e.run("unit")}))
+    if ("profile", 1) in options:  # launches, ms and algorithmic bytes per kernel class
+        print(json.dumps(e.profile()))
     e.close()
 
 
@@ -629,7 +632,7 @@ def main():
         per_launch_s = v["ms"] / v["launches"] / 1e3
         ach = per_launch_bytes / per_launch_s / 1e9
         outs = sum(cands.values()) / max(v["launches"], 1) if name == "join_emit" else 0
-        traffic = ncu_traffic(name, outs)
+        traffic = ncu_traffic(name, outs, per_launch_bytes)
         roofline = {"kernel": name, "bound": "hbm", "achieved": round(ach, 1), "peak": peak, "unit": "GB/s",
                     "frac": round(ach / peak, 4), "peak_source": peak_kind,
                     "algorithmic_bytes_per_launch": per_launch_bytes, "traffic": traffic,

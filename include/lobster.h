@@ -183,7 +183,9 @@ typedef struct lob_tune_report {
  *     bitmap_delta (bitmap read-out vs sorted candidates), emit_filter
  *     (membership filter) and cross_join (fused cross-product step).
  * Tile sizes (emission, merge, unique, sort) are compile-time constants of the
- * kernels and are not searched.
+ * kernels and are not searched.  Neither is bit_matrix: a program that runs on
+ * bit matrices does so at the default options only, so the search compares it
+ * with the general path's settings.
  * Each setting runs `repeats` times (0 = 1) and scores its median run time; a
  * change must win by 2 %.  All settings compute the same relations, so only
  * time decides.  The engine must be loaded and not yet run (LOB_E_STATE
@@ -317,7 +319,9 @@ int lob_reset(lob_engine* e);
  *                  sample ids), provided that packed_join, warp_join,
  *                  bitmap_delta, emit_filter, cross_join, join_index,
  *                  sort_algo and max_candidates (2^30 or more) are at their
- *                  defaults, which ask for no other strategy; 0: never.  The
+ *                  defaults, which ask for no other strategy, and, beyond
+ *                  32,768 values (12,288 when a rule joins derived relations),
+ *                  that the facts are many enough for it; 0: never.  The
  *                  relations and the statistics of the iterations are the
  *                  same either way                                  (default 1)
  *   "packed_backward" 1: the diff-add-mult backward pass replays packed join
