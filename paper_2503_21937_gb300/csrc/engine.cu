@@ -2150,13 +2150,16 @@ struct ToBitMatrices {};  // thrown by a run that had better start again on them
 static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
   if (e.state != 0) throw LobError(LOB_E_STATE, "run_to_fixpoint was already called; call lob_reset first");
   if (sem < 0 || sem > 6) throw LobError(LOB_E_ARG, "unknown semiring id");
-  e.peak_bytes = e.live_bytes;
-  e.launches = 0;
-  const u64 syncs0 = e.host_syncs;
+  const bool again = e.lean || e.bit_force;  // time, launches, waits and memory are the run's, not the attempt's
+  if (!again) {
+    e.peak_bytes = e.live_bytes;
+    e.launches = 0;
+    e.run_syncs = e.host_syncs;
+  }
   if (!e.run_begin) e.check(cudaEventCreate(&e.run_begin), "event");
   if (!e.run_end) e.check(cudaEventCreate(&e.run_end), "event");
   cudaEvent_t ev0 = e.run_begin, ev1 = e.run_end;
-  e.check(cudaEventRecord(ev0, e.stream), "event");
+  if (!again) e.check(cudaEventRecord(ev0, e.stream), "event");
   e.iter_counts.clear();
   e.cand_emitted = 0;
   e.stratum_begin.clear();
@@ -2265,7 +2268,7 @@ static int run_attempt(lob_engine& e, int sem, u32 max_iters, lob_stats* st) {
     if (r.idb) s.derived += r.views[0].n;
   s.peak_bytes = e.peak_bytes;
   s.kernel_launches = e.launches;
-  s.host_syncs = e.host_syncs - syncs0;
+  s.host_syncs = e.host_syncs - e.run_syncs;
   s.proof_words = e.arena_tail;
   s.strata = (u32)e.n_strata;
   e.stats = s;

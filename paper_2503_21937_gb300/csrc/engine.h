@@ -292,6 +292,7 @@ struct lob_engine {
   // facts seemed few (else 0); bit_force: they were not, and it runs on them
   u32 bit_watch = 0;
   bool bit_force = false;
+  u64 run_syncs = 0;  // host_syncs when the run began
   u32 last_iter = 0;
   lob_stats stats{};
   // scratch and transient buffers

@@ -104,6 +104,8 @@ def _profiled(program, inputs, on):
     e, st, _ = engine_run(program, inputs, options={"bit_matrix": on, "profile": 1}, read=[])
     kernels = e.profile()
     e.close()
+    assert sum(k["ms"] for k in kernels.values()) <= st["ms"]  # a second start counts
+    assert sum(k["launches"] for k in kernels.values()) <= st["kernel_launches"]
     return st, {k for k in kernels if k.startswith(("bit_gather", "bit_scatter"))}, \
         {k for k in kernels if k.startswith(("join", "pwarp", "cross"))}
 
